@@ -83,21 +83,22 @@ wpsgd_status wpsgd_destroy(wpsgd_ctx* ctx);
  *   "dense_variant"   kernel for dense rows. 0 (default): chosen from the shape. 1: any shape and alignment, model in
  *                     global memory. 2: one CTA per node, one step per round trip, model in registers. 3: the same with
  *                     one warp per node. 4: blocked form (8 samples per synchronisation), one CTA per node. 5: blocked
- *                     form, one warp per node (rows of at most 64 16-byte chunks). 8: blocked form for bf16 rows, Gram
- *                     block and margins from mma.sync tensor-core instructions, columns of a node split over a
- *                     thread-block cluster (what 0 picks for aligned bf16 rows of 2048 columns and more). 9: blocked
- *                     form (16 samples) for fp32 rows with a node's columns split over a cluster, at most 256 columns
- *                     per CTA (what 0 picks for rows of 512 columns and more when the nodes are few enough for clusters
- *                     of 4 or 8 on the GPU's SMs). The blocked forms (4, 5, 8, 9) take both step-size schedules and
- *                     need eta0 * lambda <= 0.25.
+ *                     form, one warp per node (rows of at most 64 16-byte chunks). 8: blocked form for aligned bf16 rows
+ *                     with tensor-core Gram blocks, columns of a node split over a thread-block cluster ("block_samples"
+ *                     0: 16 samples per block with margins on the tensor cores as well, or variant 10 where that is
+ *                     estimated to be faster). 9: variant 10 for aligned fp32 rows with at most 256 columns per CTA.
+ *                     10: blocked form whose margins are taken from the model one block back, any alignment, a cluster
+ *                     of 1, 2, 4 or 8 CTAs per node (what 0 picks for most runs of up to 148 nodes). 0 compares estimates
+ *                     of the whole run. The blocked forms (4, 5, 8, 9, 10) take both step-size schedules and need
+ *                     eta0 * lambda <= 0.25.
  *   "sparse_variant"  kernel for CSR rows. 0 (default) and 2: blocks of up to 64 steps run in a shared-memory cache of
  *                     the model entries they touch. 1: one step per round trip to the model in global memory.
- *   "cluster"         CTAs per node of variants 8 and 9: 0 (default) chosen from d (and the node count), else 1, 2, 4 or 8.
+ *   "cluster"         CTAs per node of variants 8, 9 and 10: 0 (default) chosen from d (and the node count), else 1, 2, 4 or 8.
  *   "block_samples"   samples per block of variant 8: 0 (default) 16 when the rows fit, else 8; 8 or 16 to force one.
  *   "threads"         threads per node of variants 2 and 4, warps x 32 per CTA of variant 5; 0 (default): chosen from d.
  *   "prefetch"        rows in flight per chain of variants 2, 3 and of sparse variant 1; 0 (default): chosen.
  *   "stages"          blocks of rows in the shared-memory ring of the blocked kernels; 0 (default): as many as fit
- *                     (up to 4), else 2..8.
+ *                     (up to 4; variant 10: up to 8), else 2..8 (variant 10 takes at least 3).
  *   "host_pipeline"   wpsgd_solve_host: 1 (default) copies the shards in up to four groups of nodes, longest chains
  *                     first, on a stream of the context and starts the chains of a group when its rows have arrived;
  *                     0 copies everything first.

@@ -49,19 +49,19 @@ constexpr int M16_WARPS = 8;           // math warps of a CTA
 
 struct Mma16Smem {
   size_t row_stride, ring, w3, red, part, tot, gam, tab, jet, bars, pbar, flag, total;
-  __host__ __device__ Mma16Smem(int stages, size_t slice_bytes, int nbuf) {
+  __host__ __device__ Mma16Smem(int stages, size_t slice_bytes) {
     row_stride = slice_bytes + 16;
     ring = 0;
     w3 = ring + (size_t)stages * M16_B * row_stride;                 // w_hi, w_mid, w_lo, one zero row
-    red = w3 + 4 * row_stride;                                       // [nbuf][slots][256] partial sums
-    part = red + (size_t)nbuf * M16_SLOTS * M16_SLOT_FLOATS * sizeof(float);  // [math warps][256] this CTA's partial sums
+    red = w3 + 4 * row_stride;                                       // [2][slots][256] partial sums
+    part = red + 2 * (size_t)M16_SLOTS * M16_SLOT_FLOATS * sizeof(float);  // [math warps][256] this CTA's partial sums
     tot = part + (size_t)M16_WARPS * M16_SLOT_FLOATS * sizeof(float);      // [256] sums over the slots
     gam = tot + M16_SLOT_FLOATS * sizeof(float);                     // gamma_0..15, 1 - a^nv, stop
     tab = gam + 32 * sizeof(float);                                  // [3][32]
     jet = tab + 3 * 32 * sizeof(float);                              // 8 x (s, s', s''/2, s'''/6) of the logistic factor
     bars = jet + 8 * 4 * sizeof(float);                             // ring barriers [8]
-    pbar = bars + 8 * sizeof(unsigned long long);                    // partial-sum barriers [nbuf <= 4]
-    flag = pbar + 4 * sizeof(unsigned long long);
+    pbar = bars + 8 * sizeof(unsigned long long);                    // partial-sum barriers [2]
+    flag = pbar + 2 * sizeof(unsigned long long);
     total = flag + 16;
   }
 };
@@ -78,14 +78,9 @@ __device__ __forceinline__ void ldmatrix_x2(uint32_t (&r)[2], const void* smem_p
   asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(a) : "memory");
 }
 
-// XT = __nv_bfloat16: the tensor-core form described above. XT = float: the same blocks, cluster exchange and recurrence
-// for fp32 rows with the Gram block and the margins on the fp32 pipes (see the math warps' second part below); there
-// the Gram part of block b + 1 is formed while the recurrence warp works on block b, so the sums exist three times.
-template <int LOSS, typename XT>
+template <int LOSS>
 __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const ClusterParams cp) {
   constexpr int B = M16_B;
-  constexpr bool F32 = sizeof(XT) == 4;
-  constexpr int NBUF = F32 ? 3 : 2;
   extern __shared__ __align__(16) unsigned char smem[];
   const BlockParams& bp = cp.b;
   const ChainParams& p = bp.c;
@@ -96,13 +91,13 @@ __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const Clust
   const int j = p.order[blockIdx.x / C];
   const long long n_run = p.n_steps[j];
   const long long d = p.d;
-  const long long chunks = d / (16 / (long long)sizeof(XT));  // 16-byte chunks of a row
+  const long long chunks = d / 8;  // 16-byte chunks of a row
   const long long chunk0 = (long long)rank * cp.chunks_per_cta;
   const long long chunk_end = chunk0 + cp.chunks_per_cta < chunks ? chunk0 + cp.chunks_per_cta : chunks;
   const int my_chunks = (int)(chunk_end > chunk0 ? chunk_end - chunk0 : 0);
   const size_t slice_bytes = (size_t)cp.chunks_per_cta * 16;
-  const size_t ld_bytes = (size_t)p.ld * sizeof(XT);
-  const Mma16Smem L(S, slice_bytes, NBUF);
+  const size_t ld_bytes = (size_t)p.ld * 2;
+  const Mma16Smem L(S, slice_bytes);
   const size_t row_stride = L.row_stride;
   unsigned char* ring = smem + L.ring;
   unsigned char* w3 = smem + L.w3;
@@ -133,7 +128,8 @@ __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const Clust
   }
   if (threadIdx.x == 32) {
     for (int s = 0; s < S; ++s) mbar_init(&bars[s], 1);
-    for (int i = 0; i < NBUF; ++i) mbar_init(&pbar[i], 1);
+    mbar_init(&pbar[0], 1);
+    mbar_init(&pbar[1], 1);
     *give_up = 0;
     mbar_fence_init();
   }
@@ -160,7 +156,7 @@ __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const Clust
 
     for (long long b = 0; b < nb; ++b) {
       const int nv = (int)((n_run - b * B) < (long long)B ? (n_run - b * B) : (long long)B);
-      const int q = (int)(b % NBUF);
+      const int q = (int)(b & 1);
       if (lane == 0) mbar_arrive_expect_tx(&pbar[q], expect_bytes);
       const float y_cur = y_nxt;  // lane l: label of sample l & 15
       if (b + 1 < nb) y_nxt = yshard[id_nxt];
@@ -176,7 +172,7 @@ __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const Clust
       }
       // ---- wait (bounded) for the partial sums of block b from every math warp of the cluster ------------------
       {
-        const uint32_t parity = (uint32_t)((b / NBUF) & 1);
+        const uint32_t parity = (uint32_t)((b >> 1) & 1);
         bool landed = false;
         for (long long i = 0; i < bp.spin_limit; ++i) {
           if (mbar_try_wait_cluster(&pbar[q], parity)) { landed = true; break; }
@@ -352,19 +348,13 @@ __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const Clust
     long long b = 0;
     bool stop = false;
     for (; b < nb; ++b) {
-      if (F32) {  // fp32 rows: the update of block b reads its stage, after gamma_b
-        __syncthreads();
-        if (gam[B + 1] != 0.0f) { stop = true; break; }
-      }
       asm volatile("bar.sync 2, %0;" ::"r"(consumed_threads) : "memory");  // the stage of block b has been read
       request(requested, st);
       ++requested;
       peek(requested);
       st = (st + 1 == S) ? 0 : st + 1;
-      if (!F32) {
-        __syncthreads();
-        if (gam[B + 1] != 0.0f) { stop = true; ++b; break; }
-      }
+      __syncthreads();
+      if (gam[B + 1] != 0.0f) { stop = true; ++b; break; }
     }
     if (stop && copy_bytes > 0) {
       // leave no copy in flight into this CTA's shared memory: wait (bounded) on the stage of every block that was
@@ -378,151 +368,6 @@ __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const Clust
   }
 
   // ============================= math warps ==============================================================
-  if constexpr (F32) {
-    // ---- fp32 rows: Gram block and margins on the fp32 pipes ------------------------------------------------------
-    // The CTA's slice is narrow here (at most 64 chunks of 4 columns: the planner spreads a chain over as many CTAs as
-    // there are idle SMs), and the math threads share it as a 16 x 16 grid: thread (i, g) holds row i's chunks g,
-    // g + 16, .. in registers and forms row i of the Gram block over those columns against the 16 staged rows (whose
-    // chunks every thread of the same g reads at the same address). Lanes l and l ^ 16 hold the same row; their sums
-    // meet with a shuffle, lanes 0..15 fill the warp's table, and the two-level sum of the tensor-core form takes over.
-    // The Gram part does not depend on the model and is formed (and sent) one block ahead, while the recurrence warp
-    // works; between two model updates lie the update itself (one column per thread, model in shared memory), the
-    // margins from the row registers and their way through the cluster.
-    // (Measured on k = 16, d = 1024, eight CTAs per chain: 2.15 ms against 2.67 ms for the 8-sample kernel with one CTA
-    // per chain. The Gram block as 4 x 4 tiles over 16 column slices with a transposing sum, and the margins by 64
-    // threads with one 4-byte store each, halve the shared-memory loads and measured 2.49 ms.)
-    constexpr int NQ = 4;  // chunks per thread at most (checked on the host: chunks per CTA <= NQ * 16)
-    const int mt = (int)threadIdx.x - 64;
-    const int i16 = mt & 15, g = mt >> 4, G16 = math_threads >> 4;
-    const int ncols = my_chunks * 4;
-    float* wsm = (float*)w3;  // this CTA's slice of the model
-    {
-      const long long c0 = chunk0 * 4;
-      const float* src = p.resume ? (p.W + (size_t)j * d + c0) : (p.w0 ? p.w0 + c0 : nullptr);
-      for (int c = mt; c < ncols; c += math_threads) wsm[c] = src ? src[c] : 0.0f;
-    }
-    const uint32_t own_base = (uint32_t)__cvta_generic_to_shared(smem);
-    uint32_t peer_base[8];
-#pragma unroll
-    for (int rr = 0; rr < 8; ++rr) peer_base[rr] = map_shared_rank(smem, (uint32_t)rr < C ? (uint32_t)rr : rank);
-    asm volatile("bar.sync 4, %0;" ::"r"(math_threads) : "memory");  // the model slice is in shared memory
-    cluster_barrier();  // start-up
-    auto wait_rows = [&](int stg, uint32_t parity) __attribute__((always_inline)) {
-      if (my_chunks > 0 && !mbar_wait_bounded(&bars[stg], parity, bp.spin_limit)) {
-        set_status(p.status, DEV_TIMEOUT, 1, (long long)blockIdx.x);
-        for (uint32_t rr = 0; rr < C; ++rr) st_shared_cluster(map_shared_rank((const void*)give_up, rr), 1);
-      }
-    };
-    // adds the math warps' tables up over the 16-byte groups [g0, g0 + n) in warp order and sends the sums to this
-    // CTA's slot in every CTA of the cluster (after a barrier among the math warps: the tables are written)
-    auto reduce_and_send = [&](int g0, int n, int q) __attribute__((always_inline)) {
-      asm volatile("bar.sync 3, %0;" ::"r"(math_threads) : "memory");
-      const uint32_t ob = (uint32_t)__cvta_generic_to_shared(&pbar[q]) - own_base;
-      for (int e = g0 + mt; e < g0 + n; e += math_threads) {
-        const float4* p4 = (const float4*)part + e;
-        float4 sum = p4[0];
-#pragma unroll
-        for (int w = 1; w < M16_WARPS; ++w)
-          if (w < math_warps) {
-            const float4 v = p4[w * (M16_SLOT_FLOATS / 4)];
-            sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
-          }
-        const uint32_t od = (uint32_t)__cvta_generic_to_shared(red + ((size_t)q * M16_SLOTS + rank) * M16_SLOT_FLOATS + 4 * e) - own_base;
-#pragma unroll
-        for (int rr = 0; rr < 8; ++rr)
-          if ((uint32_t)rr < C) st_async_f32x4(peer_base[rr] + od, sum, peer_base[rr] + ob);
-      }
-    };
-    float4 xo[NQ];  // this thread's chunks of row i16 of the block whose margins come next
-    float* tbl = part + (size_t)(warp - 2) * M16_SLOT_FLOATS;
-    auto gram_part = [&](const unsigned char* stage, int q) __attribute__((always_inline)) {
-      float acc[B];
-#pragma unroll
-      for (int k2 = 0; k2 < B; ++k2) acc[k2] = 0.0f;
-#pragma unroll
-      for (int it = 0; it < NQ; ++it) {
-        const int qi = g + G16 * it;
-        if (qi < my_chunks) {
-          xo[it] = *(const float4*)(stage + (size_t)i16 * row_stride + (size_t)qi * 16);
-#pragma unroll
-          for (int k2 = 0; k2 < B; ++k2) {
-            const float4 xk = *(const float4*)(stage + (size_t)k2 * row_stride + (size_t)qi * 16);
-            acc[k2] = fmaf(xo[it].x, xk.x, fmaf(xo[it].y, xk.y, fmaf(xo[it].z, xk.z, fmaf(xo[it].w, xk.w, acc[k2]))));
-          }
-        } else {
-          xo[it] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        }
-      }
-#pragma unroll
-      for (int k2 = 0; k2 < B; ++k2) acc[k2] += __shfl_xor_sync(0xffffffffu, acc[k2], 16);
-      if (lane < 16) {  // D0 row i16 = G[i16][0..7]; rows 8..15 also D1 row i16 - 8 = G[i16][8..15]
-        *(float4*)(tbl + i16 * 8) = make_float4(acc[0], acc[1], acc[2], acc[3]);
-        *(float4*)(tbl + i16 * 8 + 4) = make_float4(acc[4], acc[5], acc[6], acc[7]);
-        if (i16 >= 8) {
-          *(float4*)(tbl + 128 + (i16 - 8) * 8) = make_float4(acc[8], acc[9], acc[10], acc[11]);
-          *(float4*)(tbl + 128 + (i16 - 8) * 8 + 4) = make_float4(acc[12], acc[13], acc[14], acc[15]);
-        }
-      }
-      reduce_and_send(0, 48, q);
-    };
-    auto margin_part = [&](int q) __attribute__((always_inline)) {
-      float pa = 0.0f;
-#pragma unroll
-      for (int it = 0; it < NQ; ++it) {
-        const int qi = g + G16 * it;
-        if (qi < my_chunks) {
-          const float4 w4 = *(const float4*)(wsm + 4 * qi);
-          pa = fmaf(xo[it].x, w4.x, fmaf(xo[it].y, w4.y, fmaf(xo[it].z, w4.z, fmaf(xo[it].w, w4.w, pa))));
-        }
-      }
-      pa += __shfl_xor_sync(0xffffffffu, pa, 16);
-      if (lane < 16) *(float4*)(tbl + 192 + 4 * i16) = make_float4(pa, 0.0f, 0.0f, 0.0f);  // one part (the bf16 form has three)
-      reduce_and_send(48, 16, q);
-    };
-    int sg = 0, su = 0;  // stage of the next block whose Gram part is formed / whose update is applied
-    uint32_t pg = 0u;
-    auto gram_next = [&](long long blk) __attribute__((always_inline)) {
-      wait_rows(sg, pg);
-      gram_part(ring + (size_t)sg * B * row_stride, (int)(blk % NBUF));
-      if (++sg == S) { sg = 0; pg ^= 1u; }
-    };
-    if (nb > 0) {
-      gram_next(0);
-      margin_part(0);
-    }
-    for (long long b = 0; b < nb; ++b) {
-      if (b + 1 < nb) gram_next(b + 1);  // while the recurrence warp works on block b
-      __syncthreads();                   // gamma_b and the decision are in gam
-      if (gam[B + 1] != 0.0f) {
-        // giving up: sums sent just now may still be on their way to a peer; let them land before anyone exits
-        const long long t0 = clock64();
-        while (clock64() - t0 < 100000) {}
-        break;
-      }
-      // ---- w <- w - (1 - a^nv) w - sum_m gamma_m x_m, one column per thread -----------------------------------------
-      {
-        const float* xs = (const float*)(ring + (size_t)su * B * row_stride);
-        const size_t rs4 = row_stride / 4;
-        const float ndl = -gam[B];
-        for (int c = mt; c < ncols; c += math_threads) {
-          float wv = wsm[c];
-          wv = fmaf(ndl, wv, wv);
-#pragma unroll
-          for (int m = 0; m < B; ++m) wv = fmaf(-gam[m], xs[(size_t)m * rs4 + c], wv);
-          wsm[c] = wv;
-        }
-      }
-      asm volatile("bar.arrive 2, %0;" ::"r"(consumed_threads) : "memory");  // this warp is done with the stage of block b
-      if (++su == S) su = 0;
-      asm volatile("bar.sync 4, %0;" ::"r"(math_threads) : "memory");        // the model slice is up to date
-      if (b + 1 < nb) margin_part((int)((b + 1) % NBUF));
-    }
-    cluster_barrier();
-    {
-      float* dst = p.W + (size_t)j * d + chunk0 * 4;
-      for (int c = mt; c < ncols; c += math_threads) dst[c] = wsm[c];
-    }
-  } else {
   const int mw = warp - 2;
   const int lc = mw * 32 + lane;  // this thread's 16-byte chunk within the CTA's slice
   const bool act = lc < my_chunks;
@@ -689,7 +534,6 @@ __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const Clust
       dst[2 * i + 1] = w2[i].y;
     }
   }
-  }  // bf16 rows
 }
 
 }  // namespace wpsgd

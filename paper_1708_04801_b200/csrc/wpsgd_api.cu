@@ -7,8 +7,10 @@
 #include <cstdio>
 #include <cstring>
 #include <functional>
+#include <initializer_list>
 #include <numeric>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "chain_block.cuh"
@@ -17,6 +19,7 @@
 #include "chain_mma.cuh"
 #include "chain_mma16.cuh"
 #include "chain_dense.cuh"
+#include "chain_lag.cuh"
 #include "combine.cuh"
 #include "philox.cuh"
 
@@ -64,7 +67,9 @@ struct wpsgd_ctx {
   bool have_run = false;
   std::vector<long long> steps_done;
   std::vector<int> node_ids;
-  std::vector<long long> last_steps;  // step counts of the launch being prepared
+  std::vector<long long> last_steps;    // step counts of the launch being prepared
+  std::vector<long long> steps_sorted;  // the same, largest first
+  double steps_sum = 0.0;
   float eta0 = 0.f, lambda = 0.f;
   int sched = 0, loss = 0;
   uint64_t seed = 0;
@@ -432,73 +437,14 @@ bool mma_kernel_fits(const wpsgd_ctx* c, bool aligned, ClusterShape* out) {
   out->cpc = (int)cpc;
   out->math_warps = (int)mw;
   out->stages = stages;
-  // 16 samples per block (squared and hinge losses): half as many hand-offs per sample; one CTA per SM
+  // 16 samples per block: half as many hand-offs per sample; one CTA per SM
   int s16 = c->opt_stages > 0 ? std::min(c->opt_stages, 8) : 2;
-  while (s16 >= 2 && Mma16Smem(s16, (size_t)cpc * 16, 2).total > kSmemBudget) --s16;
+  while (s16 >= 2 && Mma16Smem(s16, (size_t)cpc * 16).total > kSmemBudget) --s16;
   out->stages16 = s16 >= 2 ? s16 : 0;
   const bool can16 = out->stages16 > 0;
   out->block = (c->opt_block_samples == 16 || (c->opt_block_samples == 0 && can16)) ? 16 : 8;
   if (out->block == 16 && !can16) return false;
   return true;
-}
-
-// ---- fp32 rows: the 16-sample cluster kernel with the Gram block on the fp32 pipes -------------------------------------
-// A chain is spread over as many CTAs as idle SMs allow (a cluster of 2, 4 or 8), each with at most 64 chunks of 4
-// columns: meant for few, wide chains that would otherwise hold one SM each.
-constexpr int kF16Stages = 3;
-bool f16_kernel_fits(const wpsgd_ctx* c, int nk, bool aligned, ClusterShape* out) {
-  if (!aligned || (double)c->eta0 * (double)c->lambda > 0.25) return false;
-  const long long chunks = c->d / 4;
-  int C = c->opt_cluster;
-  if (C <= 0) {
-    C = 8;
-    while (C > 1 && ((long long)nk * C > 148 || (chunks + C - 1) / C < 8)) C /= 2;
-  }
-  if (C != 1 && C != 2 && C != 4 && C != 8) return false;
-  const long long cpc = (chunks + C - 1) / C;
-  if (cpc < 1 || cpc > 64 || (long long)(C - 1) * cpc >= chunks) return false;
-  if (Mma16Smem(kF16Stages, (size_t)cpc * 16, 3).total > kSmemBudget) return false;
-  out->C = C;
-  out->cpc = (int)cpc;
-  out->math_warps = 8;
-  out->stages16 = kF16Stages;
-  out->block = 16;
-  return true;
-}
-
-wpsgd_status launch_f16(wpsgd_ctx* c, const ChainParams& p, const ClusterShape& sh) {
-  ClusterParams cp;
-  cp.b.c = p;
-  cp.b.stages = sh.stages16;
-  cp.b.eta_lambda = (double)c->eta0 * (double)c->lambda;
-  cp.b.spin_limit = c->opt_spin_limit;
-  cp.b.drop_block = c->opt_drop_block;
-  cp.b.group_order = nullptr;
-  cp.chunks_per_cta = sh.cpc;
-  const size_t smem = Mma16Smem(sh.stages16, (size_t)sh.cpc * 16, 3).total;
-  auto go = [&](auto kern) -> wpsgd_status {
-    CU_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(p.k * sh.C));
-    cfg.blockDim = dim3((unsigned)(64 + 32 * sh.math_warps));
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = c->stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)sh.C;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    CU_TRY(c, cudaLaunchKernelEx(&cfg, kern, cp));
-    c->launches++;
-    return WPSGD_OK;
-  };
-  switch (c->loss) {
-    case WPSGD_LOSS_HINGE: return go(chain_mma16_kernel<LOSS_HINGE, float>);
-    case WPSGD_LOSS_LOGISTIC: return go(chain_mma16_kernel<LOSS_LOGISTIC, float>);
-    default: return go(chain_mma16_kernel<LOSS_SQUARED, float>);
-  }
 }
 
 wpsgd_status launch_mma(wpsgd_ctx* c, const ChainParams& p, const ClusterShape& sh) {
@@ -512,7 +458,7 @@ wpsgd_status launch_mma(wpsgd_ctx* c, const ChainParams& p, const ClusterShape& 
   cp.chunks_per_cta = sh.cpc;
   const bool b16 = sh.block == 16;
   if (b16) cp.b.stages = sh.stages16;
-  const size_t smem = b16 ? Mma16Smem(sh.stages16, (size_t)sh.cpc * 16, 2).total : MmaSmem(sh.stages, (size_t)sh.cpc * 16, MMA_SLOTS).total;
+  const size_t smem = b16 ? Mma16Smem(sh.stages16, (size_t)sh.cpc * 16).total : MmaSmem(sh.stages, (size_t)sh.cpc * 16, MMA_SLOTS).total;
   auto go = [&](auto kern) -> wpsgd_status {
     CU_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     cudaLaunchConfig_t cfg = {};
@@ -533,9 +479,9 @@ wpsgd_status launch_mma(wpsgd_ctx* c, const ChainParams& p, const ClusterShape& 
   };
   if (b16) {
     switch (c->loss) {
-      case WPSGD_LOSS_HINGE: return go(chain_mma16_kernel<LOSS_HINGE, __nv_bfloat16>);
-      case WPSGD_LOSS_LOGISTIC: return go(chain_mma16_kernel<LOSS_LOGISTIC, __nv_bfloat16>);
-      default: return go(chain_mma16_kernel<LOSS_SQUARED, __nv_bfloat16>);
+      case WPSGD_LOSS_HINGE: return go(chain_mma16_kernel<LOSS_HINGE>);
+      case WPSGD_LOSS_LOGISTIC: return go(chain_mma16_kernel<LOSS_LOGISTIC>);
+      default: return go(chain_mma16_kernel<LOSS_SQUARED>);
     }
   }
   switch (c->loss) {
@@ -571,6 +517,88 @@ bool two_warp_ctas_per_sm_finish_first(const std::vector<long long>& steps, int 
     return end;
   };
   return makespan(2 * 148, 3000.0) < makespan(148, 2640.0);
+}
+
+// ---- blocked kernel with lagged margins ---------------------------------------------------------------------------------
+struct LagShape {
+  int C = 1, cpc = 0, stages = 0, teams = 1, gram_warps = 1, model_warps = 1, vb = 8, nc = 1, realign = 0, copy_warps = 2, warps = 0;
+  size_t smem = 0;
+};
+
+template <typename XT>
+bool lag_kernel_fits(const wpsgd_ctx* c, bool aligned, int C, LagShape* out) {
+  constexpr int V = XVec<XT>::V;
+  if ((double)c->eta0 * (double)c->lambda > 0.25) return false;  // keeps a^-8 harmless in fp32
+  const long long chunks = (c->d + V - 1) / V;
+  const long long cpc = (chunks + C - 1) / C;
+  if ((long long)(C - 1) * cpc >= chunks) return false;  // every CTA of the cluster owns at least one chunk
+  if (!c->steps_sorted.empty() && c->steps_sorted[0] > (1ll << 33)) return false;  // block numbers are ints
+  LagShape sh;
+  sh.C = C;
+  sh.cpc = (int)cpc;
+  sh.realign = aligned ? 0 : 1;
+  // a model thread owns one vector of 8 bytes where two warps cover the slice (the rows of two blocks then stay in
+  // registers), else one or two of 16; with realigning warps there is room for four model warps, else for eight
+  const int max_mw = sh.realign ? 4 : 8;
+  if (cpc > 32 * max_mw * 2) return false;
+  sh.vb = cpc <= 64 ? 8 : 16;
+  sh.nc = cpc <= 32 * max_mw ? 1 : 2;
+  const int per_warp = 32 * sh.vb * sh.nc;
+  sh.model_warps = (int)((cpc * 16 + per_warp - 1) / per_warp);
+  int want = c->opt_stages > 0 ? std::max(3, c->opt_stages) : 8;
+  for (; want >= 3; --want) {
+    sh.smem = LagSmem(want, (size_t)cpc * 16, C, LAG_GRAM_WARPS, sh.realign).total;
+    if (sh.smem <= kSmemBudget + 4096) break;
+  }
+  if (want < 3 || (want < 4 && C < 8 && c->opt_stages == 0 && c->opt_cluster == 0)) return false;
+  sh.stages = want;
+  // as many Gram teams as the ring feeds: a team holds two stages while it works
+  sh.teams = want >= 7 ? 4 : (want >= 5 ? 2 : 1);
+  sh.gram_warps = LAG_GRAM_WARPS / sh.teams;
+  const int others = 3 + sh.model_warps + LAG_GRAM_WARPS + (sh.realign ? LAG_REALIGN_WARPS : 0);
+  sh.copy_warps = (others + 2) * 32 <= LAG_MAX_THREADS ? 2 : 1;
+  sh.warps = others + sh.copy_warps;
+  if (sh.warps * 32 > LAG_MAX_THREADS) return false;
+  *out = sh;
+  return true;
+}
+
+template <typename XT>
+wpsgd_status launch_lag(wpsgd_ctx* c, const ChainParams& p, const LagShape& sh) {
+  LagParams lp;
+  lp.b.c = p;
+  lp.b.stages = sh.stages;
+  lp.b.eta_lambda = (double)c->eta0 * (double)c->lambda;
+  lp.b.spin_limit = c->opt_spin_limit;
+  lp.b.drop_block = c->opt_drop_block;
+  lp.b.group_order = nullptr;
+  lp.chunks_per_cta = sh.cpc;
+  lp.gram_teams = sh.teams;
+  lp.gram_warps = sh.gram_warps;
+  lp.model_warps = sh.model_warps;
+  lp.realign = sh.realign;
+  lp.copy_warps = sh.copy_warps;
+  auto go = [&](auto kern) -> wpsgd_status {
+    CU_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(p.k * sh.C));
+    cfg.blockDim = dim3((unsigned)(32 * sh.warps));
+    cfg.dynamicSmemBytes = sh.smem;
+    cfg.stream = c->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)sh.C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    CU_TRY(c, cudaLaunchKernelEx(&cfg, kern, lp));
+    c->launches++;
+    return WPSGD_OK;
+  };
+  if (sh.nc == 2) return go(chain_lag_kernel<XT, 16, 2>);
+  if (sh.vb == 16) return go(chain_lag_kernel<XT, 16, 1>);
+  return go(chain_lag_kernel<XT, 8, 1>);
 }
 
 // blocked kernel, one warp per node (small d)
@@ -649,9 +677,71 @@ wpsgd_status launch_block_warp(wpsgd_ctx* c, const ChainParams& p, int R, int st
   return R == 1 ? launch_block_warp_r<XT, 1>(c, bp, smem, ctas, warps) : launch_block_warp_r<XT, 2>(c, bp, smem, ctas, warps);
 }
 
+// ---- which dense kernel -------------------------------------------------------------------------------------------------
+// Every chain is a serial string of blocks of 8 samples, so what decides is how long a block takes in a chain that has
+// its SMs to itself (L cycles), how much of an SM's throughput it uses up when chains share one (I cycles), and how the
+// chains queue for the slots. The estimate of a run:
+//     max( longest queue of a slot x L,  all blocks x I / 148 )  +  start-up of the kernel per wave of chains,
+// with the chains in launch order (longest first) on `slots` slots. The figures are device times of runs of 300 to 4000
+// steps with k = 4 .. 2000 chains (1965 MHz); the estimates come out within about a tenth of the times measured, e.g.
+// (measured, us) fp32 d = 1024, 4000 steps, k = 16: lagged form over 8 CTAs 324, one CTA per chain 541; k = 128: lagged
+// form over 2 CTAs 594, one CTA per chain 544; fp32 d = 128, 1000 steps, k = 200: lagged 76, CTA per chain 101, warp per
+// chain 133; k = 450: 162, 115, 140; k = 2000: 656, 295, 229.
+double run_estimate(const wpsgd_ctx* c, int slots, double L, double I, double start, double restart) {
+  const std::vector<long long>& n = c->steps_sorted;
+  const size_t k = n.size(), m = (size_t)slots;
+  double q = (double)n[0];
+  // the t-th wave of a slot holds at best the (t m)-th longest chain
+  for (size_t t = 1; t < 4 && t * m < k; ++t) q = std::max(q, (double)(t + 1) * (double)n[t * m]);
+  q = std::max(q, c->steps_sum / (double)slots);
+  const double waves = (double)((k + m - 1) / m);
+  return std::max(q * L, c->steps_sum * I / 148.0) / 8.0 + start + restart * (waves - 1.0);
+}
+// piecewise linear through (x_i, y_i), x ascending
+double through(double x, std::initializer_list<std::pair<double, double>> pts) {
+  const std::pair<double, double>* a = pts.begin();
+  if (x <= a->first) return a->second;
+  for (const std::pair<double, double>* b = a + 1; b != pts.end(); a = b, ++b)
+    if (x <= b->first) return a->second + (b->second - a->second) * (x - a->first) / (b->first - a->first);
+  return a->second * x / a->first;
+}
+
+template <typename XT>
+double lag_estimate(const wpsgd_ctx* c, const LagShape& sh) {
+  constexpr bool F32 = sizeof(XT) == 4;
+  const double x = (double)sh.cpc;
+  double L;
+  if (F32) L = sh.C == 1 ? through(x, {{8, 860}, {16, 890}, {32, 1030}, {64, 1230}, {128, 1985}, {256, 3836}})
+                         : through(x, {{8, 1010}, {16, 1040}, {32, 1165}, {64, 1465}, {128, 2045}, {256, 4000}});
+  else L = sh.C == 1 ? through(x, {{16, 955}, {32, 1015}, {64, 1180}, {128, 1510}, {256, 2350}})
+                     : through(x, {{8, 1100}, {32, 1250}, {64, 1540}, {128, 1875}, {256, 2900}});
+  if (sh.C == 8) L += 90.0;
+  if (sh.realign) L = std::max(L, 850.0 + 21.0 * x);
+  // resident clusters of 1, 2, 4, 8 CTAs with one CTA per SM
+  const int slots = sh.C == 1 ? 148 : (sh.C == 2 ? 74 : (sh.C == 4 ? 36 : 16));
+  return run_estimate(c, slots, L, 0.0, 5000.0 + 40.0 * x, 10000.0);
+}
+
+// The lagged form's best cluster size (or the one asked for); the estimate, or a negative number when it does not fit.
+template <typename XT>
+double best_lag_shape(const wpsgd_ctx* c, bool aligned, LagShape* out) {
+  double best = -1.0;
+  for (int C = 1; C <= 8; C *= 2) {
+    LagShape sh;
+    if ((c->opt_cluster > 0 && C != c->opt_cluster) || !lag_kernel_fits<XT>(c, aligned, C, &sh)) continue;
+    const double t = lag_estimate<XT>(c, sh);
+    if (best < 0.0 || t < best) {
+      best = t;
+      *out = sh;
+    }
+  }
+  return best;
+}
+
 template <typename XT>
 wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
   constexpr int V = XVec<XT>::V;
+  constexpr bool F32 = sizeof(XT) == 4;
   const long long d = c->d;
   const bool aligned = ((uintptr_t)p.X % 16 == 0) && ((p.ld * (long long)sizeof(XT)) % 16 == 0) && (d % V == 0) &&
                        ((uintptr_t)c->W % 16 == 0);
@@ -661,16 +751,74 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
   const bool block_ok = block_kernel_fits<XT>(c, aligned, &bthreads, &bR, &bstages);
   int wR = 0, wstages = 0, wwarps = 0;
   const bool block_warp_ok = block_warp_kernel_fits<XT>(c, p.k, aligned, &wR, &wstages, &wwarps);
-  ClusterShape mma_shape, f16_shape;
-  const bool mma_ok = sizeof(XT) == 2 && mma_kernel_fits(c, aligned, &mma_shape);
-  const bool f16_ok = sizeof(XT) == 4 && f16_kernel_fits(c, p.k, aligned, &f16_shape);
+  ClusterShape mma_shape;
+  const bool mma_ok = !F32 && mma_kernel_fits(c, aligned, &mma_shape);
+  LagShape lag_shape;
+  double lag_t = -1.0;
+  if (variant == 0 || variant >= 8) lag_t = best_lag_shape<XT>(c, aligned, &lag_shape);
+  const double x = (double)chunks;
+  // several CTAs share an SM (as many as their shared memory lets in): a chain then takes a fifth longer
+  auto shared_estimate = [&](size_t smem, double L, double I) {
+    const int per_sm = std::max(1, std::min(4, (int)(227 * 1024 / (smem + 1024))));
+    return run_estimate(c, 148 * per_sm, c->k > 148 && per_sm > 1 ? 1.2 * L : L, I, 0.0, 6000.0);
+  };
+  double mma_t = -1.0;
+  if (mma_ok) {
+    const double w = (double)mma_shape.cpc, L = through(w, {{64, 1400}, {128, 1520}, {256, 1970}});
+    if (mma_shape.C == 1) mma_t = shared_estimate(Mma16Smem(mma_shape.stages16, (size_t)mma_shape.cpc * 16).total, L, through(w, {{32, 560}, {64, 750}, {128, 1020}, {256, 1970}}));
+    else mma_t = run_estimate(c, 148 / mma_shape.C, L, 0.0, 0.0, 6000.0);
+  }
   if (variant == 0) {
-    if (!aligned) variant = 1;
-    else if (f16_ok && f16_shape.C >= 4 && chunks >= 128) variant = 9;  // few wide fp32 chains: spread each over idle SMs
-    else if (chunks <= 64) variant = block_warp_ok ? 5 : 3;
-    else if (sizeof(XT) == 2 && chunks >= 256 && mma_ok) variant = 8;  // wide bf16 rows: tensor-core cluster kernel
-    else if (block_ok) variant = 4;
-    else variant = (chunks > 512 * 4) ? 1 : 2;
+    double best = lag_t;
+    if (best >= 0.0) variant = 10;
+    auto offer = [&](bool ok, int v, double t) {
+      if (ok && (best < 0.0 || t < best)) {
+        best = t;
+        variant = v;
+      }
+    };
+    if (block_warp_ok) {
+      // one chain per scheduler or two (see two_warp_ctas_per_sm_finish_first)
+      const double L = F32 ? (chunks <= 32 ? 1925.0 : 2520.0) : (chunks <= 32 ? 1880.0 : 2740.0);
+      const double I = F32 ? (chunks <= 32 ? 430.0 : 570.0) : (chunks <= 32 ? 480.0 : 710.0);
+      offer(true, 5, std::min(run_estimate(c, 592, L, I, 0.0, 6000.0), run_estimate(c, 1184, 1.17 * L, I, 0.0, 6000.0)));
+    }
+    if (block_ok) {
+      const double L = F32 ? through(x, {{32, 1430}, {64, 1470}, {128, 1745}, {256, 2126}, {512, 3411}})
+                           : through(x, {{64, 1870}, {128, 1965}, {256, 2700}, {512, 4480}});
+      const double I = F32 ? through(x, {{32, 550}, {64, 777}, {128, 1120}, {256, 2126}, {512, 3411}})
+                           : through(x, {{32, 740}, {64, 1034}, {128, 1388}, {256, 2700}, {512, 4480}});
+      offer(true, 4, shared_estimate(BlockSmem(bstages, (size_t)d * sizeof(XT) + (F32 ? 0 : 16), bthreads / 32 - 2).total, L, I));
+    }
+    offer(mma_ok, 8, mma_t);
+    // rows wider than the blocked kernels take, many of them: the direct kernel keeps one chain per SM
+    if (lag_t >= 0.0) offer(aligned && chunks > 512 && chunks <= 512 * 4, 2, run_estimate(c, 148, 7000.0 + 5.4 * x, 0.0, 0.0, 6000.0));
+    if (best < 0.0) variant = !aligned || chunks > 512 * 4 ? 1 : (chunks <= 64 ? 3 : 2);
+  }
+  if (variant == 8 && c->opt_block_samples == 0 && lag_t >= 0.0 && aligned && !F32 && (!mma_ok || lag_t < mma_t)) variant = 10;
+  if (variant == 9) {
+    // fp32 rows, at most 64 chunks of a row per CTA: with clusters of the size asked for, else the best one
+    double best = -1.0;
+    for (int C = 1; F32 && aligned && C <= 8; C *= 2) {
+      LagShape sh;
+      if ((c->opt_cluster > 0 && C != c->opt_cluster) || (chunks + C - 1) / C > 64 || !lag_kernel_fits<XT>(c, aligned, C, &sh)) continue;
+      const double t = lag_estimate<XT>(c, sh);
+      if (best < 0.0 || t < best) {
+        best = t;
+        lag_shape = sh;
+      }
+    }
+    if (best < 0.0)
+      return fail(c, WPSGD_ERR_UNSUPPORTED,
+                  "cluster kernel for fp32 rows needs 16-byte aligned rows, eta*lambda <= 0.25 and a cluster of "
+                  "1, 2, 4 or 8 CTAs with at most 64 chunks of a row each");
+    return launch_lag<XT>(c, p, lag_shape);
+  }
+  if (variant == 10) {
+    if (lag_t < 0.0)
+      return fail(c, WPSGD_ERR_UNSUPPORTED,
+                  "lagged kernel needs eta*lambda <= 0.25 and a cluster of 1, 2, 4 or 8 CTAs that each hold a share of the row");
+    return launch_lag<XT>(c, p, lag_shape);
   }
   if (variant == 5) {
     if (!block_warp_ok)
@@ -686,13 +834,6 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
                   "tensor-core cluster kernel needs bf16 rows, 16-byte aligned, eta*lambda <= 0.25, a "
                   "cluster of 1, 2, 4 or 8 CTAs with at most 256 chunks of a row each and at most 16 math warps in all");
     return launch_mma(c, p, sh);
-  }
-  if (variant == 9) {
-    if (!f16_ok)
-      return fail(c, WPSGD_ERR_UNSUPPORTED,
-                  "16-sample cluster kernel for fp32 rows needs 16-byte aligned rows, eta*lambda <= 0.25 and a cluster of "
-                  "1, 2, 4 or 8 CTAs with at most 64 chunks of a row each");
-    return launch_f16(c, p, f16_shape);
   }
   if (variant == 4) {
     if (!block_ok)
@@ -749,6 +890,10 @@ wpsgd_status run_dense_common(wpsgd_ctx* c, const void* X, wpsgd_xtype xt, long 
   s = upload_plan_and_stream(c, pl);
   if (s != WPSGD_OK) return s;
   c->last_steps = pl.steps;
+  c->steps_sorted.resize(c->k);
+  for (int j = 0; j < c->k; ++j) c->steps_sorted[j] = pl.steps[pl.order[j]];
+  c->steps_sum = 0.0;
+  for (long long n : pl.steps) c->steps_sum += (double)n;
   ChainParams p;
   p.X = X; p.ld = ld; p.y = y;
   p.shard_off = c->t_shard_off; p.n_steps = c->t_steps; p.first = c->t_first; p.idx_off = c->t_idx_off;
@@ -964,7 +1109,7 @@ wpsgd_status wpsgd_set_option(wpsgd_ctx* c, const char* name, int64_t value) {
   if (!c || !name) return fail(c, WPSGD_ERR_INVALID_ARG, "ctx or name is NULL");
   const std::string n(name);
   if (n == "dense_variant") {
-    if (value < 0 || value > 9 || value == 6 || value == 7) return fail(c, WPSGD_ERR_INVALID_ARG, "dense_variant must be 0..5, 8 or 9");
+    if (value < 0 || value > 10 || value == 6 || value == 7) return fail(c, WPSGD_ERR_INVALID_ARG, "dense_variant must be 0..5 or 8..10");
     c->opt_variant = (int)value;
   } else if (n == "prefetch") {
     if (value < 0 || value > 64) return fail(c, WPSGD_ERR_INVALID_ARG, "prefetch must be 0..64");

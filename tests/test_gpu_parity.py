@@ -444,8 +444,75 @@ def test_f32_cluster_kernel_bounded_waits_report_timeout_and_context_survives(P,
     assert rel_l2(v, ov) <= 1e-4
 
 
+# ---- blocked form with lagged margins (what most dense runs of up to 148 chains take) ------------------------------------
+@pytest.mark.parametrize("d,bf16,pad,cluster", [
+    (1, False, 0, 1), (3, True, 0, 1), (8, True, 0, 1), (36, False, 0, 1), (60, False, 0, 8),  # fewer columns than lanes
+    (256, False, 0, 1), (260, False, 0, 1), (512, False, 0, 1), (516, False, 0, 1),             # 64 / 65 / 128 / 129 chunks
+    (4096, False, 0, 4), (4096, False, 0, 8), (8192, True, 0, 8), (488, True, 0, 2), (2056, True, 0, 1),
+    (67, False, 0, 2), (999, False, 0, 8), (1001, True, 0, 1), (1000, True, 1, 4), (640, False, 3, 2), (4099, True, 0, 8),
+])
+@pytest.mark.parametrize("loss,sched", [(HINGE, 0), (LOGISTIC, 1), (SQUARED, 0)])
+def test_lagged_kernel_shapes(P, d, bf16, pad, cluster, loss, sched):
+    # step counts with ragged last blocks, one block, none; rows that start off 16-byte boundaries (d or the row stride not
+    # a multiple of 16 bytes) with garbage between the rows
+    wl = wi.config2(k=4, d=d, m=48, base_steps=210)
+    wl.n_steps = np.array([210, 1, 0, 67], dtype=np.int64)
+    wl.loss, wl.sched = loss, sched
+    if sched:
+        wl.eta0, wl.lam = 0.3, 0.05
+    if loss == SQUARED:
+        wl.y = (wl.y * 0.3).contiguous()
+    if bf16:
+        wl.X = wl.X.to(torch.bfloat16)
+    wl.w0 = torch.full((d,), 0.05)
+    oW = oracle.run_dense(wl.X, wl.y, wl.shard_off, wl.n_steps, d, wl.eta0, wl.sched, wl.lam, wl.loss, wl.seed, wl.w0)
+    dev = wl.to("cuda")
+    X = dev.X
+    if pad:
+        X = torch.full((X.shape[0], d + pad), float("nan"), dtype=X.dtype, device="cuda")
+        X[:, :d] = dev.X
+        X = X[:, :d]
+    with P.Context(wl.k, d) as ctx:
+        ctx.set_option("dense_variant", 10)
+        ctx.set_option("cluster", cluster)
+        ctx.run(X, dev.y, wl.shard_off, wl.n_steps, wl.eta0, wl.sched, wl.lam, wl.loss, wl.seed, dev.w0)
+        W = ctx.get_models().cpu().numpy()
+        ctx.check()
+    for j in range(wl.k):
+        assert rel_l2(W[j], oW[j]) <= TOL[loss]
+
+
+@pytest.mark.parametrize("stages", [0, 3, 4, 5])
+@pytest.mark.parametrize("n_steps", [(1, 7, 8), (9, 15, 16), (17, 0, 64), (333, 250, 3)])
+def test_lagged_kernel_block_boundaries_and_ring_depths(P, n_steps, stages):
+    wl = wi.config2(k=3, d=1024, m=64, base_steps=8)
+    wl.n_steps = np.array(n_steps, dtype=np.int64)
+    wl.w0 = torch.full((1024,), 0.1)
+    assert_parity(P, wl, {"dense_variant": 10, "cluster": 2, "stages": stages})
+
+
+@pytest.mark.parametrize("d,cluster", [(64, 1), (1024, 4), (999, 8)])
+def test_lagged_kernel_bounded_waits_report_timeout_and_context_survives(P, d, cluster):
+    wl_cpu = wi.config2(k=3, d=d, m=32, base_steps=120)
+    wl = wl_cpu.to("cuda")
+    with P.Context(wl.k, wl.d) as ctx:
+        for name, value in (("dense_variant", 10), ("cluster", cluster), ("spin_limit", 2000), ("test_drop_block", 3)):
+            ctx.set_option(name, value)
+        ctx.run_workload(wl)
+        with pytest.raises(P.WpsgdError) as e:
+            ctx.check()
+        assert e.value.status_name == "TIMEOUT"
+        ctx.set_option("test_drop_block", -1)
+        ctx.set_option("spin_limit", 1 << 20)
+        ctx.run_workload(wl)
+        v = ctx.combine().cpu().numpy()
+        ctx.check()
+    ov, _, _ = oracle.solve(wl_cpu)
+    assert rel_l2(v, ov) <= 1e-4
+
+
 # ---- logistic loss: blocks whose steps move the margins far take the direct evaluation ---------------------------------
-@pytest.mark.parametrize("variant,d", [(4, 1024), (5, 128), (8, 1024), (9, 1024)])
+@pytest.mark.parametrize("variant,d", [(4, 1024), (5, 128), (8, 1024), (9, 1024), (10, 200)])
 def test_logistic_large_steps_between_correlated_rows(P, variant, d):
     # rows that are nearly parallel (large Gram entries) and a large step size: inside a block of 8 samples the
     # margins move by much more than the range of the cubic expansion of the logistic factor
