@@ -39,13 +39,16 @@ struct CsrParams {
   DevStatus* status;
 };
 
-// u rows <- w0 (or zeros) unless keep_models, scale <- 1
+// u rows <- w0 (or zeros) unless keep_models, scale <- 1; VEC columns at a time
+template <int VEC>
 __global__ void csr_init_kernel(float* __restrict__ U, double* __restrict__ scale, const float* __restrict__ w0, int k,
                                 long long d, int keep_models) {
-  const long long total = (long long)k * d;
-  if (!keep_models)
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x)
-      U[i] = w0 ? w0[i % d] : 0.0f;
+  const long long per_row = d / VEC, total = keep_models ? 0 : (long long)k * per_row;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+    const long long c = w0 ? i - row_of(i, per_row) * per_row : 0;
+    if constexpr (VEC == 4) ((float4*)U)[i] = w0 ? ((const float4*)w0)[c] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    else U[i] = w0 ? w0[c] : 0.0f;
+  }
   if (blockIdx.x == 0)
     for (int j = threadIdx.x; j < k; j += blockDim.x) scale[j] = 1.0;
 }

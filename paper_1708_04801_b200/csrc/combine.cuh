@@ -6,134 +6,219 @@
 
 namespace wpsgd {
 
-// v[c] = sum_j (weight_j * scale_j) * W[j][c], j ascending, fp64 accumulation. scale may be null.
-__global__ void combine_kernel(const float* __restrict__ W, const double* __restrict__ weights,
-                               const double* __restrict__ scale, int k, long long d, float* __restrict__ v) {
-  for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < d; c += (long long)gridDim.x * blockDim.x) {
-    double a = 0.0;
-    int j = 0;
-    for (; j + 4 <= k; j += 4) {
-      const float f0 = W[(size_t)(j + 0) * d + c], f1 = W[(size_t)(j + 1) * d + c];
-      const float f2 = W[(size_t)(j + 2) * d + c], f3 = W[(size_t)(j + 3) * d + c];
-      // the k effective weights are the same for every thread: broadcast loads that stay in L1
-      a = fma(weights[j + 0] * (scale ? scale[j + 0] : 1.0), (double)f0, a);
-      a = fma(weights[j + 1] * (scale ? scale[j + 1] : 1.0), (double)f1, a);
-      a = fma(weights[j + 2] * (scale ? scale[j + 2] : 1.0), (double)f2, a);
-      a = fma(weights[j + 3] * (scale ? scale[j + 3] : 1.0), (double)f3, a);
+// v[c] = sum_j (weight_j * scale_j) * W[j][c] in fp64. scale may be null. Bound by the read of W. A block owns 32 VEC
+// columns and its warps split the nodes (every fourth, eighth, .. one each, j ascending), so that few columns with many
+// nodes still fill the machine; the warps' sums are added in warp order, so the result does not depend on timing. The host
+// launches up to 32 warps, four nodes or more each, and takes VEC = 4 when the column count fills the SMs with it.
+// k = 1024, d = 256: 226 us with one thread per column over all nodes, 7 us this way.
+template <int VEC>
+__global__ void __launch_bounds__(1024) combine_kernel(const float* __restrict__ W, const double* __restrict__ weights,
+                                                       const double* __restrict__ scale, int k, long long d, float* __restrict__ v) {
+  extern __shared__ __align__(16) double sums[];  // [warp][32 VEC]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const long long c = ((long long)blockIdx.x * 32 + lane) * VEC;
+  double a[VEC];
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) a[e] = 0.0;
+  if (c < d) {
+#pragma unroll 4
+    for (int j = warp; j < k; j += warps) {
+      float f[VEC];
+      const float* src = W + (size_t)j * d + c;
+      if constexpr (VEC == 4) {
+        const float4 q = __ldg((const float4*)src);
+        f[0] = q.x; f[1] = q.y; f[2] = q.z; f[3] = q.w;
+      } else {
+        f[0] = __ldg(src);
+      }
+      const double wj = weights[j] * (scale ? scale[j] : 1.0);
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) a[e] = fma(wj, (double)f[e], a[e]);
     }
-    for (; j < k; ++j) a = fma(weights[j] * (scale ? scale[j] : 1.0), (double)W[(size_t)j * d + c], a);
-    v[c] = (float)a;
+  }
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) sums[(warp * VEC + e) * 32 + lane] = a[e];
+  __syncthreads();
+  for (int e = warp; e < VEC; e += warps) {
+    double t = 0.0;
+    for (int w = 0; w < warps; ++w) t += sums[(w * VEC + e) * 32 + lane];
+    if (c < d) v[c + e] = (float)t;
   }
 }
 
-// W_out[j][c] = scale_j * W[j][c]
+// W_out[j][c] = scale_j * W[j][c], VEC columns at a time (VEC = 4: d a multiple of 4 and both matrices 16-byte aligned)
+template <int VEC>
 __global__ void export_models_kernel(const float* __restrict__ W, const double* __restrict__ scale, int k, long long d,
                                      float* __restrict__ out) {
-  const long long total = (long long)k * d;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x)
-    out[i] = scale ? (float)(scale[i / d] * (double)W[i]) : W[i];
+  const long long per_row = d / VEC, total = (long long)k * per_row;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+    const double s = scale ? scale[row_of(i, per_row)] : 1.0;
+    if constexpr (VEC == 4) {
+      float4 q = ((const float4*)W)[i];
+      if (scale) q = make_float4((float)(s * (double)q.x), (float)(s * (double)q.y), (float)(s * (double)q.z), (float)(s * (double)q.w));
+      ((float4*)out)[i] = q;
+    } else {
+      out[i] = scale ? (float)(s * (double)W[i]) : W[i];
+    }
+  }
 }
 
 // W[j][:] = v for every node; scale_j = 1
+template <int VEC>
 __global__ void broadcast_model_kernel(float* __restrict__ W, double* __restrict__ scale, const float* __restrict__ v,
                                        int k, long long d) {
-  const long long total = (long long)k * d;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x)
-    W[i] = v[i % d];
+  const long long per_row = d / VEC, total = (long long)k * per_row;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+    const long long c = i - row_of(i, per_row) * per_row;
+    if constexpr (VEC == 4) ((float4*)W)[i] = ((const float4*)v)[c];
+    else W[i] = v[c];
+  }
   if (blockIdx.x == 0)
     for (int j = threadIdx.x; j < k; j += blockDim.x) scale[j] = 1.0;
 }
 
-// Pass 1 of the objective (Eq. 3-4): one warp per row, per-block partial sums of the loss and of the
-// misclassification count, written to part[2 * blockIdx.x + {0,1}] (fixed order -> deterministic).
-template <typename XT>
-__global__ void __launch_bounds__(256) objective_rows_kernel(const XT* __restrict__ X, long long ld,
-                                                             const float* __restrict__ y, long long n_rows,
-                                                             const float* __restrict__ w, long long d, int loss,
-                                                             double* __restrict__ part) {
-  __shared__ double sl[8], se[8];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double lsum = 0.0, esum = 0.0;
-  for (long long i = (long long)blockIdx.x * 8 + warp; i < n_rows; i += (long long)gridDim.x * 8) {
-    const XT* row = X + (size_t)i * ld;
-    float acc = 0.0f;
-    for (long long c = lane; c < d; c += 32) acc = fmaf(w[c], widen_scalar<XT>(row[c]), acc);
-    const float z = warp_sum(acc);
-    const float yy = y[i];
-    double L;
-    if (loss == LOSS_HINGE) L = fmax(0.0, 1.0 - (double)yy * (double)z);
-    else if (loss == LOSS_LOGISTIC) {
-      const double t = (double)yy * (double)z;
-      L = t > 0 ? log1p(exp(-t)) : -t + log1p(exp(t));
-    } else L = 0.5 * ((double)z - (double)yy) * ((double)z - (double)yy);
-    lsum += L;
-    esum += ((z >= 0.0f) != (yy >= 0.0f)) ? 1.0 : 0.0;
+// ---- objective of Eq. 3-4 and 0/1 error ----------------------------------------------------------------------------------
+__device__ __forceinline__ double loss_value(int loss, float yy, float z) {
+  if (loss == LOSS_HINGE) return fmax(0.0, 1.0 - (double)yy * (double)z);
+  if (loss == LOSS_LOGISTIC) {
+    const double t = (double)yy * (double)z;
+    return t > 0 ? log1p(exp(-t)) : -t + log1p(exp(t));
   }
-  if (lane == 0) { sl[warp] = lsum; se[warp] = esum; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0;
-    for (int i = 0; i < 8; ++i) { a += sl[i]; b += se[i]; }
-    part[2 * blockIdx.x] = a;
-    part[2 * blockIdx.x + 1] = b;
-  }
+  return 0.5 * ((double)z - (double)yy) * ((double)z - (double)yy);
+}
+__device__ __forceinline__ double warp_sum_f64(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
-// Pass 1 on CSR rows: one warp per row, lanes over the row's nonzeros.
-__global__ void __launch_bounds__(256) objective_rows_csr_kernel(const long long* __restrict__ row_ptr,
-                                                                 const int* __restrict__ col_idx,
-                                                                 const float* __restrict__ val,
-                                                                 const float* __restrict__ y, long long n_rows,
-                                                                 const float* __restrict__ w, int loss,
-                                                                 double* __restrict__ part) {
-  __shared__ double sl[8], se[8];
+// The end of both objective kernels: sums of the block (loss, error count, its share of |w|^2) go to part[3 blockIdx.x ..];
+// the block that finishes last adds all of them up in block order and writes out (so the result does not depend on which
+// block that is) and resets the ticket for the next launch.
+__device__ __forceinline__ void objective_finish(double lsum, double esum, const float* __restrict__ w, long long d, float lambda,
+                                                 long long n_rows, double* __restrict__ part, unsigned* ticket, double* __restrict__ out) {
+  __shared__ double sh[3][8];
+  __shared__ bool last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double lsum = 0.0, esum = 0.0;
-  for (long long i = (long long)blockIdx.x * 8 + warp; i < n_rows; i += (long long)gridDim.x * 8) {
-    const long long b = row_ptr[i], e = row_ptr[i + 1];
-    float acc = 0.0f;
-    for (long long q = b + lane; q < e; q += 32) acc = fmaf(w[col_idx[q]], val[q], acc);
-    const float z = warp_sum(acc);
-    const float yy = y[i];
-    double L;
-    if (loss == LOSS_HINGE) L = fmax(0.0, 1.0 - (double)yy * (double)z);
-    else if (loss == LOSS_LOGISTIC) {
-      const double t = (double)yy * (double)z;
-      L = t > 0 ? log1p(exp(-t)) : -t + log1p(exp(t));
-    } else L = 0.5 * ((double)z - (double)yy) * ((double)z - (double)yy);
-    lsum += L;
-    esum += ((z >= 0.0f) != (yy >= 0.0f)) ? 1.0 : 0.0;
-  }
-  if (lane == 0) { sl[warp] = lsum; se[warp] = esum; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0, b2 = 0.0;
-    for (int i = 0; i < 8; ++i) { a += sl[i]; b2 += se[i]; }
-    part[2 * blockIdx.x] = a;
-    part[2 * blockIdx.x + 1] = b2;
-  }
-}
-
-// Pass 2: out[0] = (lambda/2)|w|^2 + sum(part loss)/n_rows, out[1] = sum(part err)/n_rows. One block.
-__global__ void __launch_bounds__(256) objective_finish_kernel(const double* __restrict__ part, int n_part,
-                                                               const float* __restrict__ w, long long d, float lambda,
-                                                               long long n_rows, double* __restrict__ out) {
-  __shared__ double sh[3][256];
-  double a = 0.0, b = 0.0, r = 0.0;
-  for (int i = threadIdx.x; i < n_part; i += 256) { a += part[2 * i]; b += part[2 * i + 1]; }
-  for (long long c = threadIdx.x; c < d; c += 256) r += (double)w[c] * (double)w[c];
-  sh[0][threadIdx.x] = a; sh[1][threadIdx.x] = b; sh[2][threadIdx.x] = r;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o)
-      for (int q = 0; q < 3; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + o];
+  double r = 0.0;
+  for (long long c = (long long)blockIdx.x * 256 + threadIdx.x; c < d; c += (long long)gridDim.x * 256) r += (double)w[c] * (double)w[c];
+  auto block_sums = [&](double a, double b, double c) {  // to sh[.][0], for thread 0
+    a = warp_sum_f64(a); b = warp_sum_f64(b); c = warp_sum_f64(c);
+    if (lane == 0) { sh[0][warp] = a; sh[1][warp] = b; sh[2][warp] = c; }
     __syncthreads();
+    if (threadIdx.x < 3) {
+      double t = 0.0;
+      for (int i = 0; i < 8; ++i) t += sh[threadIdx.x][i];
+      sh[threadIdx.x][0] = t;
+    }
+    __syncthreads();
+  };
+  block_sums(lsum, esum, r);
+  if (threadIdx.x == 0) {
+    for (int q = 0; q < 3; ++q) __stcg(&part[3 * blockIdx.x + q], sh[q][0]);
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double a = 0.0, b = 0.0, c = 0.0;
+  for (unsigned i = threadIdx.x; i < gridDim.x; i += 256) {
+    a += __ldcg(&part[3 * i]);
+    b += __ldcg(&part[3 * i + 1]);
+    c += __ldcg(&part[3 * i + 2]);
+  }
+  block_sums(a, b, c);
   if (threadIdx.x == 0) {
     const double n = n_rows > 0 ? (double)n_rows : 1.0;
-    out[0] = 0.5 * (double)lambda * sh[2][0] + (n_rows > 0 ? sh[0][0] / n : 0.0);
-    out[1] = n_rows > 0 ? sh[1][0] / n : 0.0;
+    out[0] = 0.5 * (double)lambda * sh[2][0] + sh[0][0] / n;
+    out[1] = sh[1][0] / n;
+    *ticket = 0u;
   }
+}
+
+// Dense rows, one warp per row. Bound by the read of X: 16 bytes per lane and load, four loads in flight per lane (VEC; rows
+// that are not 16-byte aligned go element by element, eight in flight), the model from L1. A warp keeps the margins of up
+// to 32 of its rows, one per lane, and then evaluates their fp64 losses side by side. 262144 rows of 1024 fp32 columns: 231
+// us with single 4-byte loads, a loss evaluation per row on all lanes and a second launch for the sums; 177 us this way (6.1 TB/s).
+template <typename XT, bool VEC>
+__global__ void __launch_bounds__(256) objective_rows_kernel(const XT* __restrict__ X, long long ld, const float* __restrict__ y,
+                                                             long long n_rows, const float* __restrict__ w, long long d,
+                                                             int loss, float lambda, double* __restrict__ part, unsigned* ticket,
+                                                             double* __restrict__ out) {
+  constexpr int V = XVec<XT>::V;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double lsum = 0.0, esum = 0.0;
+  float z_own = 0.0f, y_own = 0.0f;
+  int held = 0;
+  auto evaluate = [&]() {
+    if (lane < held) {
+      lsum += loss_value(loss, y_own, z_own);
+      esum += ((z_own >= 0.0f) != (y_own >= 0.0f)) ? 1.0 : 0.0;
+    }
+    held = 0;
+  };
+  for (long long i = (long long)blockIdx.x * 8 + warp; i < n_rows; i += (long long)gridDim.x * 8) {
+    const XT* row = X + (size_t)i * ld;
+    const float yy = y[i];
+    float acc = 0.0f;
+    if constexpr (VEC) {
+      const long long chunks = d / V;
+      auto add = [&](const uint4& raw, long long c) {
+        float x[V];
+        XVec<XT>::widen(raw, x);
+#pragma unroll
+        for (int e = 0; e < V; e += 4) {
+          const float4 q = __ldg((const float4*)(w + c * V + e));
+          acc = fmaf(q.x, x[e], acc); acc = fmaf(q.y, x[e + 1], acc); acc = fmaf(q.z, x[e + 2], acc); acc = fmaf(q.w, x[e + 3], acc);
+        }
+      };
+      long long c = lane;
+      for (; c + 96 < chunks; c += 128) {
+        uint4 raw[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) raw[u] = ld_stream16(row + (c + 32 * u) * V);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) add(raw[u], c + 32 * u);
+      }
+      for (; c < chunks; c += 32) add(ld_stream16(row + c * V), c);
+    } else {
+#pragma unroll 8
+      for (long long c = lane; c < d; c += 32) acc = fmaf(w[c], widen_scalar<XT>(row[c]), acc);
+    }
+    const float z = warp_sum(acc);
+    if (lane == held) { z_own = z; y_own = yy; }
+    if (++held == 32) evaluate();
+  }
+  evaluate();
+  objective_finish(lsum, esum, w, d, lambda, n_rows, part, ticket, out);
+}
+
+// CSR rows: eight lanes per row (rows of a few tens of nonzeros), four rows per warp.
+__global__ void __launch_bounds__(256) objective_rows_csr_kernel(const long long* __restrict__ row_ptr, const int* __restrict__ col_idx,
+                                                                 const float* __restrict__ val, const float* __restrict__ y,
+                                                                 long long n_rows, const float* __restrict__ w, long long d,
+                                                                 int loss, float lambda, double* __restrict__ part, unsigned* ticket,
+                                                                 double* __restrict__ out) {
+  const int l8 = threadIdx.x & 7;
+  double lsum = 0.0, esum = 0.0;
+  // the same trip count for all rows of a warp (shuffles)
+  for (long long i0 = (long long)blockIdx.x * 32; i0 < n_rows; i0 += (long long)gridDim.x * 32) {
+    const long long i = i0 + (threadIdx.x >> 3);
+    const bool in = i < n_rows;
+    const long long b = in ? row_ptr[i] : 0, e = in ? row_ptr[i + 1] : 0;
+    float acc = 0.0f;
+#pragma unroll 4
+    for (long long q = b + l8; q < e; q += 8) acc = fmaf(w[col_idx[q]], val[q], acc);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (in && l8 == 0) {
+      const float yy = y[i];
+      lsum += loss_value(loss, yy, acc);
+      esum += ((acc >= 0.0f) != (yy >= 0.0f)) ? 1.0 : 0.0;
+    }
+  }
+  objective_finish(lsum, esum, w, d, lambda, n_rows, part, ticket, out);
 }
 
 // Read-only check of a CSR matrix before it is handed to the chains: row_ptr within [0, nnz] and non-decreasing,

@@ -44,6 +44,11 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// Flat element number -> row, without a 64-bit division where 32 bits are enough.
+__device__ __forceinline__ long long row_of(long long i, long long per_row) {
+  return (i | per_row) >> 32 ? i / per_row : (long long)((uint32_t)i / (uint32_t)per_row);
+}
+
 // 16-byte vector of features, widened to fp32. V = elements per 16 bytes.
 template <typename XT>
 struct XVec;

@@ -50,6 +50,7 @@ struct wpsgd_ctx {
   DevStatus* status = nullptr;
   double* part = nullptr;  // objective partial sums
   size_t part_cap = 0;     // doubles
+  unsigned* ticket = nullptr;  // blocks of the running objective kernel that have finished (zero between launches)
   // staging of the host-buffer entry point
   void* st_X = nullptr;
   size_t st_X_cap = 0;
@@ -210,9 +211,29 @@ wpsgd_status read_status(wpsgd_ctx* c, DevStatus* dev_status, cudaStream_t strea
   return fail(c, h.code == DEV_TIMEOUT ? WPSGD_ERR_TIMEOUT : WPSGD_ERR_CUDA, buf);
 }
 
+bool aligned16(const void* p) { return (uintptr_t)p % 16 == 0; }
+
 int grid_for(long long work_items, int block, int cap = 148 * 16) {
   long long g = (work_items + block - 1) / block;
   return (int)std::max(1ll, std::min<long long>(g, cap));
+}
+
+// v_out = sum_j t_weights[j] scale_j W[j]
+wpsgd_status launch_combine(wpsgd_ctx* c, float* v_out) {
+  const double* scale = c->scaled ? c->scale : nullptr;
+  const int warps = std::max(1, std::min(32, (c->k + 3) / 4));
+  // four columns per thread once that still gives every SM several blocks
+  if (c->d % 4 == 0 && c->d >= 128 * 148 * 2 && aligned16(c->W)) {
+    const int w4 = std::min(warps, 16);  // 64 KB of sums would leave one block per SM
+    const unsigned blocks = (unsigned)((c->d + 127) / 128);
+    combine_kernel<4><<<blocks, 32 * w4, (size_t)w4 * 128 * sizeof(double), c->stream>>>(c->W, c->t_weights, scale, c->k, c->d, v_out);
+  } else {
+    const unsigned blocks = (unsigned)((c->d + 31) / 32);
+    combine_kernel<1><<<blocks, 32 * warps, (size_t)warps * 32 * sizeof(double), c->stream>>>(c->W, c->t_weights, scale, c->k, c->d, v_out);
+  }
+  CU_TRY(c, cudaGetLastError());
+  c->launches++;
+  return WPSGD_OK;
 }
 
 // ---- common part of run / continue: tables, sample stream ---------------------------------------------
@@ -940,7 +961,11 @@ wpsgd_status run_csr_common(wpsgd_ctx* c, const long long* row_ptr, const int* c
   if (s != WPSGD_OK) return s;
   if (!resume || !c->scaled) {
     // fresh chains start from w0 with scale 1; chains continued from a dense run keep their models and get scale 1
-    csr_init_kernel<<<grid_for((long long)c->k * c->d, 256), 256, 0, c->stream>>>(c->W, c->scale, w0, c->k, c->d, resume ? 1 : 0);
+    const long long n = (long long)c->k * c->d;
+    if (c->d % 4 == 0 && aligned16(c->W) && aligned16(w0))
+      csr_init_kernel<4><<<grid_for(n / 4, 256), 256, 0, c->stream>>>(c->W, c->scale, w0, c->k, c->d, resume ? 1 : 0);
+    else
+      csr_init_kernel<1><<<grid_for(n, 256), 256, 0, c->stream>>>(c->W, c->scale, w0, c->k, c->d, resume ? 1 : 0);
     CU_TRY(c, cudaGetLastError());
     c->launches++;
   }
@@ -1080,8 +1105,10 @@ wpsgd_status wpsgd_create(int device, void* cuda_stream, int32_t k, int64_t d, w
   ALLOC(c->t_group, ((size_t)k + 8) * sizeof(int));
   ALLOC(c->t_weights, (size_t)k * sizeof(double));
   ALLOC(c->status, sizeof(DevStatus));
+  ALLOC(c->ticket, sizeof(unsigned));
 #undef ALLOC
   if ((e = cudaMemsetAsync(c->status, 0, sizeof(DevStatus), c->stream)) != cudaSuccess) return bail(e, "cudaMemsetAsync");
+  if ((e = cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), c->stream)) != cudaSuccess) return bail(e, "cudaMemsetAsync");
   *out = c;
   return WPSGD_OK;
 }
@@ -1091,7 +1118,7 @@ wpsgd_status wpsgd_destroy(wpsgd_ctx* c) {
   DeviceGuard guard(c->device);
   cudaStreamSynchronize(c->stream);
   void* ptrs[] = {c->W, c->scale, c->t_shard_off, c->t_steps, c->t_first, c->t_idx_off, c->t_rows, c->t_count, c->t_order,
-                  c->t_ids, c->t_group, c->t_weights, c->idx, c->status, c->part, c->st_X, c->st_y, c->st_v, c->st_w0, c->st_rp, c->st_ci, c->st_va};
+                  c->t_ids, c->t_group, c->t_weights, c->idx, c->status, c->part, c->ticket, c->st_X, c->st_y, c->st_v, c->st_w0, c->st_rp, c->st_ci, c->st_va};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->ev0) cudaEventDestroy(c->ev0);
@@ -1272,11 +1299,7 @@ wpsgd_status wpsgd_combine(wpsgd_ctx* c, double r, float* v_out) {
   wpsgd_status s = weights_host(c->steps_done.data(), c->k, c->eta0, c->sched, c->lambda, r, w.data(), nullptr, nullptr, &why);
   if (s != WPSGD_OK) return fail(c, s, why);
   CU_TRY(c, cudaMemcpyAsync(c->t_weights, w.data(), c->k * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  combine_kernel<<<grid_for(c->d, 256), 256, 0, c->stream>>>(c->W, c->t_weights, c->scaled ? c->scale : nullptr, c->k,
-                                                            c->d, v_out);
-  CU_TRY(c, cudaGetLastError());
-  c->launches++;
-  return WPSGD_OK;
+  return launch_combine(c, v_out);
 }
 
 wpsgd_status wpsgd_combine_weighted(wpsgd_ctx* c, const double* weights, float* v_out) {
@@ -1287,11 +1310,7 @@ wpsgd_status wpsgd_combine_weighted(wpsgd_ctx* c, const double* weights, float* 
     if (!std::isfinite(weights[j])) return fail(c, WPSGD_ERR_INVALID_ARG, "a weight is not finite");
   DeviceGuard guard(c->device);
   CU_TRY(c, cudaMemcpyAsync(c->t_weights, weights, c->k * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  combine_kernel<<<grid_for(c->d, 256), 256, 0, c->stream>>>(c->W, c->t_weights, c->scaled ? c->scale : nullptr, c->k,
-                                                            c->d, v_out);
-  CU_TRY(c, cudaGetLastError());
-  c->launches++;
-  return WPSGD_OK;
+  return launch_combine(c, v_out);
 }
 
 wpsgd_status wpsgd_last_chain_ms(wpsgd_ctx* c, float* ms) {
@@ -1308,8 +1327,12 @@ wpsgd_status wpsgd_get_models(wpsgd_ctx* c, float* W_out) {
   if (!c->have_run) return fail(c, WPSGD_ERR_STATE, "get_models before run");
   if (!W_out) return fail(c, WPSGD_ERR_INVALID_ARG, "W_out is NULL");
   DeviceGuard guard(c->device);
-  export_models_kernel<<<grid_for((long long)c->k * c->d, 256), 256, 0, c->stream>>>(
-      c->W, c->scaled ? c->scale : nullptr, c->k, c->d, W_out);
+  const double* scale = c->scaled ? c->scale : nullptr;
+  const long long n = (long long)c->k * c->d;
+  if (c->d % 4 == 0 && aligned16(c->W) && aligned16(W_out))
+    export_models_kernel<4><<<grid_for(n / 4, 256), 256, 0, c->stream>>>(c->W, scale, c->k, c->d, W_out);
+  else
+    export_models_kernel<1><<<grid_for(n, 256), 256, 0, c->stream>>>(c->W, scale, c->k, c->d, W_out);
   CU_TRY(c, cudaGetLastError());
   c->launches++;
   return WPSGD_OK;
@@ -1320,7 +1343,11 @@ wpsgd_status wpsgd_set_models(wpsgd_ctx* c, const float* v) {
   if (!c->have_run) return fail(c, WPSGD_ERR_STATE, "set_models before run");
   if (!v) return fail(c, WPSGD_ERR_INVALID_ARG, "v is NULL");
   DeviceGuard guard(c->device);
-  broadcast_model_kernel<<<grid_for((long long)c->k * c->d, 256), 256, 0, c->stream>>>(c->W, c->scale, v, c->k, c->d);
+  const long long n = (long long)c->k * c->d;
+  if (c->d % 4 == 0 && aligned16(c->W) && aligned16(v))
+    broadcast_model_kernel<4><<<grid_for(n / 4, 256), 256, 0, c->stream>>>(c->W, c->scale, v, c->k, c->d);
+  else
+    broadcast_model_kernel<1><<<grid_for(n, 256), 256, 0, c->stream>>>(c->W, c->scale, v, c->k, c->d);
   CU_TRY(c, cudaGetLastError());
   c->launches++;
   return WPSGD_OK;
@@ -1348,16 +1375,17 @@ wpsgd_status wpsgd_objective(wpsgd_ctx* c, const void* X, wpsgd_xtype xt, int64_
   if (xt != WPSGD_X_F32 && xt != WPSGD_X_BF16) return fail(c, WPSGD_ERR_INVALID_ARG, "unknown feature type");
   DeviceGuard guard(c->device);
   const int nblk = grid_for((n_rows + 7) / 8, 1, 148 * 8);
-  wpsgd_status s = grow(c, &c->part, &c->part_cap, (size_t)nblk * 2);
+  wpsgd_status s = grow(c, &c->part, &c->part_cap, (size_t)nblk * 3);
   if (s != WPSGD_OK) return s;
-  if (xt == WPSGD_X_F32)
-    objective_rows_kernel<float><<<nblk, 256, 0, c->stream>>>((const float*)X, ld_elems, y, n_rows, w, c->d, (int)loss, c->part);
-  else
-    objective_rows_kernel<__nv_bfloat16><<<nblk, 256, 0, c->stream>>>((const __nv_bfloat16*)X, ld_elems, y, n_rows, w, c->d, (int)loss, c->part);
+  auto go = [&](auto kern, const auto* rows) {
+    kern<<<nblk, 256, 0, c->stream>>>(rows, ld_elems, y, n_rows, w, c->d, (int)loss, lambda, c->part, c->ticket, out);
+  };
+  const size_t es = xt == WPSGD_X_F32 ? 4 : 2;
+  const bool vec = aligned16(X) && aligned16(w) && ((size_t)ld_elems * es) % 16 == 0 && ((size_t)c->d * es) % 16 == 0;
+  if (xt == WPSGD_X_F32) vec ? go(objective_rows_kernel<float, true>, (const float*)X) : go(objective_rows_kernel<float, false>, (const float*)X);
+  else vec ? go(objective_rows_kernel<__nv_bfloat16, true>, (const __nv_bfloat16*)X) : go(objective_rows_kernel<__nv_bfloat16, false>, (const __nv_bfloat16*)X);
   CU_TRY(c, cudaGetLastError());
-  objective_finish_kernel<<<1, 256, 0, c->stream>>>(c->part, nblk, w, c->d, lambda, n_rows, out);
-  CU_TRY(c, cudaGetLastError());
-  c->launches += 2;
+  c->launches++;
   return WPSGD_OK;
 }
 
@@ -1368,15 +1396,13 @@ wpsgd_status wpsgd_objective_csr(wpsgd_ctx* c, const int64_t* row_ptr, const int
   if (!w || !out || n_rows < 0 || (int)loss < 0 || (int)loss > 2 || (n_rows > 0 && (!row_ptr || !col_idx || !val || !y)))
     return fail(c, WPSGD_ERR_INVALID_ARG, "objective_csr: bad argument");
   DeviceGuard guard(c->device);
-  const int nblk = grid_for((n_rows + 7) / 8, 1, 148 * 8);
-  wpsgd_status s = grow(c, &c->part, &c->part_cap, (size_t)nblk * 2);
+  const int nblk = grid_for((n_rows + 31) / 32, 1, 148 * 8);
+  wpsgd_status s = grow(c, &c->part, &c->part_cap, (size_t)nblk * 3);
   if (s != WPSGD_OK) return s;
-  objective_rows_csr_kernel<<<nblk, 256, 0, c->stream>>>((const long long*)row_ptr, col_idx, val, y, n_rows, w, (int)loss,
-                                                         c->part);
+  objective_rows_csr_kernel<<<nblk, 256, 0, c->stream>>>((const long long*)row_ptr, col_idx, val, y, n_rows, w, c->d, (int)loss, lambda,
+                                                         c->part, c->ticket, out);
   CU_TRY(c, cudaGetLastError());
-  objective_finish_kernel<<<1, 256, 0, c->stream>>>(c->part, nblk, w, c->d, lambda, n_rows, out);
-  CU_TRY(c, cudaGetLastError());
-  c->launches += 2;
+  c->launches++;
   return WPSGD_OK;
 }
 
