@@ -92,7 +92,7 @@ wpsgd_status wpsgd_destroy(wpsgd_ctx* ctx);
  *                     of the whole run. The blocked forms (4, 5, 8, 9, 10) take both step-size schedules and need
  *                     eta0 * lambda <= 0.25.
  *   "sparse_variant"  kernel for CSR rows. 0 (default) and 2: blocks of up to 64 steps run in a shared-memory cache of
- *                     the model entries they touch. 1: one step per round trip to the model in global memory.
+ *                     the model entries they touch, in groups of 8. 1: one step per round trip to the model in global memory.
  *   "cluster"         CTAs per node of variants 8, 9 and 10: 0 (default) chosen from d (and the node count), else 1, 2, 4 or 8.
  *   "block_samples"   samples per block of variant 8: 0 (default) 16 when the rows fit, else 8; 8 or 16 to force one.
  *   "threads"         threads per node of variants 2 and 4, warps x 32 per CTA of variant 5; 0 (default): chosen from d.

@@ -1,24 +1,41 @@
 // Per-node SGD chains on CSR rows (Eq. 5), a block of steps at a time through a shared-memory cache of the
-// model entries those steps touch. One CTA per node: warp 0 runs the chain, the other warps prepare blocks.
+// model entries those steps touch. One CTA per node: warp 0 runs the chain, warp 1 plans, the others prepare blocks.
 //
 // As in chain_csr.cuh the model of node j is w = s * u with an fp64 scalar s (the regulariser's factor
 // 1 - eta_n lambda multiplies s only), and a step is
 //     z = s_{n-1} (u . x);  g = L'(y, z);  s_n = s_{n-1} (1 - eta_n lambda);  u_c <- u_c - (eta_n g / s_n) x_c
 // on the row's nonzeros: the iterates of Eq. 5 in exact arithmetic, for any step-size schedule.
 //
-// Why blocks. In the direct kernel every step pays a round trip to the model in global memory (gather, reduce,
-// scatter) on its serial path. The sample stream does not depend on the model, so the rows of the next steps are
-// known in advance. The helper warps take the next up to 64 steps (at most CSRB_EMAX nonzeros in all), give every
-// distinct column among them a slot in a shared-memory hash table (linear probing, one compare-and-swap per
-// nonzero), store per nonzero its slot and value, and read u at the block's columns into the block's cache, all
-// while the chain warp runs the previous block. The chain warp runs a block's steps entirely in shared memory: slot
-// loads, a warp reduction, the loss derivative, slot stores.
+// Blocks. The sample stream does not depend on the model, so the rows of the next steps are known in advance. The helper
+// warps take the next up to 64 steps (at most CSRB_EMAX nonzeros in all), give every distinct column among them a slot in a
+// shared-memory hash table (linear probing, one compare-and-swap per probe), store per nonzero its slot and value, and
+// read u at the block's columns into the block's cache, all while the chain warp runs the previous block.
+//
+// Groups of 8 inside a block. In u-space nothing decays, so with kappa_n = (eta_n / s_n) L'(y_n, s_{n-1} (u . x_n)) and the
+// model u_0 before the group
+//     u before step n . x_n = u_0 . x_n - sum_{m < n} kappa_m (x_m . x_n).
+// The products x_m . x_n of a group's rows are formed ahead by helper warps: a row's values are scattered into a dense
+// array over the block's slots (one per warp) and gathered at the slots of the seven other rows. The chain warp then pays
+// once per 8 steps for the gather of the model entries and the sum over lanes (four lanes per sample), runs the 8 steps on
+// registers (the recurrence of chain_lag.cuh) and applies the 8 updates one after the other (a column of several
+// samples must see them in turn). All of it is in shared memory.
+//
+// For the hinge loss a decision within 1e-4 of its threshold sends the group through one step at a time, so that the order of
+// the sums never turns it.
+//
+// What bounds it, and what it measured (cycles per 8 steps of the longest chain, B200 at 1965 MHz): 40 Zipf-distributed
+// nonzeros per row, d = 2^20, hinge, 64 chains: 2685 (one step after the other, each with a gather, a sum over 32 lanes and a
+// scatter: 3840); 5 to 10 nonzeros, d = 100000, logistic, 10 chains: 1615 (3700). With short rows the chain warp's string is
+// the longer side: margins 160, steps 500, updates 300, boundary 130 of the 1500. With long rows the chain (2400) and the
+// helpers (insertion 700, products 1100, copies 400 per group) take about as long. Tried and taken back: margins from
+// the model one group back with a table per group and the model in L2 (5900 and 3300: everything that touches single
+// nonzeros is latency, and a table per 8 rows pays it eight times as often as one per block).
 //
 // Block boundary. The values the helpers read for block b + 1 are stale exactly at the columns block b touches, so
 // at the boundary every column of block b + 1 is looked up in block b's table and, when found, takes block b's
 // cached value (shared memory to shared memory). No global-memory latency is left on the chain's path: block b's
 // slots are written back to u by the helpers afterwards, before they reuse its tables for block b + 2. Tables and
-// caches are double buffered.
+// caches are double buffered, plans (row extents, labels, scale factors; two blocks ahead) are threefold.
 //
 // Slow boundaries (rare): a row with more than CSRB_EMAX nonzeros forms a block of its own that the chain warp runs
 // on global memory; when the scale has fallen below 1e-12 at the start of a block it is folded into u (u <- s u,
@@ -32,27 +49,35 @@
 
 #include <type_traits>
 
-#include "chain_block.cuh"
 #include "chain_csr.cuh"
+#include "chain_lag.cuh"
 
 namespace wpsgd {
 
-constexpr int CSRB_STEPS = 64;          // most steps per block
-constexpr int CSRB_EMAX = 4096;         // most nonzeros per block
-constexpr int CSRB_HASH = 8192;         // slots of the column table (power of two, > CSRB_EMAX)
-constexpr int CSRB_HASH_BITS = 13;
-constexpr int CSRB_THREADS = 256;       // warp 0: chain; warps 1..7: preparation
-constexpr int CSRB_HELPERS = CSRB_THREADS - 32;
+constexpr int CSRB_STEPS = 64;          // most steps per block, where all rows have at most 32 nonzeros
+constexpr int CSRB_LONG_STEPS = 48;     // else: as many groups as there are warps for their products
+constexpr int CSRB_GROUPS = CSRB_STEPS / LAG_B;
+constexpr int CSRB_EMAX = 2048;         // most nonzeros per block
+constexpr int CSRB_HASH = 4096;         // slots of the column table (power of two, > CSRB_EMAX)
+constexpr int CSRB_HASH_BITS = 12;
+constexpr int CSRB_THREADS = 384;       // warp 0: chain; warp 1: plans; warps 2..11: preparation
+constexpr int CSRB_HELPERS = CSRB_THREADS - 64;
+constexpr int CSRB_GRAM_WARPS = 6;      // helper warps that also form the products of a group's rows
+constexpr float CSRB_NEAR = 1e-4f;      // hinge decisions with |1 - t| below this are taken one step at a time
 constexpr int CSRB_BATCH = 8;           // independent global loads a thread keeps in flight
 
-struct CsrBlockMeta {
+// Plan of a block
+struct CsrPlan {
   int nsteps;    // steps in the block (0: the chain has ended)
   int nent;      // nonzeros of those steps
   int direct;    // 1: a single long row, run on global memory
-  int nuniq;     // distinct columns (filled while inserting; 0 again once the block has been written back)
   float fold;    // != 0: multiply u by it before the block (the scale was folded back)
-  int wide;      // 1: some row of the block has more than 64 nonzeros
-  int pad[2];
+  long long gbeg[CSRB_STEPS];          // first nonzero of the step's row in col_idx / val
+  int4 step[CSRB_STEPS];               // per step: first nonzero within the block, nonzeros, label bits, scale-before bits
+  float eos[CSRB_STEPS];               // eta_n / scale after the step
+  LagConst k[CSRB_GROUPS];             // constants of a group of 8 steps
+  int longest;                         // most nonzeros of a row of the block
+  int pad[3];
 };
 
 // One buffer of a prepared block.
@@ -61,21 +86,19 @@ struct CsrBlockBuf {
   float val[CSRB_EMAX];                // value of every nonzero, rows one after the other
   unsigned short slot[CSRB_EMAX];      // slot of every nonzero
   unsigned short uslot[CSRB_EMAX];     // the occupied slots, in order of first insertion
-  long long gbeg[CSRB_STEPS];          // first nonzero of the step's row in col_idx / val
-  int4 step[CSRB_STEPS];               // per step: first nonzero within the block, nonzeros, label bits, scale-before bits
-  float eos[CSRB_STEPS];               // eta_n / scale after the step
-  CsrBlockMeta meta;
+  float gram[CSRB_GROUPS][64];         // products of the rows of a group, [8][8], below the diagonal
+  int nuniq;                           // distinct columns (filled while inserting; 0 again once the block has been written back)
+  int pad[3];
 };
 
 struct CsrBlockSmem {
   CsrBlockBuf buf[2];
+  CsrPlan plan[3];
   float ucache[2][CSRB_HASH];          // u at the columns of a block, by slot
   int colbuf[CSRB_EMAX];               // columns of the block being prepared
+  float dense[CSRB_GRAM_WARPS][CSRB_HASH];  // one row at a time, by slot; zero in between
+  float4 jets[8];
 };
-
-__device__ __forceinline__ void named_barrier(int id, int threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
 
 // Shared-memory accesses by 32-bit shared-window address. The block buffers are chosen at run time (b & 1), so the
 // hot loops name the state space themselves instead of leaving it to address-space inference.
@@ -104,6 +127,20 @@ __device__ __forceinline__ void sts_f32(uint32_t a, float v) { asm volatile("st.
 __device__ __forceinline__ void sts_u16(uint32_t a, int v) {
   asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((unsigned short)v) : "memory");
 }
+// Where `yes`: a predicate, not a branch. (Branches around single accesses, even ones that all lanes take alike, cost more
+// than the accesses: they end the stretch of code in which loads overlap.)
+__device__ __forceinline__ void cp_async4_if(uint32_t smem_dst, const void* gmem_src, bool yes) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p cp.async.ca.shared.global [%0], [%1], 4;\n\t}" ::"r"(smem_dst), "l"(gmem_src), "r"((int)yes) : "memory");
+}
+__device__ __forceinline__ void atoms_cas_if(int& old, uint32_t a, int cmp, int val, bool yes) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %4, 0;\n\t@p atom.shared.cas.b32 %0, [%1], %2, %3;\n\t}" : "+r"(old) : "r"(a), "r"(cmp), "r"(val), "r"((int)yes) : "memory");
+}
+__device__ __forceinline__ void lds_s32_if(int& v, uint32_t a, bool yes) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p ld.shared.s32 %0, [%1];\n\t}" : "+r"(v) : "r"(a), "r"((int)yes) : "memory");
+}
+__device__ __forceinline__ void sts_f32_if(uint32_t a, float v, bool yes) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p st.shared.f32 [%0], %1;\n\t}" ::"r"(a), "f"(v), "r"((int)yes) : "memory");
+}
 __device__ __forceinline__ int atoms_cas(uint32_t a, int cmp, int val) {
   int old;
   asm volatile("atom.shared.cas.b32 %0, [%1], %2, %3;" : "=r"(old) : "r"(a), "r"(cmp), "r"(val) : "memory");
@@ -118,20 +155,19 @@ __device__ __forceinline__ int atoms_add(uint32_t a, int val) {
 __device__ __forceinline__ int csrb_hash(int col) { return (int)(((uint32_t)col * 0x9E3779B1u) >> (32 - CSRB_HASH_BITS)); }
 
 // cache[slot] <- u[column of slot] for the block's distinct columns i = t0, t0 + stride, ...; CSRB_BATCH loads in flight.
+// (Beyond the list the first column is read and written again.)
 __device__ __forceinline__ void csrb_gather(const CsrBlockBuf& B, float* cache, const float* u, int nuniq, int t0, int stride) {
   for (int base = t0; base < nuniq; base += stride * CSRB_BATCH) {
-    int h[CSRB_BATCH];
+    int h[CSRB_BATCH], c[CSRB_BATCH];
     float v[CSRB_BATCH];
 #pragma unroll
-    for (int g = 0; g < CSRB_BATCH; ++g) {
-      const int i = base + g * stride;
-      h[g] = i < nuniq ? (int)B.uslot[i] : -1;
-    }
+    for (int g = 0; g < CSRB_BATCH; ++g) h[g] = B.uslot[base + g * stride < nuniq ? base + g * stride : 0];
 #pragma unroll
-    for (int g = 0; g < CSRB_BATCH; ++g) v[g] = h[g] >= 0 ? __ldcg(u + B.keys[h[g]]) : 0.0f;
+    for (int g = 0; g < CSRB_BATCH; ++g) c[g] = B.keys[h[g]];
 #pragma unroll
-    for (int g = 0; g < CSRB_BATCH; ++g)
-      if (h[g] >= 0) cache[h[g]] = v[g];
+    for (int g = 0; g < CSRB_BATCH; ++g) v[g] = __ldcg(u + c[g]);
+#pragma unroll
+    for (int g = 0; g < CSRB_BATCH; ++g) cache[h[g]] = v[g];
   }
 }
 
@@ -160,265 +196,501 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
   for (int i = threadIdx.x; i < CSRB_HASH; i += CSRB_THREADS) {
     sm.buf[0].keys[i] = -1;
     sm.buf[1].keys[i] = -1;
+    for (int w = 0; w < CSRB_GRAM_WARPS; ++w) sm.dense[w][i] = 0.0f;
   }
-  if (threadIdx.x == 0) {
-    sm.buf[0].meta.nuniq = 0;
-    sm.buf[1].meta.nuniq = 0;
-    sm.buf[0].meta.nsteps = 0;
-    sm.buf[1].meta.nsteps = 0;
-    sm.buf[0].meta.direct = 0;
-    sm.buf[1].meta.direct = 0;
-  }
-  __syncthreads();
+  if (threadIdx.x < 2) sm.buf[threadIdx.x].nuniq = 0;
 
-  // ---- preparation of one block (helper warps only) ------------------------------------------------------------
-  long long s_next = 0;                          // first step of the next block to prepare (planner warp)
-  double sc = p.resume ? p.scale[j] : 1.0;       // scale after the last planned step (planner warp)
+  // ---- plan of the next block (planner warp) -----------------------------------------------------------------------
+  long long s_next = 0;                          // first step of the next block to plan
+  double sc = p.resume ? p.scale[j] : 1.0;       // scale after the last planned step
   const double lam = (double)p.lambda, eta0 = (double)p.eta0;
-  auto prepare = [&](CsrBlockBuf& B, float* cache) {
-    if (warp == 1) {
-      float fold = 0.0f;
-      if (sc < 1e-12 && s_next < n_run) {  // only ahead of a block that runs: the fold is applied at its start
-        fold = (float)sc;
-        sc = 1.0;
-      }
-      // row extents and labels of the next 64 steps, all loads in flight together
-      constexpr int PARTS = CSRB_STEPS / 32;
-      long long gb[PARTS], ge[PARTS];
-      float yy[PARTS];
-      uint32_t ri[PARTS];
-#pragma unroll
-      for (int part = 0; part < PARTS; ++part) {
-        const long long s = s_next + part * 32 + lane;
-        ri[part] = s < n_run ? idx[s] : 0u;
-      }
-#pragma unroll
-      for (int part = 0; part < PARTS; ++part) {
-        const long long s = s_next + part * 32 + lane;
-        gb[part] = ge[part] = 0;
-        yy[part] = 0.0f;
-        if (s < n_run) {
-          gb[part] = rp[ri[part]];
-          ge[part] = rp[ri[part] + 1];
-          yy[part] = yshard[ri[part]];
-        }
-      }
-      int nsteps = 0, nent = 0, direct = 0, wide = 0;
-      bool more = true;
-#pragma unroll
-      for (int part = 0; part < PARTS; ++part) {
-        if (!more) break;
-        const long long s = s_next + part * 32 + lane;
-        const bool valid = s < n_run;
-        const long long len = ge[part] - gb[part];
-        const int cnt = len > (long long)CSRB_EMAX ? CSRB_EMAX + 1 : (len < 0 ? 0 : (int)len);
-        const double eta = p.sched == LR_INV_SQRT ? eta0 / sqrt((double)(first + s + 1)) : eta0;
-        const double a = valid ? 1.0 - eta * lam : 1.0;
-        int icnt = cnt;
-        double ia = a;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int c2 = __shfl_up_sync(0xffffffffu, icnt, o);
-          const double a2 = __shfl_up_sync(0xffffffffu, ia, o);
-          if (lane >= o) {
-            icnt += c2;
-            ia *= a2;
-          }
-        }
-        double ea = __shfl_up_sync(0xffffffffu, ia, 1);
-        if (lane == 0) ea = 1.0;
-        const bool ok = valid && (nent + icnt <= CSRB_EMAX) && (sc * ea >= 1e-30);
-        const unsigned mask = __ballot_sync(0xffffffffu, ok);
-        const int n_ok = (mask == 0xffffffffu) ? 32 : (__ffs((int)~mask) - 1);
-        if (lane < n_ok) {
-          const int r = nsteps + lane;
-          B.gbeg[r] = gb[part];
-          B.step[r] = make_int4(nent + icnt - cnt, cnt, __float_as_int(yy[part]), __float_as_int((float)(sc * ea)));
-          B.eos[r] = (float)(eta / (sc * ia));
-        }
-        wide |= __any_sync(0xffffffffu, lane < n_ok && cnt > 64) ? 1 : 0;
-        // a first row that does not fit the tables: a block of its own, run on global memory
-        const int lone = __shfl_sync(0xffffffffu, (part == 0 && n_ok == 0 && valid) ? 1 : 0, 0);
-        if (lone) {
-          if (lane == 0) {
-            B.gbeg[0] = gb[part];
-            B.gbeg[1] = ge[part];  // the row's end travels in the unused second entry
-            B.step[0] = make_int4(0, 0, __float_as_int(yy[part]), __float_as_int((float)sc));
-            B.eos[0] = (float)(eta / (sc * a));
-          }
-          direct = 1;
-          nsteps = 1;
-          nent = 0;
-          sc *= __shfl_sync(0xffffffffu, a, 0);
-          more = false;
-        } else {
-          if (n_ok > 0) {
-            nent += __shfl_sync(0xffffffffu, icnt, n_ok - 1);
-            sc *= __shfl_sync(0xffffffffu, ia, n_ok - 1);
-            nsteps += n_ok;
-          }
-          if (n_ok < 32) more = false;
-        }
-      }
-      if (lane == 0) {
-        B.meta.nsteps = nsteps;
-        B.meta.nent = nent;
-        B.meta.direct = direct;
-        B.meta.fold = fold;
-        B.meta.wide = wide;
-      }
-      s_next += nsteps;
+  auto plan_next = [&](CsrPlan& B) {
+    float fold = 0.0f;
+    if (sc < 1e-12 && s_next < n_run) {  // only ahead of a block that runs: the fold is applied at its start
+      fold = (float)sc;
+      sc = 1.0;
     }
-    named_barrier(1, CSRB_HELPERS);  // the plan of the block is in shared memory
-    const int nsteps = B.meta.nsteps, nent = B.meta.nent;
-    if (!B.meta.direct && nsteps > 0) {
+    // row extents and labels of the next steps, all loads in flight together
+    constexpr int PARTS = (CSRB_STEPS + 31) / 32;
+    long long gb[PARTS], ge[PARTS];
+    float yy[PARTS];
+    uint32_t ri[PARTS];
+#pragma unroll
+    for (int part = 0; part < PARTS; ++part) {
+      const long long s = s_next + part * 32 + lane;
+      ri[part] = s < n_run ? idx[s] : 0u;
+    }
+#pragma unroll
+    for (int part = 0; part < PARTS; ++part) {
+      const long long s = s_next + part * 32 + lane;
+      gb[part] = ge[part] = 0;
+      yy[part] = 0.0f;
+      if (s < n_run) {
+        gb[part] = rp[ri[part]];
+        ge[part] = rp[ri[part] + 1];
+        yy[part] = yshard[ri[part]];
+      }
+    }
+    bool lean = true;
+#pragma unroll
+    for (int part = 0; part < PARTS; ++part) lean = lean && ge[part] - gb[part] <= 32;
+    const int limit = __all_sync(0xffffffffu, lean) ? CSRB_STEPS : CSRB_LONG_STEPS;
+    int nsteps = 0, nent = 0, direct = 0, longest = 0;
+    bool more = true;
+#pragma unroll
+    for (int part = 0; part < PARTS; ++part) {
+      if (!more) break;
+      const long long s = s_next + part * 32 + lane;
+      const bool valid = s < n_run;
+      const long long len = ge[part] - gb[part];
+      const int cnt = len > (long long)CSRB_EMAX ? CSRB_EMAX + 1 : (len < 0 ? 0 : (int)len);
+      const double eta = p.sched == LR_INV_SQRT ? eta0 / sqrt((double)(first + s + 1)) : eta0;
+      const double a = valid ? 1.0 - eta * lam : 1.0;
+      int icnt = cnt;
+      double ia = a;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int c2 = __shfl_up_sync(0xffffffffu, icnt, o);
+        const double a2 = __shfl_up_sync(0xffffffffu, ia, o);
+        if (lane >= o) {
+          icnt += c2;
+          ia *= a2;
+        }
+      }
+      double ea = __shfl_up_sync(0xffffffffu, ia, 1);
+      if (lane == 0) ea = 1.0;
+      const bool ok = valid && (part * 32 + lane < limit) && (nent + icnt <= CSRB_EMAX) && (sc * ea >= 1e-30);
+      const unsigned mask = __ballot_sync(0xffffffffu, ok);
+      const int n_ok = (mask == 0xffffffffu) ? 32 : (__ffs((int)~mask) - 1);
+      if (lane < n_ok) {
+        const int r = nsteps + lane;
+        const float sb = (float)(sc * ea), eos = (float)(eta / (sc * ia)), y = yy[part];
+        B.gbeg[r] = gb[part];
+        B.step[r] = make_int4(nent + icnt - cnt, cnt, __float_as_int(y), __float_as_int(sb));
+        B.eos[r] = eos;
+        // kappa_n = a f(sc r_n), see LagConst
+        LagConst& K = B.k[r >> 3];
+        if (LOSS == LOSS_SQUARED) {  // loss derivative s r - y
+          K.a[r & 7] = eos * sb;
+          K.b[r & 7] = -eos * y;
+          K.sc[r & 7] = sb;
+        } else {                     // hinge: -y where y s r < 1; logistic: -y / (1 + 2^(y s log2(e) r))
+          const float ks = LOSS == LOSS_LOGISTIC ? y * sb * 1.4426950408889634f : y * sb;
+          K.a[r & 7] = -y * eos;
+          K.b[r & 7] = -LAG_STEP * ks;
+          K.sc[r & 7] = ks;
+        }
+        // the row's nonzeros are copied a block from now
+        for (int o = 0; o < cnt; o += 32) {
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(p.col_idx + gb[part] + o));
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(p.val + gb[part] + o));
+        }
+      }
+      longest = max(longest, (int)__reduce_max_sync(0xffffffffu, lane < n_ok ? (unsigned)cnt : 0u));
+      // a first row that does not fit the tables: a block of its own, run on global memory
+      const int lone = __shfl_sync(0xffffffffu, (part == 0 && n_ok == 0 && valid) ? 1 : 0, 0);
+      if (lone) {
+        if (lane == 0) {
+          B.gbeg[0] = gb[part];
+          B.gbeg[1] = ge[part];  // the row's end travels in the unused second entry
+          B.step[0] = make_int4(0, 0, __float_as_int(yy[part]), __float_as_int((float)sc));
+          B.eos[0] = (float)(eta / (sc * a));
+        }
+        direct = 1;
+        nsteps = 1;
+        nent = 0;
+        sc *= __shfl_sync(0xffffffffu, a, 0);
+        more = false;
+      } else {
+        if (n_ok > 0) {
+          nent += __shfl_sync(0xffffffffu, icnt, n_ok - 1);
+          sc *= __shfl_sync(0xffffffffu, ia, n_ok - 1);
+          nsteps += n_ok;
+        }
+        if (n_ok < 32) more = false;
+      }
+    }
+    if (!direct) {
+      // steps that fill up the last group take no step
+      const int r = nsteps + lane;
+      if (lane < 8 && r < (nsteps + 7) / 8 * 8) {
+        B.step[r] = make_int4(nent, 0, 0, 0);
+        B.k[r >> 3].a[r & 7] = B.k[r >> 3].b[r & 7] = B.k[r >> 3].sc[r & 7] = 0.0f;
+      }
+      __syncwarp();
+      if (lane < CSRB_GROUPS && 8 * lane < nsteps) {
+        float mx = 0.0f;
+        for (int m = 0; m < 8; ++m) mx = fmaxf(mx, fabsf(B.k[lane].sc[m]));
+        B.k[lane].sc_max = mx;
+      }
+    }
+    if (lane == 0) {
+      B.nsteps = nsteps;
+      B.nent = nent;
+      B.longest = longest;
+      B.direct = direct;
+      B.fold = fold;
+    }
+    s_next += nsteps;
+  };
+
+  // ---- products of the rows of one group (a helper warp with a dense array of its own) -----------------------------------
+  // CH: chunks of 32 nonzeros of a row in registers; REST: some row may have more. Compiled for each, so that the unrolled
+  // code has no branches (with guards inside it the same loads took four times as long).
+  auto form_gram = [&](const CsrBlockBuf& B, const CsrPlan& P, int gi, float* dense, float* out, auto ch_tag, auto rest_tag) {
+    constexpr int CH = decltype(ch_tag)::value;
+    constexpr bool REST = decltype(rest_tag)::value;
+    const uint32_t dense_a = smem_addr(dense), slot_a = smem_addr(B.slot), val_a = smem_addr(B.val), step_a = smem_addr(P.step);
+    int beg[8], cnt[8];
+    uint32_t sl[CH][8];
+    float v[CH][8], acc[32];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      const int4 st = lds_s32x4(step_a + 16u * (uint32_t)(8 * gi + m));
+      beg[m] = st.x;
+      cnt[m] = st.y;
+    }
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+#pragma unroll
+      for (int c = 0; c < CH; ++c) {
+        // lanes beyond the row read the block's first nonzero and take the value 0
+        const int e = lane + 32 * c < cnt[m] ? beg[m] + lane + 32 * c : 0;
+        sl[c][m] = (uint32_t)lds_u16(slot_a + 2u * (uint32_t)e);
+        v[c][m] = lds_f32(val_a + 4u * (uint32_t)e);
+      }
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+#pragma unroll
+      for (int c = 0; c < CH; ++c) {
+        sl[c][m] = dense_a + 4u * sl[c][m];
+        if (lane + 32 * c >= cnt[m]) v[c][m] = 0.0f;
+      }
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc[i] = 0.0f;
+#pragma unroll
+    for (int m = 0; m < 7; ++m) {
+#pragma unroll
+      for (int c = 0; c < CH; ++c) sts_f32_if(sl[c][m], v[c][m], lane + 32 * c < cnt[m]);
+      if constexpr (REST)
+        for (int o = lane + 32 * CH; o < cnt[m]; o += 32) dense[B.slot[beg[m] + o]] = B.val[beg[m] + o];
+      __syncwarp();
+      float x[CH][8];
+#pragma unroll
+      for (int n = m + 1; n < 8; ++n)
+#pragma unroll
+        for (int c = 0; c < CH; ++c) x[c][n] = lds_f32(sl[c][n]);
+#pragma unroll
+      for (int n = m + 1; n < 8; ++n) {
+        float t = x[0][n] * v[0][n];
+#pragma unroll
+        for (int c = 1; c < CH; ++c) t = fmaf(x[c][n], v[c][n], t);
+        if constexpr (REST)
+          for (int o = lane + 32 * CH; o < cnt[n]; o += 32) t = fmaf(dense[B.slot[beg[n] + o]], B.val[beg[n] + o], t);
+        acc[n * (n - 1) / 2 + m] = t;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int c = 0; c < CH; ++c) sts_f32_if(sl[c][m], 0.0f, lane + 32 * c < cnt[m]);
+      if constexpr (REST)
+        for (int o = lane + 32 * CH; o < cnt[m]; o += 32) dense[B.slot[beg[m] + o]] = 0.0f;
+      __syncwarp();
+    }
+    const float tot = warp_transpose_sum32(acc);  // lane l: product number l
+    int n2 = 1, m2 = lane;
+    while (n2 < 8 && m2 >= n2) { m2 -= n2; ++n2; }
+    if (n2 < 8) out[8 * n2 + m2] = tot;
+  };
+
+  // ---- preparation of one block (helper warps only); writes the block that was in these tables back first ------------------
+  auto prepare = [&](CsrBlockBuf& B, float* cache, const CsrPlan& P) {
+    const int ht = (int)threadIdx.x - 64, hw = warp - 2;
+    const int nsteps = P.nsteps, nent = P.nent, old = B.nuniq;
+    const bool have = !P.direct && nsteps > 0;
+    if (have) {
       // nonzeros of the block's rows: asynchronous 4-byte copies, all in flight together
-      for (int r = warp - 1; r < nsteps; r += CSRB_HELPERS / 32) {
-        const long long g0 = B.gbeg[r];
-        const int off = B.step[r].x, cnt = B.step[r].y;
-        for (int o = lane; o < cnt; o += 32) {
-          cp_async4(&sm.colbuf[off + o], p.col_idx + g0 + o);
-          cp_async4(&B.val[off + o], p.val + g0 + o);
-        }
+      constexpr int W = CSRB_HELPERS / 32, ROWS = (CSRB_STEPS + W - 1) / W;
+      int off[ROWS], cnt[ROWS];
+      long long g0[ROWS];
+#pragma unroll
+      for (int i = 0; i < ROWS; ++i) {
+        const int r = hw + W * i < nsteps ? hw + W * i : 0;
+        off[i] = P.step[r].x;
+        cnt[i] = hw + W * i < nsteps ? P.step[r].y : 0;
+        g0[i] = P.gbeg[r];
       }
-      cp_async_commit();
-      cp_async_wait(0);
-      named_barrier(1, CSRB_HELPERS);  // every helper's copies have landed
-      const uint32_t keys_a = smem_addr(B.keys), slot_a = smem_addr(B.slot), uslot_a = smem_addr(B.uslot);
-      const uint32_t col_a = smem_addr(sm.colbuf), nuniq_a = smem_addr(&B.meta.nuniq);
-      for (int e0 = 0; e0 < nent; e0 += CSRB_HELPERS) {  // the same trip count for every lane of a warp
-        const int e = e0 + (int)threadIdx.x - 32;
-        bool fresh = false;
-        int h = 0;
-        if (e < nent) {
-          int col = lds_s32(col_a + 4u * (uint32_t)e);
-          if ((unsigned long long)(long long)col >= (unsigned long long)p.d) {
-            set_status(p.status, DEV_BOUNDS, 21, (long long)col);
-            col = 0;
-            B.val[e] = 0.0f;
-          }
-          h = csrb_hash(col);
-          for (int probe = 0; probe < CSRB_HASH; ++probe) {
-            const int old = atoms_cas(keys_a + 4u * (uint32_t)h, -1, col);
-            if (old == -1) {
-              fresh = true;
-              asm volatile("prefetch.global.L2 [%0];" ::"l"(u + col));  // the block's read of u[col] follows soon
-              break;
-            }
-            if (old == col) break;
-            h = (h + 1) & (CSRB_HASH - 1);
-          }
-          sts_u16(slot_a + 2u * (uint32_t)e, h);
+      const uint32_t col_a = smem_addr(sm.colbuf), val_a = smem_addr(B.val);
+#pragma unroll
+      for (int i = 0; i < ROWS; ++i)
+#pragma unroll
+        for (int o = 0; o < 64; o += 32) {
+          cp_async4_if(col_a + 4u * (uint32_t)(off[i] + lane + o), p.col_idx + g0[i] + lane + o, lane + o < cnt[i]);
+          cp_async4_if(val_a + 4u * (uint32_t)(off[i] + lane + o), p.val + g0[i] + lane + o, lane + o < cnt[i]);
         }
-        // one counter update per warp for the columns seen for the first time
-        const unsigned fm = __ballot_sync(0xffffffffu, fresh);
-        if (fm) {
-          int base = 0;
-          if (lane == 0) base = atoms_add(nuniq_a, __popc(fm));
-          base = __shfl_sync(0xffffffffu, base, 0);
-          if (fresh) sts_u16(uslot_a + 2u * (uint32_t)(base + __popc(fm & ((1u << lane) - 1u))), h);
-        }
+      if (P.longest > 64)
+        for (int i = 0; i < ROWS; ++i)
+          for (int o = lane + 64; o < cnt[i]; o += 32) {
+            cp_async4(&sm.colbuf[off[i] + o], p.col_idx + g0[i] + o);
+            cp_async4(&B.val[off[i] + o], p.val + g0[i] + o);
+          }
+    }
+    cp_async_commit();
+    csrb_scatter(B, cache, u, old, ht, CSRB_HELPERS);
+    cp_async_wait(0);
+    named_barrier(1, CSRB_HELPERS);  // every helper's copies have landed, the table is empty
+    if (ht == 0) B.nuniq = 0;
+    named_barrier(1, CSRB_HELPERS);
+    if (!have) return;
+    const uint32_t keys_a = smem_addr(B.keys), slot_a = smem_addr(B.slot), uslot_a = smem_addr(B.uslot);
+    const uint32_t col_a = smem_addr(sm.colbuf), nuniq_a = smem_addr(&B.nuniq);
+    constexpr int F = 4;  // nonzeros of a thread that probe together
+    for (int e0 = 0; e0 < nent; e0 += F * CSRB_HELPERS) {  // the same trip count for every lane of a warp
+      int e[F], col[F], h[F], k2[F];
+      bool in[F], seek[F];
+      bool any_bad = false;
+#pragma unroll
+      for (int i = 0; i < F; ++i) {
+        e[i] = e0 + ht + CSRB_HELPERS * i;
+        in[i] = seek[i] = e[i] < nent;
+        col[i] = lds_s32(col_a + 4u * (uint32_t)(in[i] ? e[i] : 0));
+        k2[i] = 0;
       }
-      named_barrier(1, CSRB_HELPERS);  // the list of distinct columns is complete
+#pragma unroll
+      for (int i = 0; i < F; ++i) any_bad |= in[i] && (unsigned long long)(long long)col[i] >= (unsigned long long)p.d;
+      if (any_bad) {
+#pragma unroll
+        for (int i = 0; i < F; ++i)
+          if (in[i] && (unsigned long long)(long long)col[i] >= (unsigned long long)p.d) {
+            set_status(p.status, DEV_BOUNDS, 21, (long long)col[i]);
+            col[i] = 0;
+            B.val[e[i]] = 0.0f;
+          }
+      }
+#pragma unroll
+      for (int i = 0; i < F; ++i) h[i] = csrb_hash(col[i]);
+      // until none of the warp's nonzeros has met another column
+      for (int probe = 0; probe < CSRB_HASH; ++probe) {
+#pragma unroll
+        for (int i = 0; i < F; ++i) atoms_cas_if(k2[i], keys_a + 4u * (uint32_t)h[i], -1, col[i], seek[i]);
+        bool any = false;
+#pragma unroll
+        for (int i = 0; i < F; ++i) {
+          seek[i] = seek[i] && k2[i] != -1 && k2[i] != col[i];
+          h[i] = seek[i] ? (h[i] + 1) & (CSRB_HASH - 1) : h[i];
+          any |= seek[i];
+        }
+        if (!__any_sync(0xffffffffu, any)) break;
+      }
+      // one counter update per warp for the columns seen for the first time
+      unsigned f[F];
+      int total = 0;
+#pragma unroll
+      for (int i = 0; i < F; ++i) {
+        f[i] = __ballot_sync(0xffffffffu, in[i] && k2[i] == -1);
+        total += __popc(f[i]);
+      }
+      int base = 0;
+      if (lane == 0) base = atoms_add(nuniq_a, total);
+      base = __shfl_sync(0xffffffffu, base, 0);
+#pragma unroll
+      for (int i = 0; i < F; ++i) {
+        if (in[i]) sts_u16(slot_a + 2u * (uint32_t)e[i], h[i]);
+        if (in[i] && k2[i] == -1) {
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(u + col[i]));  // the block's read of u[col] follows soon
+          sts_u16(uslot_a + 2u * (uint32_t)(base + __popc(f[i] & ((1u << lane) - 1u))), h[i]);
+        }
+        base += __popc(f[i]);
+      }
+    }
+    named_barrier(1, CSRB_HELPERS);  // slots and the list of distinct columns are complete
+    if (hw < CSRB_GRAM_WARPS) {
+      for (int gi = hw; 8 * gi < nsteps; gi += CSRB_GRAM_WARPS) {
+        using std::integral_constant;
+        if (P.longest <= 32) form_gram(B, P, gi, sm.dense[hw], B.gram[gi], integral_constant<int, 1>(), std::false_type());
+        else if (P.longest <= 64) form_gram(B, P, gi, sm.dense[hw], B.gram[gi], integral_constant<int, 2>(), std::false_type());
+        else form_gram(B, P, gi, sm.dense[hw], B.gram[gi], integral_constant<int, 2>(), std::true_type());
+      }
+    } else {
       // u at the block's columns (stale where the running block writes: see the boundary)
-      csrb_gather(B, cache, u, B.meta.nuniq, (int)threadIdx.x - 32, CSRB_HELPERS);
+      csrb_gather(B, cache, u, B.nuniq, ht - 32 * CSRB_GRAM_WARPS, CSRB_HELPERS - 32 * CSRB_GRAM_WARPS);
     }
   };
 
-  // ---- the steps of a block, chain warp, in shared memory ----------------------------------------------------------
-  auto run_steps = [&](CsrBlockBuf& B, float* cache, int nsteps, auto wide_tag) {
-    constexpr bool WIDE = decltype(wide_tag)::value;
-    const uint32_t cache_a = smem_addr(cache), step_a = smem_addr(B.step), eos_a = smem_addr(B.eos);
-    const uint32_t slot_a = smem_addr(B.slot) + 2u * (uint32_t)lane, val_a = smem_addr(B.val) + 4u * (uint32_t)lane;
-    // registers of the next step: its row does not depend on the running step
-    int4 n_st = lds_s32x4(step_a);
-    float n_eos = lds_f32(eos_a);
-    uint32_t n_c0 = cache_a, n_c1 = cache_a;  // addresses of the lane's two cached model entries
-    float n_v0 = 0.0f, n_v1 = 0.0f;
-    if (lane < n_st.y) {
-      n_c0 = cache_a + 4u * (uint32_t)lds_u16(slot_a + 2u * (uint32_t)n_st.x);
-      n_v0 = lds_f32(val_a + 4u * (uint32_t)n_st.x);
-    }
-    if (lane + 32 < n_st.y) {
-      n_c1 = cache_a + 4u * (uint32_t)lds_u16(slot_a + 2u * (uint32_t)(n_st.x + 32));
-      n_v1 = lds_f32(val_a + 4u * (uint32_t)(n_st.x + 32));
-    }
-    for (int r = 0; r < nsteps; ++r) {
-      const int beg = n_st.x, cnt = n_st.y;
-      const float yy = __int_as_float(n_st.z), sb = __int_as_float(n_st.w), eos = n_eos;
-      const uint32_t c0 = n_c0, c1 = n_c1;
-      const float v0 = n_v0, v1 = n_v1;
+  // ---- the steps of a block in groups of 8, chain warp, in shared memory --------------------------------------------------
+  // Steps r0 .. r1 - 1 one at a time, each margin from the model as it then is: for a group in which a hinge decision comes so
+  // near its threshold that the sums' order could turn it.
+  auto one_by_one = [&](const CsrBlockBuf& B, const CsrPlan& P, float* cache, int r0, int r1) {
+#pragma unroll 1
+    for (int r = r0; r < r1; ++r) {
+      const int4 st = P.step[r];
+      const int beg = st.x, cnt = st.y;
       const bool in0 = lane < cnt, in1 = lane + 32 < cnt;
-      float uq0 = 0.0f, uq1 = 0.0f;
-      if (in0) uq0 = lds_f32(c0);
-      if (in1) uq1 = lds_f32(c1);
-      if (r + 1 < nsteps) {
-        n_st = lds_s32x4(step_a + 16u * (uint32_t)(r + 1));
-        n_eos = lds_f32(eos_a + 4u * (uint32_t)(r + 1));
-        n_v0 = n_v1 = 0.0f;
-        if (lane < n_st.y) {
-          n_c0 = cache_a + 4u * (uint32_t)lds_u16(slot_a + 2u * (uint32_t)n_st.x);
-          n_v0 = lds_f32(val_a + 4u * (uint32_t)n_st.x);
-        }
-        if (lane + 32 < n_st.y) {
-          n_c1 = cache_a + 4u * (uint32_t)lds_u16(slot_a + 2u * (uint32_t)(n_st.x + 32));
-          n_v1 = lds_f32(val_a + 4u * (uint32_t)(n_st.x + 32));
-        }
+      const int h0 = in0 ? B.slot[beg + lane] : 0, h1 = in1 ? B.slot[beg + lane + 32] : 0;
+      const float v0 = in0 ? B.val[beg + lane] : 0.0f, v1 = in1 ? B.val[beg + lane + 32] : 0.0f;
+      const float u0 = in0 ? cache[h0] : 0.0f, u1 = in1 ? cache[h1] : 0.0f;
+      float part = fmaf(u1, v1, u0 * v0);
+      for (int o = lane + 64; o < cnt; o += 32) part = fmaf(cache[B.slot[beg + o]], B.val[beg + o], part);
+      const float acc = warp_sum(part);
+      const float coef = P.eos[r] * loss_derivative(LOSS, __int_as_float(st.z), __int_as_float(st.w) * acc);
+      if (in0) cache[h0] = fmaf(-coef, v0, u0);
+      if (in1) cache[h1] = fmaf(-coef, v1, u1);
+      for (int o = lane + 64; o < cnt; o += 32) {
+        const int h = B.slot[beg + o];
+        cache[h] = fmaf(-coef, B.val[beg + o], cache[h]);
       }
-      float part = fmaf(uq1, v1, uq0 * v0);
-      if (WIDE)
-        for (int o = lane + 64; o < cnt; o += 32) part = fmaf(cache[B.slot[beg + o]], B.val[beg + o], part);
-      const float acc = warp_sum(part);  // shuffles only: nothing here waits on shared memory
-      const float g = loss_derivative(LOSS, yy, sb * acc);
-      const float coef = eos * g;  // g == 0 (hinge off the margin): the stores below rewrite the same values
-      if (in0) sts_f32(c0, fmaf(-coef, v0, uq0));
-      if (in1) sts_f32(c1, fmaf(-coef, v1, uq1));
-      if (WIDE)
-        for (int o = lane + 64; o < cnt; o += 32) {
-          const int h = B.slot[beg + o];
-          cache[h] = fmaf(-coef, B.val[beg + o], cache[h]);
-        }
-      __syncwarp();  // the next step's slot loads see this step's stores
+      __syncwarp();
     }
   };
 
-  if (warp != 0) prepare(sm.buf[0], sm.ucache[0]);
+  // E: nonzeros per lane of a row whose slot and value wait in registers for the margins (four lanes per sample), CH: chunks
+  // of 32 of them for the updates (all lanes on one sample); REST as above
+  auto run_steps = [&](const CsrBlockBuf& B, const CsrPlan& P, float* cache, auto e_tag, auto ch_tag, auto rest_tag) {
+    constexpr int E = decltype(e_tag)::value, CH = decltype(ch_tag)::value;
+    constexpr bool REST = decltype(rest_tag)::value;
+    const uint32_t cache_a = smem_addr(cache), slot_a = smem_addr(B.slot), val_a = smem_addr(B.val), step_a = smem_addr(P.step);
+    const int n = lane >> 2, q = lane & 3, own = lane & 7;
+    uint32_t ga[E];
+    float gv[E];
+    int gbeg = 0, gcnt = 0;
+    const int groups = (P.nsteps + 7) / 8;
+    // (lanes beyond a row read the slot of the block's first nonzero; what they read is not used)
+    auto entries = [&](int gi) __attribute__((always_inline)) {
+      const int4 st = lds_s32x4(step_a + 16u * (uint32_t)(8 * gi + n));
+      gbeg = st.x;
+      gcnt = st.y;
+#pragma unroll
+      for (int i = 0; i < E; ++i) {
+        const int e = q + 4 * i < gcnt ? gbeg + q + 4 * i : 0;
+        ga[i] = (uint32_t)lds_u16(slot_a + 2u * (uint32_t)e);
+        gv[i] = lds_f32(val_a + 4u * (uint32_t)e);
+      }
+    };
+    entries(0);
+#pragma unroll 1
+    for (int gi = 0; gi < groups; ++gi) {
+      const float* T = B.gram[gi];
+      const LagConst& K = P.k[gi];
+      float uq[E];
+#pragma unroll
+      for (int i = 0; i < E; ++i) uq[i] = lds_f32(cache_a + 4u * ga[i]);
+      // slots and values for the updates
+      int ub[8], uc[8];
+      uint32_t c[CH][8];
+      float w[CH][8];
+#pragma unroll
+      for (int m = 0; m < 8; ++m) {
+        const int4 st = lds_s32x4(step_a + 16u * (uint32_t)(8 * gi + m));
+        ub[m] = st.x;
+        uc[m] = st.y;
+      }
+      LagBlock<LOSS> blk;
+      blk.load(T, K, own);
+      float a0 = 0.0f, a1 = 0.0f;
+#pragma unroll
+      for (int i = 0; i < E; i += 2) {
+        a0 = q + 4 * i < gcnt ? fmaf(uq[i], gv[i], a0) : a0;
+        a1 = q + 4 * i + 4 < gcnt ? fmaf(uq[i + 1], gv[i + 1], a1) : a1;
+      }
+      if constexpr (REST)
+        for (int e = q + 4 * E; e < gcnt; e += 4) a0 = fmaf(cache[B.slot[gbeg + e]], B.val[gbeg + e], a0);
+      float r = a0 + a1;
+      r += __shfl_xor_sync(0xffffffffu, r, 1);
+#pragma unroll
+      for (int m = 0; m < 8; ++m)
+#pragma unroll
+        for (int k2 = 0; k2 < CH; ++k2) {
+          const int e = lane + 32 * k2 < uc[m] ? ub[m] + lane + 32 * k2 : 0;
+          c[k2][m] = (uint32_t)lds_u16(slot_a + 2u * (uint32_t)e);
+          w[k2][m] = lds_f32(val_a + 4u * (uint32_t)e);
+        }
+      r += __shfl_xor_sync(0xffffffffu, r, 2);
+      float kappa[LAG_B], margin;
+      blk.steps(__shfl_sync(0xffffffffu, r, 4 * own), T, K, sm.jets, kappa, margin);
+      if (gi + 1 < groups) entries(gi + 1);  // on their way while the updates run
+      if (LOSS == LOSS_HINGE && margin < CSRB_NEAR * LAG_STEP) {
+        one_by_one(B, P, cache, 8 * gi, min(8 * gi + 8, P.nsteps));
+        continue;
+      }
+      // u <- u - kappa_m x_m, m ascending
+#pragma unroll
+      for (int m = 0; m < LAG_B; ++m) {
+        float um[CH];
+#pragma unroll
+        for (int k2 = 0; k2 < CH; ++k2) um[k2] = lds_f32(cache_a + 4u * c[k2][m]);
+#pragma unroll
+        for (int k2 = 0; k2 < CH; ++k2) sts_f32_if(cache_a + 4u * c[k2][m], fmaf(-kappa[m], w[k2][m], um[k2]), lane + 32 * k2 < uc[m]);
+        if constexpr (REST)
+          for (int o = lane + 32 * CH; o < uc[m]; o += 32) {
+            const int h = B.slot[ub[m] + o];
+            cache[h] = fmaf(-kappa[m], B.val[ub[m] + o], cache[h]);
+          }
+        __syncwarp();  // the next sample's loads see this sample's stores
+      }
+    }
+  };
+
+  __syncthreads();
+  if (warp == 1) plan_next(sm.plan[0]);
+  __syncthreads();
+  if (warp == 1) plan_next(sm.plan[1]);
+  if (warp > 1) prepare(sm.buf[0], sm.ucache[0], sm.plan[0]);
   __syncthreads();
 
-  int prev_direct = 0;
+  int prev_direct = 0, cur = 0;  // cur = b mod 3
   for (long long b = 0;; ++b) {
     CsrBlockBuf& B = sm.buf[b & 1];
     CsrBlockBuf& Bp = sm.buf[(b + 1) & 1];  // the block that has just run (and the buffer of the next preparation)
     float* cache = sm.ucache[b & 1];
     float* cache_p = sm.ucache[(b + 1) & 1];
-    const int nsteps = B.meta.nsteps, nuniq = B.meta.nuniq, direct = B.meta.direct;
-    const int nuniq_p = Bp.meta.nuniq;
-    const float fold = B.meta.fold;
+    const CsrPlan& P = sm.plan[cur];
+    const CsrPlan& P1 = sm.plan[cur == 2 ? 0 : cur + 1];
+    CsrPlan& P2 = sm.plan[cur == 0 ? 2 : cur - 1];
+    const int nsteps = P.nsteps, nuniq = B.nuniq, direct = P.direct;
+    const int nuniq_p = Bp.nuniq;
+    const float fold = P.fold;
     const bool slow = b == 0 || nsteps == 0 || fold != 0.0f || direct || prev_direct;
     if (!slow) {
       // ---- boundary: columns that the block that has just run also holds take its values -----------------------------
       const uint32_t uslot_a = smem_addr(B.uslot), keys_a = smem_addr(B.keys), keysp_a = smem_addr(Bp.keys);
       const uint32_t cache_a = smem_addr(cache), cachep_a = smem_addr(cache_p);
-      for (int i = threadIdx.x; i < nuniq; i += CSRB_THREADS) {
-        const int h2 = lds_u16(uslot_a + 2u * (uint32_t)i);
-        const int col = lds_s32(keys_a + 4u * (uint32_t)h2);
-        int h = csrb_hash(col);
-        for (int probe = 0; probe < CSRB_HASH; ++probe) {
-          const int k2 = lds_s32(keysp_a + 4u * (uint32_t)h);
-          if (k2 == col) {
-            sts_f32(cache_a + 4u * (uint32_t)h2, lds_f32(cachep_a + 4u * (uint32_t)h));
-            break;
-          }
-          if (k2 == -1) break;
-          h = (h + 1) & (CSRB_HASH - 1);
+      constexpr int F = 3;  // columns of a thread in flight
+      for (int i0 = threadIdx.x; i0 - (int)threadIdx.x < nuniq; i0 += F * CSRB_THREADS) {
+        int h2[F], col[F], h[F], k2[F];
+        bool seek[F];
+#pragma unroll
+        for (int i = 0; i < F; ++i) {
+          seek[i] = i0 + i * CSRB_THREADS < nuniq;
+          h2[i] = lds_u16(uslot_a + 2u * (uint32_t)(seek[i] ? i0 + i * CSRB_THREADS : 0));
+          k2[i] = -1;
         }
+#pragma unroll
+        for (int i = 0; i < F; ++i) col[i] = lds_s32(keys_a + 4u * (uint32_t)h2[i]);
+#pragma unroll
+        for (int i = 0; i < F; ++i) h[i] = csrb_hash(col[i]);
+        for (int probe = 0; probe < CSRB_HASH; ++probe) {
+#pragma unroll
+          for (int i = 0; i < F; ++i) lds_s32_if(k2[i], keysp_a + 4u * (uint32_t)h[i], seek[i]);
+          bool any = false;
+#pragma unroll
+          for (int i = 0; i < F; ++i) {
+            seek[i] = seek[i] && k2[i] != col[i] && k2[i] != -1;
+            h[i] = seek[i] ? (h[i] + 1) & (CSRB_HASH - 1) : h[i];
+            any |= seek[i];
+          }
+          if (!__any_sync(0xffffffffu, any)) break;
+        }
+        float v[F];
+#pragma unroll
+        for (int i = 0; i < F; ++i) v[i] = lds_f32(cachep_a + 4u * (uint32_t)h[i]);
+#pragma unroll
+        for (int i = 0; i < F; ++i) sts_f32_if(cache_a + 4u * (uint32_t)h2[i], v[i], k2[i] == col[i]);
       }
       __syncthreads();
     } else {
       // ---- slow boundary: write back, fold, read again ------------------------------------------------------------------
       csrb_scatter(Bp, cache_p, u, nuniq_p, threadIdx.x, CSRB_THREADS);
       __syncthreads();
-      if (threadIdx.x == 0) Bp.meta.nuniq = 0;
+      if (threadIdx.x == 0) Bp.nuniq = 0;
       if (nsteps == 0) break;
       if (fold != 0.0f) {
         for (long long c = threadIdx.x; c < p.d; c += CSRB_THREADS) u[c] = __ldcg(u + c) * fold;
@@ -427,17 +699,15 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
       csrb_gather(B, cache, u, nuniq, threadIdx.x, CSRB_THREADS);
       __syncthreads();
     }
-    if (warp != 0) {
+    if (warp > 1) {
       // the block that has just run goes back to u (a slow boundary has done it already: nothing left to do), then its
       // tables and cache take the block after this one
-      csrb_scatter(Bp, cache_p, u, Bp.meta.nuniq, (int)threadIdx.x - 32, CSRB_HELPERS);
-      named_barrier(1, CSRB_HELPERS);
-      if (threadIdx.x == 32) Bp.meta.nuniq = 0;
-      named_barrier(1, CSRB_HELPERS);
-      prepare(Bp, cache_p);
+      prepare(Bp, cache_p, P1);
+    } else if (warp == 1) {
+      plan_next(P2);
     } else if (direct) {
       // ---- a single long row, on global memory ---------------------------------------------------------------
-      const long long g0 = B.gbeg[0], g1 = B.gbeg[1];
+      const long long g0 = P.gbeg[0], g1 = P.gbeg[1];
       float acc = 0.0f;
       for (long long o = g0 + lane; o < g1; o += 32) {
         const int c = p.col_idx[o];
@@ -445,20 +715,23 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
         else set_status(p.status, DEV_BOUNDS, 22, (long long)c);
       }
       acc = warp_sum(acc);
-      const float g = loss_derivative(LOSS, __int_as_float(B.step[0].z), __int_as_float(B.step[0].w) * acc);
+      const float g = loss_derivative(LOSS, __int_as_float(P.step[0].z), __int_as_float(P.step[0].w) * acc);
       if (g != 0.0f) {
-        const float coef = B.eos[0] * g;
+        const float coef = P.eos[0] * g;
         for (long long o = g0 + lane; o < g1; o += 32) {
           const int c = p.col_idx[o];
           if ((unsigned long long)(long long)c < (unsigned long long)p.d) u[c] = fmaf(-coef, p.val[o], __ldcg(u + c));
         }
       }
-    } else if (B.meta.wide) {
-      run_steps(B, cache, nsteps, std::true_type());
     } else {
-      run_steps(B, cache, nsteps, std::false_type());
+      using std::integral_constant;
+      if (P.longest <= 16) run_steps(B, P, cache, integral_constant<int, 4>(), integral_constant<int, 1>(), std::false_type());
+      else if (P.longest <= 32) run_steps(B, P, cache, integral_constant<int, 8>(), integral_constant<int, 1>(), std::false_type());
+      else if (P.longest <= 64) run_steps(B, P, cache, integral_constant<int, 16>(), integral_constant<int, 2>(), std::false_type());
+      else run_steps(B, P, cache, integral_constant<int, 16>(), integral_constant<int, 2>(), std::true_type());
     }
     prev_direct = direct;
+    cur = cur == 2 ? 0 : cur + 1;
     __syncthreads();
   }
   if (warp == 1 && lane == 0) p.scale[j] = sc;

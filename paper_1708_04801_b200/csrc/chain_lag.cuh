@@ -60,7 +60,6 @@
 
 #include "chain_block.cuh"
 #include "chain_mma16.cuh"
-#include "chain_csr_block.cuh"
 
 namespace wpsgd {
 
@@ -134,6 +133,9 @@ struct LagSmem {
 // (two of each where the arriving side can be a block ahead)
 enum { LAG_BAR_GAMMA = 1, LAG_BAR_Q = 3, LAG_BAR_MODEL = 5, LAG_BAR_TEAM = 7, LAG_BAR_START = 15 };
 
+__device__ __forceinline__ void named_barrier(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
 __device__ __forceinline__ void named_arrive(int id, int threads) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
@@ -207,9 +209,9 @@ struct LagWait {
   uint32_t flag, C;
   int polls;  // a poll lasts up to 20 microseconds
   bool dead;
-  __device__ __forceinline__ LagWait(const BlockParams& bp, volatile int* g, uint32_t C_)
-      : status(bp.c.status), flag((uint32_t)__cvta_generic_to_shared((const void*)g)), C(C_), dead(false) {
-    polls = bp.spin_limit < 64 ? 1 : (bp.spin_limit > (1ll << 26) ? 1 << 20 : (int)(bp.spin_limit >> 6));
+  __device__ __forceinline__ LagWait(DevStatus* st, long long spin_limit, volatile int* g, uint32_t C_)
+      : status(st), flag((uint32_t)__cvta_generic_to_shared((const void*)g)), C(C_), dead(false) {
+    polls = spin_limit < 64 ? 1 : (spin_limit > (1ll << 26) ? 1 << 20 : (int)(spin_limit >> 6));
   }
   // the answer of a poll taken earlier (`ok`) decides whether there is anything to wait for
   __device__ __forceinline__ void finish(bool ok, unsigned long long* bar, uint32_t parity, int where) {
@@ -222,35 +224,16 @@ struct LagWait {
   }
 };
 
-// The recurrence warp's loop. Every lane steps through the block redundantly; lane l forms the margin of sample l & 7.
-// r_n = p_n - sum_m beta_m G_mn is the bracket of the blocked form; the loss is taken at sc_n r_n. What is published and
-// kept for the next block is -gamma_m.
+// Registers of the recurrence warp for one block and its eight steps, every lane the same except for the *_own values, which
+// belong to sample lane & 7. r_n = p_n - sum_m beta_m G_mn is the bracket of the blocked form; the loss is taken at sc_n r_n.
 template <int LOSS>
-__device__ __forceinline__ void lag_recurrence(int nb, int TB, int C, int NM, const float* tabs, const LagConst* cst, const float* q,
-                                               const float* qpart, float* gam, float4* jets, unsigned long long* qbar,
-                                               unsigned long long* cempty, LagWait& wait) {
-  constexpr int B = LAG_B;
-  const int lane = threadIdx.x & 31, n = lane & 7;
-  const int bar_threads = 32 * (2 + NM);
-  // where this lane finds its share of the q sums: [slot][sample][4]; slots are the model warps of this CTA, or the CTAs
-  const int slots = C == 1 ? NM : C;
-  const int q_stride = C == 1 ? LAG_MAX_MODEL_WARPS * 32 : C * 32;
-  const float* q_src = (C == 1 ? qpart : q) + (lane >> 3) * 32 + n * 4;
-  const int q_mask = C == 1 ? 1 : LAG_QBUF - 1;
-  const bool have0 = (lane >> 3) < slots, have1 = (lane >> 3) + 4 < slots;
-  float ng[B], ndl_prev = 0.0f;
+struct LagBlock {
+  float G[BLK_PAIRS], ca[LAG_B], cb[LAG_B];
+  float sc_own, ca_own, sc_max;
+  // T: sums of the block, [8][8] Gram entries and [8][8] C^T
+  __device__ __forceinline__ void load(const float* T, const LagConst& K, int n) {
 #pragma unroll
-  for (int m = 0; m < B; ++m) ng[m] = 0.0f;
-  const float* T = tabs;
-  const float* T_end = tabs + TB * LAG_SUMS;
-  named_barrier(LAG_BAR_START, 64);  // sums and constants of block 0
-#pragma unroll 1
-  for (int b = 0; b < nb; ++b) {
-    if (C > 1 && lane == 0 && !wait.dead) mbar_arrive_expect_tx(&qbar[b & (LAG_QBUF - 1)], C * 128u);
-    const LagConst& K = cst[b & (LAG_GROUP * LAG_GROUPS - 1)];
-    float G[BLK_PAIRS], ca[B], cb[B];
-#pragma unroll
-    for (int n2 = 1; n2 < B; ++n2) {
+    for (int n2 = 1; n2 < LAG_B; ++n2) {
       const float4 lo = *(const float4*)&T[n2 * 8];
       const float l4[4] = {lo.x, lo.y, lo.z, lo.w};
 #pragma unroll
@@ -264,14 +247,6 @@ __device__ __forceinline__ void lag_recurrence(int nb, int TB, int C, int NM, co
           if (m < n2) G[n2 * (n2 - 1) / 2 + m] = h4[m - 4];
       }
     }
-    float acc0 = 0.0f, acc1 = 0.0f;
-#pragma unroll
-    for (int m = 0; m < B; m += 2) {
-      acc0 = fmaf(ng[m], T[64 + m * 8 + n], acc0);
-      acc1 = fmaf(ng[m + 1], T[64 + (m + 1) * 8 + n], acc1);
-    }
-    const float na_nv = K.na_nv, ndl_nv = K.ndl_nv;
-    float sc_own = 0.0f, ca_own = 0.0f, sc_max = 0.0f;
     if (LOSS == LOSS_LOGISTIC) {
       sc_own = K.sc[n];
       ca_own = K.a[n];
@@ -284,23 +259,21 @@ __device__ __forceinline__ void lag_recurrence(int nb, int TB, int C, int NM, co
         cb[4 * i] = u.x; cb[4 * i + 1] = u.y; cb[4 * i + 2] = u.z; cb[4 * i + 3] = u.w;
       }
     }
-    const float acc = acc0 + acc1;
-    named_barrier(LAG_BAR_Q + (b & 1), bar_threads);  // q_b is formed (and sent); sums and constants of block b + 1 are there
-    if (C > 1) wait(&qbar[b & (LAG_QBUF - 1)], (uint32_t)(b / LAG_QBUF) & 1u, 4);
-    const float* qs = q_src + (b & q_mask) * q_stride;
-    float4 s4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    if (have0) s4 = *(const float4*)qs;
-    if (have1) {
-      const float4 v = *(const float4*)(qs + 4 * 32);
-      s4.x += v.x; s4.y += v.y; s4.z += v.z; s4.w += v.w;
+  }
+  // sum_m ng_m C[n][m]: what the block before adds to the margin of sample n
+  __device__ __forceinline__ float correction(const float* T, const float (&ng)[LAG_B], int n) const {
+    float acc0 = 0.0f, acc1 = 0.0f;
+#pragma unroll
+    for (int m = 0; m < LAG_B; m += 2) {
+      acc0 = fmaf(ng[m], T[64 + m * 8 + n], acc0);
+      acc1 = fmaf(ng[m + 1], T[64 + (m + 1) * 8 + n], acc1);
     }
-    float qv = (s4.x + s4.y) + (s4.z + s4.w);
-    if (slots > 1) qv += __shfl_xor_sync(0xffffffffu, qv, 8);
-    if (slots > 2) qv += __shfl_xor_sync(0xffffffffu, qv, 16);
-    if (slots == 1) qv = __shfl_sync(0xffffffffu, qv, n);
-    if (slots == 2) qv = __shfl_sync(0xffffffffu, qv, n);
-    const float r_own = fmaf(ndl_prev, qv, qv) + acc;
-    float beta[B];
+    return acc0 + acc1;
+  }
+  // `margin`: for the hinge loss the smallest 2^40 |1 - t| of the samples, how near a decision came to its threshold
+  __device__ __forceinline__ void steps(float r_own, const float* T, const LagConst& K, float4* jets, float (&beta)[LAG_B], float& margin) const {
+    constexpr int B = LAG_B;
+    const int lane = threadIdx.x & 31, n = lane & 7;
     if (LOSS == LOSS_LOGISTIC) {
       // the factor expanded around the block's margins as a cubic in r; beta's constant is in the coefficients
       float4 jet = logistic_jet(sc_own * r_own);
@@ -340,22 +313,75 @@ __device__ __forceinline__ void lag_recurrence(int nb, int TB, int C, int NM, co
       for (int m = 0; m < B; ++m) r[m] = __shfl_sync(0xffffffffu, r_own, m);
 #pragma unroll
       for (int m = 0; m < B; ++m) {
-        if (LOSS == LOSS_HINGE) beta[m] = ca[m] * __saturatef(fmaf(cb[m], r[m], LAG_STEP));  // 1 where sc r < 1, else 0
-        else beta[m] = fmaf(ca[m], r[m], cb[m]);
+        if (LOSS == LOSS_HINGE) {
+          const float far = fmaf(cb[m], r[m], LAG_STEP);
+          beta[m] = ca[m] * __saturatef(far);  // 1 where sc r < 1, else 0
+          margin = m == 0 ? fabsf(far) : fminf(margin, fabsf(far));
+        } else beta[m] = fmaf(ca[m], r[m], cb[m]);
 #pragma unroll
         for (int n2 = m + 1; n2 < B; ++n2) r[n2] = fmaf(-beta[m], G[n2 * (n2 - 1) / 2 + m], r[n2]);
       }
     }
+  }
+};
+// -gamma_0..7 and -delta to the model warps, every value twice: the operand form of the packed FMA
+__device__ __forceinline__ void lag_publish(float* dst, const float (&ng)[LAG_B], float ndl) {
+  float4* gd = (float4*)dst;
+  gd[0] = make_float4(ng[0], ng[0], ng[1], ng[1]);
+  gd[1] = make_float4(ng[2], ng[2], ng[3], ng[3]);
+  gd[2] = make_float4(ng[4], ng[4], ng[5], ng[5]);
+  gd[3] = make_float4(ng[6], ng[6], ng[7], ng[7]);
+  ((float2*)gd)[8] = make_float2(ndl, ndl);
+}
+
+// The recurrence warp's loop. What is published and kept for the next block is -gamma_m.
+template <int LOSS>
+__device__ __forceinline__ void lag_recurrence(int nb, int TB, int C, int NM, const float* tabs, const LagConst* cst, const float* q,
+                                               const float* qpart, float* gam, float4* jets, unsigned long long* qbar,
+                                               unsigned long long* cempty, LagWait& wait) {
+  constexpr int B = LAG_B;
+  const int lane = threadIdx.x & 31, n = lane & 7;
+  const int bar_threads = 32 * (2 + NM);
+  // where this lane finds its share of the q sums: [slot][sample][4]; slots are the model warps of this CTA, or the CTAs
+  const int slots = C == 1 ? NM : C;
+  const int q_stride = C == 1 ? LAG_MAX_MODEL_WARPS * 32 : C * 32;
+  const float* q_src = (C == 1 ? qpart : q) + (lane >> 3) * 32 + n * 4;
+  const int q_mask = C == 1 ? 1 : LAG_QBUF - 1;
+  const bool have0 = (lane >> 3) < slots, have1 = (lane >> 3) + 4 < slots;
+  float ng[B], ndl_prev = 0.0f;
+#pragma unroll
+  for (int m = 0; m < B; ++m) ng[m] = 0.0f;
+  const float* T = tabs;
+  const float* T_end = tabs + TB * LAG_SUMS;
+  named_barrier(LAG_BAR_START, 64);  // sums and constants of block 0
+#pragma unroll 1
+  for (int b = 0; b < nb; ++b) {
+    if (C > 1 && lane == 0 && !wait.dead) mbar_arrive_expect_tx(&qbar[b & (LAG_QBUF - 1)], C * 128u);
+    const LagConst& K = cst[b & (LAG_GROUP * LAG_GROUPS - 1)];
+    LagBlock<LOSS> blk;
+    blk.load(T, K, n);
+    const float acc = blk.correction(T, ng, n);
+    const float na_nv = K.na_nv, ndl_nv = K.ndl_nv;
+    named_barrier(LAG_BAR_Q + (b & 1), bar_threads);  // q_b is formed (and sent); sums and constants of block b + 1 are there
+    if (C > 1) wait(&qbar[b & (LAG_QBUF - 1)], (uint32_t)(b / LAG_QBUF) & 1u, 4);
+    const float* qs = q_src + (b & q_mask) * q_stride;
+    float4 s4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (have0) s4 = *(const float4*)qs;
+    if (have1) {
+      const float4 v = *(const float4*)(qs + 4 * 32);
+      s4.x += v.x; s4.y += v.y; s4.z += v.z; s4.w += v.w;
+    }
+    float qv = (s4.x + s4.y) + (s4.z + s4.w);
+    if (slots > 1) qv += __shfl_xor_sync(0xffffffffu, qv, 8);
+    if (slots > 2) qv += __shfl_xor_sync(0xffffffffu, qv, 16);
+    if (slots == 1) qv = __shfl_sync(0xffffffffu, qv, n);
+    if (slots == 2) qv = __shfl_sync(0xffffffffu, qv, n);
+    const float r_own = fmaf(ndl_prev, qv, qv) + acc;
+    float beta[B], margin;
+    blk.steps(r_own, T, K, jets, beta, margin);
 #pragma unroll
     for (int m = 0; m < B; ++m) ng[m] = beta[m] * na_nv;
-    if (lane == 0) {  // every value twice: the operand form of the packed FMA
-      float4* gd = (float4*)(gam + (b & 1) * LAG_GAM);
-      gd[0] = make_float4(ng[0], ng[0], ng[1], ng[1]);
-      gd[1] = make_float4(ng[2], ng[2], ng[3], ng[3]);
-      gd[2] = make_float4(ng[4], ng[4], ng[5], ng[5]);
-      gd[3] = make_float4(ng[6], ng[6], ng[7], ng[7]);
-      ((float2*)gd)[8] = make_float2(ndl_nv, ndl_nv);
-    }
+    if (lane == 0) lag_publish(gam + (b & 1) * LAG_GAM, ng, ndl_nv);
     named_arrive(LAG_BAR_GAMMA + (b & 1), bar_threads);
     ndl_prev = ndl_nv;
     if ((b & (LAG_GROUP - 1)) == LAG_GROUP - 1 && lane == 0 && !wait.dead) mbar_arrive(&cempty[(b / LAG_GROUP) & (LAG_GROUPS - 1)]);
@@ -474,7 +500,7 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
   __syncthreads();
   cluster_barrier();  // every CTA of the cluster runs and has set up its shared memory
 
-  LagWait wait(bp, give_up, C);
+  LagWait wait(bp.c.status, bp.spin_limit, give_up, C);
   const int place = warp;  // recurrence, model warps, copy, constants, feeder, gram, realign
   const int first_part = 1 + NM;
   const int pl_copy = first_part, pl_const = pl_copy + lp.copy_warps, pl_feed = pl_const + 1, pl_gram = pl_feed + 1,

@@ -994,3 +994,30 @@ def test_csr_rows_without_nonzeros_and_single_nonzero(P):
     wl = wi.Workload("gaps", 1, 8, np.array([0, 5]), np.array([200]), 0.1, 1, 0.05, LOGISTIC, 2, y, row_ptr=rp, col_idx=ci,
                      val=va, w0=torch.full((8,), 0.3))
     assert_parity(P, wl)
+
+
+# ---- CSR kernel: groups of 8 steps, forms by row length, rows at the edges of the chunks ---------------------------------
+@pytest.mark.parametrize("lengths", [(1, 4, 5, 16), (16, 17, 31, 32), (33, 48, 63, 64), (65, 96, 97, 200), (0, 0, 1, 128)])
+@pytest.mark.parametrize("loss", [HINGE, LOGISTIC, SQUARED])
+def test_csr_group_forms(P, lengths, loss):
+    # 16, 32 and 64 nonzeros are the limits of the compiled forms; step counts leave groups of 1, 7 and 8
+    d = 1024
+    rp, ci, va, y = _rows_with_given_lengths(list(lengths) * 3, d, 5)
+    wl = wi.Workload("forms", 3, d, np.array([0, 4, 8, 12]), np.array([135, 96, 49]), 0.2, 1, 0.01, loss, 5, y, row_ptr=rp,
+                     col_idx=ci, val=va, w0=torch.full((d,), 0.01))
+    assert_parity(P, wl, {"sparse_variant": 2})
+
+
+def test_csr_hinge_decisions_at_the_threshold(P):
+    # two rows of the same columns with values chosen so that margins come within rounding of 1: the decisions have to be
+    # those of one step at a time, as in the direct kernel (bit for bit the same models but for the fp64 scale's last bits)
+    d, n = 64, 400
+    g = torch.Generator().manual_seed(2)
+    lengths = [8] * 40
+    rp, ci, va, y = _rows_with_given_lengths(lengths, d, 3)
+    va = (va * (1.0 + 1e-6 * torch.randn(va.shape, generator=g))).contiguous()
+    wl = wi.Workload("ties", 2, d, np.array([0, 20, 40]), np.array([n, n // 2]), 0.25, 0, 0.0, HINGE, 5, y, row_ptr=rp, col_idx=ci, val=va)
+    _, W2, _, _ = gpu_solve(P, wl, {"sparse_variant": 2})
+    _, W1, _, _ = gpu_solve(P, wl, {"sparse_variant": 1})
+    for j in range(2):
+        assert rel_l2(W2[j], W1[j]) <= 1e-6
