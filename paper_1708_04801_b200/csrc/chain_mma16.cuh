@@ -115,7 +115,6 @@ __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const Clust
   const uint32_t* idx = p.idx + p.idx_off[j];  // padded to a multiple of 64 entries, all valid rows
   const long long nb = (n_run + B - 1) / B;
   const int consumed_threads = (math_warps + 1) * 32;  // math warps arrive, the copy warp waits: named barrier 2
-  const int math_threads = math_warps * 32;
 
   // ---- set-up: tables, barriers, zeroed ring / model rows / partial-sum tables ------------------------------------
   if (threadIdx.x <= B) {  // power tables in fp64, rounded once

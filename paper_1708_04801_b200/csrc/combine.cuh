@@ -11,10 +11,18 @@ namespace wpsgd {
 // nodes still fill the machine; the warps' sums are added in warp order, so the result does not depend on timing. The host
 // launches up to 32 warps, four nodes or more each, and takes VEC = 4 when the column count fills the SMs with it.
 // k = 1024, d = 256: 226 us with one thread per column over all nodes, 7 us this way.
-template <int VEC>
-__global__ void __launch_bounds__(1024) combine_kernel(const float* __restrict__ W, const double* __restrict__ weights,
+// N > 0: the weights are the argument `iw` (no copy is enqueued for them), else they lie at `far_weights`.
+template <int N>
+struct InlineWeights {
+  double w[N];
+};
+constexpr int COMBINE_INLINE = 256;
+template <int VEC, int N>
+__global__ void __launch_bounds__(1024) combine_kernel(const __grid_constant__ InlineWeights<(N > 0 ? N : 1)> iw,
+                                                       const float* __restrict__ W, const double* __restrict__ far_weights,
                                                        const double* __restrict__ scale, int k, long long d, float* __restrict__ v) {
   extern __shared__ __align__(16) double sums[];  // [warp][32 VEC]
+  const double* weights = N > 0 ? iw.w : far_weights;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   const long long c = ((long long)blockIdx.x * 32 + lane) * VEC;
   double a[VEC];

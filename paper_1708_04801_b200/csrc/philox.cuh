@@ -93,20 +93,47 @@ __host__ __device__ __forceinline__ void emit_indices(int sampling, uint64_t see
   }
 }
 
-// All nodes' streams for one launch of the chains. Node = blockIdx.y (+ gridDim.y per pass).
-//   idx_off[j]   position of node j's first entry in idx (prefix sums of count)
-//   first[j]     number of steps node j has already run (its entries start at step first[j]+1)
-//   count[j]     entries to produce for node j
-//   rows[j]      shard size m_j
-//   ids[j]       node number that enters the counter (j itself unless the caller renumbers nodes)
-__global__ void index_stream_kernel(int sampling, uint64_t seed, int k, const long long* __restrict__ idx_off,
-                                    const long long* __restrict__ first, const long long* __restrict__ count,
-                                    const long long* __restrict__ rows, const int* __restrict__ ids,
-                                    uint32_t* __restrict__ idx) {
+// Per-node tables of a launch, one after the other in one buffer (built on the host, read by the kernels).
+struct TableLayout {
+  size_t shard_off, steps, first, idx_off, order, ids, total;
+  __host__ __device__ explicit TableLayout(int k) {
+    const size_t n = (size_t)k;
+    shard_off = 0;                                     // [k+1] row offsets
+    steps = shard_off + (n + 1) * sizeof(long long);   // [k] steps of this launch
+    first = steps + n * sizeof(long long);             // [k] steps already run
+    idx_off = first + n * sizeof(long long);           // [k+1] position of the node's stream: prefix sums of stream_entries
+    order = idx_off + (n + 1) * sizeof(long long);     // [k+8] nodes, longest chain first, then -1
+    ids = order + (n + 8) * sizeof(int);               // [k] node numbers that enter the counter
+    total = (ids + n * sizeof(int) + 15) / 16 * 16;
+  }
+};
+// The stream of a node is produced up to the next multiple of 64 steps (the draws simply continue), so that kernels that
+// take samples in groups always read valid rows.
+__host__ __device__ __forceinline__ long long stream_entries(long long steps) { return (steps + 63) / 64 * 64; }
+
+// Tables small enough travel as a kernel argument: no copy is enqueued for them.
+template <int BYTES>
+struct InlineTables {
+  alignas(16) unsigned char b[BYTES];
+};
+
+// All nodes' streams for one launch of the chains. Node = blockIdx.y (+ gridDim.y per pass). BYTES > 0: the tables are the
+// argument `t`, and block (0, 0) writes them to `tables` for the kernels that follow.
+template <int BYTES>
+__global__ void __launch_bounds__(256) index_stream_kernel(const __grid_constant__ InlineTables<(BYTES > 0 ? BYTES : 16)> t, int sampling,
+                                                           uint64_t seed, int k, unsigned char* __restrict__ tables,
+                                                           uint32_t* __restrict__ idx) {
+  const TableLayout L(k);
+  const unsigned char* src = BYTES > 0 ? t.b : tables;
+  if (BYTES > 0 && blockIdx.x == 0 && blockIdx.y == 0)
+    for (size_t i = threadIdx.x; i < L.total / 16; i += blockDim.x) ((uint4*)tables)[i] = ((const uint4*)t.b)[i];
+  const long long *off = (const long long*)(src + L.shard_off), *steps = (const long long*)(src + L.steps),
+                  *first = (const long long*)(src + L.first), *idx_off = (const long long*)(src + L.idx_off);
+  const int* ids = (const int*)(src + L.ids);
   for (int j = blockIdx.y; j < k; j += gridDim.y) {
-    const long long cnt = count[j];
+    const long long cnt = stream_entries(steps[j]);
     if (cnt <= 0) continue;
-    emit_indices(sampling, seed, (uint32_t)ids[j], first[j], cnt, (uint32_t)rows[j], idx + idx_off[j],
+    emit_indices(sampling, seed, (uint32_t)ids[j], first[j], cnt, (uint32_t)(off[j + 1] - off[j]), idx + idx_off[j],
                  (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
   }
 }

@@ -34,16 +34,11 @@ struct wpsgd_ctx {
   float* W = nullptr;       // [k, d]
   double* scale = nullptr;  // [k] (sparse path: w_j = scale_j * W[j])
   bool scaled = false;
-  // per-launch tables on the device
-  long long* t_shard_off = nullptr;  // [k+1]
-  long long* t_steps = nullptr;      // [k]
-  long long* t_first = nullptr;      // [k]
-  long long* t_idx_off = nullptr;    // [k+1]
-  long long* t_rows = nullptr;       // [k]
-  long long* t_count = nullptr;      // [k] entries of the sample stream per node (steps rounded up to 8)
-  int* t_order = nullptr;            // [k]
-  int* t_ids = nullptr;              // [k] node numbers entering the sample stream
-  int* t_group = nullptr;            // [k + 8] node of every (CTA, warp) slot of the warp-per-node blocked kernel
+  // per-launch tables on the device: one buffer laid out by TableLayout(k), and where its parts are
+  unsigned char* tables = nullptr;
+  long long *t_shard_off = nullptr, *t_steps = nullptr, *t_first = nullptr, *t_idx_off = nullptr;
+  int* t_order = nullptr;
+  std::vector<unsigned char> h_tables;
   double* t_weights = nullptr;       // [k]
   uint32_t* idx = nullptr;
   size_t idx_cap = 0;  // entries
@@ -218,27 +213,31 @@ int grid_for(long long work_items, int block, int cap = 148 * 16) {
   return (int)std::max(1ll, std::min<long long>(g, cap));
 }
 
-// v_out = sum_j t_weights[j] scale_j W[j]
-wpsgd_status launch_combine(wpsgd_ctx* c, float* v_out) {
+// v_out = sum_j weights[j] scale_j W[j] (weights HOST)
+template <int VEC, int N>
+wpsgd_status launch_combine_form(wpsgd_ctx* c, const double* weights, float* v_out) {
   const double* scale = c->scaled ? c->scale : nullptr;
-  const int warps = std::max(1, std::min(32, (c->k + 3) / 4));
-  // four columns per thread once that still gives every SM several blocks
-  if (c->d % 4 == 0 && c->d >= 128 * 148 * 2 && aligned16(c->W)) {
-    const int w4 = std::min(warps, 16);  // 64 KB of sums would leave one block per SM
-    const unsigned blocks = (unsigned)((c->d + 127) / 128);
-    combine_kernel<4><<<blocks, 32 * w4, (size_t)w4 * 128 * sizeof(double), c->stream>>>(c->W, c->t_weights, scale, c->k, c->d, v_out);
-  } else {
-    const unsigned blocks = (unsigned)((c->d + 31) / 32);
-    combine_kernel<1><<<blocks, 32 * warps, (size_t)warps * 32 * sizeof(double), c->stream>>>(c->W, c->t_weights, scale, c->k, c->d, v_out);
-  }
+  InlineWeights<(N > 0 ? N : 1)> iw;
+  if (N > 0) memcpy(iw.w, weights, c->k * sizeof(double));
+  else CU_TRY(c, cudaMemcpyAsync(c->t_weights, weights, c->k * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+  const int warps = std::max(1, std::min(VEC == 4 ? 16 : 32, (c->k + 3) / 4));  // (64 KB of sums would leave one block per SM)
+  const unsigned blocks = (unsigned)((c->d + 32 * VEC - 1) / (32 * VEC));
+  combine_kernel<VEC, N><<<blocks, 32 * warps, (size_t)warps * 32 * VEC * sizeof(double), c->stream>>>(iw, c->W, c->t_weights, scale, c->k, c->d, v_out);
   CU_TRY(c, cudaGetLastError());
   c->launches++;
   return WPSGD_OK;
 }
+wpsgd_status launch_combine(wpsgd_ctx* c, const double* weights, float* v_out) {
+  const bool few = c->k <= COMBINE_INLINE;
+  // four columns per thread once that still gives every SM several blocks
+  if (c->d % 4 == 0 && c->d >= 128 * 148 * 2 && aligned16(c->W))
+    return few ? launch_combine_form<4, COMBINE_INLINE>(c, weights, v_out) : launch_combine_form<4, 0>(c, weights, v_out);
+  return few ? launch_combine_form<1, COMBINE_INLINE>(c, weights, v_out) : launch_combine_form<1, 0>(c, weights, v_out);
+}
 
 // ---- common part of run / continue: tables, sample stream ---------------------------------------------
 struct Plan {
-  std::vector<long long> off, steps, first, idx_off, rows, count;
+  std::vector<long long> off, steps, first, idx_off;
   std::vector<int> order;
   long long total = 0;
 };
@@ -252,19 +251,13 @@ wpsgd_status make_plan(wpsgd_ctx* c, const long long* shard_off, const long long
   pl->steps.assign(n_steps, n_steps + k);
   pl->first = first;
   pl->idx_off.assign(k + 1, 0);
-  pl->rows.assign(k, 0);
-  pl->count.assign(k, 0);
   for (int j = 0; j < k; ++j) {
     const long long m = shard_off[j + 1] - shard_off[j];
     if (m < 0) return fail(c, WPSGD_ERR_INVALID_ARG, "shard_off is not non-decreasing");
     if (n_steps[j] < 0) return fail(c, WPSGD_ERR_INVALID_ARG, "negative step count");
     if (n_steps[j] > 0 && m < 1) return fail(c, WPSGD_ERR_INVALID_ARG, "a node with steps has an empty shard");
     if (m > 0xFFFFFFFFll) return fail(c, WPSGD_ERR_INVALID_ARG, "a shard has 2^32 rows or more");
-    pl->rows[j] = m;
-    // the stream of a node is produced up to the next multiple of 64 steps (the draws simply continue), so
-    // that kernels that take samples in groups of 8 or 64 always read valid rows
-    pl->count[j] = (n_steps[j] + 63) / 64 * 64;
-    pl->idx_off[j + 1] = pl->idx_off[j] + pl->count[j];
+    pl->idx_off[j + 1] = pl->idx_off[j] + stream_entries(n_steps[j]);
   }
   pl->total = pl->idx_off[k];
   pl->order.resize(k);
@@ -273,23 +266,50 @@ wpsgd_status make_plan(wpsgd_ctx* c, const long long* shard_off, const long long
   return WPSGD_OK;
 }
 
+// Where the tables' parts are inside the device buffer
+void bind_tables(wpsgd_ctx* c, unsigned char* base) {
+  const TableLayout L(c->k);
+  c->tables = base;
+  c->t_shard_off = (long long*)(base + L.shard_off);
+  c->t_steps = (long long*)(base + L.steps);
+  c->t_first = (long long*)(base + L.first);
+  c->t_idx_off = (long long*)(base + L.idx_off);
+  c->t_order = (int*)(base + L.order);
+}
+
+template <int BYTES>
+void launch_index_stream(wpsgd_ctx* c, dim3 grid, size_t bytes) {
+  InlineTables<(BYTES > 0 ? BYTES : 16)> t;
+  if (BYTES > 0) memcpy(t.b, c->h_tables.data(), bytes);
+  index_stream_kernel<BYTES><<<grid, 256, 0, c->stream>>>(t, c->opt_sampling, c->seed, c->k, c->tables, c->idx);
+}
+
 wpsgd_status upload_plan_and_stream(wpsgd_ctx* c, const Plan& pl) {
   const int k = c->k;
   wpsgd_status s = grow(c, &c->idx, &c->idx_cap, (size_t)std::max(1ll, pl.total));
   if (s != WPSGD_OK) return s;
-  // pageable sources: the copy has left the host buffer when cudaMemcpyAsync returns
-  CU_TRY(c, cudaMemcpyAsync(c->t_shard_off, pl.off.data(), (k + 1) * sizeof(long long), cudaMemcpyHostToDevice, c->stream));
-  CU_TRY(c, cudaMemcpyAsync(c->t_steps, pl.steps.data(), k * sizeof(long long), cudaMemcpyHostToDevice, c->stream));
-  CU_TRY(c, cudaMemcpyAsync(c->t_first, pl.first.data(), k * sizeof(long long), cudaMemcpyHostToDevice, c->stream));
-  CU_TRY(c, cudaMemcpyAsync(c->t_idx_off, pl.idx_off.data(), (k + 1) * sizeof(long long), cudaMemcpyHostToDevice, c->stream));
-  CU_TRY(c, cudaMemcpyAsync(c->t_rows, pl.rows.data(), k * sizeof(long long), cudaMemcpyHostToDevice, c->stream));
-  CU_TRY(c, cudaMemcpyAsync(c->t_count, pl.count.data(), k * sizeof(long long), cudaMemcpyHostToDevice, c->stream));
-  CU_TRY(c, cudaMemcpyAsync(c->t_order, pl.order.data(), k * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  CU_TRY(c, cudaMemcpyAsync(c->t_ids, c->node_ids.data(), k * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+  const TableLayout L(k);
+  c->h_tables.assign(L.total, 0);
+  unsigned char* h = c->h_tables.data();
+  memcpy(h + L.shard_off, pl.off.data(), (k + 1) * sizeof(long long));
+  memcpy(h + L.steps, pl.steps.data(), k * sizeof(long long));
+  memcpy(h + L.first, pl.first.data(), k * sizeof(long long));
+  memcpy(h + L.idx_off, pl.idx_off.data(), (k + 1) * sizeof(long long));
+  int* order = (int*)(h + L.order);
+  std::copy(pl.order.begin(), pl.order.end(), order);
+  std::fill(order + k, order + k + 8, -1);
+  memcpy(h + L.ids, c->node_ids.data(), k * sizeof(int));
+  // Up to 8 KB of tables (some 200 nodes) travel as an argument of the stream kernel, in one of two sizes; the eight copies
+  // this replaces took 14 us of a 53 us round (32 nodes, 250 steps): 848 -> 622 us for 16 rounds.
+  const bool as_argument = pl.total > 0 && L.total <= 8192;
+  // pageable source: the copy has left the host buffer when cudaMemcpyAsync returns
+  if (!as_argument) CU_TRY(c, cudaMemcpyAsync(c->tables, h, L.total, cudaMemcpyHostToDevice, c->stream));
   if (pl.total > 0) {
     const long long longest = *std::max_element(pl.steps.begin(), pl.steps.end());
     dim3 grid((unsigned)grid_for(c->opt_sampling ? longest + 8 : (longest + 3) / 4 + 3, 256, 1024), (unsigned)std::min(k, 65535));
-    index_stream_kernel<<<grid, 256, 0, c->stream>>>(c->opt_sampling, c->seed, k, c->t_idx_off, c->t_first, c->t_count, c->t_rows, c->t_ids, c->idx);
+    if (!as_argument) launch_index_stream<0>(c, grid, 0);
+    else if (L.total <= 2048) launch_index_stream<2048>(c, grid, L.total);
+    else launch_index_stream<8192>(c, grid, L.total);
     CU_TRY(c, cudaGetLastError());
     c->launches++;
   }
@@ -653,18 +673,6 @@ bool block_warp_kernel_fits(const wpsgd_ctx* c, int nk, bool aligned, int* R_out
   return true;
 }
 
-// Nodes of every CTA of the warp-per-node kernel: longest first, consecutive ranks share a CTA; -1 fills the last one.
-wpsgd_status upload_groups(wpsgd_ctx* c, const long long* n_steps_host, int warps, int* ctas_out) {
-  const int k = c->k;
-  const int ctas = (k + warps - 1) / warps;
-  std::vector<int> group((size_t)ctas * warps, -1);
-  std::iota(group.begin(), group.begin() + k, 0);
-  std::stable_sort(group.begin(), group.begin() + k, [&](int a, int b) { return n_steps_host[a] > n_steps_host[b]; });
-  CU_TRY(c, cudaMemcpyAsync(c->t_group, group.data(), group.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  *ctas_out = ctas;
-  return WPSGD_OK;
-}
-
 template <typename XT, int R>
 wpsgd_status launch_block_warp_r(wpsgd_ctx* c, const BlockParams& bp, size_t smem, int ctas, int warps) {
   auto go = [&](auto kern) -> wpsgd_status {
@@ -690,10 +698,8 @@ wpsgd_status launch_block_warp(wpsgd_ctx* c, const ChainParams& p, int R, int st
   bp.eta_lambda = (double)c->eta0 * (double)c->lambda;
   bp.spin_limit = c->opt_spin_limit;
   bp.drop_block = -1;
-  bp.group_order = c->t_group;
-  int ctas = 0;
-  wpsgd_status s = upload_groups(c, c->last_steps.data(), warps, &ctas);
-  if (s != WPSGD_OK) return s;
+  bp.group_order = c->t_order;  // longest first, consecutive ranks share a CTA; -1 fills the last one
+  const int ctas = (c->k + warps - 1) / warps;
   const size_t smem = BlockWarpSmem(stages, (size_t)c->d * sizeof(XT), warps).total;
   return R == 1 ? launch_block_warp_r<XT, 1>(c, bp, smem, ctas, warps) : launch_block_warp_r<XT, 2>(c, bp, smem, ctas, warps);
 }
@@ -1017,16 +1023,8 @@ constexpr size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 struct StaticLayout {
   size_t W = 0;
   size_t idx = align256(W + sizeof(float) * (size_t)WPSGD_STATIC_MAX_MODEL_ELEMS);
-  size_t shard_off = align256(idx + sizeof(uint32_t) * ((size_t)WPSGD_STATIC_MAX_STEPS + 64 * WPSGD_STATIC_MAX_NODES));
-  size_t steps = align256(shard_off + sizeof(long long) * (WPSGD_STATIC_MAX_NODES + 1));
-  size_t first = align256(steps + sizeof(long long) * WPSGD_STATIC_MAX_NODES);
-  size_t idx_off = align256(first + sizeof(long long) * WPSGD_STATIC_MAX_NODES);
-  size_t rows = align256(idx_off + sizeof(long long) * (WPSGD_STATIC_MAX_NODES + 1));
-  size_t count = align256(rows + sizeof(long long) * WPSGD_STATIC_MAX_NODES);
-  size_t order = align256(count + sizeof(long long) * WPSGD_STATIC_MAX_NODES);
-  size_t ids = align256(order + sizeof(int) * WPSGD_STATIC_MAX_NODES);
-  size_t group = align256(ids + sizeof(int) * WPSGD_STATIC_MAX_NODES);
-  size_t weights = align256(group + sizeof(int) * (WPSGD_STATIC_MAX_NODES + 8));
+  size_t tables = align256(idx + sizeof(uint32_t) * ((size_t)WPSGD_STATIC_MAX_STEPS + 64 * WPSGD_STATIC_MAX_NODES));
+  size_t weights = align256(tables + TableLayout(WPSGD_STATIC_MAX_NODES).total);
   size_t scale = align256(weights + sizeof(double) * WPSGD_STATIC_MAX_NODES);
   size_t status = align256(scale + sizeof(double) * WPSGD_STATIC_MAX_NODES);
   size_t total = align256(status + sizeof(DevStatus));
@@ -1094,15 +1092,8 @@ wpsgd_status wpsgd_create(int device, void* cuda_stream, int32_t k, int64_t d, w
   if ((e = cudaMalloc((void**)&(ptr), (bytes))) != cudaSuccess) return bail(e, "cudaMalloc(" #ptr ")");
   ALLOC(c->W, (size_t)k * (size_t)d * sizeof(float));
   ALLOC(c->scale, (size_t)k * sizeof(double));
-  ALLOC(c->t_shard_off, (size_t)(k + 1) * sizeof(long long));
-  ALLOC(c->t_steps, (size_t)k * sizeof(long long));
-  ALLOC(c->t_first, (size_t)k * sizeof(long long));
-  ALLOC(c->t_idx_off, (size_t)(k + 1) * sizeof(long long));
-  ALLOC(c->t_rows, (size_t)k * sizeof(long long));
-  ALLOC(c->t_count, (size_t)k * sizeof(long long));
-  ALLOC(c->t_order, (size_t)k * sizeof(int));
-  ALLOC(c->t_ids, (size_t)k * sizeof(int));
-  ALLOC(c->t_group, ((size_t)k + 8) * sizeof(int));
+  ALLOC(c->tables, TableLayout(k).total);
+  bind_tables(c, c->tables);
   ALLOC(c->t_weights, (size_t)k * sizeof(double));
   ALLOC(c->status, sizeof(DevStatus));
   ALLOC(c->ticket, sizeof(unsigned));
@@ -1117,8 +1108,7 @@ wpsgd_status wpsgd_destroy(wpsgd_ctx* c) {
   if (!c) return WPSGD_OK;
   DeviceGuard guard(c->device);
   cudaStreamSynchronize(c->stream);
-  void* ptrs[] = {c->W, c->scale, c->t_shard_off, c->t_steps, c->t_first, c->t_idx_off, c->t_rows, c->t_count, c->t_order,
-                  c->t_ids, c->t_group, c->t_weights, c->idx, c->status, c->part, c->ticket, c->st_X, c->st_y, c->st_v, c->st_w0, c->st_rp, c->st_ci, c->st_va};
+  void* ptrs[] = {c->W, c->scale, c->tables, c->t_weights, c->idx, c->status, c->part, c->ticket, c->st_X, c->st_y, c->st_v, c->st_w0, c->st_rp, c->st_ci, c->st_va};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->ev0) cudaEventDestroy(c->ev0);
@@ -1298,8 +1288,7 @@ wpsgd_status wpsgd_combine(wpsgd_ctx* c, double r, float* v_out) {
   std::string why;
   wpsgd_status s = weights_host(c->steps_done.data(), c->k, c->eta0, c->sched, c->lambda, r, w.data(), nullptr, nullptr, &why);
   if (s != WPSGD_OK) return fail(c, s, why);
-  CU_TRY(c, cudaMemcpyAsync(c->t_weights, w.data(), c->k * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  return launch_combine(c, v_out);
+  return launch_combine(c, w.data(), v_out);
 }
 
 wpsgd_status wpsgd_combine_weighted(wpsgd_ctx* c, const double* weights, float* v_out) {
@@ -1309,8 +1298,7 @@ wpsgd_status wpsgd_combine_weighted(wpsgd_ctx* c, const double* weights, float* 
   for (int j = 0; j < c->k; ++j)
     if (!std::isfinite(weights[j])) return fail(c, WPSGD_ERR_INVALID_ARG, "a weight is not finite");
   DeviceGuard guard(c->device);
-  CU_TRY(c, cudaMemcpyAsync(c->t_weights, weights, c->k * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  return launch_combine(c, v_out);
+  return launch_combine(c, weights, v_out);
 }
 
 wpsgd_status wpsgd_last_chain_ms(wpsgd_ctx* c, float* ms) {
@@ -1579,15 +1567,7 @@ wpsgd_status wpsgd_solve_static(int device, void* cuda_stream, const void* X, wp
   c.W = (float*)(base + L.W);
   c.idx = (uint32_t*)(base + L.idx);
   c.idx_cap = (size_t)WPSGD_STATIC_MAX_STEPS + 64 * WPSGD_STATIC_MAX_NODES;  // never regrown: padding included
-  c.t_shard_off = (long long*)(base + L.shard_off);
-  c.t_steps = (long long*)(base + L.steps);
-  c.t_first = (long long*)(base + L.first);
-  c.t_idx_off = (long long*)(base + L.idx_off);
-  c.t_rows = (long long*)(base + L.rows);
-  c.t_count = (long long*)(base + L.count);
-  c.t_order = (int*)(base + L.order);
-  c.t_ids = (int*)(base + L.ids);
-  c.t_group = (int*)(base + L.group);
+  bind_tables(&c, base + L.tables);
   c.t_weights = (double*)(base + L.weights);
   c.scale = (double*)(base + L.scale);
   c.status = (DevStatus*)(base + L.status);
