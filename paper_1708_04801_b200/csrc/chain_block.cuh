@@ -47,6 +47,16 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src)
   const uint32_t s = (uint32_t)__cvta_generic_to_shared(smem_dst);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem_src) : "memory");
 }
+// the copy happens where `yes`: a predicate, not a branch (branches inside unrolled code end the stretch in which accesses
+// overlap, and cost more than the accesses)
+__device__ __forceinline__ void cp_async16_if(uint32_t smem_dst, const void* gmem_src, bool yes) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p cp.async.cg.shared.global [%0], [%1], 16;\n\t}" ::"r"(smem_dst), "l"(gmem_src), "r"((int)yes) : "memory");
+}
+__device__ __forceinline__ uint4 lds_u32x4(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+  return v;
+}
 __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gmem_src) {
   const uint32_t s = (uint32_t)__cvta_generic_to_shared(smem_dst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(gmem_src) : "memory");
@@ -345,7 +355,7 @@ __device__ __forceinline__ void block8_recurrence(float (&t)[BLK_B], const float
 
 // Shared-memory carve-up (bytes). Ring first (16-byte aligned), then the small arrays.
 struct BlockSmem {
-  size_t ring, redG, redP, totG, gam, tab, jet, bars, flag, total;
+  size_t ring, redG, redP, totG, gam, tab, jet, bars, flag, zero, total;
   __host__ __device__ BlockSmem(int stages, size_t row_bytes, int math_warps) {
     ring = 0;
     redG = ring + (size_t)stages * BLK_B * row_bytes;
@@ -357,7 +367,8 @@ struct BlockSmem {
     jet = tab + 3 * 16 * sizeof(float);  // 8 x (s, s', s''/2, s'''/6) of the logistic factor
     bars = jet + 8 * 4 * sizeof(float);  // one arrival barrier per ring stage (up to 8)
     flag = bars + 8 * sizeof(unsigned long long);
-    total = flag + 16;
+    zero = flag + 16;  // what threads without columns read
+    total = zero + 16;
   }
 };
 
@@ -404,6 +415,7 @@ __global__ void __launch_bounds__(64 + 32 * MAXW, 1) chain_block_kernel(const Bl
   if (threadIdx.x == 32) {
     for (int s = 0; s < S; ++s) mbar_init(&bars[s], 1);
     *give_up = 0;
+    *(uint4*)(smem + L.zero) = make_uint4(0u, 0u, 0u, 0u);
     mbar_fence_init();
   }
   __syncthreads();  // tables and barriers are set up
@@ -585,15 +597,20 @@ __global__ void __launch_bounds__(64 + 32 * MAXW, 1) chain_block_kernel(const Bl
       *give_up = 1;
     }
   };
-  // this thread's chunks of the 8 rows of a landed block, shared memory -> registers (the only read of them)
+  // this thread's chunks of the 8 rows of a landed block, shared memory -> registers (the only read of them); a chunk
+  // beyond the row is the zero bytes, at strides of zero
+  uint32_t at[R], row_step[R], stage_step[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    at[r] = (uint32_t)__cvta_generic_to_shared(act[r] ? ring + ((size_t)r * TM + tm) * 16 : smem + L.zero);
+    row_step[r] = act[r] ? (uint32_t)row_bytes : 0u;
+    stage_step[r] = act[r] ? (uint32_t)(B * row_bytes) : 0u;
+  }
   auto load_raw = [&](int stg, uint4 (&raw)[R][B]) {
-    const unsigned char* stage = ring + (size_t)stg * B * row_bytes;
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
-      for (int m = 0; m < B; ++m)
-        raw[r][m] = act[r] ? *(const uint4*)(stage + (size_t)m * row_bytes + ((size_t)r * TM + tm) * 16)
-                           : make_uint4(0u, 0u, 0u, 0u);
+      for (int m = 0; m < B; ++m) raw[r][m] = lds_u32x4(at[r] + (uint32_t)stg * stage_step[r] + (uint32_t)m * row_step[r]);
   };
   // Gram partials (and, when WITH_P, p partials against the current model) of the block held in raw
   auto products = [&](const uint4 (&raw)[R][B], float (&acc)[32], float (&accp)[B], bool with_g, bool with_p) {
@@ -741,12 +758,13 @@ namespace wpsgd {
 constexpr int BLKW_MAX_WARPS = 4;  // most nodes per CTA
 
 struct BlockWarpSmem {
-  size_t ring, scratch, tab, total;
+  size_t ring, scratch, tab, zero, total;
   __host__ __device__ BlockWarpSmem(int stages, size_t row_bytes, int warps) {
     ring = 0;
     scratch = ring + (size_t)warps * stages * BLK_B * row_bytes;
     tab = scratch + (size_t)warps * 72 * sizeof(float);
-    total = tab + 3 * 16 * sizeof(float);
+    zero = tab + 3 * 16 * sizeof(float);  // what lanes without columns read
+    total = zero + 16;
   }
 };
 
@@ -754,7 +772,6 @@ struct BlockWarpSmem {
 template <typename XT, int R, int LOSS, bool DECAY>
 __global__ void __launch_bounds__(32 * BLKW_MAX_WARPS) chain_block_warp_kernel(const BlockParams bp) {
   constexpr int V = XVec<XT>::V;
-  constexpr int QV = V / 4;
   constexpr int B = BLK_B;
   extern __shared__ __align__(16) unsigned char smem[];
   const ChainParams& p = bp.c;
@@ -777,6 +794,7 @@ __global__ void __launch_bounds__(32 * BLKW_MAX_WARPS) chain_block_warp_kernel(c
     tab[16 + threadIdx.x] = (float)((double)p.eta0 / (pw * a));
     tab[32 + threadIdx.x] = (float)(1.0 - pw);
   }
+  if (threadIdx.x == 31) *(uint4*)(smem + L.zero) = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();  // the only CTA-wide barrier; every warp passes it exactly once
   // slot -> node table (group_order): the nodes of a CTA are chosen on the host so that every CTA carries about
   // the same total number of steps; -1 marks an unused slot
@@ -818,16 +836,24 @@ __global__ void __launch_bounds__(32 * BLKW_MAX_WARPS) chain_block_warp_kernel(c
       hi = __ldg(q + 1);
     }
   };
+  // this lane's chunks in the ring; a chunk beyond the row is the zero bytes, at strides of zero
+  uint32_t at[R], row_step[R], stage_step[R];
+  const char* src[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    at[r] = (uint32_t)__cvta_generic_to_shared(act[r] ? ring + ((size_t)r * 32 + lane) * 16 : smem + L.zero);
+    row_step[r] = act[r] ? (uint32_t)row_bytes : 0u;
+    stage_step[r] = act[r] ? (uint32_t)(B * row_bytes) : 0u;
+    src[r] = shard + ((size_t)r * 32 + lane) * 16;
+  }
   auto prefetch_block = [&](long long blk, int stg, const uint4& i_lo, const uint4& i_hi) {
     if (blk < nb) {
-      unsigned char* stage = ring + (size_t)stg * B * row_bytes;
       const uint32_t ib[B] = {i_lo.x, i_lo.y, i_lo.z, i_lo.w, i_hi.x, i_hi.y, i_hi.z, i_hi.w};
 #pragma unroll
       for (int m = 0; m < B; ++m) {
-        const char* row = shard + (size_t)ib[m] * ld_bytes;
+        const size_t row = (size_t)ib[m] * ld_bytes;
 #pragma unroll
-        for (int r = 0; r < R; ++r)
-          if (act[r]) cp_async16(stage + (size_t)m * row_bytes + ((size_t)r * 32 + lane) * 16, row + ((size_t)r * 32 + lane) * 16);
+        for (int r = 0; r < R; ++r) cp_async16_if(at[r] + (uint32_t)stg * stage_step[r] + (uint32_t)m * row_step[r], src[r] + row, act[r]);
       }
     }
     cp_async_commit();
@@ -853,15 +879,10 @@ __global__ void __launch_bounds__(32 * BLKW_MAX_WARPS) chain_block_warp_kernel(c
     // ---- rows of block b: shared memory -> registers, then refill the stage --------------------------------
     cp_async_wait(S - 1 < 3 ? S - 1 : 3);  // groups committed: S + b; block b must be complete
     uint4 raw[R][B];
-    {
-      const unsigned char* stage = ring + (size_t)st * B * row_bytes;
 #pragma unroll
-      for (int r = 0; r < R; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int m = 0; m < B; ++m)
-          raw[r][m] = act[r] ? *(const uint4*)(stage + (size_t)m * row_bytes + ((size_t)r * 32 + lane) * 16)
-                             : make_uint4(0u, 0u, 0u, 0u);
-    }
+      for (int m = 0; m < B; ++m) raw[r][m] = lds_u32x4(at[r] + (uint32_t)st * stage_step[r] + (uint32_t)m * row_step[r]);
     prefetch_block(b + S, st, id_lo, id_hi);
     load_ids(b + 1 + S, id_lo, id_hi);
     // ---- G_b and p_b in one pass -----------------------------------------------------------------------

@@ -78,7 +78,8 @@ __device__ __forceinline__ void ldmatrix_x2(uint32_t (&r)[2], const void* smem_p
   asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(a) : "memory");
 }
 
-template <int LOSS>
+// FULL: every math warp of every CTA owns 32 chunks, so that the unrolled pass has no guards (see the note above).
+template <int LOSS, bool FULL>
 __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const ClusterParams cp) {
   constexpr int B = M16_B;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -369,9 +370,9 @@ __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const Clust
   // ============================= math warps ==============================================================
   const int mw = warp - 2;
   const int lc = mw * 32 + lane;  // this thread's 16-byte chunk within the CTA's slice
-  const bool act = lc < my_chunks;
+  const bool act = FULL || lc < my_chunks;
   const int warp_chunks = my_chunks - mw * 32 < 0 ? 0 : (my_chunks - mw * 32 > 32 ? 32 : my_chunks - mw * 32);
-  const int ksteps = (warp_chunks + 1) / 2;  // 16 columns (two chunks) per tensor-core step
+  const int ksteps = FULL ? 16 : (warp_chunks + 1) / 2;  // 16 columns (two chunks) per tensor-core step
   float2 w2[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) w2[i] = make_float2(0.0f, 0.0f);

@@ -519,10 +519,11 @@ wpsgd_status launch_mma(wpsgd_ctx* c, const ChainParams& p, const ClusterShape& 
     return WPSGD_OK;
   };
   if (b16) {
+    const bool full = sh.cpc % 32 == 0 && (long long)sh.cpc * sh.C * 8 == c->d;
     switch (c->loss) {
-      case WPSGD_LOSS_HINGE: return go(chain_mma16_kernel<LOSS_HINGE>);
-      case WPSGD_LOSS_LOGISTIC: return go(chain_mma16_kernel<LOSS_LOGISTIC>);
-      default: return go(chain_mma16_kernel<LOSS_SQUARED>);
+      case WPSGD_LOSS_HINGE: return full ? go(chain_mma16_kernel<LOSS_HINGE, true>) : go(chain_mma16_kernel<LOSS_HINGE, false>);
+      case WPSGD_LOSS_LOGISTIC: return full ? go(chain_mma16_kernel<LOSS_LOGISTIC, true>) : go(chain_mma16_kernel<LOSS_LOGISTIC, false>);
+      default: return full ? go(chain_mma16_kernel<LOSS_SQUARED, true>) : go(chain_mma16_kernel<LOSS_SQUARED, false>);
     }
   }
   switch (c->loss) {
