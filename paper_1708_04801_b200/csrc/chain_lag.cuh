@@ -110,7 +110,7 @@ struct LagSmem {
     part = red + (C > 1 ? (size_t)(stages + 6) * C * LAG_SUMS * sizeof(float) : 0);  // [buffer][CTA][128]
     tabs = part + 2 * (size_t)gram_warps_all * LAG_SUMS * sizeof(float);             // [parity][gram warp][128]
     q = tabs + (size_t)(stages + 4) * LAG_SUMS * sizeof(float);
-    qpart = q + (C > 1 ? LAG_QBUF * (size_t)C * 32 * sizeof(float) : 0);             // [LAG_QBUF][CTA][32]
+    qpart = q + (C > 1 ? LAG_QBUF * LAG_MAX_CLUSTER * 32 * sizeof(float) : 0);       // [LAG_QBUF][8][32]
     cst = qpart + 2 * LAG_MAX_MODEL_WARPS * 32 * sizeof(float);                      // [2][model warp][32]
     gam = cst + LAG_GROUPS * LAG_GROUP * sizeof(LagConst);
     tab = gam + 2 * LAG_GAM * sizeof(float);                                       // powers of 1 - eta lambda
@@ -342,12 +342,11 @@ __device__ __forceinline__ void lag_recurrence(int nb, int TB, int C, int NM, co
   constexpr int B = LAG_B;
   const int lane = threadIdx.x & 31, n = lane & 7;
   const int bar_threads = 32 * (2 + NM);
-  // where this lane finds its share of the q sums: [slot][sample][4]; slots are the model warps of this CTA, or the CTAs
-  const int slots = C == 1 ? NM : C;
-  const int q_stride = C == 1 ? LAG_MAX_MODEL_WARPS * 32 : C * 32;
+  // where this lane finds its share of the q sums: [slot][sample][4]; slots are the model warps of this CTA, or the CTAs, eight
+  // in either case (absent ones are zero)
+  const int q_stride = LAG_MAX_MODEL_WARPS * 32;
   const float* q_src = (C == 1 ? qpart : q) + (lane >> 3) * 32 + n * 4;
   const int q_mask = C == 1 ? 1 : LAG_QBUF - 1;
-  const bool have0 = (lane >> 3) < slots, have1 = (lane >> 3) + 4 < slots;
   float ng[B], ndl_prev = 0.0f;
 #pragma unroll
   for (int m = 0; m < B; ++m) ng[m] = 0.0f;
@@ -365,17 +364,10 @@ __device__ __forceinline__ void lag_recurrence(int nb, int TB, int C, int NM, co
     named_barrier(LAG_BAR_Q + (b & 1), bar_threads);  // q_b is formed (and sent); sums and constants of block b + 1 are there
     if (C > 1) wait(&qbar[b & (LAG_QBUF - 1)], (uint32_t)(b / LAG_QBUF) & 1u, 4);
     const float* qs = q_src + (b & q_mask) * q_stride;
-    float4 s4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    if (have0) s4 = *(const float4*)qs;
-    if (have1) {
-      const float4 v = *(const float4*)(qs + 4 * 32);
-      s4.x += v.x; s4.y += v.y; s4.z += v.z; s4.w += v.w;
-    }
-    float qv = (s4.x + s4.y) + (s4.z + s4.w);
-    if (slots > 1) qv += __shfl_xor_sync(0xffffffffu, qv, 8);
-    if (slots > 2) qv += __shfl_xor_sync(0xffffffffu, qv, 16);
-    if (slots == 1) qv = __shfl_sync(0xffffffffu, qv, n);
-    if (slots == 2) qv = __shfl_sync(0xffffffffu, qv, n);
+    const float4 s4 = *(const float4*)qs, t4 = *(const float4*)(qs + 4 * 32);
+    float qv = ((s4.x + t4.x) + (s4.y + t4.y)) + ((s4.z + t4.z) + (s4.w + t4.w));
+    qv += __shfl_xor_sync(0xffffffffu, qv, 8);
+    qv += __shfl_xor_sync(0xffffffffu, qv, 16);
     const float r_own = fmaf(ndl_prev, qv, qv) + acc;
     float beta[B], margin;
     blk.steps(r_own, T, K, jets, beta, margin);
@@ -565,15 +557,21 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
         }
         if (mw == 0 && !wait.dead) {
           // lane l sends the four values of sample l & 7 to the CTAs l >> 3 and (l >> 3) + 4
-          float4 s = *(const float4*)(qp + (lane & 7) * 4);
-#pragma unroll 1
-          for (int k2 = 1; k2 < NM; ++k2) {
-            const float4 u = *(const float4*)(qp + k2 * 32 + (lane & 7) * 4);
-            s.x += u.x; s.y += u.y; s.z += u.z; s.w += u.w;
+          float4 t[4];  // (rows of absent warps stay zero)
+#pragma unroll
+          for (int k2 = 0; k2 < 4; ++k2) t[k2] = *(const float4*)(qp + k2 * 32 + (lane & 7) * 4);
+          if (NM > 4) {
+#pragma unroll
+            for (int k2 = 0; k2 < 4; ++k2) {
+              const float4 u = *(const float4*)(qp + (k2 + 4) * 32 + (lane & 7) * 4);
+              t[k2].x += u.x; t[k2].y += u.y; t[k2].z += u.z; t[k2].w += u.w;
+            }
           }
+          const float4 s = make_float4((t[0].x + t[1].x) + (t[2].x + t[3].x), (t[0].y + t[1].y) + (t[2].y + t[3].y),
+                                       (t[0].z + t[1].z) + (t[2].z + t[3].z), (t[0].w + t[1].w) + (t[2].w + t[3].w));
           const uint32_t qb = (uint32_t)(blk & (LAG_QBUF - 1));
-          if ((uint32_t)(lane >> 3) < C) st_async_f32x4(q_dst0 + qb * C * 128u, s, q_bar0 + qb * 8u);
-          if ((uint32_t)(lane >> 3) + 4u < C) st_async_f32x4(q_dst1 + qb * C * 128u, s, q_bar1 + qb * 8u);
+          st_async_f32x4_if(q_dst0 + qb * 1024u, s, q_bar0 + qb * 8u, (uint32_t)(lane >> 3) < C);
+          st_async_f32x4_if(q_dst1 + qb * 1024u, s, q_bar1 + qb * 8u, (uint32_t)(lane >> 3) + 4u < C);
         }
       }
       named_arrive(LAG_BAR_Q + (blk & 1), bar_threads);
