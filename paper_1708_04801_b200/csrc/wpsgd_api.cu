@@ -533,12 +533,12 @@ wpsgd_status launch_mma(wpsgd_ctx* c, const ChainParams& p, const ClusterShape& 
   }
 }
 
-// Warp-per-node kernel: one CTA of four warps per SM, or two? A warp alone on its scheduler takes about 2640 cycles
-// per block of 8 samples, two warps sharing one about 3000 each (measured, k = 1024, d = 256). With one CTA per SM
+// Warp-per-node kernel: one CTA of four warps per SM, or two? A warp alone on its scheduler takes about 1990 cycles
+// per block of 8 samples, two warps sharing one about 3500 each (measured, d = 256 fp32). With one CTA per SM
 // there are 148 CTA slots and the remaining CTAs queue behind, longest first; with two there are 296 slots. Which
-// finishes first depends on the step counts (equal work: 3.57 ms with two against 5.28 ms with one; speed ratio 16:
-// 5.69 ms against 4.97 ms), so both schedules are played through on the host: CTAs in launch order (a CTA lasts as long
-// as its longest chain) onto the slot that frees first.
+// finishes first depends on the step counts (k = 1024: equal work is one wave of 3500 against two of 1990; with a speed
+// ratio of 4 one CTA per SM is ahead), so both schedules are played through on the host: CTAs in launch order (a CTA lasts
+// as long as its longest chain) onto the slot that frees first.
 bool two_warp_ctas_per_sm_finish_first(const std::vector<long long>& steps, int warps) {
   std::vector<long long> sorted(steps);
   std::sort(sorted.begin(), sorted.end(), [](long long a, long long b) { return a > b; });
@@ -558,7 +558,7 @@ bool two_warp_ctas_per_sm_finish_first(const std::vector<long long>& steps, int 
     }
     return end;
   };
-  return makespan(2 * 148, 3000.0) < makespan(148, 2640.0);
+  return makespan(2 * 148, 3500.0) < makespan(148, 1990.0);
 }
 
 // ---- blocked kernel with lagged margins ---------------------------------------------------------------------------------
@@ -712,9 +712,9 @@ wpsgd_status launch_block_warp(wpsgd_ctx* c, const ChainParams& p, int R, int st
 //     max( longest queue of a slot x L,  all blocks x I / 148 )  +  start-up of the kernel per wave of chains,
 // with the chains in launch order (longest first) on `slots` slots. The figures are device times of runs of 300 to 4000
 // steps with k = 4 .. 2000 chains (1965 MHz); the estimates come out within about a tenth of the times measured, e.g.
-// (measured, us) fp32 d = 1024, 4000 steps, k = 16: lagged form over 8 CTAs 324, one CTA per chain 541; k = 128: lagged
-// form over 2 CTAs 594, one CTA per chain 544; fp32 d = 128, 1000 steps, k = 200: lagged 76, CTA per chain 101, warp per
-// chain 133; k = 450: 162, 115, 140; k = 2000: 656, 295, 229.
+// (measured, us) fp32 d = 1024, 4000 steps, k = 16: lagged form over 8 CTAs 322, one CTA per chain 464; k = 148: lagged
+// form over 2 CTAs 651, one CTA per chain 467; fp32 d = 128, 1000 steps, k = 200: lagged 73, CTA per chain 96, warp per
+// chain 113; k = 450: 156, 111, 123; k = 2000: 631, 285, 196.
 double run_estimate(const wpsgd_ctx* c, int slots, double L, double I, double start, double restart) {
   const std::vector<long long>& n = c->steps_sorted;
   const size_t k = n.size(), m = (size_t)slots;
@@ -723,6 +723,7 @@ double run_estimate(const wpsgd_ctx* c, int slots, double L, double I, double st
   for (size_t t = 1; t < 4 && t * m < k; ++t) q = std::max(q, (double)(t + 1) * (double)n[t * m]);
   q = std::max(q, c->steps_sum / (double)slots);
   const double waves = (double)((k + m - 1) / m);
+  if (waves > 1.0) q *= 1.06;  // chains of a second wave do not fall into place perfectly
   return std::max(q * L, c->steps_sum * I / 148.0) / 8.0 + start + restart * (waves - 1.0);
 }
 // piecewise linear through (x_i, y_i), x ascending
@@ -739,12 +740,12 @@ double lag_estimate(const wpsgd_ctx* c, const LagShape& sh) {
   constexpr bool F32 = sizeof(XT) == 4;
   const double x = (double)sh.cpc;
   double L;
-  if (F32) L = sh.C == 1 ? through(x, {{8, 860}, {16, 890}, {32, 1030}, {64, 1230}, {128, 1985}, {256, 3836}})
-                         : through(x, {{8, 1010}, {16, 1040}, {32, 1165}, {64, 1465}, {128, 2045}, {256, 4000}});
-  else L = sh.C == 1 ? through(x, {{16, 955}, {32, 1015}, {64, 1180}, {128, 1510}, {256, 2350}})
-                     : through(x, {{8, 1100}, {32, 1250}, {64, 1540}, {128, 1875}, {256, 2900}});
-  if (sh.C == 8) L += 90.0;
-  if (sh.realign) L = std::max(L, 850.0 + 21.0 * x);
+  if (F32) L = sh.C == 1 ? through(x, {{8, 860}, {16, 890}, {32, 990}, {64, 1210}, {128, 1945}, {256, 3800}, {512, 9600}})
+                         : through(x, {{8, 1020}, {16, 1045}, {32, 1155}, {64, 1345}, {128, 2025}, {256, 3890}, {512, 10200}});
+  else L = sh.C == 1 ? through(x, {{8, 955}, {32, 1005}, {64, 1165}, {128, 1460}, {256, 2490}, {512, 7100}})
+                     : through(x, {{8, 1150}, {32, 1245}, {64, 1390}, {128, 1740}, {256, 2670}, {512, 7800}});
+  if (sh.C == 8) L += 80.0;
+  if (sh.realign) L = std::max(L, through(x, {{8, 1150}, {32, 1310}, {64, 1880}, {128, 3050}, {256, 9100}}));
   // resident clusters of 1, 2, 4, 8 CTAs with one CTA per SM
   const int slots = sh.C == 1 ? 148 : (sh.C == 2 ? 74 : (sh.C == 4 ? 36 : 16));
   return run_estimate(c, slots, L, 0.0, 5000.0 + 40.0 * x, 10000.0);
@@ -790,10 +791,14 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
     const int per_sm = std::max(1, std::min(4, (int)(227 * 1024 / (smem + 1024))));
     return run_estimate(c, 148 * per_sm, c->k > 148 && per_sm > 1 ? 1.2 * L : L, I, 0.0, 6000.0);
   };
+  const bool decay = c->sched == WPSGD_LR_INV_SQRT;
   double mma_t = -1.0;
   if (mma_ok) {
-    const double w = (double)mma_shape.cpc, L = through(w, {{64, 1400}, {128, 1520}, {256, 1970}});
-    if (mma_shape.C == 1) mma_t = shared_estimate(Mma16Smem(mma_shape.stages16, (size_t)mma_shape.cpc * 16).total, L, through(w, {{32, 560}, {64, 750}, {128, 1020}, {256, 1970}}));
+    // (guarded passes where some warp is not full; the decaying schedule's tables are formed on the chain's path)
+    const bool full = mma_shape.cpc % 32 == 0 && (long long)mma_shape.cpc * mma_shape.C == chunks;
+    const double w = (double)mma_shape.cpc;
+    const double L = through(w, {{64, 1260}, {128, 1330}, {256, 1820}}) * (full || mma_shape.C > 1 ? 1.0 : 1.14) * (decay ? 1.1 : 1.0);
+    if (mma_shape.C == 1) mma_t = shared_estimate(Mma16Smem(mma_shape.stages16, (size_t)mma_shape.cpc * 16).total, L, through(w, {{32, 620}, {64, 800}, {128, 1090}, {256, 1820}}));
     else mma_t = run_estimate(c, 148 / mma_shape.C, L, 0.0, 0.0, 6000.0);
   }
   if (variant == 0) {
@@ -807,15 +812,15 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
     };
     if (block_warp_ok) {
       // one chain per scheduler or two (see two_warp_ctas_per_sm_finish_first)
-      const double L = F32 ? (chunks <= 32 ? 1925.0 : 2520.0) : (chunks <= 32 ? 1880.0 : 2740.0);
-      const double I = F32 ? (chunks <= 32 ? 430.0 : 570.0) : (chunks <= 32 ? 480.0 : 710.0);
-      offer(true, 5, std::min(run_estimate(c, 592, L, I, 0.0, 6000.0), run_estimate(c, 1184, 1.17 * L, I, 0.0, 6000.0)));
+      const double L = (F32 ? (chunks <= 32 ? 1655.0 : 1990.0) : (chunks <= 32 ? 1700.0 : 2270.0)) * (decay ? 1.25 : 1.0);
+      const double I = (F32 ? (chunks <= 32 ? 365.0 : 446.0) : (chunks <= 32 ? 440.0 : 655.0)) * (decay ? 1.25 : 1.0);
+      offer(true, 5, std::min(run_estimate(c, 592, L, I, 0.0, 6000.0), run_estimate(c, 1184, 1.76 * L, I, 0.0, 6000.0)));
     }
     if (block_ok) {
-      const double L = F32 ? through(x, {{32, 1430}, {64, 1470}, {128, 1745}, {256, 2126}, {512, 3411}})
-                           : through(x, {{64, 1870}, {128, 1965}, {256, 2700}, {512, 4480}});
-      const double I = F32 ? through(x, {{32, 550}, {64, 777}, {128, 1120}, {256, 2126}, {512, 3411}})
-                           : through(x, {{32, 740}, {64, 1034}, {128, 1388}, {256, 2700}, {512, 4480}});
+      const double L = F32 ? through(x, {{32, 1310}, {64, 1320}, {128, 1655}, {256, 1825}, {512, 3140}})
+                           : through(x, {{64, 1780}, {128, 1855}, {256, 2560}, {512, 4250}});
+      const double I = F32 ? through(x, {{32, 530}, {64, 745}, {128, 1080}, {256, 1825}, {512, 3140}})
+                           : through(x, {{32, 730}, {64, 1020}, {128, 1345}, {256, 2560}, {512, 4250}});
       offer(true, 4, shared_estimate(BlockSmem(bstages, (size_t)d * sizeof(XT) + (F32 ? 0 : 16), bthreads / 32 - 2).total, L, I));
     }
     offer(mma_ok, 8, mma_t);
