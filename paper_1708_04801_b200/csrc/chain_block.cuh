@@ -382,6 +382,7 @@ __global__ void __launch_bounds__(64 + 32 * MAXW, 1) chain_block_kernel(const Bl
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int math_warps = (blockDim.x >> 5) - 2;  // warp 0: recurrence, warp 1: row copies, the rest: math
   const int TM = math_warps * 32;
+  kernel_inputs_ready();
   const int S = bp.stages;
   const int j = p.order[blockIdx.x];
   const long long n_run = p.n_steps[j];
@@ -776,6 +777,7 @@ __global__ void __launch_bounds__(32 * BLKW_MAX_WARPS) chain_block_warp_kernel(c
   extern __shared__ __align__(16) unsigned char smem[];
   const ChainParams& p = bp.c;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  kernel_inputs_ready();
   const int S = bp.stages;
   const long long d = p.d;
   const size_t row_bytes = (size_t)d * sizeof(XT);

@@ -43,6 +43,8 @@ struct CsrParams {
 template <int VEC>
 __global__ void csr_init_kernel(float* __restrict__ U, double* __restrict__ scale, const float* __restrict__ w0, int k,
                                 long long d, int keep_models) {
+  kernel_started();
+  kernel_inputs_ready();
   const long long per_row = d / VEC, total = keep_models ? 0 : (long long)k * per_row;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
     const long long c = w0 ? i - row_of(i, per_row) * per_row : 0;
@@ -56,6 +58,7 @@ __global__ void csr_init_kernel(float* __restrict__ U, double* __restrict__ scal
 template <int P>
 __global__ void __launch_bounds__(32) chain_csr_kernel(const CsrParams p) {
   constexpr int Q = 2;  // nonzeros per lane kept in registers (rows up to 64 nonzeros); longer rows loop
+  kernel_inputs_ready();
   const int lane = threadIdx.x;
   const int j = p.order[blockIdx.x];
   const long long n_run = p.n_steps[j];

@@ -185,6 +185,14 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CsrBlockSmem& sm = *reinterpret_cast<CsrBlockSmem*>(smem_raw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i < CSRB_HASH; i += CSRB_THREADS) {
+    sm.buf[0].keys[i] = -1;
+    sm.buf[1].keys[i] = -1;
+    for (int w = 0; w < CSRB_GRAM_WARPS; ++w) sm.dense[w][i] = 0.0f;
+  }
+  if (threadIdx.x < 2) sm.buf[threadIdx.x].nuniq = 0;
+
+  kernel_inputs_ready();
   const int j = p.order[blockIdx.x];
   const long long n_run = p.n_steps[j];
   const long long first = p.resume ? p.first[j] : 0;
@@ -192,13 +200,6 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
   const float* yshard = p.y + p.shard_off[j];
   const uint32_t* idx = p.idx + p.idx_off[j];
   float* u = p.U + (size_t)j * p.d;
-
-  for (int i = threadIdx.x; i < CSRB_HASH; i += CSRB_THREADS) {
-    sm.buf[0].keys[i] = -1;
-    sm.buf[1].keys[i] = -1;
-    for (int w = 0; w < CSRB_GRAM_WARPS; ++w) sm.dense[w][i] = 0.0f;
-  }
-  if (threadIdx.x < 2) sm.buf[threadIdx.x].nuniq = 0;
 
   // ---- plan of the next block (planner warp) -----------------------------------------------------------------------
   long long s_next = 0;                          // first step of the next block to plan

@@ -40,6 +40,7 @@ struct ChainParams {
 template <typename XT, int R, int PF, bool BLOCK_PER_NODE>
 __global__ void __launch_bounds__(BLOCK_PER_NODE ? 512 : 128)
 chain_reg_kernel(const ChainParams p) {
+  kernel_inputs_ready();
   constexpr int V = XVec<XT>::V;
   __shared__ float red[2][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -162,6 +163,7 @@ chain_reg_kernel(const ChainParams p) {
 template <typename XT>
 __global__ void __launch_bounds__(256) chain_generic_kernel(const ChainParams p) {
   __shared__ float red[2][32];
+  kernel_inputs_ready();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int j = p.order[blockIdx.x];
   const long long n_run = p.n_steps[j], n_first = p.first[j], d = p.d;

@@ -422,8 +422,6 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
   const int S = bp.stages, TB = S + 4, GB = S + 6;
   const int NT = lp.gram_teams, NW = lp.gram_warps, NM = lp.model_warps;
   const uint32_t C = cluster_nctarank(), rank = cluster_ctarank();
-  const int j = p.order[blockIdx.x / C];
-  const long long n_run = p.n_steps[j];
   const long long d = p.d;
   const long long c_first = (long long)rank * lp.chunks_per_cta * V;  // first column of the slice
   const long long c_left = d - c_first;
@@ -450,11 +448,6 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
   unsigned long long* cfull = (unsigned long long*)(smem + L.cfull);
   unsigned long long* cempty = (unsigned long long*)(smem + L.cempty);
   volatile int* give_up = (volatile int*)(smem + L.flag);
-  const char* shard = (const char*)p.X + (size_t)p.shard_off[j] * ld_bytes + (size_t)c_first * sizeof(XT);
-  const float* yshard = p.y + p.shard_off[j];
-  const uint32_t* idx = p.idx + p.idx_off[j];  // padded to a multiple of 64 entries, all valid rows
-  const int nb = (int)((n_run + B - 1) / B);  // the host sends chains of up to 2^33 steps here
-
   if (threadIdx.x <= B) {  // power tables in fp64, rounded once
     const double a = 1.0 - bp.eta_lambda;
     double pw = 1.0;
@@ -489,6 +482,13 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
     for (int i = threadIdx.x; i < n16; i += blockDim.x) z[i] = make_uint4(0u, 0u, 0u, 0u);
   }
   fence_proxy_async_shared();
+  kernel_inputs_ready();
+  const int j = p.order[blockIdx.x / C];
+  const long long n_run = p.n_steps[j];
+  const char* shard = (const char*)p.X + (size_t)p.shard_off[j] * ld_bytes + (size_t)c_first * sizeof(XT);
+  const float* yshard = p.y + p.shard_off[j];
+  const uint32_t* idx = p.idx + p.idx_off[j];  // padded to a multiple of 64 entries, all valid rows
+  const int nb = (int)((n_run + B - 1) / B);  // the host sends chains of up to 2^33 steps here
   __syncthreads();
   cluster_barrier();  // every CTA of the cluster runs and has set up its shared memory
 

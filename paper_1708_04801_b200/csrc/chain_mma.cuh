@@ -136,6 +136,7 @@ __global__ void __launch_bounds__(NPL == 4 ? 64 + 32 * 8 : 64 + 32 * 16, 1) chai
   const int math_warps = (blockDim.x >> 5) - 2;
   const int S = bp.stages;
   const uint32_t C = cluster_nctarank(), rank = cluster_ctarank();
+  kernel_inputs_ready();
   const int j = p.order[blockIdx.x / C];
   const long long n_run = p.n_steps[j];
   const long long d = p.d;

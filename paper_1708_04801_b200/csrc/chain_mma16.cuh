@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const Clust
   const int math_warps = (blockDim.x >> 5) - 2;
   const int S = bp.stages;
   const uint32_t C = cluster_nctarank(), rank = cluster_ctarank();
+  kernel_inputs_ready();
   const int j = p.order[blockIdx.x / C];
   const long long n_run = p.n_steps[j];
   const long long d = p.d;

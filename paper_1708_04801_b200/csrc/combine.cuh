@@ -23,6 +23,8 @@ __global__ void __launch_bounds__(1024) combine_kernel(const __grid_constant__ I
                                                        const double* __restrict__ scale, int k, long long d, float* __restrict__ v) {
   extern __shared__ __align__(16) double sums[];  // [warp][32 VEC]
   const double* weights = N > 0 ? iw.w : far_weights;
+  kernel_started();
+  kernel_inputs_ready();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   const long long c = ((long long)blockIdx.x * 32 + lane) * VEC;
   double a[VEC];
@@ -58,6 +60,8 @@ __global__ void __launch_bounds__(1024) combine_kernel(const __grid_constant__ I
 template <int VEC>
 __global__ void export_models_kernel(const float* __restrict__ W, const double* __restrict__ scale, int k, long long d,
                                      float* __restrict__ out) {
+  kernel_started();
+  kernel_inputs_ready();
   const long long per_row = d / VEC, total = (long long)k * per_row;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
     const double s = scale ? scale[row_of(i, per_row)] : 1.0;
@@ -75,6 +79,8 @@ __global__ void export_models_kernel(const float* __restrict__ W, const double* 
 template <int VEC>
 __global__ void broadcast_model_kernel(float* __restrict__ W, double* __restrict__ scale, const float* __restrict__ v,
                                        int k, long long d) {
+  kernel_started();
+  kernel_inputs_ready();
   const long long per_row = d / VEC, total = (long long)k * per_row;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
     const long long c = i - row_of(i, per_row) * per_row;
@@ -154,6 +160,8 @@ __global__ void __launch_bounds__(256) objective_rows_kernel(const XT* __restric
                                                              long long n_rows, const float* __restrict__ w, long long d,
                                                              int loss, float lambda, double* __restrict__ part, unsigned* ticket,
                                                              double* __restrict__ out) {
+  kernel_started();
+  kernel_inputs_ready();
   constexpr int V = XVec<XT>::V;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double lsum = 0.0, esum = 0.0;
@@ -208,6 +216,8 @@ __global__ void __launch_bounds__(256) objective_rows_csr_kernel(const long long
                                                                  long long n_rows, const float* __restrict__ w, long long d,
                                                                  int loss, float lambda, double* __restrict__ part, unsigned* ticket,
                                                                  double* __restrict__ out) {
+  kernel_started();
+  kernel_inputs_ready();
   const int l8 = threadIdx.x & 7;
   double lsum = 0.0, esum = 0.0;
   // the same trip count for all rows of a warp (shuffles)
@@ -235,6 +245,8 @@ __global__ void __launch_bounds__(256) objective_rows_csr_kernel(const long long
 // 32 column range, 33 column order; detail = the row). Nothing is read outside [0, nnz).
 __global__ void validate_csr_kernel(const long long* __restrict__ row_ptr, const int* __restrict__ col_idx, long long n_rows,
                                     long long nnz, long long d, DevStatus* status) {
+  kernel_started();
+  kernel_inputs_ready();
   const int lane = threadIdx.x & 31;
   const long long warp0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;

@@ -123,6 +123,8 @@ template <int BYTES>
 __global__ void __launch_bounds__(256) index_stream_kernel(const __grid_constant__ InlineTables<(BYTES > 0 ? BYTES : 16)> t, int sampling,
                                                            uint64_t seed, int k, unsigned char* __restrict__ tables,
                                                            uint32_t* __restrict__ idx) {
+  kernel_started();
+  kernel_inputs_ready();
   const TableLayout L(k);
   const unsigned char* src = BYTES > 0 ? t.b : tables;
   if (BYTES > 0 && blockIdx.x == 0 && blockIdx.y == 0)
@@ -141,6 +143,8 @@ __global__ void __launch_bounds__(256) index_stream_kernel(const __grid_constant
 // One node's stream, for callers that want to look at it.
 __global__ void index_single_kernel(int sampling, uint64_t seed, int node, long long m, long long n_begin,
                                     long long count, uint32_t* __restrict__ out) {
+  kernel_started();
+  kernel_inputs_ready();
   if (count > 0)
     emit_indices(sampling, seed, (uint32_t)node, n_begin, count, (uint32_t)m, out,
                  (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);

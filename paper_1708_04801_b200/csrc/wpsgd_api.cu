@@ -206,6 +206,22 @@ wpsgd_status read_status(wpsgd_ctx* c, DevStatus* dev_status, cudaStream_t strea
   return fail(c, h.code == DEV_TIMEOUT ? WPSGD_ERR_TIMEOUT : WPSGD_ERR_CUDA, buf);
 }
 
+// Kernel launch that may start while the kernel before it on the stream ends (see kernel_started in common.cuh).
+template <typename... P, typename... A>
+cudaError_t launch(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
+
 bool aligned16(const void* p) { return (uintptr_t)p % 16 == 0; }
 
 int grid_for(long long work_items, int block, int cap = 148 * 16) {
@@ -222,7 +238,7 @@ wpsgd_status launch_combine_form(wpsgd_ctx* c, const double* weights, float* v_o
   else CU_TRY(c, cudaMemcpyAsync(c->t_weights, weights, c->k * sizeof(double), cudaMemcpyHostToDevice, c->stream));
   const int warps = std::max(1, std::min(VEC == 4 ? 16 : 32, (c->k + 3) / 4));  // (64 KB of sums would leave one block per SM)
   const unsigned blocks = (unsigned)((c->d + 32 * VEC - 1) / (32 * VEC));
-  combine_kernel<VEC, N><<<blocks, 32 * warps, (size_t)warps * 32 * VEC * sizeof(double), c->stream>>>(iw, c->W, c->t_weights, scale, c->k, c->d, v_out);
+  launch(combine_kernel<VEC, N>, blocks, 32 * warps, (size_t)warps * 32 * VEC * sizeof(double), c->stream, iw, c->W, c->t_weights, scale, c->k, c->d, v_out);
   CU_TRY(c, cudaGetLastError());
   c->launches++;
   return WPSGD_OK;
@@ -281,7 +297,7 @@ template <int BYTES>
 void launch_index_stream(wpsgd_ctx* c, dim3 grid, size_t bytes) {
   InlineTables<(BYTES > 0 ? BYTES : 16)> t;
   if (BYTES > 0) memcpy(t.b, c->h_tables.data(), bytes);
-  index_stream_kernel<BYTES><<<grid, 256, 0, c->stream>>>(t, c->opt_sampling, c->seed, c->k, c->tables, c->idx);
+  launch(index_stream_kernel<BYTES>, grid, 256, 0, c->stream, t, c->opt_sampling, c->seed, c->k, c->tables, c->idx);
 }
 
 wpsgd_status upload_plan_and_stream(wpsgd_ctx* c, const Plan& pl) {
@@ -347,10 +363,10 @@ wpsgd_status timing_end(wpsgd_ctx* c) {
 template <typename XT, int R, int PF>
 wpsgd_status launch_reg(wpsgd_ctx* c, const ChainParams& p, bool block_per_node, int threads) {
   if (block_per_node) {
-    chain_reg_kernel<XT, R, PF, true><<<p.k, threads, 0, c->stream>>>(p);
+    launch(chain_reg_kernel<XT, R, PF, true>, p.k, threads, 0, c->stream, p);
   } else {
     const int nodes_per_cta = 4;
-    chain_reg_kernel<XT, R, PF, false><<<(p.k + nodes_per_cta - 1) / nodes_per_cta, 32 * nodes_per_cta, 0, c->stream>>>(p);
+    launch(chain_reg_kernel<XT, R, PF, false>, (p.k + nodes_per_cta - 1) / nodes_per_cta, 32 * nodes_per_cta, 0, c->stream, p);
   }
   CU_TRY(c, cudaGetLastError());
   c->launches++;
@@ -401,7 +417,7 @@ template <typename XT, int R, bool OVL, int MAXW>
 wpsgd_status launch_block_r(wpsgd_ctx* c, const BlockParams& bp, int threads, size_t smem) {
   auto go = [&](auto kern) -> wpsgd_status {
     CU_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kern<<<bp.c.k, threads, smem, c->stream>>>(bp);
+    launch(kern, bp.c.k, threads, smem, c->stream, bp);
     CU_TRY(c, cudaGetLastError());
     c->launches++;
     return WPSGD_OK;
@@ -507,13 +523,15 @@ wpsgd_status launch_mma(wpsgd_ctx* c, const ChainParams& p, const ClusterShape& 
     cfg.blockDim = dim3((unsigned)(64 + 32 * sh.math_warps));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = c->stream;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)sh.C;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     CU_TRY(c, cudaLaunchKernelEx(&cfg, kern, cp));
     c->launches++;
     return WPSGD_OK;
@@ -627,13 +645,15 @@ wpsgd_status launch_lag(wpsgd_ctx* c, const ChainParams& p, const LagShape& sh) 
     cfg.blockDim = dim3((unsigned)(32 * sh.warps));
     cfg.dynamicSmemBytes = sh.smem;
     cfg.stream = c->stream;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)sh.C;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     CU_TRY(c, cudaLaunchKernelEx(&cfg, kern, lp));
     c->launches++;
     return WPSGD_OK;
@@ -678,7 +698,7 @@ template <typename XT, int R>
 wpsgd_status launch_block_warp_r(wpsgd_ctx* c, const BlockParams& bp, size_t smem, int ctas, int warps) {
   auto go = [&](auto kern) -> wpsgd_status {
     CU_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kern<<<ctas, 32 * warps, smem, c->stream>>>(bp);
+    launch(kern, ctas, 32 * warps, smem, c->stream, bp);
     CU_TRY(c, cudaGetLastError());
     c->launches++;
     return WPSGD_OK;
@@ -879,7 +899,7 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
   if (variant == 3 && chunks > 32 * 4) return fail(c, WPSGD_ERR_UNSUPPORTED, "warp-per-node kernel: d too large");
   if (variant == 2 && chunks > 512 * 4) return fail(c, WPSGD_ERR_UNSUPPORTED, "CTA-per-node kernel: d too large");
   if (variant == 1) {
-    chain_generic_kernel<XT><<<p.k, 256, 0, c->stream>>>(p);
+    launch(chain_generic_kernel<XT>, p.k, 256, 0, c->stream, p);
     CU_TRY(c, cudaGetLastError());
     c->launches++;
     return WPSGD_OK;
@@ -975,9 +995,9 @@ wpsgd_status run_csr_common(wpsgd_ctx* c, const long long* row_ptr, const int* c
     // fresh chains start from w0 with scale 1; chains continued from a dense run keep their models and get scale 1
     const long long n = (long long)c->k * c->d;
     if (c->d % 4 == 0 && aligned16(c->W) && aligned16(w0))
-      csr_init_kernel<4><<<grid_for(n / 4, 256), 256, 0, c->stream>>>(c->W, c->scale, w0, c->k, c->d, resume ? 1 : 0);
+      launch(csr_init_kernel<4>, grid_for(n / 4, 256), 256, 0, c->stream, c->W, c->scale, w0, c->k, c->d, resume ? 1 : 0);
     else
-      csr_init_kernel<1><<<grid_for(n, 256), 256, 0, c->stream>>>(c->W, c->scale, w0, c->k, c->d, resume ? 1 : 0);
+      launch(csr_init_kernel<1>, grid_for(n, 256), 256, 0, c->stream, c->W, c->scale, w0, c->k, c->d, resume ? 1 : 0);
     CU_TRY(c, cudaGetLastError());
     c->launches++;
   }
@@ -991,15 +1011,15 @@ wpsgd_status run_csr_common(wpsgd_ctx* c, const long long* row_ptr, const int* c
   if (s != WPSGD_OK) return s;
   if (c->opt_sparse_variant == 1) {
     const int pf = c->opt_prefetch > 0 ? c->opt_prefetch : 4;
-    if (pf >= 8) chain_csr_kernel<8><<<c->k, 32, 0, c->stream>>>(p);
-    else if (pf >= 4) chain_csr_kernel<4><<<c->k, 32, 0, c->stream>>>(p);
-    else chain_csr_kernel<2><<<c->k, 32, 0, c->stream>>>(p);
+    if (pf >= 8) launch(chain_csr_kernel<8>, c->k, 32, 0, c->stream, p);
+    else if (pf >= 4) launch(chain_csr_kernel<4>, c->k, 32, 0, c->stream, p);
+    else launch(chain_csr_kernel<2>, c->k, 32, 0, c->stream, p);
     CU_TRY(c, cudaGetLastError());
   } else {
     const size_t smem = sizeof(CsrBlockSmem);
     auto go = [&](auto kern) -> wpsgd_status {
       CU_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      kern<<<c->k, CSRB_THREADS, smem, c->stream>>>(p);
+      launch(kern, c->k, CSRB_THREADS, smem, c->stream, p);
       CU_TRY(c, cudaGetLastError());
       return WPSGD_OK;
     };
@@ -1279,7 +1299,7 @@ wpsgd_status wpsgd_validate_csr(wpsgd_ctx* c, const int64_t* row_ptr, const int3
   if (n_rows < 0 || nnz < 0 || !row_ptr || (nnz > 0 && !col_idx)) return fail(c, WPSGD_ERR_INVALID_ARG, "validate_csr: bad argument");
   if (n_rows == 0) return WPSGD_OK;
   DeviceGuard guard(c->device);
-  validate_csr_kernel<<<grid_for(n_rows, 8), 256, 0, c->stream>>>((const long long*)row_ptr, col_idx, n_rows, nnz, c->d, c->status);
+  launch(validate_csr_kernel, grid_for(n_rows, 8), 256, 0, c->stream, (const long long*)row_ptr, col_idx, n_rows, nnz, c->d, c->status);
   CU_TRY(c, cudaGetLastError());
   c->launches++;
   return WPSGD_OK;
@@ -1324,9 +1344,9 @@ wpsgd_status wpsgd_get_models(wpsgd_ctx* c, float* W_out) {
   const double* scale = c->scaled ? c->scale : nullptr;
   const long long n = (long long)c->k * c->d;
   if (c->d % 4 == 0 && aligned16(c->W) && aligned16(W_out))
-    export_models_kernel<4><<<grid_for(n / 4, 256), 256, 0, c->stream>>>(c->W, scale, c->k, c->d, W_out);
+    launch(export_models_kernel<4>, grid_for(n / 4, 256), 256, 0, c->stream, c->W, scale, c->k, c->d, W_out);
   else
-    export_models_kernel<1><<<grid_for(n, 256), 256, 0, c->stream>>>(c->W, scale, c->k, c->d, W_out);
+    launch(export_models_kernel<1>, grid_for(n, 256), 256, 0, c->stream, c->W, scale, c->k, c->d, W_out);
   CU_TRY(c, cudaGetLastError());
   c->launches++;
   return WPSGD_OK;
@@ -1339,9 +1359,9 @@ wpsgd_status wpsgd_set_models(wpsgd_ctx* c, const float* v) {
   DeviceGuard guard(c->device);
   const long long n = (long long)c->k * c->d;
   if (c->d % 4 == 0 && aligned16(c->W) && aligned16(v))
-    broadcast_model_kernel<4><<<grid_for(n / 4, 256), 256, 0, c->stream>>>(c->W, c->scale, v, c->k, c->d);
+    launch(broadcast_model_kernel<4>, grid_for(n / 4, 256), 256, 0, c->stream, c->W, c->scale, v, c->k, c->d);
   else
-    broadcast_model_kernel<1><<<grid_for(n, 256), 256, 0, c->stream>>>(c->W, c->scale, v, c->k, c->d);
+    launch(broadcast_model_kernel<1>, grid_for(n, 256), 256, 0, c->stream, c->W, c->scale, v, c->k, c->d);
   CU_TRY(c, cudaGetLastError());
   c->launches++;
   return WPSGD_OK;
@@ -1355,7 +1375,7 @@ wpsgd_status wpsgd_sample_indices(wpsgd_ctx* c, uint64_t seed, int32_t node, int
   if (count == 0) return WPSGD_OK;
   if (!out) return fail(c, WPSGD_ERR_INVALID_ARG, "out is NULL");
   DeviceGuard guard(c->device);
-  index_single_kernel<<<grid_for(c->opt_sampling ? count : (count + 3) / 4 + 1, 256), 256, 0, c->stream>>>(c->opt_sampling, seed, node, m, n_begin, count, out);
+  launch(index_single_kernel, grid_for(c->opt_sampling ? count : (count + 3) / 4 + 1, 256), 256, 0, c->stream, c->opt_sampling, seed, node, m, n_begin, count, out);
   CU_TRY(c, cudaGetLastError());
   c->launches++;
   return WPSGD_OK;
@@ -1372,7 +1392,7 @@ wpsgd_status wpsgd_objective(wpsgd_ctx* c, const void* X, wpsgd_xtype xt, int64_
   wpsgd_status s = grow(c, &c->part, &c->part_cap, (size_t)nblk * 3);
   if (s != WPSGD_OK) return s;
   auto go = [&](auto kern, const auto* rows) {
-    kern<<<nblk, 256, 0, c->stream>>>(rows, ld_elems, y, n_rows, w, c->d, (int)loss, lambda, c->part, c->ticket, out);
+    launch(kern, nblk, 256, 0, c->stream, rows, ld_elems, y, n_rows, w, c->d, (int)loss, lambda, c->part, c->ticket, out);
   };
   const size_t es = xt == WPSGD_X_F32 ? 4 : 2;
   const bool vec = aligned16(X) && aligned16(w) && ((size_t)ld_elems * es) % 16 == 0 && ((size_t)c->d * es) % 16 == 0;
@@ -1393,7 +1413,7 @@ wpsgd_status wpsgd_objective_csr(wpsgd_ctx* c, const int64_t* row_ptr, const int
   const int nblk = grid_for((n_rows + 31) / 32, 1, 148 * 8);
   wpsgd_status s = grow(c, &c->part, &c->part_cap, (size_t)nblk * 3);
   if (s != WPSGD_OK) return s;
-  objective_rows_csr_kernel<<<nblk, 256, 0, c->stream>>>((const long long*)row_ptr, col_idx, val, y, n_rows, w, c->d, (int)loss, lambda,
+  launch(objective_rows_csr_kernel, nblk, 256, 0, c->stream, (const long long*)row_ptr, col_idx, val, y, n_rows, w, c->d, (int)loss, lambda,
                                                          c->part, c->ticket, out);
   CU_TRY(c, cudaGetLastError());
   c->launches++;
