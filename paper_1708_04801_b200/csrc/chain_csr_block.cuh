@@ -20,6 +20,12 @@
 // registers (the recurrence of chain_lag.cuh) and applies the 8 updates one after the other (a column of several
 // samples must see them in turn). All of it is in shared memory.
 //
+// Short form (blocks of at most 640 nonzeros in rows of at most 32). Most columns are held by one row of a group only. The
+// helpers find the ones that several rows hold and give each a record with its value in all 8 rows; the products come from the
+// records alone. After the 8 steps the lane that read a column's entry for the margins writes it back, and one lane per record
+// applies all rows' updates in order: two passes where the long form makes eight. Why the limit: longer blocks take longer
+// this way, their helpers being the longer side (see form_short).
+//
 // For the hinge loss a decision within 1e-4 of its threshold sends the group through one step at a time, so that the order of
 // the sums never turns it.
 //
@@ -27,7 +33,8 @@
 // nonzeros per row, d = 2^20, hinge, 64 chains: 2685 (one step after the other, each with a gather, a sum over 32 lanes and a
 // scatter: 3840); 5 to 10 nonzeros, d = 100000, logistic, 10 chains: 1615 (3700). With short rows the chain warp's string is
 // the longer side: margins 160, steps 500, updates 300, boundary 130 of the 1500. With long rows the chain (2400) and the
-// helpers (insertion 700, products 1100, copies 400 per group) take about as long. Tried and taken back: margins from
+// helpers (insertion 700, products 1100, copies 400 per group) take about as long; the short form took 1615 to 1230 and, at 8
+// Zipf-distributed nonzeros, 1480 to 1270. Tried and taken back: margins from
 // the model one group back with a table per group and the model in L2 (5900 and 3300: everything that touches single
 // nonzeros is latency, and a table per 8 rows pays it eight times as often as one per block).
 //
@@ -63,6 +70,10 @@ constexpr int CSRB_HASH_BITS = 12;
 constexpr int CSRB_THREADS = 384;       // warp 0: chain; warp 1: plans; warps 2..11: preparation
 constexpr int CSRB_HELPERS = CSRB_THREADS - 64;
 constexpr int CSRB_GRAM_WARPS = 6;      // helper warps that also form the products of a group's rows
+constexpr int CSRB_SHORT_ENT = 2 * CSRB_HELPERS;  // blocks of at most that many nonzeros in rows of at most
+constexpr int CSRB_SHORT_ROW = 32;      // these take the short form
+constexpr int CSRB_SLOT = CSRB_HASH - 1;  // bits of a nonzero's slot entry: the slot,
+constexpr int CSRB_SHARED = 0x8000;     // and (short form) whether another row of its group holds the column
 constexpr float CSRB_NEAR = 1e-4f;      // hinge decisions with |1 - t| below this are taken one step at a time
 constexpr int CSRB_BATCH = 8;           // independent global loads a thread keeps in flight
 
@@ -77,7 +88,8 @@ struct CsrPlan {
   float eos[CSRB_STEPS];               // eta_n / scale after the step
   LagConst k[CSRB_GROUPS];             // constants of a group of 8 steps
   int longest;                         // most nonzeros of a row of the block
-  int pad[3];
+  int brief;                           // the block takes the short form
+  int pad[2];
 };
 
 // One buffer of a prepared block.
@@ -87,6 +99,12 @@ struct CsrBlockBuf {
   unsigned short slot[CSRB_EMAX];      // slot of every nonzero
   unsigned short uslot[CSRB_EMAX];     // the occupied slots, in order of first insertion
   float gram[CSRB_GROUPS][64];         // products of the rows of a group, [8][8], below the diagonal
+  union {
+    int col[CSRB_EMAX];                // columns of the nonzeros, until they have their slots
+    float shared_x[CSRB_SHORT_ENT / 2][8];  // short form: value of every shared column in each of the 8 rows of its group,
+  };
+  unsigned short shared_slot[CSRB_SHORT_ENT / 2];  // its slot,
+  int2 records[CSRB_GROUPS];           // first shared column of a group and how many
   int nuniq;                           // distinct columns (filled while inserting; 0 again once the block has been written back)
   int pad[3];
 };
@@ -95,8 +113,9 @@ struct CsrBlockSmem {
   CsrBlockBuf buf[2];
   CsrPlan plan[3];
   float ucache[2][CSRB_HASH];          // u at the columns of a block, by slot
-  int colbuf[CSRB_EMAX];               // columns of the block being prepared
   float dense[CSRB_GRAM_WARPS][CSRB_HASH];  // one row at a time, by slot; zero in between
+  unsigned votes[32];                  // per 32 nonzeros: which are the first of a shared column in their group
+  int before[32];                      // how many there are before these
   float4 jets[8];
 };
 
@@ -118,6 +137,16 @@ __device__ __forceinline__ int lds_u16(uint32_t a) {
   asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
   return (int)v;
 }
+__device__ __forceinline__ int lds_u8(uint32_t a) {
+  int v;
+  asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ int2 lds_s32x2(uint32_t a) {
+  int2 v;
+  asm volatile("ld.shared.v2.s32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+  return v;
+}
 __device__ __forceinline__ int4 lds_s32x4(uint32_t a) {
   int4 v;
   asm volatile("ld.shared.v4.s32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
@@ -137,6 +166,21 @@ __device__ __forceinline__ void atoms_cas_if(int& old, uint32_t a, int cmp, int 
 }
 __device__ __forceinline__ void lds_s32_if(int& v, uint32_t a, bool yes) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p ld.shared.s32 %0, [%1];\n\t}" : "+r"(v) : "r"(a), "r"((int)yes) : "memory");
+}
+__device__ __forceinline__ void sts_u16_if(uint32_t a, int v, bool yes) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p st.shared.u16 [%0], %1;\n\t}" ::"r"(a), "h"((unsigned short)v), "r"((int)yes) : "memory");
+}
+__device__ __forceinline__ void reds_or_if(uint32_t a, uint32_t v, bool yes) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p red.shared.or.b32 [%0], %1;\n\t}" ::"r"(a), "r"(v), "r"((int)yes) : "memory");
+}
+__device__ __forceinline__ void sts_u8_if(uint32_t a, int v, bool yes) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p st.shared.u8 [%0], %1;\n\t}" ::"r"(a), "r"(v), "r"((int)yes) : "memory");
+}
+__device__ __forceinline__ void sts_zero32_if(uint32_t a, bool yes) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p st.shared.v4.f32 [%0], {%1, %1, %1, %1};\n\t@p st.shared.v4.f32 [%0+16], {%1, %1, %1, %1};\n\t}" ::"r"(a), "f"(0.0f), "r"((int)yes) : "memory");
+}
+__device__ __forceinline__ void prefetch_l2_if(const void* a, bool yes) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %1, 0;\n\t@p prefetch.global.L2 [%0];\n\t}" ::"l"(a), "r"((int)yes) : "memory");
 }
 __device__ __forceinline__ void sts_f32_if(uint32_t a, float v, bool yes) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p st.shared.f32 [%0], %1;\n\t}" ::"r"(a), "f"(v), "r"((int)yes) : "memory");
@@ -185,13 +229,6 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CsrBlockSmem& sm = *reinterpret_cast<CsrBlockSmem*>(smem_raw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < CSRB_HASH; i += CSRB_THREADS) {
-    sm.buf[0].keys[i] = -1;
-    sm.buf[1].keys[i] = -1;
-    for (int w = 0; w < CSRB_GRAM_WARPS; ++w) sm.dense[w][i] = 0.0f;
-  }
-  if (threadIdx.x < 2) sm.buf[threadIdx.x].nuniq = 0;
-
   kernel_inputs_ready();
   const int j = p.order[blockIdx.x];
   const long long n_run = p.n_steps[j];
@@ -200,6 +237,13 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
   const float* yshard = p.y + p.shard_off[j];
   const uint32_t* idx = p.idx + p.idx_off[j];
   float* u = p.U + (size_t)j * p.d;
+
+  for (int i = threadIdx.x; i < CSRB_HASH; i += CSRB_THREADS) {
+    sm.buf[0].keys[i] = -1;
+    sm.buf[1].keys[i] = -1;
+    for (int w = 0; w < CSRB_GRAM_WARPS; ++w) sm.dense[w][i] = 0.0f;
+  }
+  if (threadIdx.x < 2) sm.buf[threadIdx.x].nuniq = 0;
 
   // ---- plan of the next block (planner warp) -----------------------------------------------------------------------
   long long s_next = 0;                          // first step of the next block to plan
@@ -329,6 +373,7 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
       B.nsteps = nsteps;
       B.nent = nent;
       B.longest = longest;
+      B.brief = !direct && longest <= CSRB_SHORT_ROW && nent <= CSRB_SHORT_ENT;
       B.direct = direct;
       B.fold = fold;
     }
@@ -403,6 +448,176 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
     if (n2 < 8) out[8 * n2 + m2] = tot;
   };
 
+  // ---- short form of a block (few nonzeros, short rows; helper warps) -----------------------------------------------------
+  // Slots, then the columns that rows of a group share: only these contribute to the products of its rows, and only these need
+  // their updates one after the other. Thread ht takes the nonzeros ht + 320 i, i < F, whatever their rows, and keeps
+  // what it knows of them in registers; a cell per group and slot collects the rows that hold the column and then the number
+  // of its record. (For blocks of 2000 nonzeros the same form takes longer than form_gram, which leaves four warps to read
+  // the model meanwhile: 3950 against 2950 cycles per 8 steps at 40 Zipf-distributed nonzeros per row.)
+  auto form_short = [&](CsrBlockBuf& B, float* cache, const CsrPlan& P) __attribute__((always_inline)) {
+    constexpr int F = CSRB_SHORT_ENT / CSRB_HELPERS;
+    constexpr int W = CSRB_HELPERS / 32;
+    static_assert(F * W <= 31, "one lane per 32 nonzeros, and one more");
+    const int ht = (int)threadIdx.x - 64, hw = warp - 2;
+    const int nsteps = P.nsteps, nent = P.nent;
+    const unsigned below = (1u << lane) - 1u;
+    const uint32_t keys_a = smem_addr(B.keys), slot_a = smem_addr(B.slot), uslot_a = smem_addr(B.uslot), val_a = smem_addr(B.val);
+    const uint32_t col_a = smem_addr(B.col), nuniq_a = smem_addr(&B.nuniq), cell_a = smem_addr(sm.dense);
+    const uint32_t rslot_a = smem_addr(B.shared_slot), rec_a = smem_addr(B.shared_x), cache_a = smem_addr(cache);
+    int col[F], h[F], k2[F], r[F];
+    bool in[F], seek[F], several[F], first[F];
+    bool any_bad = false;
+#pragma unroll
+    for (int i = 0; i < F; ++i) {
+      in[i] = seek[i] = ht + CSRB_HELPERS * i < nent;
+      const uint32_t e = (uint32_t)(in[i] ? ht + CSRB_HELPERS * i : 0);
+      col[i] = lds_s32(col_a + 4u * e);
+      r[i] = lds_u16(slot_a + 2u * e) & (CSRB_STEPS - 1);  // the copies' note
+      k2[i] = 0;
+    }
+#pragma unroll
+    for (int i = 0; i < F; ++i) any_bad |= in[i] && (unsigned long long)(long long)col[i] >= (unsigned long long)p.d;
+    if (any_bad) {
+#pragma unroll
+      for (int i = 0; i < F; ++i)
+        if (in[i] && (unsigned long long)(long long)col[i] >= (unsigned long long)p.d) {
+          set_status(p.status, DEV_BOUNDS, 21, (long long)col[i]);
+          col[i] = 0;
+          B.val[ht + CSRB_HELPERS * i] = 0.0f;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < F; ++i) h[i] = csrb_hash(col[i]);
+    // until none of the warp's nonzeros has met another column
+    for (int probe = 0; probe < CSRB_HASH; ++probe) {
+#pragma unroll
+      for (int i = 0; i < F; ++i) atoms_cas_if(k2[i], keys_a + 4u * (uint32_t)h[i], -1, col[i], seek[i]);
+      bool any = false;
+#pragma unroll
+      for (int i = 0; i < F; ++i) {
+        seek[i] = seek[i] && k2[i] != -1 && k2[i] != col[i];
+        h[i] = seek[i] ? (h[i] + 1) & (CSRB_HASH - 1) : h[i];
+        any |= seek[i];
+      }
+      if (!__any_sync(0xffffffffu, any)) break;
+    }
+    // which rows of its group hold a column: one bit per row in the cell of group and slot
+    uint32_t ca[F];
+#pragma unroll
+    for (int i = 0; i < F; ++i) {
+      ca[i] = cell_a + (uint32_t)((r[i] >> 3) * CSRB_HASH + h[i]);
+      reds_or_if(ca[i] & ~3u, 1u << (8 * (ca[i] & 3u) + (r[i] & 7)), in[i]);
+    }
+    // one counter update per warp for the columns seen for the first time
+    unsigned votes[F];
+    int total = 0;
+#pragma unroll
+    for (int i = 0; i < F; ++i) {
+      votes[i] = __ballot_sync(0xffffffffu, in[i] && k2[i] == -1);
+      total += __popc(votes[i]);
+    }
+    int base = 0;
+    if (lane == 0) base = atoms_add(nuniq_a, total);
+    base = __shfl_sync(0xffffffffu, base, 0);
+#pragma unroll
+    for (int i = 0; i < F; ++i) {
+      const bool fresh = in[i] && k2[i] == -1;
+      prefetch_l2_if(u + col[i], fresh);  // the block's read of u[col] follows soon
+      sts_u16_if(uslot_a + 2u * (uint32_t)(base + __popc(votes[i] & below)), h[i], fresh);
+      base += __popc(votes[i]);
+    }
+    named_barrier(1, CSRB_HELPERS);  // table, list of distinct columns and cells are complete
+    int gh[F];
+    float gu[F];
+    const int nuniq = B.nuniq;
+#pragma unroll
+    for (int i = 0; i < F; ++i) gh[i] = lds_u16(uslot_a + 2u * (uint32_t)(ht + CSRB_HELPERS * i < nuniq ? ht + CSRB_HELPERS * i : 0)) & CSRB_SLOT;
+#pragma unroll
+    for (int i = 0; i < F; ++i) k2[i] = lds_s32(keys_a + 4u * (uint32_t)gh[i]);
+#pragma unroll
+    for (int i = 0; i < F; ++i) gu[i] = __ldcg(u + (ht + CSRB_HELPERS * i < nuniq ? k2[i] : 0));
+    // the first row to hold a shared column gives it a record; records are numbered in the order of the nonzeros
+#pragma unroll
+    for (int i = 0; i < F; ++i) col[i] = lds_u8(ca[i]);
+#pragma unroll
+    for (int i = 0; i < F; ++i) {
+      several[i] = in[i] && (col[i] & (col[i] - 1)) != 0;
+      first[i] = several[i] && (col[i] & ((1 << (r[i] & 7)) - 1)) == 0;
+      votes[i] = __ballot_sync(0xffffffffu, first[i]);
+      if (lane == 0) sm.votes[i * W + hw] = votes[i];
+    }
+    named_barrier(1, CSRB_HELPERS);
+    {  // (every warp writes the same numbers)
+      const int n = lane < F * W ? __popc(sm.votes[lane]) : 0;
+      int sum = n;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, sum, o);
+        sum += lane >= o ? v : 0;
+      }
+      sm.before[lane] = sum - n;
+    }
+    __syncwarp();
+    int rec0;  // lane g: the first record of group g
+    {
+      const int x = 8 * lane < nsteps && lane < CSRB_GROUPS ? P.step[8 * lane].x : nent;
+      rec0 = min(sm.before[x >> 5] + __popc(sm.votes[x >> 5] & ((1u << (x & 31)) - 1u)), CSRB_SHORT_ENT / 2);
+      const int next = __shfl_down_sync(0xffffffffu, rec0, 1);
+      if (hw == 0 && lane < CSRB_GROUPS) B.records[lane] = make_int2(rec0, next - rec0);
+    }
+#pragma unroll
+    for (int i = 0; i < F; ++i) {
+      const int rec = sm.before[i * W + hw] + __popc(votes[i] & below);
+      const int rel = rec - __shfl_sync(0xffffffffu, rec0, r[i] >> 3);
+      const bool write = in[i] && first[i] == several[i];
+      sts_u8_if(ca[i], first[i] ? rel : 0, write);
+      const bool mine = first[i] && rec < CSRB_SHORT_ENT / 2;  // (more only where a row holds a column twice)
+      sts_u16_if(rslot_a + 2u * (uint32_t)rec, h[i], mine);
+      sts_zero32_if(rec_a + 32u * (uint32_t)rec, mine);
+    }
+    named_barrier(1, CSRB_HELPERS);
+    float v[F];
+#pragma unroll
+    for (int i = 0; i < F; ++i) {
+      col[i] = lds_u8(ca[i]);
+      v[i] = lds_f32(val_a + 4u * (uint32_t)(in[i] ? ht + CSRB_HELPERS * i : 0));
+    }
+#pragma unroll
+    for (int i = 0; i < F; ++i) {
+      const int rec = __shfl_sync(0xffffffffu, rec0, r[i] >> 3) + col[i];
+      sts_f32_if(rec_a + 32u * (uint32_t)rec + 4u * (uint32_t)(r[i] & 7), v[i], several[i] && rec < CSRB_SHORT_ENT / 2);
+      sts_u16_if(slot_a + 2u * (uint32_t)(ht + CSRB_HELPERS * i), several[i] ? h[i] | CSRB_SHARED : h[i], in[i]);
+      sts_f32_if(cache_a + 4u * (uint32_t)gh[i], gu[i], ht + CSRB_HELPERS * i < nuniq);
+    }
+    named_barrier(1, CSRB_HELPERS);  // records are complete
+#pragma unroll
+    for (int i = 0; i < F; ++i) sts_u8_if(ca[i], 0, several[i]);
+    // products of the rows of a group: only shared columns contribute
+    if (8 * hw < nsteps) {
+      const int g0 = __shfl_sync(0xffffffffu, rec0, hw), n_rec = __shfl_sync(0xffffffffu, rec0, hw + 1) - g0;
+      float acc[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) acc[i] = 0.0f;
+#pragma unroll 1
+      for (int i = lane; i - lane < n_rec; i += 32) {
+        const float4* r4 = (const float4*)B.shared_x[i < n_rec ? g0 + i : 0];
+        const float in_f = i < n_rec ? 1.0f : 0.0f;
+        const float4 lo = r4[0], hi = r4[1];
+        const float x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+        for (int n = 1; n < 8; ++n) {
+          const float xn = in_f != 0.0f ? x[n] : 0.0f;
+#pragma unroll
+          for (int m = 0; m < n; ++m) acc[n * (n - 1) / 2 + m] = fmaf(xn, in_f != 0.0f ? x[m] : 0.0f, acc[n * (n - 1) / 2 + m]);
+        }
+      }
+      const float tot = warp_transpose_sum32(acc);  // lane l: product number l
+      int n2 = 1, m2 = lane;
+      while (n2 < 8 && m2 >= n2) { m2 -= n2; ++n2; }
+      if (n2 < 8) B.gram[hw][8 * n2 + m2] = tot;
+    }
+  };
+
   // ---- preparation of one block (helper warps only); writes the block that was in these tables back first ------------------
   auto prepare = [&](CsrBlockBuf& B, float* cache, const CsrPlan& P) {
     const int ht = (int)threadIdx.x - 64, hw = warp - 2;
@@ -420,7 +635,7 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
         cnt[i] = hw + W * i < nsteps ? P.step[r].y : 0;
         g0[i] = P.gbeg[r];
       }
-      const uint32_t col_a = smem_addr(sm.colbuf), val_a = smem_addr(B.val);
+      const uint32_t col_a = smem_addr(B.col), val_a = smem_addr(B.val);
 #pragma unroll
       for (int i = 0; i < ROWS; ++i)
 #pragma unroll
@@ -428,10 +643,14 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
           cp_async4_if(col_a + 4u * (uint32_t)(off[i] + lane + o), p.col_idx + g0[i] + lane + o, lane + o < cnt[i]);
           cp_async4_if(val_a + 4u * (uint32_t)(off[i] + lane + o), p.val + g0[i] + lane + o, lane + o < cnt[i]);
         }
+      if (P.brief) {  // a nonzero's row, for form_short
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) sts_u16_if(smem_addr(B.slot) + 2u * (uint32_t)(off[i] + lane), hw + W * i, lane < cnt[i]);
+      }
       if (P.longest > 64)
         for (int i = 0; i < ROWS; ++i)
           for (int o = lane + 64; o < cnt[i]; o += 32) {
-            cp_async4(&sm.colbuf[off[i] + o], p.col_idx + g0[i] + o);
+            cp_async4(&B.col[off[i] + o], p.col_idx + g0[i] + o);
             cp_async4(&B.val[off[i] + o], p.val + g0[i] + o);
           }
     }
@@ -442,8 +661,12 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
     if (ht == 0) B.nuniq = 0;
     named_barrier(1, CSRB_HELPERS);
     if (!have) return;
+    if (P.brief) {
+      form_short(B, cache, P);
+      return;
+    }
     const uint32_t keys_a = smem_addr(B.keys), slot_a = smem_addr(B.slot), uslot_a = smem_addr(B.uslot);
-    const uint32_t col_a = smem_addr(sm.colbuf), nuniq_a = smem_addr(&B.nuniq);
+    const uint32_t col_a = smem_addr(B.col), nuniq_a = smem_addr(&B.nuniq);
     constexpr int F = 4;  // nonzeros of a thread that probe together
     for (int e0 = 0; e0 < nent; e0 += F * CSRB_HELPERS) {  // the same trip count for every lane of a warp
       int e[F], col[F], h[F], k2[F];
@@ -526,17 +749,17 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
       const int4 st = P.step[r];
       const int beg = st.x, cnt = st.y;
       const bool in0 = lane < cnt, in1 = lane + 32 < cnt;
-      const int h0 = in0 ? B.slot[beg + lane] : 0, h1 = in1 ? B.slot[beg + lane + 32] : 0;
+      const int h0 = in0 ? B.slot[beg + lane] & CSRB_SLOT : 0, h1 = in1 ? B.slot[beg + lane + 32] & CSRB_SLOT : 0;
       const float v0 = in0 ? B.val[beg + lane] : 0.0f, v1 = in1 ? B.val[beg + lane + 32] : 0.0f;
       const float u0 = in0 ? cache[h0] : 0.0f, u1 = in1 ? cache[h1] : 0.0f;
       float part = fmaf(u1, v1, u0 * v0);
-      for (int o = lane + 64; o < cnt; o += 32) part = fmaf(cache[B.slot[beg + o]], B.val[beg + o], part);
+      for (int o = lane + 64; o < cnt; o += 32) part = fmaf(cache[B.slot[beg + o] & CSRB_SLOT], B.val[beg + o], part);
       const float acc = warp_sum(part);
       const float coef = P.eos[r] * loss_derivative(LOSS, __int_as_float(st.z), __int_as_float(st.w) * acc);
       if (in0) cache[h0] = fmaf(-coef, v0, u0);
       if (in1) cache[h1] = fmaf(-coef, v1, u1);
       for (int o = lane + 64; o < cnt; o += 32) {
-        const int h = B.slot[beg + o];
+        const int h = B.slot[beg + o] & CSRB_SLOT;
         cache[h] = fmaf(-coef, B.val[beg + o], cache[h]);
       }
       __syncwarp();
@@ -627,6 +850,92 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
           }
         __syncwarp();  // the next sample's loads see this sample's stores
       }
+    }
+  };
+
+  // Four lanes per sample hold E nonzeros each in registers, from the margins to the updates (short form). A column that
+  // only one row of the group holds is updated by the lane that read it; a shared one by a lane that takes all rows' values.
+  auto run_short = [&](const CsrBlockBuf& B, const CsrPlan& P, float* cache, auto e_tag) {
+    constexpr int E = decltype(e_tag)::value;
+    const uint32_t cache_a = smem_addr(cache), slot_a = smem_addr(B.slot), val_a = smem_addr(B.val), step_a = smem_addr(P.step);
+    const uint32_t rslot_a = smem_addr(B.shared_slot), records_a = smem_addr(B.records);
+    const int n = lane >> 2, q = lane & 3, own = lane & 7;
+    uint32_t ga[E], ga2[E];
+    float gv[E];
+    int gbeg, gcnt, gbeg2, gcnt2, rec0, rec02, n_rec, n_rec2;
+    const int groups = (P.nsteps + 7) / 8;
+    // (lanes beyond a row read the slot of the block's first nonzero; what they read is not used)
+    auto entries = [&](int gi) __attribute__((always_inline)) {
+      const int4 st = lds_s32x4(step_a + 16u * (uint32_t)(8 * gi + n));
+      const int2 rr = lds_s32x2(records_a + 8u * (uint32_t)gi);
+      rec02 = rr.x;
+      n_rec2 = rr.y;
+      gbeg2 = st.x;
+      gcnt2 = st.y;
+#pragma unroll
+      for (int i = 0; i < E; ++i) ga2[i] = (uint32_t)lds_u16(slot_a + 2u * (uint32_t)(q + 4 * i < gcnt2 ? gbeg2 + q + 4 * i : 0));
+    };
+    entries(0);
+#pragma unroll 1
+    for (int gi = 0; gi < groups; ++gi) {
+      const float* T = B.gram[gi];
+      const LagConst& K = P.k[gi];
+      gbeg = gbeg2;
+      gcnt = gcnt2;
+      rec0 = rec02;
+      n_rec = n_rec2;
+      float uq[E];
+#pragma unroll
+      for (int i = 0; i < E; ++i) {
+        ga[i] = ga2[i];
+        uq[i] = lds_f32(cache_a + 4u * (ga[i] & CSRB_SLOT));
+        gv[i] = lds_f32(val_a + 4u * (uint32_t)(q + 4 * i < gcnt ? gbeg + q + 4 * i : 0));
+      }
+      // this lane's shared column: its value in each row, its model entry
+      const int rec = lane < n_rec ? rec0 + lane : 0;
+      const uint32_t rs = (uint32_t)lds_u16(rslot_a + 2u * (uint32_t)rec);
+      const float4 xl = *(const float4*)B.shared_x[rec], xh = *(const float4*)(B.shared_x[rec] + 4);
+      LagBlock<LOSS> blk;
+      blk.load(T, K, own);
+      float ru = lds_f32(cache_a + 4u * (rs & CSRB_SLOT));
+      float a0 = 0.0f, a1 = 0.0f;
+#pragma unroll
+      for (int i = 0; i < E; i += 2) {
+        a0 = q + 4 * i < gcnt ? fmaf(uq[i], gv[i], a0) : a0;
+        a1 = q + 4 * i + 4 < gcnt ? fmaf(uq[i + 1], gv[i + 1], a1) : a1;
+      }
+      float r = a0 + a1;
+      r += __shfl_xor_sync(0xffffffffu, r, 1);
+      entries(gi + 1 < groups ? gi + 1 : gi);  // of the next group, on their way while the steps run
+      r += __shfl_xor_sync(0xffffffffu, r, 2);
+      float kappa[LAG_B], margin;
+      blk.steps(__shfl_sync(0xffffffffu, r, 4 * own), T, K, sm.jets, kappa, margin);
+      if (LOSS == LOSS_HINGE && margin < CSRB_NEAR * LAG_STEP) {
+        one_by_one(B, P, cache, 8 * gi, min(8 * gi + 8, P.nsteps));
+        continue;
+      }
+      // u <- u - kappa_m x_m, m ascending
+      const float k01 = n & 1 ? kappa[1] : kappa[0], k23 = n & 1 ? kappa[3] : kappa[2];
+      const float k45 = n & 1 ? kappa[5] : kappa[4], k67 = n & 1 ? kappa[7] : kappa[6];
+      const float k03 = n & 2 ? k23 : k01, k47 = n & 2 ? k67 : k45;
+      const float k_row = n & 4 ? k47 : k03;
+#pragma unroll
+      for (int i = 0; i < E; ++i)
+        sts_f32_if(cache_a + 4u * (ga[i] & CSRB_SLOT), fmaf(-k_row, gv[i], uq[i]), q + 4 * i < gcnt && !(ga[i] & CSRB_SHARED));
+      auto all_rows = [&](float v, const float4& lo, const float4& hi) __attribute__((always_inline)) {
+        const float x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+        for (int m = 0; m < 8; ++m) v = x[m] != 0.0f ? fmaf(-kappa[m], x[m], v) : v;  // 0: not in this row
+        return v;
+      };
+      ru = all_rows(ru, xl, xh);
+      sts_f32_if(cache_a + 4u * (rs & CSRB_SLOT), ru, lane < n_rec);
+      for (int i = lane + 32; i < n_rec; i += 32) {
+        const int h = B.shared_slot[rec0 + i];
+        const float4* x4 = (const float4*)B.shared_x[rec0 + i];
+        cache[h] = all_rows(cache[h], x4[0], x4[1]);
+      }
+      __syncwarp();  // the next group's loads see these stores
     }
   };
 
@@ -726,7 +1035,8 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
       }
     } else {
       using std::integral_constant;
-      if (P.longest <= 16) run_steps(B, P, cache, integral_constant<int, 4>(), integral_constant<int, 1>(), std::false_type());
+      if (P.brief && P.longest <= 16) run_short(B, P, cache, integral_constant<int, 4>());
+      else if (P.brief) run_short(B, P, cache, integral_constant<int, 8>());
       else if (P.longest <= 32) run_steps(B, P, cache, integral_constant<int, 8>(), integral_constant<int, 1>(), std::false_type());
       else if (P.longest <= 64) run_steps(B, P, cache, integral_constant<int, 16>(), integral_constant<int, 2>(), std::false_type());
       else run_steps(B, P, cache, integral_constant<int, 16>(), integral_constant<int, 2>(), std::true_type());

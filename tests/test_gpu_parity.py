@@ -1008,6 +1008,19 @@ def test_csr_group_forms(P, lengths, loss):
     assert_parity(P, wl, {"sparse_variant": 2})
 
 
+@pytest.mark.parametrize("d, lengths", [(32, (32,)), (34, (32, 31)), (33, (1, 32, 0, 7)), (2048, (10,)), (48, (20, 21)), (40, (5, 6, 10))])
+@pytest.mark.parametrize("loss", [HINGE, LOGISTIC, SQUARED])
+def test_csr_short_form_of_a_block(P, d, lengths, loss):
+    # rows of at most 32 nonzeros, blocks of at most 640: every column shared by all rows of a group (d = 32), more shared
+    # columns than lanes, hardly any (d = 2048); blocks on both sides of 640 follow one another where the rows differ
+    rp, ci, va, y = _rows_with_given_lengths(list(lengths) * (24 // len(lengths)), d, 7)
+    n = len(rp) - 1
+    steps = np.array([203, 64, 17])
+    wl = wi.Workload("short", 3, d, np.array([0, n // 3, 2 * (n // 3), n]), steps, 0.1, 1, 0.01, loss, 5, y, row_ptr=rp,
+                     col_idx=ci, val=va, w0=torch.full((d,), 0.01))
+    assert_parity(P, wl, {"sparse_variant": 2})
+
+
 def test_csr_hinge_decisions_at_the_threshold(P):
     # two rows of the same columns with values chosen so that margins come within rounding of 1: the decisions have to be
     # those of one step at a time, as in the direct kernel (bit for bit the same models but for the fp64 scale's last bits)
