@@ -229,7 +229,6 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   CsrBlockSmem& sm = *reinterpret_cast<CsrBlockSmem*>(smem_raw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  kernel_inputs_ready();
   const int j = p.order[blockIdx.x];
   const long long n_run = p.n_steps[j];
   const long long first = p.resume ? p.first[j] : 0;
