@@ -152,6 +152,30 @@ def test_large_d_falls_back_and_matches(P):
     assert_parity(P, wl)
 
 
+# ---- rounding of the update: eta lambda far below 2^-24 of the model -----------------------------------------------------
+@pytest.mark.parametrize("variant,d,bf16", [(0, 17, False), (0, 999, False), (0, 1001, True), (1, 67, False), (1, 256, True), (2, 256, False),
+                                            (2, 1000, True), (3, 64, False)])
+def test_small_decays_are_not_rounded_away(P, variant, d, bf16):
+    # eta lambda from 1e-6 down to 1.6e-8: where w (1 - eta lambda) is rounded on its own in every step, its error has the same
+    # sign step after step (4e-5 after these 4000 steps). One rounding of w per step, half a unit in the last place at most and
+    # of either sign, leaves sqrt(4000) 2^-24 = 3.8e-6 at three times its standard deviation, twice that with the margins' sums.
+    g = torch.Generator().manual_seed(4)
+    k, m, n = 2, 512, 4000
+    X = torch.randn(k * m, d, generator=g) / np.sqrt(d)
+    if bf16:
+        X = X.to(torch.bfloat16)
+    y = (X.float() @ torch.randn(d, generator=g) + 0.1 * torch.randn(k * m, generator=g)).contiguous()
+    off, steps = np.array([0, m, 2 * m], dtype=np.int64), np.array([n, n // 2], dtype=np.int64)
+    oW = oracle.run_dense(X, y, off, steps, d, 0.01, 1, 1e-4, SQUARED, 7)
+    with P.Context(k, d) as ctx:
+        ctx.set_option("dense_variant", variant)
+        ctx.run(X.cuda(), y.cuda(), off, steps, 0.01, 1, 1e-4, SQUARED, 7)
+        W = ctx.get_models().cpu().numpy()
+        ctx.check()
+    for j in range(k):
+        assert rel_l2(W[j], oW[j]) <= 8e-6
+
+
 # ---- blocked kernels with the decaying step size eta0 / sqrt(n): per-block tables instead of powers of one factor -------
 @pytest.mark.parametrize("loss", [HINGE, LOGISTIC, SQUARED])
 @pytest.mark.parametrize("kind", ["block_fp32", "block_bf16", "warp", "mma8", "mma16", "f32x16"])
