@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(64 + 32 * MAXW, 1) chain_block_kernel(const Bl
   volatile int* give_up = (volatile int*)(smem + L.flag);           // set when a bounded wait ran out
   const char* shard = (const char*)p.X + (size_t)p.shard_off[j] * ld_bytes;
   const float* yshard = p.y + p.shard_off[j];
-  const uint32_t* idx = p.idx + p.idx_off[j];  // padded to a multiple of B entries, all valid rows
+  const uint32_t* idx = p.idx + p.idx_off[j];  // padded to a multiple of B entries with the last step's row
   const long long nb = (n_run + B - 1) / B;
 
   if (threadIdx.x <= B) {  // power tables in fp64, rounded once

@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
   const long long n_run = p.n_steps[j];
   const char* shard = (const char*)p.X + (size_t)p.shard_off[j] * ld_bytes + (size_t)c_first * sizeof(XT);
   const float* yshard = p.y + p.shard_off[j];
-  const uint32_t* idx = p.idx + p.idx_off[j];  // padded to a multiple of 64 entries, all valid rows
+  const uint32_t* idx = p.idx + p.idx_off[j];  // padded to a multiple of 64 entries with the last step's row
   const int nb = (int)((n_run + B - 1) / B);  // the host sends chains of up to 2^33 steps here
   __syncthreads();
   cluster_barrier();  // every CTA of the cluster runs and has set up its shared memory

@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const Clust
   volatile int* give_up = (volatile int*)(smem + L.flag);
   const char* shard = (const char*)p.X + (size_t)p.shard_off[j] * ld_bytes + (size_t)chunk0 * 16;
   const float* yshard = p.y + p.shard_off[j];
-  const uint32_t* idx = p.idx + p.idx_off[j];  // padded to a multiple of 64 entries, all valid rows
+  const uint32_t* idx = p.idx + p.idx_off[j];  // padded to a multiple of 64 entries with the last step's row
   const long long nb = (n_run + B - 1) / B;
   const int consumed_threads = (math_warps + 1) * 32;  // math warps arrive, the copy warp waits: named barrier 2
 

@@ -71,16 +71,25 @@ __host__ __device__ __forceinline__ uint32_t shuffled_row(const uint4& keys, lon
   return (uint32_t)(x < m ? x : 0ull);
 }
 
-// Entries of steps b+1 .. b+cnt of node j (shard of m rows) into out[0 .. cnt). sampling 0: one counter value q
-// (four consecutive steps) per (t0 + i * stride); sampling 1: one step per (t0 + i * stride).
-__host__ __device__ __forceinline__ void emit_indices(int sampling, uint64_t seed, uint32_t j, long long b, long long cnt, uint32_t m,
+// Row of step s + 1 of node j in a shard of m rows.
+__host__ __device__ __forceinline__ uint32_t drawn_row(uint64_t seed, uint32_t j, long long s, uint32_t m) {
+  const unsigned long long q = (unsigned long long)s >> 2;
+  const uint4 o = philox4x32_10(make_uint4((uint32_t)q, (uint32_t)(q >> 32), j, 0u), (uint32_t)seed, (uint32_t)(seed >> 32));
+  const int e = (int)(s & 3);
+  return mulhi32(e == 0 ? o.x : (e == 1 ? o.y : (e == 2 ? o.z : o.w)), m);  // floor(u m / 2^32)
+}
+
+// Entries of steps b+1 .. b+steps of node j (shard of m rows) into out[0 .. steps), and the last one's row again into
+// out[steps .. cnt). sampling 0: one counter value q (four consecutive steps) per (t0 + i * stride); sampling 1: one step
+// per (t0 + i * stride).
+__host__ __device__ __forceinline__ void emit_indices(int sampling, uint64_t seed, uint32_t j, long long b, long long steps, long long cnt, uint32_t m,
                                              uint32_t* __restrict__ out, long long t0, long long stride) {
   if (sampling == 1) {
     const uint4 keys = philox4x32_10(make_uint4(0u, 0u, j, 1u), (uint32_t)seed, (uint32_t)(seed >> 32));
-    for (long long i = t0; i < cnt; i += stride) out[i] = shuffled_row(keys, b + i, m);
+    for (long long i = t0; i < cnt; i += stride) out[i] = shuffled_row(keys, b + (i < steps ? i : steps - 1), m);
     return;
   }
-  const long long q_lo = b >> 2, q_hi = (b + cnt - 1) >> 2;  // zero-based step s = n-1 lies in [b, b+cnt)
+  const long long q_lo = b >> 2, q_hi = (b + steps - 1) >> 2;  // zero-based step s = n-1 lies in [b, b+steps)
   for (long long q = q_lo + t0; q <= q_hi; q += stride) {
     const uint4 o = philox4x32_10(make_uint4((uint32_t)q, (uint32_t)((unsigned long long)q >> 32), j, 0u),
                                   (uint32_t)seed, (uint32_t)(seed >> 32));
@@ -88,8 +97,13 @@ __host__ __device__ __forceinline__ void emit_indices(int sampling, uint64_t see
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const long long s = (q << 2) + e;
-      if (s >= b && s < b + cnt) out[s - b] = mulhi32(w[e], m);  // floor(u m / 2^32)
+      if (s >= b && s < b + steps) out[s - b] = mulhi32(w[e], m);  // floor(u m / 2^32)
     }
+  }
+  const long long t1 = stride - 1 - t0;  // the threads with the least to do above
+  if (t1 < cnt - steps) {
+    const uint32_t last = drawn_row(seed, j, b + steps - 1, m);
+    for (long long i = steps + t1; i < cnt; i += stride) out[i] = last;
   }
 }
 
@@ -107,8 +121,9 @@ struct TableLayout {
     total = (ids + n * sizeof(int) + 15) / 16 * 16;
   }
 };
-// The stream of a node is produced up to the next multiple of 64 steps (the draws simply continue), so that kernels that
-// take samples in groups always read valid rows.
+// The stream of a node is filled up to the next multiple of 64 steps with the row of its last step, so that kernels that take
+// samples in groups always read valid rows, and only rows that the chain has visited: what fills a group up has the weight
+// zero, but zero times a value that is not finite would reach the model.
 __host__ __device__ __forceinline__ long long stream_entries(long long steps) { return (steps + 63) / 64 * 64; }
 
 // Tables small enough travel as a kernel argument: no copy is enqueued for them.
@@ -135,7 +150,7 @@ __global__ void __launch_bounds__(256) index_stream_kernel(const __grid_constant
   for (int j = blockIdx.y; j < k; j += gridDim.y) {
     const long long cnt = stream_entries(steps[j]);
     if (cnt <= 0) continue;
-    emit_indices(sampling, seed, (uint32_t)ids[j], first[j], cnt, (uint32_t)(off[j + 1] - off[j]), idx + idx_off[j],
+    emit_indices(sampling, seed, (uint32_t)ids[j], first[j], steps[j], cnt, (uint32_t)(off[j + 1] - off[j]), idx + idx_off[j],
                  (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
   }
 }
@@ -146,7 +161,7 @@ __global__ void index_single_kernel(int sampling, uint64_t seed, int node, long 
   kernel_started();
   kernel_inputs_ready();
   if (count > 0)
-    emit_indices(sampling, seed, (uint32_t)node, n_begin, count, (uint32_t)m, out,
+    emit_indices(sampling, seed, (uint32_t)node, n_begin, count, count, (uint32_t)m, out,
                  (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
 }
 

@@ -1292,7 +1292,7 @@ wpsgd_status wpsgd_sample_indices_host(uint64_t seed, int32_t node, int64_t m, i
                 "sample_indices_host: need node >= 0, 1 <= m < 2^32, n_begin >= 0, count >= 0, sampling 0 or 1");
   if (count == 0) return WPSGD_OK;
   if (!out) return fail(nullptr, WPSGD_ERR_INVALID_ARG, "out is NULL");
-  emit_indices(sampling, seed, (uint32_t)node, n_begin, count, (uint32_t)m, out, 0, 1);  // the kernels' own function
+  emit_indices(sampling, seed, (uint32_t)node, n_begin, count, count, (uint32_t)m, out, 0, 1);  // the kernels' own function
   return WPSGD_OK;
 }
 

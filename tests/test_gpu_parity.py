@@ -583,6 +583,34 @@ def test_nodes_without_work_keep_w0(P):
     assert_parity(P, wl)
 
 
+@pytest.mark.parametrize("sampling", [0, 1])
+@pytest.mark.parametrize("d,bf16,loss,opts", [
+    (999, False, SQUARED, {}), (999, False, LOGISTIC, {}), (999, False, HINGE, {}), (1000, True, HINGE, {}), (64, False, HINGE, {}),
+    (8192, False, LOGISTIC, {}), (1024, False, SQUARED, {"dense_variant": 4}), (128, False, SQUARED, {"dense_variant": 5}),
+    (4096, True, SQUARED, {"dense_variant": 8, "block_samples": 16}), (4096, True, LOGISTIC, {"dense_variant": 8, "block_samples": 8}),
+])
+def test_rows_that_no_step_visits_do_not_reach_the_model(P, d, bf16, loss, opts, sampling):
+    # 21 steps end inside a block of 8 or 16: what fills the block up must not bring in other rows (here NaN) or labels
+    wl = wi.config2(k=2, d=d, m=512, base_steps=21)
+    wl.n_steps = np.array([21, 1], dtype=np.int64)
+    wl.loss = loss
+    if loss == SQUARED:
+        wl.y = (wl.y * 0.3).contiguous()
+    if bf16:
+        wl.X = wl.X.to(torch.bfloat16)
+    opts = dict(opts, sampling=sampling)
+    _, clean, _, _ = gpu_solve(P, wl, opts)
+    unseen = torch.ones(len(wl.y), dtype=torch.bool)
+    for j in range(2):
+        rows = P.sample_indices_host(wl.seed, j, 512, 0, int(wl.n_steps[j]), sampling).astype(np.int64) + int(wl.shard_off[j])
+        unseen[torch.from_numpy(rows)] = False
+    wl.X, wl.y = wl.X.clone(), wl.y.clone()
+    wl.X[unseen] = float("nan")
+    wl.y[unseen] = float("nan")
+    _, W, _, _ = gpu_solve(P, wl, opts)
+    np.testing.assert_array_equal(W, clean)
+
+
 def test_no_work_at_all_returns_w0(P):
     wl = wi.config1(k=3, d=64, m=8, n_steps=(0, 0, 0))
     wl.w0 = torch.arange(64, dtype=torch.float32)
