@@ -23,8 +23,10 @@
 // Short form (blocks of at most 640 nonzeros in rows of at most 32). Most columns are held by one row of a group only. The
 // helpers find the ones that several rows hold and give each a record with its value in all 8 rows; the products come from the
 // records alone. After the 8 steps the lane that read a column's entry for the margins writes it back, and one lane per record
-// applies all rows' updates in order: two passes where the long form makes eight. Why the limit: longer blocks take longer
-// this way, their helpers being the longer side (see form_short).
+// applies all rows' updates in order: two passes where the long form makes eight. 640 is two nonzeros per helper thread: what
+// it knows of them then stays in registers. Up to 10 nonzeros per row a block of 64 steps fits (a row of 12 takes 1590
+// cycles per 8 steps in the long form, one of 10 takes 1270 in this); with as many nonzeros per thread as blocks of 40 per row
+// need, this form was the slower one (see form_short). Blocks of fewer steps, which would let rows of 11 to 32 take it, were not measured.
 //
 // For the hinge loss a decision within 1e-4 of its threshold sends the group through one step at a time, so that the order of
 // the sums never turns it.
@@ -224,10 +226,9 @@ __device__ __forceinline__ void csrb_scatter(CsrBlockBuf& B, const float* cache,
   }
 }
 
-template <int LOSS>
-__global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const CsrParams p) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  CsrBlockSmem& sm = *reinterpret_cast<CsrBlockSmem*>(smem_raw);
+// SHORT: the chain's blocks may take the short form
+template <int LOSS, bool SHORT>
+__device__ __forceinline__ void chain_csr_block(const CsrParams& p, CsrBlockSmem& sm) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int j = p.order[blockIdx.x];
   const long long n_run = p.n_steps[j];
@@ -642,7 +643,7 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
           cp_async4_if(col_a + 4u * (uint32_t)(off[i] + lane + o), p.col_idx + g0[i] + lane + o, lane + o < cnt[i]);
           cp_async4_if(val_a + 4u * (uint32_t)(off[i] + lane + o), p.val + g0[i] + lane + o, lane + o < cnt[i]);
         }
-      if (P.brief) {  // a nonzero's row, for form_short
+      if (SHORT && P.brief) {  // a nonzero's row, for form_short
 #pragma unroll
         for (int i = 0; i < ROWS; ++i) sts_u16_if(smem_addr(B.slot) + 2u * (uint32_t)(off[i] + lane), hw + W * i, lane < cnt[i]);
       }
@@ -660,7 +661,7 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
     if (ht == 0) B.nuniq = 0;
     named_barrier(1, CSRB_HELPERS);
     if (!have) return;
-    if (P.brief) {
+    if (SHORT && P.brief) {
       form_short(B, cache, P);
       return;
     }
@@ -1034,8 +1035,8 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
       }
     } else {
       using std::integral_constant;
-      if (P.brief && P.longest <= 16) run_short(B, P, cache, integral_constant<int, 4>());
-      else if (P.brief) run_short(B, P, cache, integral_constant<int, 8>());
+      if (SHORT && P.brief && P.longest <= 16) run_short(B, P, cache, integral_constant<int, 4>());
+      else if (SHORT && P.brief) run_short(B, P, cache, integral_constant<int, 8>());
       else if (P.longest <= 32) run_steps(B, P, cache, integral_constant<int, 8>(), integral_constant<int, 1>(), std::false_type());
       else if (P.longest <= 64) run_steps(B, P, cache, integral_constant<int, 16>(), integral_constant<int, 2>(), std::false_type());
       else run_steps(B, P, cache, integral_constant<int, 16>(), integral_constant<int, 2>(), std::true_type());
@@ -1045,6 +1046,24 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
     __syncthreads();
   }
   if (warp == 1 && lane == 0) p.scale[j] = sc;
+}
+
+// The short form is compiled into a body of its own, for chains whose shard has at most 10 nonzeros per row on average (640
+// nonzeros in 64 steps, the limit of that form). Code that a chain never runs costs it time all the same, through the registers
+// and the schedule of the one body: 64 chains with 40 Zipf-distributed nonzeros per row take 11.55 ms with two bodies and 12.25 with
+// one; 10 chains of 5 to 10 nonzeros take the same in both.
+constexpr int CSRB_SHORT_MEAN = CSRB_SHORT_ENT / CSRB_STEPS;
+template <int LOSS>
+__global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const CsrParams p) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  CsrBlockSmem& sm = *reinterpret_cast<CsrBlockSmem*>(smem_raw);
+  const int j = p.order[blockIdx.x];
+  const long long r0 = p.shard_off[j], r1 = p.shard_off[j + 1];
+  if (p.row_ptr[r1] - p.row_ptr[r0] > CSRB_SHORT_MEAN * (r1 - r0)) {
+    chain_csr_block<LOSS, false>(p, sm);
+    return;
+  }
+  chain_csr_block<LOSS, true>(p, sm);
 }
 
 }  // namespace wpsgd

@@ -1019,8 +1019,8 @@ wpsgd_status run_csr_common(wpsgd_ctx* c, const long long* row_ptr, const int* c
     const size_t smem = sizeof(CsrBlockSmem);
     auto go = [&](auto kern) -> wpsgd_status {
       CU_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      // Launched after its predecessor, without the wait that an early start needs inside the kernel: with it the kernel itself
-      // was slower (64 chains, 40 nonzeros per row: 12.2 against 11.4 ms).
+      // Launched after its predecessor, without the wait that an early start needs inside the kernel: the wait, with the set-up of
+      // shared memory before it, was measured by itself at 12.0 against 11.16 ms (64 chains, 40 nonzeros per row).
       kern<<<c->k, CSRB_THREADS, smem, c->stream>>>(p);
       CU_TRY(c, cudaGetLastError());
       return WPSGD_OK;

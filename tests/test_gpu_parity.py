@@ -1073,6 +1073,20 @@ def test_csr_short_form_of_a_block(P, d, lengths, loss):
     assert_parity(P, wl, {"sparse_variant": 2})
 
 
+@pytest.mark.parametrize("loss", [HINGE, LOGISTIC, SQUARED])
+def test_csr_chains_of_both_bodies_in_one_run(P, loss):
+    # shards of 10 nonzeros per row on average (the limit of the body with the short form), just above, and far above; the
+    # first also holds rows that fit no short block; the last shard is a single row without nonzeros
+    d = 3000
+    shards = [[3, 4, 5, 2, 40, 6, 20, 0], [10, 11, 9, 11, 10, 10, 10, 10], [40, 64, 33, 7], [0]]
+    assert sum(shards[0]) == 10 * len(shards[0]) and sum(shards[1]) == 81
+    rp, ci, va, y = _rows_with_given_lengths([n for s in shards for n in s], d, 9)
+    off = np.concatenate([[0], np.cumsum([len(s) for s in shards])])
+    wl = wi.Workload("bodies", 4, d, off, np.array([230, 230, 150, 20]), 0.1, 1, 0.01, loss, 5, y, row_ptr=rp, col_idx=ci, val=va,
+                     w0=torch.full((d,), 0.01))
+    assert_parity(P, wl, {"sparse_variant": 2})
+
+
 def test_csr_hinge_decisions_at_the_threshold(P):
     # two rows of the same columns with values chosen so that margins come within rounding of 1: the decisions have to be
     # those of one step at a time, as in the direct kernel (bit for bit the same models but for the fp64 scale's last bits)
