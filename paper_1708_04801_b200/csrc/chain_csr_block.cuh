@@ -28,6 +28,11 @@
 // cycles per 8 steps in the long form, one of 10 takes 1270 in this); with as many nonzeros per thread as blocks of 40 per row
 // need, this form was the slower one (see form_short). Blocks of fewer steps, which would let rows of 11 to 32 take it, were not measured.
 //
+// Blocks of long rows (more than 64 nonzeros per step on average) take their steps one at a time: the products cost their
+// helpers time in proportion to eight times the nonzeros, and with rows of more than two chunks of 32 the group is the slower
+// form (uniform columns, hinge, cycles per 8 steps, group against one at a time: 64 nonzeros 6470 / 7660, 72 nonzeros 10470 / 8210,
+// 200 nonzeros 34500 / 21000).
+//
 // For the hinge loss a decision within 1e-4 of its threshold sends the group through one step at a time, so that the order of
 // the sums never turns it.
 //
@@ -47,8 +52,9 @@
 // caches are double buffered, plans (row extents, labels, scale factors; two blocks ahead) are threefold.
 //
 // Slow boundaries (rare): a row with more than CSRB_EMAX nonzeros forms a block of its own that the chain warp runs
-// on global memory; when the scale has fallen below 1e-12 at the start of a block it is folded into u (u <- s u,
-// s <- 1). In both cases, and for the first block, all threads write the previous block back, apply the fold, and
+// on global memory, 16 loads of a lane in flight (rows of 2500 nonzeros: 32500 cycles a step, 162000 with single loads); when
+// the scale has fallen below 1e-12 at the start of a block it is folded into u (u <- s u, s <- 1). In both cases, and for the
+// first block, all threads write the previous block back, apply the fold, and
 // read the block's columns again from global memory. A block also ends early before the scale would leave the fp32
 // range of the per-step factors.
 //
@@ -76,7 +82,9 @@ constexpr int CSRB_SHORT_ENT = 2 * CSRB_HELPERS;  // blocks of at most that many
 constexpr int CSRB_SHORT_ROW = 32;      // these take the short form
 constexpr int CSRB_SLOT = CSRB_HASH - 1;  // bits of a nonzero's slot entry: the slot,
 constexpr int CSRB_SHARED = 0x8000;     // and (short form) whether another row of its group holds the column
+constexpr int CSRB_APART = 64;          // blocks with more nonzeros per step on average take their steps one at a time
 constexpr float CSRB_NEAR = 1e-4f;      // hinge decisions with |1 - t| below this are taken one step at a time
+constexpr int CSRB_DIRECT = 16;         // the same of the chain warp on a row longer than the tables
 constexpr int CSRB_BATCH = 8;           // independent global loads a thread keeps in flight
 
 // Plan of a block
@@ -91,7 +99,8 @@ struct CsrPlan {
   LagConst k[CSRB_GROUPS];             // constants of a group of 8 steps
   int longest;                         // most nonzeros of a row of the block
   int brief;                           // the block takes the short form
-  int pad[2];
+  int apart;                           // its steps are run one at a time
+  int pad[1];
 };
 
 // One buffer of a prepared block.
@@ -374,6 +383,7 @@ __device__ __forceinline__ void chain_csr_block(const CsrParams& p, CsrBlockSmem
       B.nent = nent;
       B.longest = longest;
       B.brief = !direct && longest <= CSRB_SHORT_ROW && nent <= CSRB_SHORT_ENT;
+      B.apart = nent > CSRB_APART * nsteps;
       B.direct = direct;
       B.fold = fold;
     }
@@ -727,10 +737,13 @@ __device__ __forceinline__ void chain_csr_block(const CsrParams& p, CsrBlockSmem
       }
     }
     named_barrier(1, CSRB_HELPERS);  // slots and the list of distinct columns are complete
-    if (hw < CSRB_GRAM_WARPS) {
+    if (!SHORT && P.apart) {
+      csrb_gather(B, cache, u, B.nuniq, ht, CSRB_HELPERS);
+    } else if (hw < CSRB_GRAM_WARPS) {
       for (int gi = hw; 8 * gi < nsteps; gi += CSRB_GRAM_WARPS) {
         using std::integral_constant;
         if (P.longest <= 32) form_gram(B, P, gi, sm.dense[hw], B.gram[gi], integral_constant<int, 1>(), std::false_type());
+        else if (SHORT) form_gram(B, P, gi, sm.dense[hw], B.gram[gi], integral_constant<int, 1>(), std::true_type());
         else if (P.longest <= 64) form_gram(B, P, gi, sm.dense[hw], B.gram[gi], integral_constant<int, 2>(), std::false_type());
         else form_gram(B, P, gi, sm.dense[hw], B.gram[gi], integral_constant<int, 2>(), std::true_type());
       }
@@ -762,6 +775,70 @@ __device__ __forceinline__ void chain_csr_block(const CsrParams& p, CsrBlockSmem
         const int h = B.slot[beg + o] & CSRB_SLOT;
         cache[h] = fmaf(-coef, B.val[beg + o], cache[h]);
       }
+      __syncwarp();
+    }
+  };
+
+  // Blocks of long rows: their steps one at a time, all lanes on a row. The first 128 nonzeros of a row and of the next one wait
+  // in registers, the others are read again for the update.
+  auto run_long = [&](const CsrBlockBuf& B, const CsrPlan& P, float* cache) __attribute__((always_inline)) {
+    constexpr int U = 4;
+    const uint32_t cache_a = smem_addr(cache), slot_a = smem_addr(B.slot), val_a = smem_addr(B.val), step_a = smem_addr(P.step);
+    uint32_t c2[U];
+    float v2[U];
+    int4 st2;
+    auto entries = [&](int r) __attribute__((always_inline)) {
+      st2 = lds_s32x4(step_a + 16u * (uint32_t)r);
+#pragma unroll
+      for (int i = 0; i < U; ++i) {
+        const int e = lane + 32 * i < st2.y ? st2.x + lane + 32 * i : 0;
+        c2[i] = cache_a + 4u * (uint32_t)lds_u16(slot_a + 2u * (uint32_t)e);
+        v2[i] = lds_f32(val_a + 4u * (uint32_t)e);
+      }
+    };
+    entries(0);
+#pragma unroll 1
+    for (int r = 0; r < P.nsteps; ++r) {
+      const int4 st = st2;
+      uint32_t c[U];
+      float v[U], x[U];
+#pragma unroll
+      for (int i = 0; i < U; ++i) {
+        c[i] = c2[i];
+        v[i] = lane + 32 * i < st.y ? v2[i] : 0.0f;
+        x[i] = lds_f32(c[i]);
+      }
+      entries(r + 1 < P.nsteps ? r + 1 : r);
+      const float eos = P.eos[r];
+      float a0 = 0.0f, a1 = 0.0f;
+#pragma unroll
+      for (int i = 0; i < U; i += 2) {
+        a0 = lane + 32 * i < st.y ? fmaf(x[i], v[i], a0) : a0;
+        a1 = lane + 32 * i + 32 < st.y ? fmaf(x[i + 1], v[i + 1], a1) : a1;
+      }
+      auto rest = [&](auto use) __attribute__((always_inline)) {
+#pragma unroll 1
+        for (int o = lane + 32 * U; o - lane < st.y; o += 32 * U) {
+          uint32_t cr[U];
+          float vr[U], xr[U];
+#pragma unroll
+          for (int i = 0; i < U; ++i) {
+            const int e = o + 32 * i < st.y ? st.x + o + 32 * i : 0;
+            cr[i] = cache_a + 4u * (uint32_t)lds_u16(slot_a + 2u * (uint32_t)e);
+            vr[i] = lds_f32(val_a + 4u * (uint32_t)e);
+          }
+#pragma unroll
+          for (int i = 0; i < U; ++i) xr[i] = lds_f32(cr[i]);
+#pragma unroll
+          for (int i = 0; i < U; ++i) use(cr[i], vr[i], xr[i], o + 32 * i < st.y);
+        }
+      };
+      rest([&](uint32_t, float vv, float xx, bool in) { a0 = in ? fmaf(xx, vv, a0) : a0; });
+      const float acc = warp_sum(a0 + a1);
+      const float coef = eos * loss_derivative(LOSS, __int_as_float(st.z), __int_as_float(st.w) * acc);
+#pragma unroll
+      for (int i = 0; i < U; ++i) sts_f32_if(c[i], fmaf(-coef, v[i], x[i]), lane + 32 * i < st.y);
+      rest([&](uint32_t a, float vv, float xx, bool in) { sts_f32_if(a, fmaf(-coef, vv, xx), in); });
       __syncwarp();
     }
   };
@@ -1018,19 +1095,44 @@ __device__ __forceinline__ void chain_csr_block(const CsrParams& p, CsrBlockSmem
     } else if (direct) {
       // ---- a single long row, on global memory ---------------------------------------------------------------
       const long long g0 = P.gbeg[0], g1 = P.gbeg[1];
+      // CSRB_DIRECT loads in flight per lane; lanes beyond the row take its first nonzero and the value 0
+      auto batch = [&](long long o, long long (&e)[CSRB_DIRECT], int (&c)[CSRB_DIRECT], float (&v)[CSRB_DIRECT], float (&x)[CSRB_DIRECT]) __attribute__((always_inline)) {
+#pragma unroll
+        for (int i = 0; i < CSRB_DIRECT; ++i) {
+          e[i] = o + 32 * i < g1 ? o + 32 * i : g0;
+          c[i] = p.col_idx[e[i]];
+          v[i] = o + 32 * i < g1 ? p.val[e[i]] : 0.0f;
+        }
+#pragma unroll
+        for (int i = 0; i < CSRB_DIRECT; ++i)
+          if ((unsigned long long)(long long)c[i] >= (unsigned long long)p.d) {
+            set_status(p.status, DEV_BOUNDS, 22, (long long)c[i]);
+            c[i] = 0;
+            v[i] = 0.0f;
+          }
+#pragma unroll
+        for (int i = 0; i < CSRB_DIRECT; ++i) x[i] = __ldcg(u + c[i]);
+      };
+      long long e[CSRB_DIRECT];
+      int c[CSRB_DIRECT];
+      float v[CSRB_DIRECT], x[CSRB_DIRECT];
       float acc = 0.0f;
-      for (long long o = g0 + lane; o < g1; o += 32) {
-        const int c = p.col_idx[o];
-        if ((unsigned long long)(long long)c < (unsigned long long)p.d) acc = fmaf(__ldcg(u + c), p.val[o], acc);
-        else set_status(p.status, DEV_BOUNDS, 22, (long long)c);
+#pragma unroll 1
+      for (long long o = g0 + lane; o - lane < g1; o += 32 * CSRB_DIRECT) {
+        batch(o, e, c, v, x);
+#pragma unroll
+        for (int i = 0; i < CSRB_DIRECT; ++i) acc = v[i] != 0.0f ? fmaf(x[i], v[i], acc) : acc;
       }
       acc = warp_sum(acc);
       const float g = loss_derivative(LOSS, __int_as_float(P.step[0].z), __int_as_float(P.step[0].w) * acc);
       if (g != 0.0f) {
         const float coef = P.eos[0] * g;
-        for (long long o = g0 + lane; o < g1; o += 32) {
-          const int c = p.col_idx[o];
-          if ((unsigned long long)(long long)c < (unsigned long long)p.d) u[c] = fmaf(-coef, p.val[o], __ldcg(u + c));
+#pragma unroll 1
+        for (long long o = g0 + lane; o - lane < g1; o += 32 * CSRB_DIRECT) {
+          batch(o, e, c, v, x);
+#pragma unroll
+          for (int i = 0; i < CSRB_DIRECT; ++i)
+            if (v[i] != 0.0f) u[c[i]] = fmaf(-coef, v[i], x[i]);
         }
       }
     } else {
@@ -1038,6 +1140,8 @@ __device__ __forceinline__ void chain_csr_block(const CsrParams& p, CsrBlockSmem
       if (SHORT && P.brief && P.longest <= 16) run_short(B, P, cache, integral_constant<int, 4>());
       else if (SHORT && P.brief) run_short(B, P, cache, integral_constant<int, 8>());
       else if (P.longest <= 32) run_steps(B, P, cache, integral_constant<int, 8>(), integral_constant<int, 1>(), std::false_type());
+      else if (SHORT) run_steps(B, P, cache, integral_constant<int, 8>(), integral_constant<int, 1>(), std::true_type());
+      else if (P.apart) run_long(B, P, cache);
       else if (P.longest <= 64) run_steps(B, P, cache, integral_constant<int, 16>(), integral_constant<int, 2>(), std::false_type());
       else run_steps(B, P, cache, integral_constant<int, 16>(), integral_constant<int, 2>(), std::true_type());
     }
@@ -1059,11 +1163,11 @@ __global__ void __launch_bounds__(CSRB_THREADS, 1) chain_csr_block_kernel(const 
   CsrBlockSmem& sm = *reinterpret_cast<CsrBlockSmem*>(smem_raw);
   const int j = p.order[blockIdx.x];
   const long long r0 = p.shard_off[j], r1 = p.shard_off[j + 1];
-  if (p.row_ptr[r1] - p.row_ptr[r0] > CSRB_SHORT_MEAN * (r1 - r0)) {
-    chain_csr_block<LOSS, false>(p, sm);
+  if (p.row_ptr[r1] - p.row_ptr[r0] <= CSRB_SHORT_MEAN * (r1 - r0)) {
+    chain_csr_block<LOSS, true>(p, sm);
     return;
   }
-  chain_csr_block<LOSS, true>(p, sm);
+  chain_csr_block<LOSS, false>(p, sm);
 }
 
 }  // namespace wpsgd

@@ -1087,6 +1087,21 @@ def test_csr_chains_of_both_bodies_in_one_run(P, loss):
     assert_parity(P, wl, {"sparse_variant": 2})
 
 
+@pytest.mark.parametrize("loss", [HINGE, LOGISTIC, SQUARED])
+def test_csr_long_rows_one_step_at_a_time(P, loss):
+    # blocks with more than 64 nonzeros per step (65; rows at the edges of the 128 that wait in registers; 2048, the most a block
+    # takes; 2049 and 2560, which run on global memory), blocks just below, both kinds in turn, and long rows in a shard of
+    # few nonzeros on average
+    d = 6000
+    shards = [[65, 65, 64, 66, 127, 128, 129, 256, 257], [2048, 65, 2049, 700, 2560, 513], [64, 63, 64, 65, 64, 64],
+              [70, 300] + [2] * 60, [40, 40, 40, 400, 40, 40, 40, 40]]
+    rp, ci, va, y = _rows_with_given_lengths([n for s in shards for n in s], d, 13)
+    off = np.concatenate([[0], np.cumsum([len(s) for s in shards])])
+    wl = wi.Workload("apart", 5, d, off, np.array([133, 60, 101, 400, 200]), 0.1, 1, 0.01, loss, 5, y, row_ptr=rp, col_idx=ci, val=va,
+                     w0=torch.full((d,), 0.01))
+    assert_parity(P, wl, {"sparse_variant": 2})
+
+
 def test_csr_hinge_decisions_at_the_threshold(P):
     # two rows of the same columns with values chosen so that margins come within rounding of 1: the decisions have to be
     # those of one step at a time, as in the direct kernel (bit for bit the same models but for the fp64 scale's last bits)
