@@ -152,11 +152,16 @@ __device__ __forceinline__ void objective_finish(double lsum, double esum, const
 }
 
 // Dense rows, one warp per row. Bound by the read of X: 16 bytes per lane and load, four loads in flight per lane (VEC; rows
-// that are not 16-byte aligned go element by element, eight in flight), the model from L1. A warp keeps the margins of up
-// to 32 of its rows, one per lane, and then evaluates their fp64 losses side by side. 262144 rows of 1024 fp32 columns: 231
-// us with single 4-byte loads, a loss evaluation per row on all lanes and a second launch for the sums; 177 us this way (6.1 TB/s).
-template <typename XT, bool VEC>
-__global__ void __launch_bounds__(256) objective_rows_kernel(const XT* __restrict__ X, long long ld, const float* __restrict__ y,
+// that are not 16-byte aligned go element by element, four or eight in flight), the model from L1. The end of such a row is a matter of predicates,
+// not of a loop of its own, in which each load would be waited for; rows of at most 32 chunks (64 elements), NARROW, go four at a time. A
+// warp keeps the margins of up to 32 of its rows, one per lane, and then evaluates their fp64 losses side by side. 262144 rows of
+// 1024 fp32 columns: 231 us with single 4-byte loads, a loss evaluation per row on all lanes and a second launch for the sums;
+// 177 us this way (6.1 TB/s). 300000 fp32 rows of 166 columns: 179 us with a loop for the row's
+// end, 98 without; 300000 bf16 rows of 8 columns: 63 us one at a time, 42 four at a time. Four or five blocks per SM: with six (40
+// registers) the rows that do not start on 16 bytes lose the cache lines that neighbouring loads share (30000 rows of 4673 fp32
+// columns: 181 us against 111).
+template <typename XT, bool VEC, bool NARROW>
+__global__ void __launch_bounds__(256, sizeof(XT) == 2 ? 5 : 4) objective_rows_kernel(const XT* __restrict__ X, long long ld, const float* __restrict__ y,
                                                              long long n_rows, const float* __restrict__ w, long long d,
                                                              int loss, float lambda, double* __restrict__ part, unsigned* ticket,
                                                              double* __restrict__ out) {
@@ -174,37 +179,90 @@ __global__ void __launch_bounds__(256) objective_rows_kernel(const XT* __restric
     }
     held = 0;
   };
-  for (long long i = (long long)blockIdx.x * 8 + warp; i < n_rows; i += (long long)gridDim.x * 8) {
-    const XT* row = X + (size_t)i * ld;
-    const float yy = y[i];
-    float acc = 0.0f;
-    if constexpr (VEC) {
-      const long long chunks = d / V;
-      auto add = [&](const uint4& raw, long long c) {
-        float x[V];
-        XVec<XT>::widen(raw, x);
-#pragma unroll
-        for (int e = 0; e < V; e += 4) {
-          const float4 q = __ldg((const float4*)(w + c * V + e));
-          acc = fmaf(q.x, x[e], acc); acc = fmaf(q.y, x[e + 1], acc); acc = fmaf(q.z, x[e + 2], acc); acc = fmaf(q.w, x[e + 3], acc);
-        }
-      };
-      long long c = lane;
-      for (; c + 96 < chunks; c += 128) {
-        uint4 raw[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) raw[u] = ld_stream16(row + (c + 32 * u) * V);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) add(raw[u], c + 32 * u);
-      }
-      for (; c < chunks; c += 32) add(ld_stream16(row + c * V), c);
-    } else {
-#pragma unroll 8
-      for (long long c = lane; c < d; c += 32) acc = fmaf(w[c], widen_scalar<XT>(row[c]), acc);
-    }
-    const float z = warp_sum(acc);
+  auto hold = [&](float z, float yy) {
     if (lane == held) { z_own = z; y_own = yy; }
     if (++held == 32) evaluate();
+  };
+  auto add = [&](const uint4& raw, long long c, float& acc) {
+    float x[V];
+    XVec<XT>::widen(raw, x);
+#pragma unroll
+    for (int e = 0; e < V; e += 4) {
+      const float4 q = __ldg((const float4*)(w + c * V + e));
+      acc = fmaf(q.x, x[e], acc); acc = fmaf(q.y, x[e + 1], acc); acc = fmaf(q.z, x[e + 2], acc); acc = fmaf(q.w, x[e + 3], acc);
+    }
+  };
+  const long long warps = (long long)gridDim.x * 8, units = VEC ? d / V : d;
+  long long i = (long long)blockIdx.x * 8 + warp;
+  if constexpr (NARROW) {
+    constexpr int R = 4, U = VEC ? 1 : 2;
+    for (; i < n_rows; i += R * warps) {
+      float yy[R], acc[R];
+      uint4 raw[R];
+      float x[R][U];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const bool in = i + r * warps < n_rows;
+        const XT* row = X + (size_t)(in ? i + r * warps : i) * ld;
+        yy[r] = y[in ? i + r * warps : i];
+        if constexpr (VEC) {
+          raw[r] = ld_stream16_if(row + lane * V, lane < units);
+        } else {
+#pragma unroll
+          for (int u = 0; u < U; ++u) x[r][u] = lane + 32 * u < units ? widen_scalar<XT>(row[lane + 32 * u]) : 0.0f;
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        acc[r] = 0.0f;
+        if constexpr (VEC) {
+          if (lane < units) add(raw[r], lane, acc[r]);
+        } else {
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (lane + 32 * u < units) acc[r] = fmaf(w[lane + 32 * u], x[r][u], acc[r]);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r) acc[r] = warp_sum(acc[r]);
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (i + r * warps < n_rows) hold(acc[r], yy[r]);
+    }
+  } else {
+    for (; i < n_rows; i += warps) {
+      const XT* row = X + (size_t)i * ld;
+      const float yy = y[i];
+      float acc = 0.0f;
+      long long c = lane;
+      if constexpr (VEC) {
+        for (; c + 96 < units; c += 128) {
+          uint4 raw[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) raw[u] = ld_stream16(row + (c + 32 * u) * V);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) add(raw[u], c + 32 * u, acc);
+        }
+        for (; c < units; c += 32) add(ld_stream16(row + c * V), c, acc);
+      } else {
+        float x[4], q[4];
+#pragma unroll 2
+        for (; c + 96 < units; c += 128) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) { x[u] = widen_scalar<XT>(row[c + 32 * u]); q[u] = w[c + 32 * u]; }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) acc = fmaf(q[u], x[u], acc);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          x[u] = c + 32 * u < units ? widen_scalar<XT>(row[c + 32 * u]) : 0.0f;
+          q[u] = c + 32 * u < units ? w[c + 32 * u] : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc = fmaf(q[u], x[u], acc);
+      }
+      hold(warp_sum(acc), yy);
+    }
   }
   evaluate();
   objective_finish(lsum, esum, w, d, lambda, n_rows, part, ticket, out);

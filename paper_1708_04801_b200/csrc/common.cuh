@@ -104,5 +104,13 @@ __device__ __forceinline__ uint4 ld_stream16(const void* p) {
                : "l"(p));
   return r;
 }
+// The same where `yes` (zeros elsewhere): a predicate, not a branch.
+__device__ __forceinline__ uint4 ld_stream16_if(const void* p, bool yes) {
+  uint4 r = make_uint4(0u, 0u, 0u, 0u);
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %5, 0;\n\t@p ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];\n\t}"
+               : "+r"(r.x), "+r"(r.y), "+r"(r.z), "+r"(r.w)
+               : "l"(p), "r"((int)yes));
+  return r;
+}
 
 }  // namespace wpsgd

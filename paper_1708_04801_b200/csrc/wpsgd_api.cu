@@ -1398,8 +1398,13 @@ wpsgd_status wpsgd_objective(wpsgd_ctx* c, const void* X, wpsgd_xtype xt, int64_
   };
   const size_t es = xt == WPSGD_X_F32 ? 4 : 2;
   const bool vec = aligned16(X) && aligned16(w) && ((size_t)ld_elems * es) % 16 == 0 && ((size_t)c->d * es) % 16 == 0;
-  if (xt == WPSGD_X_F32) vec ? go(objective_rows_kernel<float, true>, (const float*)X) : go(objective_rows_kernel<float, false>, (const float*)X);
-  else vec ? go(objective_rows_kernel<__nv_bfloat16, true>, (const __nv_bfloat16*)X) : go(objective_rows_kernel<__nv_bfloat16, false>, (const __nv_bfloat16*)X);
+  const bool narrow = (size_t)c->d * es <= 32 * (vec ? 16 : 2 * es);  // at most one load (two where they are of single elements) per lane
+  auto pick = [&](auto vec_tag, auto narrow_tag) {
+    if (xt == WPSGD_X_F32) go(objective_rows_kernel<float, vec_tag.value, narrow_tag.value>, (const float*)X);
+    else go(objective_rows_kernel<__nv_bfloat16, vec_tag.value, narrow_tag.value>, (const __nv_bfloat16*)X);
+  };
+  if (vec) narrow ? pick(std::true_type(), std::true_type()) : pick(std::true_type(), std::false_type());
+  else narrow ? pick(std::false_type(), std::true_type()) : pick(std::false_type(), std::false_type());
   CU_TRY(c, cudaGetLastError());
   c->launches++;
   return WPSGD_OK;

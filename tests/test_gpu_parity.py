@@ -765,6 +765,27 @@ def test_objective_and_error_rate(P, loss, bf16):
     assert abs(out[1] - err) <= 2.0 / 666  # a margin within fp32 rounding of 0 may flip
 
 
+@pytest.mark.parametrize("d", [1, 31, 33, 64, 65, 96, 97, 128, 129, 160, 161, 256, 257, 264, 520])
+@pytest.mark.parametrize("bf16,shift", [(False, 0), (True, 0), (False, 1)])
+def test_objective_row_widths(P, d, bf16, shift):
+    # around the ends of the loads in flight: 32 and 128 chunks of 16 bytes, 64 and 128 single elements; rows that start off 16
+    # bytes (shift); row counts that leave warps with one to four rows in flight (37) and with several turns of them (40000)
+    for rows in (37, 40000 if d <= 64 else 9600):
+        g = torch.Generator().manual_seed(d)
+        X = torch.randn(rows * d + shift, generator=g)
+        X = (X.to(torch.bfloat16) if bf16 else X)
+        w = torch.randn(d, generator=g) / np.sqrt(d)
+        y = torch.sign(torch.randn(rows, generator=g))
+        with P.Context(1, d) as ctx:
+            out = ctx.objective(X.cuda()[shift:].view(rows, d), y.cuda(), w.cuda(), 0.01, LOGISTIC).cpu().numpy()
+            ctx.check()
+        Xr = X[shift:].view(rows, d).contiguous()
+        obj, err = oracle.objective_dense(Xr, y, w.numpy().astype(np.float64), 0.01, LOGISTIC)
+        # the rounding of a margin (some units of 2^-24 of sum |w x|) is of either sign and averages out over the rows
+        assert out[0] == pytest.approx(obj, rel=1e-6)
+        assert abs(out[1] - err) <= 2.0 / rows
+
+
 # ---- host-buffer entry point --------------------------------------------------------------------------------
 def test_solve_host_equals_device_path(P):
     wl = wi.config2(k=5, d=256, m=128, base_steps=200)
