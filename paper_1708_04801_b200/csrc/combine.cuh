@@ -268,7 +268,36 @@ __global__ void __launch_bounds__(256, sizeof(XT) == 2 ? 5 : 4) objective_rows_k
   objective_finish(lsum, esum, w, d, lambda, n_rows, part, ticket, out);
 }
 
-// CSR rows: eight lanes per row (rows of a few tens of nonzeros), four rows per warp.
+// Lane l of L: its share of w . x over the nonzeros b .. e - 1 of a row
+template <int L>
+__device__ __forceinline__ float csr_margin_part(const int* __restrict__ col_idx, const float* __restrict__ val, const float* __restrict__ w,
+                                                 long long b, long long e, int l) {
+  float acc = 0.0f;
+  if constexpr (L == 8) {  // (short rows: predicated batches as below cost them 3 to 6 %)
+#pragma unroll 4
+    for (long long q = b + l; q < e; q += 8) acc = fmaf(w[col_idx[q]], val[q], acc);
+  } else {
+    for (long long q = b + l; q - l < e; q += 4 * L) {
+      int c[4];
+      float v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        c[u] = q + L * u < e ? col_idx[q + L * u] : 0;
+        v[u] = q + L * u < e ? val[q + L * u] : 0.0f;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (q + L * u < e) acc = fmaf(w[c[u]], v[u], acc);
+    }
+  }
+  return acc;
+}
+
+// CSR rows. LANES = 8: four rows per warp (rows of a few tens of nonzeros), except that a warp with a row of more than 512 takes
+// its rows in turn with all lanes. LANES = 32: for so few rows that every warp has one at most, whatever their length (the host
+// decides by the row count: 100 rows of 10000 nonzeros take 62 us with all lanes of a warp, 206 with eight; 9000 rows of 30 take
+// 22.1 and 20.7).
+template <int LANES>
 __global__ void __launch_bounds__(256) objective_rows_csr_kernel(const long long* __restrict__ row_ptr, const int* __restrict__ col_idx,
                                                                  const float* __restrict__ val, const float* __restrict__ y,
                                                                  long long n_rows, const float* __restrict__ w, long long d,
@@ -276,19 +305,28 @@ __global__ void __launch_bounds__(256) objective_rows_csr_kernel(const long long
                                                                  double* __restrict__ out) {
   kernel_started();
   kernel_inputs_ready();
-  const int l8 = threadIdx.x & 7;
+  constexpr int ROWS = 256 / LANES;  // of a block
+  const int lane = threadIdx.x & 31, sub = threadIdx.x & (LANES - 1);
   double lsum = 0.0, esum = 0.0;
   // the same trip count for all rows of a warp (shuffles)
-  for (long long i0 = (long long)blockIdx.x * 32; i0 < n_rows; i0 += (long long)gridDim.x * 32) {
-    const long long i = i0 + (threadIdx.x >> 3);
+  for (long long i0 = (long long)blockIdx.x * ROWS; i0 < n_rows; i0 += (long long)gridDim.x * ROWS) {
+    const long long i = i0 + threadIdx.x / LANES;
     const bool in = i < n_rows;
     const long long b = in ? row_ptr[i] : 0, e = in ? row_ptr[i + 1] : 0;
     float acc = 0.0f;
-#pragma unroll 4
-    for (long long q = b + l8; q < e; q += 8) acc = fmaf(w[col_idx[q]], val[q], acc);
+    if (LANES < 32 && __any_sync(0xffffffffu, e - b > 512)) {
+#pragma unroll 1
+      for (int r = 0; r < 32 / LANES; ++r) {
+        const long long rb = __shfl_sync(0xffffffffu, b, r * LANES), re = __shfl_sync(0xffffffffu, e, r * LANES);
+        const float z = warp_sum(csr_margin_part<32>(col_idx, val, w, rb, re, lane));
+        if (lane / LANES == r) acc = z;
+      }
+    } else {
+      acc = csr_margin_part<LANES>(col_idx, val, w, b, e, sub);
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (in && l8 == 0) {
+      for (int o = LANES / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    }
+    if (in && sub == 0) {
       const float yy = y[i];
       lsum += loss_value(loss, yy, acc);
       esum += ((acc >= 0.0f) != (yy >= 0.0f)) ? 1.0 : 0.0;

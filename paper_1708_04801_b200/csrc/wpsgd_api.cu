@@ -1417,11 +1417,12 @@ wpsgd_status wpsgd_objective_csr(wpsgd_ctx* c, const int64_t* row_ptr, const int
   if (!w || !out || n_rows < 0 || (int)loss < 0 || (int)loss > 2 || (n_rows > 0 && (!row_ptr || !col_idx || !val || !y)))
     return fail(c, WPSGD_ERR_INVALID_ARG, "objective_csr: bad argument");
   DeviceGuard guard(c->device);
-  const int nblk = grid_for((n_rows + 31) / 32, 1, 148 * 8);
+  const bool few = n_rows <= 148 * 8 * 4;  // half the warps that the GPU holds
+  const int nblk = grid_for(few ? (n_rows + 7) / 8 : (n_rows + 31) / 32, 1, 148 * 8);
   wpsgd_status s = grow(c, &c->part, &c->part_cap, (size_t)nblk * 3);
   if (s != WPSGD_OK) return s;
-  launch(objective_rows_csr_kernel, nblk, 256, 0, c->stream, (const long long*)row_ptr, col_idx, val, y, n_rows, w, c->d, (int)loss, lambda,
-                                                         c->part, c->ticket, out);
+  launch(few ? objective_rows_csr_kernel<32> : objective_rows_csr_kernel<8>, nblk, 256, 0, c->stream, (const long long*)row_ptr, col_idx, val, y, n_rows, w,
+         c->d, (int)loss, lambda, c->part, c->ticket, out);
   CU_TRY(c, cudaGetLastError());
   c->launches++;
   return WPSGD_OK;

@@ -786,6 +786,30 @@ def test_objective_row_widths(P, d, bf16, shift):
         assert abs(out[1] - err) <= 2.0 / rows
 
 
+@pytest.mark.parametrize("rows", [1, 300, 4736, 4737])
+def test_objective_csr_rows_of_all_lengths(P, rows):
+    # 4736 rows are the most that get a warp each; above, four rows share a warp unless one is longer than 512
+    g = torch.Generator().manual_seed(rows)
+    d = 3000
+    kinds = [0, 1, 7, 8, 33, 127, 128, 129] + [2] * 20
+    lengths = [kinds[i % len(kinds)] for i in range(rows)]
+    for i, n in ((0, 513), (5, 512), (9, 2900), (rows - 1, 1025)):
+        if i < rows:
+            lengths[i] = n
+    rp = torch.zeros(rows + 1, dtype=torch.int64)
+    rp[1:] = torch.cumsum(torch.tensor(lengths), 0)
+    ci = torch.cat([torch.sort(torch.randint(0, d, (n,), generator=g))[0] for n in lengths]).to(torch.int32)
+    va = torch.randn(len(ci), generator=g) / 8
+    y = torch.sign(torch.randn(rows, generator=g))
+    w = torch.randn(d, generator=g)
+    with P.Context(1, d) as ctx:
+        out = ctx.objective_csr(rp.cuda(), ci.cuda(), va.cuda(), y.cuda(), w.cuda(), 0.01, SQUARED).cpu().numpy()
+        ctx.check()
+    obj, err = oracle.objective_csr(rp, ci, va, y, w.numpy().astype(np.float64), 0.01, SQUARED)
+    assert out[0] == pytest.approx(obj, rel=1e-6)
+    assert abs(out[1] - err) <= 2.0 / rows
+
+
 # ---- host-buffer entry point --------------------------------------------------------------------------------
 def test_solve_host_equals_device_path(P):
     wl = wi.config2(k=5, d=256, m=128, base_steps=200)
