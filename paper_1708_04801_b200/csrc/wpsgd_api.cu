@@ -3,6 +3,7 @@
 #include "../../include/wpsgd.h"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -755,6 +756,40 @@ double through(double x, std::initializer_list<std::pair<double, double>> pts) {
   return a->second * x / a->first;
 }
 
+// Clusters of C CTAs, one CTA per SM, that are resident at once. A cluster lies within one GPC and the GPCs differ in size from
+// GPU to GPU, so the driver is asked, once per device: where 148 / 8 = 18 or 16 of 8 were taken for granted, 16 equally long
+// chains over 8 CTAs each ran in two waves (measured: 15 of 8, 33 of 4, 74 of 2).
+int cluster_slots(int device, int C, size_t chains) {
+  if (C == 1) return 148;
+  const int i = C == 2 ? 0 : (C == 4 ? 1 : 2);
+  const int nominal = 148 / C;
+  if (chains * (size_t)C <= 64) return nominal;  // these fit in any case
+  static std::atomic<int> known[64][3];  // 0: not asked yet
+  if (device < 64 && known[device][i] > 0) return known[device][i];
+  auto kern = chain_lag_kernel<float, 8, 1>;
+  const size_t smem = 200 * 1024;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(nominal * C));
+  cfg.blockDim = dim3(LAG_MAX_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)C;
+  at.val.clusterDim.y = 1;
+  at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    n = C == 2 ? 74 : (C == 4 ? 32 : 14);
+  }
+  n = std::min(n, nominal);
+  if (device < 64) known[device][i] = n;
+  return n;
+}
+
 template <typename XT>
 double lag_estimate(const wpsgd_ctx* c, const LagShape& sh) {
   constexpr bool F32 = sizeof(XT) == 4;
@@ -766,9 +801,7 @@ double lag_estimate(const wpsgd_ctx* c, const LagShape& sh) {
                      : through(x, {{8, 1150}, {32, 1245}, {64, 1390}, {128, 1740}, {256, 2670}, {512, 7800}});
   if (sh.C == 8) L += 80.0;
   if (sh.realign) L = std::max(L, through(x, {{8, 1150}, {32, 1310}, {64, 1880}, {128, 3050}, {256, 9100}}));
-  // resident clusters of 1, 2, 4, 8 CTAs with one CTA per SM
-  const int slots = sh.C == 1 ? 148 : (sh.C == 2 ? 74 : (sh.C == 4 ? 36 : 16));
-  return run_estimate(c, slots, L, 0.0, 5000.0 + 40.0 * x, 10000.0);
+  return run_estimate(c, cluster_slots(c->device, sh.C, c->steps_sorted.size()), L, 0.0, 5000.0 + 40.0 * x, 10000.0);
 }
 
 // The lagged form's best cluster size (or the one asked for); the estimate, or a negative number when it does not fit.
@@ -819,7 +852,7 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
     const double w = (double)mma_shape.cpc;
     const double L = through(w, {{64, 1260}, {128, 1330}, {256, 1820}}) * (full || mma_shape.C > 1 ? 1.0 : 1.14) * (decay ? 1.1 : 1.0);
     if (mma_shape.C == 1) mma_t = shared_estimate(Mma16Smem(mma_shape.stages16, (size_t)mma_shape.cpc * 16).total, L, through(w, {{32, 620}, {64, 800}, {128, 1090}, {256, 1820}}));
-    else mma_t = run_estimate(c, 148 / mma_shape.C, L, 0.0, 0.0, 6000.0);
+    else mma_t = run_estimate(c, cluster_slots(c->device, mma_shape.C, c->steps_sorted.size()), L, 0.0, 0.0, 6000.0);
   }
   if (variant == 0) {
     double best = lag_t;
