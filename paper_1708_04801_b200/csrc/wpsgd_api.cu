@@ -65,7 +65,7 @@ struct wpsgd_ctx {
   std::vector<long long> steps_done;
   std::vector<int> node_ids;
   std::vector<long long> last_steps;    // step counts of the launch being prepared
-  std::vector<long long> steps_sorted;  // the same, largest first
+  std::vector<long long> steps_sorted;  // step counts that the estimates of a launch go by, largest first (see estimate_for)
   double steps_sum = 0.0;
   float eta0 = 0.f, lambda = 0.f;
   int sched = 0, loss = 0;
@@ -842,7 +842,7 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
   // several CTAs share an SM (as many as their shared memory lets in): a chain then takes a fifth longer
   auto shared_estimate = [&](size_t smem, double L, double I) {
     const int per_sm = std::max(1, std::min(4, (int)(227 * 1024 / (smem + 1024))));
-    return run_estimate(c, 148 * per_sm, c->k > 148 && per_sm > 1 ? 1.2 * L : L, I, 0.0, 6000.0);
+    return run_estimate(c, 148 * per_sm, c->steps_sorted.size() > 148 && per_sm > 1 ? 1.2 * L : L, I, 0.0, 6000.0);
   };
   const bool decay = c->sched == WPSGD_LR_INV_SQRT;
   double mma_t = -1.0;
@@ -976,10 +976,6 @@ wpsgd_status run_dense_common(wpsgd_ctx* c, const void* X, wpsgd_xtype xt, long 
   s = upload_plan_and_stream(c, pl);
   if (s != WPSGD_OK) return s;
   c->last_steps = pl.steps;
-  c->steps_sorted.resize(c->k);
-  for (int j = 0; j < c->k; ++j) c->steps_sorted[j] = pl.steps[pl.order[j]];
-  c->steps_sum = 0.0;
-  for (long long n : pl.steps) c->steps_sum += (double)n;
   ChainParams p;
   p.X = X; p.ld = ld; p.y = y;
   p.shard_off = c->t_shard_off; p.n_steps = c->t_steps; p.first = c->t_first; p.idx_off = c->t_idx_off;
@@ -988,7 +984,21 @@ wpsgd_status run_dense_common(wpsgd_ctx* c, const void* X, wpsgd_xtype xt, long 
   p.status = c->status;
   s = timing_begin(c);
   if (s != WPSGD_OK) return s;
+  // The estimates go by the chains of one launch. For groups of nodes that run one after another these are the group's, with its
+  // step counts scaled to the longest chain of the run: groups of a run then differ in the number of chains only, and where all
+  // of them fit the GPU at once anyway every group takes the kernel, and gives the bits, of a run on rows that lie on the device.
+  auto estimate_for = [&](int first_slot, int count) {
+    const long long longest = pl.steps[pl.order[0]], own = pl.steps[pl.order[first_slot]];
+    c->steps_sorted.resize(count);
+    c->steps_sum = 0.0;
+    for (int i = 0; i < count; ++i) {
+      const long long n = pl.steps[pl.order[first_slot + i]];
+      c->steps_sorted[i] = own == longest ? n : (own > 0 ? (long long)((double)n / (double)own * (double)longest) : longest);
+      c->steps_sum += (double)c->steps_sorted[i];
+    }
+  };
   if (!groups) {
+    estimate_for(0, c->k);
     s = (xt == WPSGD_X_F32) ? launch_dense<float>(c, p) : launch_dense<__nv_bfloat16>(c, p);
     if (s != WPSGD_OK) return s;
   } else {
@@ -997,6 +1007,7 @@ wpsgd_status run_dense_common(wpsgd_ctx* c, const void* X, wpsgd_xtype xt, long 
     for (const LaunchGroup& g : *groups) {
       CU_TRY(c, cudaStreamWaitEvent(c->stream, g.ready, 0));
       if (g.count > 0) {
+        estimate_for(first_slot, g.count);
         ChainParams q = p;
         q.order = c->t_order + first_slot;
         q.k = g.count;

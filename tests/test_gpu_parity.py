@@ -846,6 +846,26 @@ def test_solve_host_pipelined_equals_device_path(P, d, bf16, k, pipeline):
         ctx.check()
 
 
+def test_solve_host_pipelined_groups_take_the_kernel_of_their_own_size(P):
+    # 64 chains in four launches of 16: each launch has the GPU to itself and has to run what a context of these 16 nodes
+    # runs (a cluster of CTAs per chain), not what 64 chains at once would take (one CTA per chain)
+    wl = wi.config2(k=64, d=1024, m=48, base_steps=8)
+    wl.n_steps = 420 - np.arange(64, dtype=np.int64)
+    dev = wl.to("cuda")
+    with P.Context(wl.k, wl.d) as ctx:
+        ctx.solve_host(wl.X.pin_memory(), wl.y.pin_memory(), wl.shard_off, wl.n_steps, wl.eta0, wl.sched, wl.lam, wl.loss, wl.seed)
+        W = ctx.get_models().cpu().numpy()
+        ctx.check()
+    for g in range(0, 64, 16):
+        lo, hi = int(wl.shard_off[g]), int(wl.shard_off[g + 16])
+        with P.Context(16, wl.d) as ctx:
+            ctx.set_node_ids(np.arange(g, g + 16))
+            ctx.run(dev.X[lo:hi], dev.y[lo:hi], wl.shard_off[g:g + 17] - lo, wl.n_steps[g:g + 16], wl.eta0, wl.sched, wl.lam, wl.loss,
+                    wl.seed)
+            np.testing.assert_array_equal(W[g:g + 16], ctx.get_models().cpu().numpy())
+            ctx.check()
+
+
 def test_solve_host_csr_equals_device_path(P):
     wl = wi.config4(k=5, d=4096, m=200, base_steps=500, mean_nnz=25.0)
     wl.w0 = torch.full((4096,), 0.02)
