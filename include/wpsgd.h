@@ -85,8 +85,7 @@ wpsgd_status wpsgd_destroy(wpsgd_ctx* ctx);
  *                     one warp per node. 4: blocked form (8 samples per synchronisation), one CTA per node. 5: blocked
  *                     form, one warp per node (rows of at most 64 16-byte chunks). 8: blocked form for aligned bf16 rows
  *                     with tensor-core Gram blocks, columns of a node split over a thread-block cluster ("block_samples"
- *                     0: 16 samples per block with margins on the tensor cores as well, or variant 10 where that is
- *                     estimated to be faster). 9: variant 10 for aligned fp32 rows with at most 256 columns per CTA.
+ *                     0: 16 samples per block, with margins on the tensor cores as well, where that fits). 9: variant 10 for aligned fp32 rows with at most 256 columns per CTA.
  *                     10: blocked form whose margins are taken from the model one block back, any alignment, a cluster
  *                     of 1, 2, 4 or 8 CTAs per node (what 0 picks for most runs of up to 148 nodes). 0 compares estimates
  *                     of the whole run. The blocked forms (4, 5, 8, 9, 10) take both step-size schedules and need

@@ -837,7 +837,7 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
   const bool mma_ok = !F32 && mma_kernel_fits(c, aligned, &mma_shape);
   LagShape lag_shape;
   double lag_t = -1.0;
-  if (variant == 0 || variant >= 8) lag_t = best_lag_shape<XT>(c, aligned, &lag_shape);
+  if (variant == 0 || variant == 10) lag_t = best_lag_shape<XT>(c, aligned, &lag_shape);
   const double x = (double)chunks;
   // several CTAs share an SM (as many as their shared memory lets in): a chain then takes a fifth longer
   auto shared_estimate = [&](size_t smem, double L, double I) {
@@ -881,7 +881,6 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
     if (lag_t >= 0.0) offer(aligned && chunks > 512 && chunks <= 512 * 4, 2, run_estimate(c, 148, 7000.0 + 5.4 * x, 0.0, 0.0, 6000.0));
     if (best < 0.0) variant = !aligned || chunks > 512 * 4 ? 1 : (chunks <= 64 ? 3 : 2);
   }
-  if (variant == 8 && c->opt_block_samples == 0 && lag_t >= 0.0 && aligned && !F32 && (!mma_ok || lag_t < mma_t)) variant = 10;
   if (variant == 9) {
     // fp32 rows, at most 64 chunks of a row per CTA: with clusters of the size asked for, else the best one
     double best = -1.0;

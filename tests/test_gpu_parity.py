@@ -398,7 +398,7 @@ def test_mma_kernel_bounded_waits_report_timeout_and_context_survives(P, d, clus
     assert rel_l2(v, ov) <= 1e-4
 
 
-# ---- fp32 rows, 16 samples per block, a chain spread over a cluster (Gram block on the fp32 pipes) ----------------------
+# ---- fp32 rows, a chain spread over a cluster: variant 9, the lagged form with at most 64 chunks of a row per CTA ------------------------
 @pytest.mark.parametrize("d,cluster", [(1024, 8), (1024, 4), (512, 2), (256, 1), (1000, 8), (36, 1), (2048, 8)])
 @pytest.mark.parametrize("loss", [HINGE, LOGISTIC, SQUARED])
 def test_f32_cluster_kernel_losses_and_widths(P, d, cluster, loss):
@@ -552,7 +552,7 @@ def test_logistic_large_steps_between_correlated_rows(P, variant, d):
 
 @pytest.mark.parametrize("k,variant", [(4, 9), (40, 4)])
 def test_default_kernels_for_large_aligned_fp32_rows(P, k, variant):
-    # few chains: each spread over a cluster of idle SMs (16 samples per block); many chains: one CTA each (8 per block)
+    # few chains: each spread over a cluster of idle SMs (lagged form); many chains: one CTA each
     wl = wi.config2(k=k, d=1024, m=64, base_steps=100).to("cuda")
     with P.Context(wl.k, wl.d) as a, P.Context(wl.k, wl.d) as b:
         a.run_workload(wl)
@@ -572,6 +572,38 @@ def test_tensor_core_cluster_kernel_is_the_default_for_wide_bf16_rows(P):
         np.testing.assert_array_equal(a.get_models().cpu().numpy(), b.get_models().cpu().numpy())
         a.check()
         b.check()
+
+
+def _models(P, wl, **opts):
+    with P.Context(wl.k, wl.d) as ctx:
+        for name, value in opts.items():
+            ctx.set_option(name, value)
+        ctx.run_workload(wl)
+        W = ctx.get_models().cpu().numpy()
+        ctx.check()
+    return W
+
+
+def test_dense_variant_8_forces_the_tensor_core_kernel(P):
+    # few chains of 1000 steps: variant 10 is the default there, and an explicit 8 is not
+    wl = wi.config3(k=3, d=1024, m=64, n_lo=1000, n_hi=1000).to("cuda")
+    W8 = _models(P, wl, dense_variant=8)
+    np.testing.assert_array_equal(W8, _models(P, wl, dense_variant=8, block_samples=16))
+    W10 = _models(P, wl, dense_variant=10)
+    assert not np.array_equal(W8, W10)
+    np.testing.assert_array_equal(_models(P, wl), W10)
+
+
+def test_default_kernels_far_from_the_crossover(P):
+    # every form sums in another order, so equal bits name the kernel
+    wide = wi.config3(k=128, d=4096, m=16, n_lo=60, n_hi=120).to("cuda")
+    W = _models(P, wide)
+    np.testing.assert_array_equal(W, _models(P, wide, dense_variant=8, block_samples=16))
+    assert not np.array_equal(W, _models(P, wide, dense_variant=10))
+    few = wi.config2(k=4, d=1024, m=64, base_steps=400).to("cuda")
+    W = _models(P, few)
+    np.testing.assert_array_equal(W, _models(P, few, dense_variant=10))
+    assert not np.array_equal(W, _models(P, few, dense_variant=4))
 
 
 # ---- degenerate cases -----------------------------------------------------------------------------------
