@@ -43,10 +43,6 @@ struct BlockParams {
   const int* group_order;  // warp-per-node kernel: node of every (CTA, warp) slot, -1 = none
 };
 
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
-  const uint32_t s = (uint32_t)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem_src) : "memory");
-}
 // the copy happens where `yes`: a predicate, not a branch (branches inside unrolled code end the stretch in which accesses
 // overlap, and cost more than the accesses)
 __device__ __forceinline__ void cp_async16_if(uint32_t smem_dst, const void* gmem_src, bool yes) {

@@ -163,7 +163,6 @@ __device__ __forceinline__ int4 lds_s32x4(uint32_t a) {
   asm volatile("ld.shared.v4.s32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
   return v;
 }
-__device__ __forceinline__ void sts_f32(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
 __device__ __forceinline__ void sts_u16(uint32_t a, int v) {
   asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((unsigned short)v) : "memory");
 }
@@ -195,11 +194,6 @@ __device__ __forceinline__ void prefetch_l2_if(const void* a, bool yes) {
 }
 __device__ __forceinline__ void sts_f32_if(uint32_t a, float v, bool yes) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p st.shared.f32 [%0], %1;\n\t}" ::"r"(a), "f"(v), "r"((int)yes) : "memory");
-}
-__device__ __forceinline__ int atoms_cas(uint32_t a, int cmp, int val) {
-  int old;
-  asm volatile("atom.shared.cas.b32 %0, [%1], %2, %3;" : "=r"(old) : "r"(a), "r"(cmp), "r"(val) : "memory");
-  return old;
 }
 __device__ __forceinline__ int atoms_add(uint32_t a, int val) {
   int old;

@@ -143,11 +143,6 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
   const uint32_t a = (uint32_t)__cvta_generic_to_shared(bar);
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(a) : "memory");
 }
-// 4-byte store into the shared memory of a CTA of the cluster, counted on that CTA's barrier `mbar`
-__device__ __forceinline__ void st_async_f32(uint32_t addr, float v, uint32_t mbar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(addr), "f"(v), "r"(mbar)
-               : "memory");
-}
 // try_wait with a suspend-time hint: the warp sleeps until the phase completes or about 20 microseconds have passed, so
 // waiting roles take no issue slots from the ones that work
 __device__ __forceinline__ bool mbar_sleep_wait(uint32_t a, uint32_t parity) {

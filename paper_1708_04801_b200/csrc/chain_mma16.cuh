@@ -41,7 +41,6 @@
 namespace wpsgd {
 
 constexpr int M16_B = 16;
-constexpr int M16_PAIRS = M16_B * (M16_B - 1) / 2;  // 120
 constexpr int M16_SLOT_FLOATS = 256;   // D0 [16][8] | D1 rows 8..15 [8][8] | p parts [16][4]
 constexpr uint32_t M16_SLOT_BYTES = M16_SLOT_FLOATS * sizeof(float);
 constexpr int M16_SLOTS = 8;           // one slot per CTA of the cluster
