@@ -124,7 +124,8 @@ def input_bytes(wl) -> int:
 
 
 def ctas_of(wl) -> int:
-    """CTAs the default chain kernel of this workload launches (for the SM coverage figure)."""
+    """CTAs the default chain kernel of this workload launches (for the SM coverage figure): the library's choice restated for
+    the shapes timed here."""
     if wl.sparse:
         return wl.k
     chunks = wl.d // (8 if wl.xtype == 1 else 4)
@@ -134,8 +135,8 @@ def ctas_of(wl) -> int:
             c //= 2
         if c >= 4 and (chunks + c - 1) // c <= 64:
             return wl.k * c
-    if chunks <= 64:
-        return (wl.k + 3) // 4            # four nodes (warps) per CTA
+    if chunks <= 64:                      # few chains: a CTA each; many: four nodes (warps) per CTA
+        return wl.k if wl.k <= N_SMS else (wl.k + 3) // 4
     if wl.xtype == 1 and chunks >= 256:
         c = 1
         while (chunks + c - 1) // c > 256 and c < 8:

@@ -237,7 +237,7 @@ wpsgd_status launch_combine_form(wpsgd_ctx* c, const double* weights, float* v_o
   InlineWeights<(N > 0 ? N : 1)> iw;
   if (N > 0) memcpy(iw.w, weights, c->k * sizeof(double));
   else CU_TRY(c, cudaMemcpyAsync(c->t_weights, weights, c->k * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  const int warps = std::max(1, std::min(VEC == 4 ? 16 : 32, (c->k + 3) / 4));  // (64 KB of sums would leave one block per SM)
+  const int warps = std::max(1, std::min(VEC == 4 ? 16 : 32, (c->k + 3) / 4));  // (32 warps of four columns were not measured)
   const unsigned blocks = (unsigned)((c->d + 32 * VEC - 1) / (32 * VEC));
   launch(combine_kernel<VEC, N>, blocks, 32 * warps, (size_t)warps * 32 * VEC * sizeof(double), c->stream, iw, c->W, c->t_weights, scale, c->k, c->d, v_out);
   CU_TRY(c, cudaGetLastError());
@@ -1062,8 +1062,9 @@ wpsgd_status run_csr_common(wpsgd_ctx* c, const long long* row_ptr, const int* c
     const size_t smem = sizeof(CsrBlockSmem);
     auto go = [&](auto kern) -> wpsgd_status {
       CU_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      // Launched after its predecessor, without the wait that an early start needs inside the kernel: the wait, with the set-up of
-      // shared memory before it, was measured by itself at 12.0 against 11.16 ms (64 chains, 40 nonzeros per row).
+      // Launched after its predecessor, without the wait that an early start needs inside the kernel. With one body for all chains
+      // the wait made no difference by itself (64 chains, 40 nonzeros per row: 12.18 ms with it and without; see
+      // chain_csr_block_kernel for what did); the chains are long, so the plain launch costs nothing.
       kern<<<c->k, CSRB_THREADS, smem, c->stream>>>(p);
       CU_TRY(c, cudaGetLastError());
       return WPSGD_OK;

@@ -125,7 +125,7 @@ def test_losses_and_schedules(P, loss, sched, variant):
 
 
 def test_generic_kernel_handles_unaligned_shapes(P):
-    # d = 67 (not a multiple of 4), row stride 71: only the generic kernel applies, and auto must pick it
+    # d = 67 (not a multiple of 4), row stride 71: the register and the aligned blocked kernels do not apply
     g = torch.Generator().manual_seed(3)
     k, d, ld, m = 3, 67, 71, 50
     Xp = torch.randn(k * m, ld, generator=g) / 8
@@ -148,7 +148,7 @@ def test_generic_kernel_handles_unaligned_shapes(P):
 
 
 def test_large_d_falls_back_and_matches(P):
-    wl = wi.config2(k=2, d=8200, m=16, base_steps=40)  # beyond the register kernels' reach
+    wl = wi.config2(k=2, d=8200, m=16, base_steps=40)  # beyond the register kernels' reach (the default spreads a row over a cluster)
     assert_parity(P, wl)
 
 
