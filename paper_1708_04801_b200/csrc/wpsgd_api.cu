@@ -582,7 +582,7 @@ bool two_warp_ctas_per_sm_finish_first(const std::vector<long long>& steps, int 
 
 // ---- blocked kernel with lagged margins ---------------------------------------------------------------------------------
 struct LagShape {
-  int C = 1, cpc = 0, stages = 0, teams = 1, gram_warps = 1, model_warps = 1, vb = 8, nc = 1, realign = 0, copy_warps = 2, warps = 0;
+  int C = 1, cpc = 0, stages = 0, teams = 1, gram_warps = 1, model_warps = 1, vb = 8, nc = 1, raw_stages = 0, realign_warps = 0, realign_rows = 1, copy_warps = 2, warps = 0;
   size_t smem = 0;
 };
 
@@ -597,26 +597,40 @@ bool lag_kernel_fits(const wpsgd_ctx* c, bool aligned, int C, LagShape* out) {
   LagShape sh;
   sh.C = C;
   sh.cpc = (int)cpc;
-  sh.realign = aligned ? 0 : 1;
-  // a model thread owns one vector of 8 bytes where two warps cover the slice (the rows of two blocks then stay in
-  // registers), else one or two of 16; with realigning warps there is room for four model warps, else for eight
-  const int max_mw = sh.realign ? 4 : 8;
-  if (cpc > 32 * max_mw * 2) return false;
-  sh.vb = cpc <= 64 ? 8 : 16;
-  sh.nc = cpc <= 32 * max_mw ? 1 : 2;
+  // A model thread owns one vector of 8 bytes in narrow slices (the rows of two blocks then stay in registers), else one or two of
+  // 16: 64 fp32 chunks 1143 cycles per block with 16-byte vectors, 1236 with 8-byte ones (twice as many warps); 63 bf16 chunks
+  // 1106 and 1054.
+  if (cpc > (aligned ? 512 : 256)) return false;
+  sh.vb = cpc <= (sizeof(XT) == 4 ? 32 : 64) ? 8 : 16;
+  sh.nc = cpc <= 32 * (aligned ? (C > 1 ? 6 : 8) : 4) ? 1 : 2;
   const int per_warp = 32 * sh.vb * sh.nc;
   sh.model_warps = (int)((cpc * 16 + per_warp - 1) / per_warp);
-  int want = c->opt_stages > 0 ? std::max(3, c->opt_stages) : 8;
+  // As deep a ring as there is room for. Realigning warps: a block each and both rings in multiples of four up to 64 chunks (fp32,
+  // 31 chunks, 12 chains: 1314 cycles per block, 1490 with all warps on every block), else all on a block (128 chunks: 3050, 5100).
+  if (!aligned) {
+    sh.realign_warps = LAG_REALIGN_WARPS;
+    sh.realign_rows = cpc <= 64 && (c->opt_stages == 0 || c->opt_stages >= 4) ? 1 : LAG_REALIGN_WARPS;
+  }
+  int want = c->opt_stages > 0 ? std::max(3, c->opt_stages) : LAG_MAX_STAGES;
   for (; want >= 3; --want) {
-    sh.smem = LagSmem(want, (size_t)cpc * 16, C, LAG_GRAM_WARPS, sh.realign).total;
+    if (!aligned && sh.realign_rows == 1 && want % LAG_REALIGN_WARPS != 0) continue;
+    sh.raw_stages = aligned ? 0 : (sh.realign_rows > 1 ? 3 : (want >= 8 ? LAG_MAX_RAW_STAGES : 4));
+    sh.smem = LagSmem(want, (size_t)cpc * 16, C, LAG_GRAM_WARPS, sh.raw_stages).total;
     if (sh.smem <= kSmemBudget + 4096) break;
   }
   if (want < 3 || (want < 4 && C < 8 && c->opt_stages == 0 && c->opt_cluster == 0)) return false;
+  // Gram teams: four of one warp, two of two or one of all, as the ring feeds them (a team holds two stages while it works). With more
+  // than two teams the ring is a multiple of their number, so that a team has seen every earlier block of the stages it
+  // waits for (else a barrier's parity could stand for an older phase).
+  int others = 3 + (C > 1 ? 1 : 0) + sh.model_warps + sh.realign_warps;
+  const int gram = (others + LAG_GRAM_WARPS + 1) * 32 > LAG_MAX_THREADS ? LAG_GRAM_WARPS - 1 : LAG_GRAM_WARPS;
+  others += gram;
+  if (want >= 8) want -= want % 4;
+  sh.teams = want >= 8 ? 4 : (want >= 5 ? 2 : 1);
+  if (gram == 3) sh.teams = want % 3 == 0 ? 3 : 1;
+  sh.gram_warps = gram / sh.teams;
   sh.stages = want;
-  // as many Gram teams as the ring feeds: a team holds two stages while it works
-  sh.teams = want >= 7 ? 4 : (want >= 5 ? 2 : 1);
-  sh.gram_warps = LAG_GRAM_WARPS / sh.teams;
-  const int others = 3 + sh.model_warps + LAG_GRAM_WARPS + (sh.realign ? LAG_REALIGN_WARPS : 0);
+  sh.smem = LagSmem(want, (size_t)cpc * 16, C, LAG_GRAM_WARPS, sh.raw_stages).total;
   sh.copy_warps = (others + 2) * 32 <= LAG_MAX_THREADS ? 2 : 1;
   sh.warps = others + sh.copy_warps;
   if (sh.warps * 32 > LAG_MAX_THREADS) return false;
@@ -627,6 +641,7 @@ bool lag_kernel_fits(const wpsgd_ctx* c, bool aligned, int C, LagShape* out) {
 template <typename XT>
 wpsgd_status launch_lag(wpsgd_ctx* c, const ChainParams& p, const LagShape& sh) {
   LagParams lp;
+  int launch_warps = 0;
   lp.b.c = p;
   lp.b.stages = sh.stages;
   lp.b.eta_lambda = (double)c->eta0 * (double)c->lambda;
@@ -637,13 +652,39 @@ wpsgd_status launch_lag(wpsgd_ctx* c, const ChainParams& p, const LagShape& sh) 
   lp.gram_teams = sh.teams;
   lp.gram_warps = sh.gram_warps;
   lp.model_warps = sh.model_warps;
-  lp.realign = sh.realign;
+  lp.raw_stages = sh.raw_stages;
+  lp.realign_warps = sh.realign_warps;
+  lp.realign_rows = sh.realign_rows;
   lp.copy_warps = sh.copy_warps;
+  // Warp w runs on scheduler w mod 4. The scheduler of the recurrence warp gets only the two short loops beside it (sums of q,
+  // constants); the others are dealt out over the other three (16 chains of 1024 fp32 columns, logistic: 1058 cycles per block
+  // with the roles in plain order, 908 this way; all four gram warps on one scheduler: 1136).
+  {
+    const int sums = sh.C > 1 ? 1 : 0, constants = 1 + sh.model_warps + sums + sh.copy_warps, gram = constants + 2;
+    std::vector<int> first = {0}, rest;
+    if (sums) first.push_back(1 + sh.model_warps);
+    first.push_back(constants);
+    for (int i = 0; i < sh.model_warps; ++i) rest.push_back(1 + i);
+    const int g0 = sizeof(XT) == 4 && sh.cpc > 40 ? 1 : 0;
+    if (g0) first.push_back(gram);
+    for (int i = g0; i < sh.teams * sh.gram_warps; ++i) rest.push_back(gram + i);
+    rest.push_back(constants + 1);  // feeder
+    for (int i = 0; i < sh.copy_warps; ++i) rest.push_back(1 + sh.model_warps + sums + i);
+    for (int i = gram + sh.teams * sh.gram_warps; i < sh.warps; ++i) rest.push_back(i);  // realign
+    for (; rest.size() > 12; rest.pop_back()) first.push_back(rest.back());
+    const int warps = 4 * (int)std::max(first.size(), (rest.size() + 2) / 3);
+    size_t a = 0, b = 0;
+    for (int w = 0; w < LAG_MAX_THREADS / 32; ++w) {
+      if (w % 4 == 0) lp.role[w] = a < first.size() ? (unsigned char)first[a++] : 255;
+      else lp.role[w] = b < rest.size() ? (unsigned char)rest[b++] : 255;
+    }
+    launch_warps = warps;
+  }
   auto go = [&](auto kern) -> wpsgd_status {
     CU_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p.k * sh.C));
-    cfg.blockDim = dim3((unsigned)(32 * sh.warps));
+    cfg.blockDim = dim3((unsigned)(32 * launch_warps));
     cfg.dynamicSmemBytes = sh.smem;
     cfg.stream = c->stream;
     cudaLaunchAttribute at[2];
@@ -659,9 +700,13 @@ wpsgd_status launch_lag(wpsgd_ctx* c, const ChainParams& p, const LagShape& sh) 
     c->launches++;
     return WPSGD_OK;
   };
-  if (sh.nc == 2) return go(chain_lag_kernel<XT, 16, 2>);
-  if (sh.vb == 16) return go(chain_lag_kernel<XT, 16, 1>);
-  return go(chain_lag_kernel<XT, 8, 1>);
+  auto pick = [&](auto multi, auto realign) -> wpsgd_status {
+    if (sh.nc == 2) return go(chain_lag_kernel<XT, 16, 2, multi.value, realign.value>);
+    if (sh.vb == 16) return go(chain_lag_kernel<XT, 16, 1, multi.value, realign.value>);
+    return go(chain_lag_kernel<XT, 8, 1, multi.value, realign.value>);
+  };
+  if (sh.C > 1) return sh.raw_stages ? pick(std::true_type(), std::true_type()) : pick(std::true_type(), std::false_type());
+  return sh.raw_stages ? pick(std::false_type(), std::true_type()) : pick(std::false_type(), std::false_type());
 }
 
 // blocked kernel, one warp per node (small d)
@@ -766,7 +811,7 @@ int cluster_slots(int device, int C, size_t chains) {
   if (chains * (size_t)C <= 64) return nominal;  // these fit in any case
   static std::atomic<int> known[64][3];  // 0: not asked yet
   if (device < 64 && known[device][i] > 0) return known[device][i];
-  auto kern = chain_lag_kernel<float, 8, 1>;
+  auto kern = chain_lag_kernel<float, 8, 1, true, false>;
   const size_t smem = 200 * 1024;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(nominal * C));
@@ -795,12 +840,12 @@ double lag_estimate(const wpsgd_ctx* c, const LagShape& sh) {
   constexpr bool F32 = sizeof(XT) == 4;
   const double x = (double)sh.cpc;
   double L;
-  if (F32) L = sh.C == 1 ? through(x, {{8, 860}, {16, 890}, {32, 990}, {64, 1210}, {128, 1945}, {256, 3800}, {512, 9600}})
-                         : through(x, {{8, 1020}, {16, 1045}, {32, 1155}, {64, 1345}, {128, 2025}, {256, 3890}, {512, 10200}});
-  else L = sh.C == 1 ? through(x, {{8, 955}, {32, 1005}, {64, 1165}, {128, 1460}, {256, 2490}, {512, 7100}})
-                     : through(x, {{8, 1150}, {32, 1245}, {64, 1390}, {128, 1740}, {256, 2670}, {512, 7800}});
-  if (sh.C == 8) L += 80.0;
-  if (sh.realign) L = std::max(L, through(x, {{8, 1150}, {32, 1310}, {64, 1880}, {128, 3050}, {256, 9100}}));
+  if (F32) L = sh.C == 1 ? through(x, {{8, 725}, {16, 740}, {32, 815}, {48, 920}, {64, 1090}, {96, 1430}, {128, 1875}, {256, 3490}, {512, 6850}})
+                         : through(x, {{8, 790}, {16, 800}, {32, 840}, {48, 1000}, {64, 1130}, {96, 1500}, {128, 1940}, {256, 3640}, {384, 5560}, {512, 11200}});
+  else L = sh.C == 1 ? through(x, {{16, 785}, {32, 890}, {64, 1025}, {96, 1320}, {128, 1560}, {192, 1890}, {256, 2410}, {384, 3730}, {512, 5450}})
+                     : through(x, {{16, 885}, {48, 935}, {64, 1035}, {96, 1265}, {128, 1510}, {192, 1970}, {256, 2790}, {384, 4300}, {512, 6130}});
+  if (sh.C == 8) L += 25.0;
+  if (sh.realign_warps) L = std::max(L, through(x, {{8, 850}, {16, 920}, {32, 1180}, {48, 1500}, {64, 1800}, {96, 2450}, {128, 3050}, {256, 9100}}));
   return run_estimate(c, cluster_slots(c->device, sh.C, c->steps_sorted.size()), L, 0.0, 5000.0 + 40.0 * x, 10000.0);
 }
 
@@ -837,9 +882,12 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
   const bool mma_ok = !F32 && mma_kernel_fits(c, aligned, &mma_shape);
   LagShape lag_shape;
   double lag_t = -1.0;
-  if (variant == 0 || variant == 10) lag_t = best_lag_shape<XT>(c, aligned, &lag_shape);
+  if ((variant == 0 || variant == 10) && p.ld * (long long)sizeof(XT) < (1ll << 31)) lag_t = best_lag_shape<XT>(c, aligned, &lag_shape);
   const double x = (double)chunks;
   // several CTAs share an SM (as many as their shared memory lets in): a chain then takes a fifth longer
+  // Where the tensor-core kernel takes the shape it keeps the runs of few blocks (up to 16 at 2048 columns): both forms then last 14 to
+  // 25 us, most of it launch and start-up.
+  if (mma_ok && lag_t >= 0.0) lag_t += 7500.0;
   auto shared_estimate = [&](size_t smem, double L, double I) {
     const int per_sm = std::max(1, std::min(4, (int)(227 * 1024 / (smem + 1024))));
     return run_estimate(c, 148 * per_sm, c->steps_sorted.size() > 148 && per_sm > 1 ? 1.2 * L : L, I, 0.0, 6000.0);
@@ -884,7 +932,7 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
   if (variant == 9) {
     // fp32 rows, at most 64 chunks of a row per CTA: with clusters of the size asked for, else the best one
     double best = -1.0;
-    for (int C = 1; F32 && aligned && C <= 8; C *= 2) {
+    for (int C = 1; F32 && aligned && p.ld * (long long)sizeof(XT) < (1ll << 31) && C <= 8; C *= 2) {
       LagShape sh;
       if ((c->opt_cluster > 0 && C != c->opt_cluster) || (chunks + C - 1) / C > 64 || !lag_kernel_fits<XT>(c, aligned, C, &sh)) continue;
       const double t = lag_estimate<XT>(c, sh);
