@@ -86,7 +86,7 @@ __device__ __forceinline__ void ldmatrix_x2(uint32_t (&r)[2], const void* smem_p
 }
 
 // FULL: every math warp of every CTA owns 32 chunks, so that the unrolled pass has no guards (see the note above).
-template <int LOSS, bool FULL>
+template <int LOSS, bool FULL, int MAXC>
 __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const ClusterParams cp) {
   constexpr int B = M16_B;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const Clust
         float4 s0 = r4[lane], s1 = r4[32 + lane];
 #pragma unroll
         for (int w = 1; w < M16_SLOTS; ++w) {
-          if ((uint32_t)w >= C) break;
+          if (w >= MAXC || (uint32_t)w >= C) break;
           const float4 v0 = r4[w * (M16_SLOT_FLOATS / 4) + lane], v1 = r4[w * (M16_SLOT_FLOATS / 4) + 32 + lane];
           s0.x += v0.x; s0.y += v0.y; s0.z += v0.z; s0.w += v0.w;
           s1.x += v1.x; s1.y += v1.y; s1.z += v1.z; s1.w += v1.w;
@@ -419,9 +419,9 @@ __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const Clust
   const unsigned char* w_src = w3 + (size_t)((lane & 7) < 3 ? (lane & 7) : 3) * row_stride + warp_col_bytes + (size_t)((lane >> 3) & 1) * 16;
   // shared-memory window of every CTA of the cluster (the same offsets apply inside each window)
   const uint32_t own_base = (uint32_t)__cvta_generic_to_shared(smem);
-  uint32_t peer_base[8];
+  uint32_t peer_base[MAXC];
 #pragma unroll
-  for (int rr = 0; rr < 8; ++rr) peer_base[rr] = map_shared_rank(smem, (uint32_t)rr < C ? (uint32_t)rr : rank);
+  for (int rr = 0; rr < MAXC; ++rr) peer_base[rr] = map_shared_rank(smem, (uint32_t)rr < C ? (uint32_t)rr : rank);
   cluster_barrier();  // start-up
 
   const int g8 = lane >> 2, t4 = lane & 3;
@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(64 + 32 * 8, 1) chain_mma16_kernel(const Clust
         }
       const uint32_t od = (uint32_t)__cvta_generic_to_shared(red + ((size_t)q * M16_SLOTS + rank) * M16_SLOT_FLOATS + 4 * e) - own_base;
 #pragma unroll
-      for (int rr = 0; rr < 8; ++rr)
+      for (int rr = 0; rr < MAXC; ++rr)
         if ((uint32_t)rr < C) st_async_f32x4(peer_base[rr] + od, sum, peer_base[rr] + ob);
     }
   };

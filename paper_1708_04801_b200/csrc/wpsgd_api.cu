@@ -539,11 +539,17 @@ wpsgd_status launch_mma(wpsgd_ctx* c, const ChainParams& p, const ClusterShape& 
   };
   if (b16) {
     const bool full = sh.cpc % 32 == 0 && (long long)sh.cpc * sh.C * 8 == c->d;
-    switch (c->loss) {
-      case WPSGD_LOSS_HINGE: return full ? go(chain_mma16_kernel<LOSS_HINGE, true>) : go(chain_mma16_kernel<LOSS_HINGE, false>);
-      case WPSGD_LOSS_LOGISTIC: return full ? go(chain_mma16_kernel<LOSS_LOGISTIC, true>) : go(chain_mma16_kernel<LOSS_LOGISTIC, false>);
-      default: return full ? go(chain_mma16_kernel<LOSS_SQUARED, true>) : go(chain_mma16_kernel<LOSS_SQUARED, false>);
-    }
+    auto pick = [&](auto loss, auto is_full) -> wpsgd_status {
+      return sh.C <= 2 ? go(chain_mma16_kernel<loss.value, is_full.value, 2>) : go(chain_mma16_kernel<loss.value, is_full.value, 8>);
+    };
+    auto with_loss = [&](auto is_full) -> wpsgd_status {
+      switch (c->loss) {
+        case WPSGD_LOSS_HINGE: return pick(std::integral_constant<int, LOSS_HINGE>(), is_full);
+        case WPSGD_LOSS_LOGISTIC: return pick(std::integral_constant<int, LOSS_LOGISTIC>(), is_full);
+        default: return pick(std::integral_constant<int, LOSS_SQUARED>(), is_full);
+      }
+    };
+    return full ? with_loss(std::true_type()) : with_loss(std::false_type());
   }
   switch (c->loss) {
     case WPSGD_LOSS_HINGE: return go(chain_mma_kernel<LOSS_HINGE, 4>);
