@@ -868,32 +868,6 @@ __global__ void __launch_bounds__(32 * BLKW_MAX_WARPS) chain_block_warp_kernel(c
   if (nb > 0) y_nxt = yshard[idx[n]];
   if (nb > 1) id_nxt = idx[B + n];
 
-  // Gram entries of the rows in raw: lane l gets the total of entry l. Packed two-wide fp32 FMAs: even and odd columns accumulate
-  // side by side and are added at the end.
-  constexpr int NP = XPairs<XT>::NP;
-  auto gram_total = [&](const uint4 (&raw)[R][B]) __attribute__((always_inline)) -> float {
-    float2 acc2[BLK_PAIRS];
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        float2 x2[B];
-#pragma unroll
-        for (int m = 0; m < B; ++m) x2[m] = XPairs<XT>::get(raw[r][m], i);
-#pragma unroll
-        for (int n2 = 1; n2 < B; ++n2)
-#pragma unroll
-          for (int m = 0; m < n2; ++m) {
-            float2& t = acc2[n2 * (n2 - 1) / 2 + m];
-            t = r == 0 && i == 0 ? __fmul2_rn(x2[m], x2[n2]) : __ffma2_rn(x2[m], x2[n2], t);
-          }
-      }
-    float acc[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) acc[i] = i < BLK_PAIRS ? acc2[i].x + acc2[i].y : 0.0f;
-    return warp_transpose_sum32(acc);
-  };
-  // (Forming the Gram entries one block ahead, beside the steps, took 3850 cycles per block at d = 256 instead of 2370: 13 KB more code.)
   int st = 0;
   for (long long b = 0; b < nb; ++b) {
     const int nv = (int)((n_run - b * B) < (long long)B ? (n_run - b * B) : (long long)B);
@@ -909,21 +883,43 @@ __global__ void __launch_bounds__(32 * BLKW_MAX_WARPS) chain_block_warp_kernel(c
       for (int m = 0; m < B; ++m) raw[r][m] = lds_u32x4(at[r] + (uint32_t)st * stage_step[r] + (uint32_t)m * row_step[r]);
     prefetch_block(b + S, st, id_lo, id_hi);
     load_ids(b + 1 + S, id_lo, id_hi);
-    scratch[lane] = gram_total(raw);
-    // ---- p_b ---------------------------------------------------------------------------------------------------
-    float accp[B];
+    // ---- G_b and p_b in one pass -----------------------------------------------------------------------
+    // packed two-wide fp32 FMAs: even and odd columns accumulate side by side and are added at the end
+    float acc[32], accp[B];
+    {
+      constexpr int NP = XPairs<XT>::NP;
+      float2 acc2[BLK_PAIRS], accp2[B];
 #pragma unroll
-    for (int m = 0; m < B; ++m) {
-      float2 t = __fmul2_rn(make_float2(w[0][0], w[0][1]), XPairs<XT>::get(raw[0][m], 0));
+      for (int i = 0; i < BLK_PAIRS; ++i) acc2[i] = make_float2(0.0f, 0.0f);
 #pragma unroll
-      for (int r = 0; r < R; ++r)
+      for (int m = 0; m < B; ++m) accp2[m] = make_float2(0.0f, 0.0f);
 #pragma unroll
-        for (int i = 0; i < NP; ++i)
-          if (r > 0 || i > 0) t = __ffma2_rn(make_float2(w[r][2 * i], w[r][2 * i + 1]), XPairs<XT>::get(raw[r][m], i), t);
-      accp[m] = t.x + t.y;
+      for (int r = 0; r < R; ++r) {
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+          float2 x2[B];
+#pragma unroll
+          for (int m = 0; m < B; ++m) x2[m] = XPairs<XT>::get(raw[r][m], i);
+#pragma unroll
+          for (int n2 = 1; n2 < B; ++n2)
+#pragma unroll
+            for (int m = 0; m < n2; ++m) acc2[n2 * (n2 - 1) / 2 + m] = __ffma2_rn(x2[m], x2[n2], acc2[n2 * (n2 - 1) / 2 + m]);
+          const float2 wp = make_float2(w[r][2 * i], w[r][2 * i + 1]);
+#pragma unroll
+          for (int m = 0; m < B; ++m) accp2[m] = __ffma2_rn(wp, x2[m], accp2[m]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < BLK_PAIRS; ++i) acc[i] = acc2[i].x + acc2[i].y;
+#pragma unroll
+      for (int i = BLK_PAIRS; i < 32; ++i) acc[i] = 0.0f;
+#pragma unroll
+      for (int m = 0; m < B; ++m) accp[m] = accp2[m].x + accp2[m].y;
     }
     const float ptot = warp_transpose_sum8(accp);   // every lane: total of p_{lane >> 2}
+    const float gtot = warp_transpose_sum32(acc);   // lane l: total of Gram entry l
     // all 28 + 8 totals into every lane (through the warp's scratch line)
+    scratch[lane] = gtot;
     if ((lane & 3) == 0) scratch[32 + (lane >> 2)] = ptot;
     __syncwarp();
     float Gs[BLK_PAIRS], pv[B];
@@ -955,6 +951,7 @@ __global__ void __launch_bounds__(32 * BLKW_MAX_WARPS) chain_block_warp_kernel(c
     block8_recurrence<LOSS>(t, Gs, cf, yv, y_cur * apw_own * 1.4426950408889634f * pv_own, (float4*)(scratch + 40), beta);
     // ---- w <- w - (1 - a^nv) w - sum_m gamma_m x_m,  gamma_m = beta_m a^nv ----------------------------------
     {
+      constexpr int NP = XPairs<XT>::NP;
       float2 ngm2[B];
 #pragma unroll
       for (int m = 0; m < B; ++m) {
