@@ -25,8 +25,8 @@ __device__ __forceinline__ void set_status(DevStatus* st, int code, int where, l
 
 // Launches of the library overlap their start-up with the end of the kernel before them (programmatic dependent launch): a
 // kernel is launched once every block of its predecessor has called kernel_started() or ended, and every block calls
-// kernel_inputs_ready(), which waits until the predecessor has completed, before it touches memory; so a kernel's completion
-// implies that of all before it (chain_csr_block_kernel is launched without the overlap, which comes to the same). The short
+// kernel_inputs_ready(), which waits until the predecessor has completed, before it touches memory (index_stream_kernel: before it
+// ends); so a kernel's completion implies that of all before it (chain_csr_block_kernel is launched without the overlap, which comes to the same). The short
 // kernels call kernel_started() at once. The chains do not: the blocks that wait would hold shared memory and thread slots of
 // the SMs for as long as the chains run, which kernels of other streams can use.
 // Measured: 16 rounds of set models, stream, short chains, combine (fp32, 32 chains of 512 columns): 622 -> 461 us; objective of

@@ -133,13 +133,18 @@ struct InlineTables {
 };
 
 // All nodes' streams for one launch of the chains. Node = blockIdx.y (+ gridDim.y per pass). BYTES > 0: the tables are the
-// argument `t`, and block (0, 0) writes them to `tables` for the kernels that follow.
+// argument `t`, and block (0, 0) writes them to `tables` for the kernels that follow. What is written is read by chain kernels only, and
+// those let the kernel after them start when their last block has ended (they do not call kernel_started): whoever read the
+// old tables and streams is done when this kernel starts. So nothing has to be waited for first, and the streams are formed while
+// the kernels before are still at work; the wait stands at the end (a kernel's completion implies that of all before it).
+// `wait_first`: a stream kernel before this one was not followed by chains and may still be writing. 16 rounds of combine, set
+// models, stream and short chains, squared loss: 32 x 512 fp32 369 -> 342 us; logistic, 100 x 200: 424 -> 388.
 template <int BYTES>
-__global__ void __launch_bounds__(256) index_stream_kernel(const __grid_constant__ InlineTables<(BYTES > 0 ? BYTES : 16)> t, int sampling,
+__global__ void __launch_bounds__(256) index_stream_kernel(const __grid_constant__ InlineTables<(BYTES > 0 ? BYTES : 16)> t, int wait_first, int sampling,
                                                            uint64_t seed, int k, unsigned char* __restrict__ tables,
                                                            uint32_t* __restrict__ idx) {
   kernel_started();
-  kernel_inputs_ready();
+  if (BYTES == 0 || wait_first) kernel_inputs_ready();
   const TableLayout L(k);
   const unsigned char* src = BYTES > 0 ? t.b : tables;
   if (BYTES > 0 && blockIdx.x == 0 && blockIdx.y == 0)
@@ -153,6 +158,7 @@ __global__ void __launch_bounds__(256) index_stream_kernel(const __grid_constant
     emit_indices(sampling, seed, (uint32_t)ids[j], first[j], steps[j], cnt, (uint32_t)(off[j + 1] - off[j]), idx + idx_off[j],
                  (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
   }
+  kernel_inputs_ready();
 }
 
 // One node's stream, for callers that want to look at it.

@@ -43,6 +43,7 @@ struct wpsgd_ctx {
   double* t_weights = nullptr;       // [k]
   uint32_t* idx = nullptr;
   size_t idx_cap = 0;  // entries
+  bool streams_read = false;  // every stream kernel so far has been followed by a launch of chains
   DevStatus* status = nullptr;
   double* part = nullptr;  // objective partial sums
   size_t part_cap = 0;     // doubles
@@ -298,7 +299,7 @@ template <int BYTES>
 void launch_index_stream(wpsgd_ctx* c, dim3 grid, size_t bytes) {
   InlineTables<(BYTES > 0 ? BYTES : 16)> t;
   if (BYTES > 0) memcpy(t.b, c->h_tables.data(), bytes);
-  launch(index_stream_kernel<BYTES>, grid, 256, 0, c->stream, t, c->opt_sampling, c->seed, c->k, c->tables, c->idx);
+  launch(index_stream_kernel<BYTES>, grid, 256, 0, c->stream, t, c->streams_read ? 0 : 1, c->opt_sampling, c->seed, c->k, c->tables, c->idx);
 }
 
 wpsgd_status upload_plan_and_stream(wpsgd_ctx* c, const Plan& pl) {
@@ -327,6 +328,7 @@ wpsgd_status upload_plan_and_stream(wpsgd_ctx* c, const Plan& pl) {
     if (!as_argument) launch_index_stream<0>(c, grid, 0);
     else if (L.total <= 2048) launch_index_stream<2048>(c, grid, L.total);
     else launch_index_stream<8192>(c, grid, L.total);
+    c->streams_read = false;
     CU_TRY(c, cudaGetLastError());
     c->launches++;
   }
@@ -1073,7 +1075,7 @@ wpsgd_status run_dense_common(wpsgd_ctx* c, const void* X, wpsgd_xtype xt, long 
   s = timing_end(c);
   if (s != WPSGD_OK) return s;
   for (int j = 0; j < c->k; ++j) c->steps_done[j] = first[j] + n_steps[j];
-  c->have_run = true;
+  c->have_run = c->streams_read = true;
   c->scaled = false;
   return WPSGD_OK;
 }
@@ -1134,7 +1136,7 @@ wpsgd_status run_csr_common(wpsgd_ctx* c, const long long* row_ptr, const int* c
   s = timing_end(c);
   if (s != WPSGD_OK) return s;
   for (int j = 0; j < c->k; ++j) c->steps_done[j] = first[j] + n_steps[j];
-  c->have_run = true;
+  c->have_run = c->streams_read = true;
   c->scaled = true;
   return WPSGD_OK;
 }

@@ -506,6 +506,53 @@ def test_lagged_kernel_shapes(P, d, bf16, pad, cluster, loss, sched):
         assert rel_l2(W[j], oW[j]) <= TOL[loss]
 
 
+@pytest.mark.parametrize("d,bf16,cluster", [
+    (1024, False, 8), (1056, False, 8), (1284, False, 8), (1320, False, 8),  # 32 / 33 / 41 / 42 chunks of a CTA: 8- and 16-byte vectors, Gram warps on all schedulers
+    (1024, True, 2), (1040, True, 2),                                        # 64 / 65 bf16 chunks
+    (1536, False, 2), (1544, False, 2), (3072, False, 2), (2000, False, 1),  # 192 / 193 / 384 chunks: one and two vectors per thread, three Gram warps
+    (1023, False, 4), (1025, False, 4), (1021, False, 2), (2049, True, 1),   # unaligned: 64 / 65 chunks (a block per warp, all warps per block), 128, 257
+    (2047, False, 4), (3071, False, 4), (5999, False, 8),
+])
+@pytest.mark.parametrize("loss,sched", [(LOGISTIC, 0), (SQUARED, 1)])
+def test_lagged_kernel_roles_at_their_limits(P, d, bf16, cluster, loss, sched):
+    wl = wi.config2(k=3, d=d, m=48, base_steps=260)
+    wl.n_steps = np.array([260, 129, 5], dtype=np.int64)
+    wl.loss, wl.sched = loss, sched
+    if loss == SQUARED:
+        wl.y = (wl.y * 0.3).contiguous()
+    if bf16:
+        wl.X = wl.X.to(torch.bfloat16)
+    if (d * (2 if bf16 else 4) + 15) // 16 > (256 if d % 2 else 512) * cluster:
+        with pytest.raises(P.WpsgdError):  # more chunks of a row than the CTAs take
+            gpu_solve(P, wl, {"dense_variant": 10, "cluster": cluster})
+        return
+    assert_parity(P, wl, {"dense_variant": 10, "cluster": cluster})
+
+
+@pytest.mark.parametrize("k", [3, 240])  # tables as an argument of the stream kernel, and copied
+def test_runs_in_a_row_do_not_read_each_others_streams(P, k):
+    # the stream of a run is formed while kernels before it are still at work; a run that is refused after its stream was
+    # launched must not disturb the next one
+    wl = wi.config2(k=k, d=40, m=32, base_steps=90).to("cuda")
+    want = []
+    for seed in (1, 2):
+        with P.Context(wl.k, wl.d) as ctx:
+            wl.seed = seed
+            ctx.run_workload(wl)
+            want.append(ctx.combine().cpu().numpy())
+    with P.Context(wl.k, wl.d) as ctx:
+        for rep in range(6):
+            wl.seed = 1 + rep % 2
+            if rep >= 2:
+                ctx.set_option("dense_variant", 8)  # fp32 rows: refused
+                with pytest.raises(P.WpsgdError):
+                    ctx.run_workload(wl)
+                ctx.set_option("dense_variant", 0)
+            ctx.run_workload(wl)
+            v = ctx.combine()
+            np.testing.assert_array_equal(v.cpu().numpy(), want[rep % 2])
+
+
 @pytest.mark.parametrize("stages", [0, 3, 4, 5])
 @pytest.mark.parametrize("n_steps", [(1, 7, 8), (9, 15, 16), (17, 0, 64), (333, 250, 3)])
 def test_lagged_kernel_block_boundaries_and_ring_depths(P, n_steps, stages):
