@@ -1,6 +1,7 @@
 """The C-ABI library: it builds, loads and exports every symbol the header declares; its host-side
 logic (weights, argument checks) is checked against the oracle. No GPU compute here."""
 import ctypes
+import math
 import os
 import re
 
@@ -74,6 +75,23 @@ def test_host_weights_match_oracle(wpsgd_lib, case):
     assert holds == wholds
     assert tot == pytest.approx(wtot, rel=1e-12)
     assert abs(got.sum() - 1.0) < 1e-14
+
+
+@pytest.mark.parametrize("eta,lam", [(0.3, 1e-3), (1.0, 0.09), (9.0, 0.111), (0.1, 0.0)])
+@pytest.mark.parametrize("t", [1, 255, 256, 257, 288, 289, 5000, 70000])
+def test_host_weights_of_the_decaying_step_size_sum_every_skipped_step(wpsgd_lib, eta, lam, t):
+    # around the step from which the sums come from a formula, and the last steps, which do not: against every factor's
+    # logarithm added up without rounding. Weights are exponentials of sums of up to 8 c sqrt(t): 1e-12 allows for their rounding.
+    import paper_1708_04801_b200 as P
+
+    n = np.unique(np.clip(np.array([0, 1, 2, 254, 255, 256, 257, 300, t // 3, t - 33, t - 32, t - 31, t - 1, t]), 0, t)).astype(np.int64)
+    c = float(np.float32(eta)) * float(np.float32(lam))
+    f = np.log1p(-c / np.sqrt(np.arange(1, t + 1, dtype=np.float64)))
+    lg = np.array([math.fsum(f[int(m):]) for m in n])
+    want = np.exp(lg - lg.max())
+    got, _, tot = P.weights(n, eta, 1, lam)
+    np.testing.assert_allclose(got, want / want.sum(), rtol=1e-12, atol=0)
+    assert tot == pytest.approx(np.exp(lg).sum(), rel=1e-12)
 
 
 def test_host_weights_reject_bad_input(wpsgd_lib):
