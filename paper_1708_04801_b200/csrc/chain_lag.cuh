@@ -47,7 +47,7 @@
 //
 // What bounds a block, and what it measured (B200, 1965 MHz; cycles per block of 8 samples, 4 chains that have their SMs to
 // themselves, squared and logistic loss alike): fp32, one CTA, 16 / 32 / 64 chunks of a row 740 / 815 / 1090; eight CTAs, 32 / 64 / 128
-// chunks each 845 / 1160 / 1980; bf16, 32 / 64 / 128 chunks 890 / 1030 / 1510; rows that do not start on 16 bytes, 32 / 64 / 128
+// chunks each 845 / 1160 / 1980, 256 chunks 3720; bf16, 32 / 64 / 128 chunks 890 / 1030 / 1510; rows that do not start on 16 bytes, 32 / 64 / 128
 // chunks about 1050 / 1500 / 3000. With few chunks it is the string gamma -> update -> shares -> sum (430) -> cluster (280) -> steps
 // over two blocks, and the instruction supply; from about 64 fp32 chunks per CTA on the Gram block (shared-memory reads, 8 wavefronts
 // per chunk). Before the sums of q had a warp of their own and the code was cut: 16 / 32 (eight CTAs) / 64 bf16 chunks 815 / 1235 / 1350.
@@ -74,7 +74,9 @@ constexpr int LAG_MAX_CLUSTER = 8;
 constexpr int LAG_SUMS = 128;        // [8][8] G, then [8][8] C (a row per sample of the block)
 constexpr int LAG_MAX_MODEL_WARPS = 8;
 constexpr int LAG_GRAM_WARPS = 4;
-constexpr int LAG_QROW = 132;        // shares of q of a sample: one per model thread (or pair of them), padded
+// Shares of q of a sample: one per model thread (or pair of them), padded. (Realigned rows in 16-byte vectors have at most four model
+// warps, and their rings need the room.)
+__host__ __device__ constexpr int lag_q_row(int vb, bool realign) { return vb == 16 && realign ? 68 : 132; }
 constexpr int LAG_REALIGN_WARPS = 4;
 constexpr int LAG_MAX_THREADS = 512;
 constexpr int LAG_GROUP = 4;         // blocks whose constants are formed together
@@ -106,7 +108,7 @@ struct LagConst {
 
 struct LagSmem {
   size_t row_stride, raw_stride, ring, raw, red, part, tabs, q, qpart, cst, gam, tab, jet, full, empty, rfull, rempty, gbar, tbar, qbar, cfull, cempty, flag, total;
-  __host__ __device__ LagSmem(int stages, size_t slice_bytes, int C, int gram_warps_all, int raw_stages) {
+  __host__ __device__ LagSmem(int stages, size_t slice_bytes, int C, int gram_warps_all, int raw_stages, int q_row) {
     // odd multiples of 16 bytes: tile loads of 8 (or 4) rows at the same column never meet in a bank
     row_stride = slice_bytes + 16;
     if (row_stride % 32 == 0) row_stride += 16;
@@ -118,7 +120,7 @@ struct LagSmem {
     tabs = part + 2 * (size_t)gram_warps_all * LAG_SUMS * sizeof(float);             // [parity][gram warp][128]
     q = tabs + (size_t)(stages + 4) * LAG_SUMS * sizeof(float);
     qpart = q + (C > 1 ? LAG_QBUF * 64 * sizeof(float) : 0);                         // [LAG_QBUF][CTA / 4][sample][CTA % 4]
-    cst = qpart + 2 * LAG_B * LAG_QROW * sizeof(float);                              // [2][sample][model thread]
+    cst = qpart + 2 * LAG_B * (size_t)q_row * sizeof(float);                              // [2][sample][model thread]
     gam = cst + LAG_GROUPS * LAG_GROUP * sizeof(LagConst);
     tab = gam + 2 * LAG_GAM * sizeof(float);                                       // powers of 1 - eta lambda
     jet = tab + 3 * 16 * sizeof(float);
@@ -365,9 +367,10 @@ __device__ __forceinline__ void lag_publish(float* dst, const float (&ng)[LAG_B]
 
 // Sum of the model threads' shares of q for sample lane & 7, over this lane's quarter of them (lane >> 3): `n16` groups of 16
 // entries, those from n16 on are zero
+template <int QROW>
 __device__ __forceinline__ float lag_sum_q(const float* qp, int n16) {
   const int lane = threadIdx.x & 31;
-  const uint32_t src = (uint32_t)__cvta_generic_to_shared(qp) + (uint32_t)((lane & 7) * LAG_QROW + (lane >> 3) * 4) * 4u;
+  const uint32_t src = (uint32_t)__cvta_generic_to_shared(qp) + (uint32_t)((lane & 7) * QROW + (lane >> 3) * 4) * 4u;
   const float4 a = lds_f32x4(src), b = lds_f32x4(src + 64u), c = lds_f32x4(src + 128u), d = lds_f32x4(src + 192u);
   float v = (((a.x + b.x) + (c.x + d.x)) + ((a.y + b.y) + (c.y + d.y))) + (((a.z + b.z) + (c.z + d.z)) + ((a.w + b.w) + (c.w + d.w)));
   if (n16 > 4) {
@@ -378,7 +381,7 @@ __device__ __forceinline__ float lag_sum_q(const float* qp, int n16) {
 }
 
 // The recurrence warp's loop. What is published and kept for the next block is -gamma_m.
-template <int LOSS, bool MULTI>
+template <int LOSS, bool MULTI, int QROW>
 __device__ __forceinline__ void lag_recurrence(int nb, int TB, int C, int NM, int n16, const float* tabs, const LagConst* cst, const float* q,
                                                const float* qpart, float* gam, float4* jets, unsigned long long* qbar,
                                                unsigned long long* cempty, LagWait& wait) {
@@ -402,7 +405,7 @@ __device__ __forceinline__ void lag_recurrence(int nb, int TB, int C, int NM, in
     named_barrier(LAG_BAR_Q + (b & 1), q_threads);  // sums and constants of block b + 1 are there (one CTA: and the shares of q_b)
     float qv;
     if constexpr (!MULTI) {
-      qv = lag_sum_q(qpart + (b & 1) * (B * LAG_QROW), n16);
+      qv = lag_sum_q<QROW>(qpart + (b & 1) * (B * QROW), n16);
       qv += __shfl_xor_sync(0xffffffffu, qv, 8);
       qv += __shfl_xor_sync(0xffffffffu, qv, 16);
     } else {
@@ -460,6 +463,7 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
   constexpr int B = LAG_B;
   constexpr int V = 16 / (int)sizeof(XT);
   constexpr int VW = VB / (int)sizeof(XT);
+  constexpr int QROW = lag_q_row(VB, REALIGN);
   extern __shared__ __align__(16) unsigned char smem[];
   const BlockParams& bp = lp.b;
   const ChainParams& p = bp.c;
@@ -473,7 +477,7 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
   const int ncols = (int)(c_left < 0 ? 0 : (c_left < (long long)lp.chunks_per_cta * V ? c_left : (long long)lp.chunks_per_cta * V));
   const int my_chunks = (ncols + V - 1) / V;
   const uint32_t ld_bytes = (uint32_t)p.ld * (uint32_t)sizeof(XT);  // (the host sees to it that 32 bits hold it)
-  const LagSmem L(S, (size_t)lp.chunks_per_cta * 16, (int)C, NT * NW, REALIGN ? lp.raw_stages : 0);
+  const LagSmem L(S, (size_t)lp.chunks_per_cta * 16, (int)C, NT * NW, REALIGN ? lp.raw_stages : 0, QROW);
   const uint32_t row_stride = (uint32_t)L.row_stride;
   unsigned char* ring = smem + L.ring;
   float* red = (float*)(smem + L.red);
@@ -550,9 +554,9 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
     // =========================== recurrence ==============================================================
     float4* jets = (float4*)(smem + L.jet);
     switch (p.loss) {
-      case LOSS_HINGE: lag_recurrence<LOSS_HINGE, MULTI>(nb, TB, (int)C, NM, n16, tabs, cst, q, qpart, gam, jets, qbar, cempty, wait); break;
-      case LOSS_LOGISTIC: lag_recurrence<LOSS_LOGISTIC, MULTI>(nb, TB, (int)C, NM, n16, tabs, cst, q, qpart, gam, jets, qbar, cempty, wait); break;
-      default: lag_recurrence<LOSS_SQUARED, MULTI>(nb, TB, (int)C, NM, n16, tabs, cst, q, qpart, gam, jets, qbar, cempty, wait); break;
+      case LOSS_HINGE: lag_recurrence<LOSS_HINGE, MULTI, QROW>(nb, TB, (int)C, NM, n16, tabs, cst, q, qpart, gam, jets, qbar, cempty, wait); break;
+      case LOSS_LOGISTIC: lag_recurrence<LOSS_LOGISTIC, MULTI, QROW>(nb, TB, (int)C, NM, n16, tabs, cst, q, qpart, gam, jets, qbar, cempty, wait); break;
+      default: lag_recurrence<LOSS_SQUARED, MULTI, QROW>(nb, TB, (int)C, NM, n16, tabs, cst, q, qpart, gam, jets, qbar, cempty, wait); break;
     }
   } else if (place < first_part) {
     // =========================== model ===================================================================
@@ -580,7 +584,7 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
     }
     // this thread's shares of q_blk (16-byte vectors: added up with those of the lane 16 away, half of the samples each)
     auto put_q = [&](float (&v)[B], int blk) __attribute__((always_inline)) {
-      float* qp = qpart + (blk & 1) * (B * LAG_QROW);
+      float* qp = qpart + (blk & 1) * (B * QROW);
       if constexpr (VB == 16) {
         const bool hi = (lane & 16) != 0;
 #pragma unroll
@@ -588,13 +592,13 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
           const float send = hi ? v[i] : v[i + 4], keep = hi ? v[i + 4] : v[i];
           v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
         }
-        qp += (lane >> 4) * (4 * LAG_QROW) + mw * 16 + (lane & 15);
+        qp += (lane >> 4) * (4 * QROW) + mw * 16 + (lane & 15);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) qp[i * LAG_QROW] = v[i];
+        for (int i = 0; i < 4; ++i) qp[i * QROW] = v[i];
       } else {
         qp += mt;
 #pragma unroll
-        for (int i = 0; i < B; ++i) qp[i * LAG_QROW] = v[i];
+        for (int i = 0; i < B; ++i) qp[i * QROW] = v[i];
       }
       if (MULTI) named_arrive(LAG_BAR_SUM + (blk & 1), TM + 32);
       else named_arrive(LAG_BAR_Q + (blk & 1), bar_threads);
@@ -719,7 +723,7 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
       }
       wait.dead = wait.dead || *give_up != 0;
       named_barrier(LAG_BAR_SUM + (b & 1), sum_threads);
-      float v = lag_sum_q(qpart + (b & 1) * (B * LAG_QROW), n16);
+      float v = lag_sum_q<QROW>(qpart + (b & 1) * (B * QROW), n16);
       v += __shfl_xor_sync(0xffffffffu, v, 8);
       v += __shfl_xor_sync(0xffffffffu, v, 16);
       const uint32_t qb = (uint32_t)(b & (LAG_QBUF - 1));

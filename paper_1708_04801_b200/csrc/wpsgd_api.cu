@@ -642,26 +642,27 @@ bool lag_kernel_fits(const wpsgd_ctx* c, bool aligned, int C, LagShape* out) {
     sh.realign_warps = LAG_REALIGN_WARPS;
     sh.realign_rows = cpc <= 64 && (c->opt_stages == 0 || c->opt_stages >= 4) ? 1 : LAG_REALIGN_WARPS;
   }
+  int others = 3 + (C > 1 ? 1 : 0) + sh.model_warps + sh.realign_warps;
+  const int gram = (others + LAG_GRAM_WARPS + 1) * 32 > LAG_MAX_THREADS ? LAG_GRAM_WARPS - 1 : LAG_GRAM_WARPS;
+  others += gram;
+  const int q_row = lag_q_row(sh.vb, !aligned);
   int want = c->opt_stages > 0 ? std::max(3, c->opt_stages) : LAG_MAX_STAGES;
   for (; want >= 3; --want) {
     if (!aligned && sh.realign_rows == 1 && want % LAG_REALIGN_WARPS != 0) continue;
     sh.raw_stages = aligned ? 0 : (sh.realign_rows > 1 ? 3 : (want >= 8 ? LAG_MAX_RAW_STAGES : 4));
-    sh.smem = LagSmem(want, (size_t)cpc * 16, C, LAG_GRAM_WARPS, sh.raw_stages).total;
-    if (sh.smem <= kSmemBudget + 4096) break;
+    sh.smem = LagSmem(want, (size_t)cpc * 16, C, gram, sh.raw_stages, q_row).total;
+    if (sh.smem <= 227 * 1024) break;
   }
   if (want < 3 || (want < 4 && C < 8 && c->opt_stages == 0 && c->opt_cluster == 0)) return false;
   // Gram teams: four of one warp, two of two or one of all, as the ring feeds them (a team holds two stages while it works). With more
   // than two teams the ring is a multiple of their number, so that a team has seen every earlier block of the stages it
   // waits for (else a barrier's parity could stand for an older phase).
-  int others = 3 + (C > 1 ? 1 : 0) + sh.model_warps + sh.realign_warps;
-  const int gram = (others + LAG_GRAM_WARPS + 1) * 32 > LAG_MAX_THREADS ? LAG_GRAM_WARPS - 1 : LAG_GRAM_WARPS;
-  others += gram;
   if (want >= 8) want -= want % 4;
   sh.teams = want >= 8 ? 4 : (want >= 5 ? 2 : 1);
   if (gram == 3) sh.teams = want % 3 == 0 ? 3 : 1;
   sh.gram_warps = gram / sh.teams;
   sh.stages = want;
-  sh.smem = LagSmem(want, (size_t)cpc * 16, C, LAG_GRAM_WARPS, sh.raw_stages).total;
+  sh.smem = LagSmem(want, (size_t)cpc * 16, C, gram, sh.raw_stages, q_row).total;
   sh.copy_warps = (others + 2) * 32 <= LAG_MAX_THREADS ? 2 : 1;
   sh.warps = others + sh.copy_warps;
   if (sh.warps * 32 > LAG_MAX_THREADS) return false;
@@ -809,11 +810,10 @@ wpsgd_status launch_block_warp(wpsgd_ctx* c, const ChainParams& p, int R, int st
 // its SMs to itself (L cycles), how much of an SM's throughput it uses up when chains share one (I cycles), and how the
 // chains queue for the slots. The estimate of a run:
 //     max( longest queue of a slot x L,  all blocks x I / 148 )  +  start-up of the kernel per wave of chains,
-// with the chains in launch order (longest first) on `slots` slots. The figures are device times of runs of 300 to 4000
+// with the chains in launch order (longest first) on `slots` slots. The figures are device times of runs of 64 to 4000
 // steps with k = 4 .. 2000 chains (1965 MHz); the estimates come out within about a tenth of the times measured, e.g.
-// (measured, us) fp32 d = 1024, 4000 steps, k = 16: lagged form over 8 CTAs 322, one CTA per chain 464; k = 148: lagged
-// form over 2 CTAs 651, one CTA per chain 467; fp32 d = 128, 1000 steps, k = 200: lagged 73, CTA per chain 96, warp per
-// chain 113; k = 450: 156, 111, 123; k = 2000: 631, 285, 196.
+// (measured, us, logistic, 2048 steps) fp32 d = 1024, k = 16: lagged form 160, one CTA per chain 242; k = 100: 475, 247; d = 256,
+// k = 148: lagged 154, CTA per chain 178, warp per chain 275; k = 300: 445, 265, 275; d = 128, k = 200: 225, 202, 227.
 double run_estimate(const wpsgd_ctx* c, int slots, double L, double I, double start, double restart) {
   const std::vector<long long>& n = c->steps_sorted;
   const size_t k = n.size(), m = (size_t)slots;
