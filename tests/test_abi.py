@@ -94,6 +94,22 @@ def test_host_weights_of_the_decaying_step_size_sum_every_skipped_step(wpsgd_lib
     assert tot == pytest.approx(np.exp(lg).sum(), rel=1e-12)
 
 
+@pytest.mark.parametrize("eta,lam", [(0.3, 1e-3), (1.0, 0.09), (9.0, 0.111)])
+@pytest.mark.parametrize("t", [5000, 4000000])
+def test_host_weights_of_long_chains_do_not_cancel(wpsgd_lib, eta, lam, t):
+    # nodes a few hundred steps short of the longest chain: their sums are small differences of values of up to 2 c sqrt(t). A sum of
+    # logarithms lg, correct to a few units in its last place, gives weights correct to a few (1 + |lg|) units; 16 allowed.
+    import paper_1708_04801_b200 as P
+
+    n = np.array([t - 5000, t - 2000, t - 1000, t - 200, t - 33, t - 32, t - 1, t], dtype=np.int64)
+    c = float(np.float32(eta)) * float(np.float32(lam))
+    f = np.log1p(-c / np.sqrt(np.arange(n[0] + 1, t + 1, dtype=np.float64)))
+    lg = np.array([math.fsum(f[int(m - n[0]):]) for m in n])
+    got, _, _ = P.weights(n, eta, 1, lam)
+    err = np.abs(got / got[-1] / np.exp(lg) - 1.0)
+    assert np.all(err <= 16 * 2.0 ** -53 * (1.0 + np.abs(lg))), err
+
+
 def test_host_weights_reject_bad_input(wpsgd_lib):
     import paper_1708_04801_b200 as P
 
