@@ -391,6 +391,15 @@ wpsgd_status timing_end(wpsgd_ctx* c) {
   return WPSGD_OK;
 }
 
+// Lets a kernel take up to all of an SM's shared memory. The limit belongs to the function and so to every thread and context of
+// the process: set to the size of the launch at hand, a thread with a small ring lowered it between another's call and its
+// launch, which was then refused. It is therefore only ever set to this one value; a launch names its own size.
+constexpr size_t kSmemMax = 227 * 1024;
+template <typename Kernel>
+cudaError_t allow_all_smem(Kernel kern) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+}
+
 // ---- dense chain launch ---------------------------------------------------------------------------------
 template <typename XT, int R, int PF>
 wpsgd_status launch_reg(wpsgd_ctx* c, const ChainParams& p, bool block_per_node, int threads) {
@@ -448,7 +457,7 @@ bool block_kernel_fits(const wpsgd_ctx* c, bool aligned, int* threads_out, int* 
 template <typename XT, int R, bool OVL, int MAXW>
 wpsgd_status launch_block_r(wpsgd_ctx* c, const BlockParams& bp, int threads, size_t smem) {
   auto go = [&](auto kern) -> wpsgd_status {
-    CU_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CU_TRY(c, allow_all_smem(kern));
     launch(kern, bp.c.k, threads, smem, c->stream, bp);
     CU_TRY(c, cudaGetLastError());
     c->launches++;
@@ -549,7 +558,7 @@ wpsgd_status launch_mma(wpsgd_ctx* c, const ChainParams& p, const ClusterShape& 
   if (b16) cp.b.stages = sh.stages16;
   const size_t smem = b16 ? Mma16Smem(sh.stages16, (size_t)sh.cpc * 16).total : MmaSmem(sh.stages, (size_t)sh.cpc * 16, MMA_SLOTS).total;
   auto go = [&](auto kern) -> wpsgd_status {
-    CU_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CU_TRY(c, allow_all_smem(kern));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p.k * sh.C));
     cfg.blockDim = dim3((unsigned)(64 + 32 * sh.math_warps));
@@ -657,7 +666,7 @@ bool lag_kernel_fits(const wpsgd_ctx* c, bool aligned, int C, LagShape* out) {
     if (!aligned && sh.realign_rows == 1 && want % LAG_REALIGN_WARPS != 0) continue;
     sh.raw_stages = aligned ? 0 : (sh.realign_rows > 1 ? 3 : (want >= 8 ? LAG_MAX_RAW_STAGES : 4));
     sh.smem = LagSmem(want, (size_t)cpc * 16, C, gram, sh.raw_stages, q_row).total;
-    if (sh.smem <= 227 * 1024) break;
+    if (sh.smem <= kSmemMax) break;
   }
   if (want < 3 || (want < 4 && C < 8 && c->opt_stages == 0 && c->opt_cluster == 0)) return false;
   // Gram teams: four of one warp, two of two or one of all, as the ring feeds them (a team holds two stages while it works). With more
@@ -721,7 +730,7 @@ wpsgd_status launch_lag(wpsgd_ctx* c, const ChainParams& p, const LagShape& sh) 
     launch_warps = warps;
   }
   auto go = [&](auto kern) -> wpsgd_status {
-    CU_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem));
+    CU_TRY(c, allow_all_smem(kern));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p.k * sh.C));
     cfg.blockDim = dim3((unsigned)(32 * launch_warps));
@@ -783,7 +792,7 @@ bool block_warp_kernel_fits(const wpsgd_ctx* c, int nk, bool aligned, int* R_out
 template <typename XT, int R>
 wpsgd_status launch_block_warp_r(wpsgd_ctx* c, const BlockParams& bp, size_t smem, int ctas, int warps) {
   auto go = [&](auto kern) -> wpsgd_status {
-    CU_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CU_TRY(c, allow_all_smem(kern));
     launch(kern, ctas, 32 * warps, smem, c->stream, bp);
     CU_TRY(c, cudaGetLastError());
     c->launches++;
@@ -864,7 +873,7 @@ int cluster_slots(int device, int C, size_t chains) {
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+  if (allow_all_smem(kern) != cudaSuccess ||
       cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
     cudaGetLastError();
     n = C == 2 ? 74 : (C == 4 ? 32 : 14);
@@ -1148,7 +1157,7 @@ wpsgd_status run_csr_common(wpsgd_ctx* c, const long long* row_ptr, const int* c
   } else {
     const size_t smem = sizeof(CsrBlockSmem);
     auto go = [&](auto kern) -> wpsgd_status {
-      CU_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      CU_TRY(c, allow_all_smem(kern));
       // Launched after its predecessor, without the wait that an early start needs inside the kernel. With one body for all chains
       // the wait made no difference by itself (64 chains, 40 nonzeros per row: 12.18 ms with it and without; see
       // chain_csr_block_kernel for what did); the chains are long, so the plain launch costs nothing.

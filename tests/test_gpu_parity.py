@@ -553,6 +553,38 @@ def test_runs_in_a_row_do_not_read_each_others_streams(P, k):
             np.testing.assert_array_equal(v.cpu().numpy(), want[rep % 2])
 
 
+def test_contexts_of_two_threads_launch_one_kernel_with_different_shared_memory(P):
+    # the limit on a kernel's shared memory belongs to the process: the launch of a large ring must not meet the limit of a small one
+    import ctypes
+    import threading
+
+    failed = []
+
+    def work(d, stages):
+        X, y = torch.randn(16, d, device="cuda"), torch.ones(16, device="cuda")
+        n, off = np.array([8], dtype=np.int64), np.array([0, 16], dtype=np.int64)
+        with torch.cuda.stream(torch.cuda.Stream()), P.Context(1, d) as ctx:
+            ctx.set_option("dense_variant", 10)
+            ctx.set_option("cluster", 1)
+            ctx.set_option("stages", stages)
+            args = (ctx._h, ctypes.c_void_p(X.data_ptr()), P.X_F32, d, ctypes.c_void_p(y.data_ptr()), off.ctypes.data, n.ctypes.data, 0.01,
+                    P.LR_CONST, 1e-4, P.LOSS_SQUARED, 1, None)
+            for i in range(3000):  # the bare entry point: little between two calls but the launch
+                if ctx._lib.wpsgd_run(*args):
+                    failed.append((d, i, ctx._lib.wpsgd_last_error(ctx._h).decode()))
+                if i % 64 == 0:
+                    torch.cuda.current_stream().synchronize()
+            ctx.check()
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=a) for a in ((160, 3), (960, 6))]  # one form of the kernel, about 30 and 200 KB
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, (len(failed), failed[:3])
+
+
 @pytest.mark.parametrize("stages", [0, 3, 4, 5])
 @pytest.mark.parametrize("n_steps", [(1, 7, 8), (9, 15, 16), (17, 0, 64), (333, 250, 3)])
 def test_lagged_kernel_block_boundaries_and_ring_depths(P, n_steps, stages):
