@@ -115,6 +115,7 @@ wpsgd_status fail(wpsgd_ctx* c, wpsgd_status s, const std::string& msg) {
   do {                                                                                             \
     cudaError_t e_ = (expr);                                                                       \
     if (e_ != cudaSuccess) {                                                                       \
+      cudaGetLastError(); /* reported here, and not by the next call's look at the last error too */ \
       const bool oom_ = (e_ == cudaErrorMemoryAllocation);                                         \
       return fail(ctx, oom_ ? WPSGD_ERR_ALLOC : WPSGD_ERR_CUDA,                                    \
                   std::string(#expr) + ": " + cudaGetErrorString(e_));                             \

@@ -553,6 +553,16 @@ def test_runs_in_a_row_do_not_read_each_others_streams(P, k):
             np.testing.assert_array_equal(v.cpu().numpy(), want[rep % 2])
 
 
+def test_a_failed_allocation_does_not_fail_the_next_call(P):
+    wl = wi.config2(k=2, d=40, m=16, base_steps=40).to("cuda")
+    with P.Context(wl.k, wl.d) as ctx:
+        with pytest.raises(P.WpsgdError) as e:  # a sample stream of 1.6 TB
+            ctx.run(wl.X, wl.y, wl.shard_off, np.array([200 * 10 ** 9] * 2, dtype=np.int64), wl.eta0, wl.sched, wl.lam, wl.loss, wl.seed)
+        assert e.value.status_name == "ALLOC"
+        ctx.run_workload(wl)
+        ctx.check()
+
+
 def test_contexts_of_two_threads_launch_one_kernel_with_different_shared_memory(P):
     # the limit on a kernel's shared memory belongs to the process: the launch of a large ring must not meet the limit of a small one
     import ctypes
