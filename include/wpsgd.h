@@ -91,8 +91,7 @@ wpsgd_status wpsgd_destroy(wpsgd_ctx* ctx);
  *                     of the whole run. The blocked forms (4, 5, 8, 9, 10) take both step-size schedules and need
  *                     eta0 * lambda <= 0.25. Variant 10 reads rows that do not start on 16 bytes in whole aligned 16-byte
  *                     units: up to 15 bytes before the first and after the last byte of a row are read and not used, also
- *                     outside X, within the unit that holds the row's first or last byte (never across a page). It takes row
- *                     strides below 2 GiB.
+ *                     outside X, within the unit that holds the row's first or last byte (never across a page).
  *   "sparse_variant"  kernel for CSR rows. 0 (default) and 2: blocks of up to 64 steps run in a shared-memory cache of
  *                     the model entries they touch, in groups of 8. 1: one step per round trip to the model in global memory.
  *   "cluster"         CTAs per node of variants 8, 9 and 10: 0 (default) chosen from d (and the node count), else 1, 2, 4 or 8.

@@ -931,7 +931,7 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
   const bool mma_ok = !F32 && mma_kernel_fits(c, aligned, &mma_shape);
   LagShape lag_shape;
   double lag_t = -1.0;
-  if ((variant == 0 || variant == 10) && p.ld * (long long)sizeof(XT) < (1ll << 31)) lag_t = best_lag_shape<XT>(c, aligned, &lag_shape);
+  if (variant == 0 || variant == 10) lag_t = best_lag_shape<XT>(c, aligned, &lag_shape);
   const double x = (double)chunks;
   // several CTAs share an SM (as many as their shared memory lets in): a chain then takes a fifth longer
   // Where the tensor-core kernel takes the shape it keeps the runs of few blocks (up to 16 at 2048 columns): both forms then last 14 to
@@ -981,7 +981,7 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
   if (variant == 9) {
     // fp32 rows, at most 64 chunks of a row per CTA: with clusters of the size asked for, else the best one
     double best = -1.0;
-    for (int C = 1; F32 && aligned && p.ld * (long long)sizeof(XT) < (1ll << 31) && C <= 8; C *= 2) {
+    for (int C = 1; F32 && aligned && C <= 8; C *= 2) {
       LagShape sh;
       if ((c->opt_cluster > 0 && C != c->opt_cluster) || (chunks + C - 1) / C > 64 || !lag_kernel_fits<XT>(c, aligned, C, &sh)) continue;
       const double t = lag_estimate<XT>(c, sh);

@@ -553,6 +553,25 @@ def test_runs_in_a_row_do_not_read_each_others_streams(P, k):
             np.testing.assert_array_equal(v.cpu().numpy(), want[rep % 2])
 
 
+@pytest.mark.parametrize("variant,bf16,stride", [(9, False, 2 ** 31), (10, False, 2 ** 31 + 4), (10, True, 2 ** 32 + 16), (0, False, 2 ** 31 + 16)])
+def test_lagged_kernel_takes_row_strides_of_2_gib_and_more(P, variant, bf16, stride):
+    # three rows, 2 or 4 GiB apart (the third one beyond what 32 bits of a byte offset hold); rows off 16-byte boundaries too
+    wl = wi.config2(k=1, d=40, m=3, base_steps=40)
+    if bf16:
+        wl.X = wl.X.to(torch.bfloat16)
+    oW = oracle.run_dense(wl.X, wl.y, wl.shard_off, wl.n_steps, wl.d, wl.eta0, wl.sched, wl.lam, wl.loss, wl.seed)
+    dev = wl.to("cuda")
+    ld = stride // wl.X.element_size()
+    X = torch.empty(2 * ld + 64, dtype=wl.X.dtype, device="cuda").as_strided((3, 40), (ld, 1))
+    X.copy_(dev.X)
+    with P.Context(wl.k, wl.d) as ctx:
+        ctx.set_option("dense_variant", variant)
+        ctx.run(X, dev.y, wl.shard_off, wl.n_steps, wl.eta0, wl.sched, wl.lam, wl.loss, wl.seed)
+        W = ctx.get_models().cpu().numpy()
+        ctx.check()
+    assert rel_l2(W[0], oW[0]) <= TOL[wl.loss]
+
+
 def test_a_failed_allocation_does_not_fail_the_next_call(P):
     wl = wi.config2(k=2, d=40, m=16, base_steps=40).to("cuda")
     with P.Context(wl.k, wl.d) as ctx:
