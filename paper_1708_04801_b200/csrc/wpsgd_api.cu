@@ -934,9 +934,6 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
   if (variant == 0 || variant == 10) lag_t = best_lag_shape<XT>(c, aligned, &lag_shape);
   const double x = (double)chunks;
   // several CTAs share an SM (as many as their shared memory lets in): a chain then takes a fifth longer
-  // Where the tensor-core kernel takes the shape it keeps the runs of few blocks (up to 16 at 2048 columns): both forms then last 14 to
-  // 25 us, most of it launch and start-up.
-  if (mma_ok && lag_t >= 0.0) lag_t += 7500.0;
   auto shared_estimate = [&](size_t smem, double L, double I) {
     const int per_sm = std::max(1, std::min(4, (int)(227 * 1024 / (smem + 1024))));
     return run_estimate(c, 148 * per_sm, c->steps_sorted.size() > 148 && per_sm > 1 ? 1.2 * L : L, I, 0.0, 6000.0);
@@ -973,7 +970,12 @@ wpsgd_status launch_dense(wpsgd_ctx* c, const ChainParams& p) {
                            : through(x, {{32, 730}, {64, 1020}, {128, 1345}, {256, 2560}, {512, 4250}});
       offer(true, 4, shared_estimate(BlockSmem(bstages, (size_t)d * sizeof(XT) + (F32 ? 0 : 16), bthreads / 32 - 2).total, L, I));
     }
-    offer(mma_ok, 8, mma_t);
+    // Rows of 2048 columns and more: the tensor-core kernel keeps the runs of up to about 16 blocks, whatever the start-up in the lagged
+    // form's estimate (4 to 74 chains of 2048, 8 to 64 steps: 12 to 20 us there, 10 to 16; narrower rows 14 against 25 us after 128 steps).
+    if (mma_ok && (best < 0.0 || mma_t < best + (variant == 10 && chunks >= 256 ? 7500.0 : 0.0))) {
+      best = mma_t;
+      variant = 8;
+    }
     // rows wider than the blocked kernels take, many of them: the direct kernel keeps one chain per SM
     if (lag_t >= 0.0) offer(aligned && chunks > 512 && chunks <= 512 * 4, 2, run_estimate(c, 148, 7000.0 + 5.4 * x, 0.0, 0.0, 6000.0));
     if (best < 0.0) variant = !aligned || chunks > 512 * 4 ? 1 : (chunks <= 64 ? 3 : 2);

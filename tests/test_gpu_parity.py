@@ -614,6 +614,13 @@ def test_contexts_of_two_threads_launch_one_kernel_with_different_shared_memory(
     assert not failed, (len(failed), failed[:3])
 
 
+@pytest.mark.parametrize("k,d,steps", [(4, 64, 128), (148, 128, 128), (37, 256, 256), (4, 1000, 128)])
+def test_short_runs_of_few_bf16_chains_take_the_lagged_kernel(P, k, d, steps):
+    # 14 to 25 us there, 25 to 70 % more in the kernels that share the shape (and other bits: their sums are in another order)
+    wl = wi.config3(k=k, d=d, m=16, n_lo=steps, n_hi=steps)
+    np.testing.assert_array_equal(gpu_solve(P, wl)[0], gpu_solve(P, wl, {"dense_variant": 10})[0])
+
+
 @pytest.mark.parametrize("stages", [0, 3, 4, 5])
 @pytest.mark.parametrize("n_steps", [(1, 7, 8), (9, 15, 16), (17, 0, 64), (333, 250, 3)])
 def test_lagged_kernel_block_boundaries_and_ring_depths(P, n_steps, stages):
