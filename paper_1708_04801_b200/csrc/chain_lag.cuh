@@ -70,13 +70,19 @@ constexpr int LAG_B = 8;
 constexpr int LAG_MAX_STAGES = 16;
 constexpr int LAG_MAX_RAW_STAGES = 8;
 constexpr int LAG_QBUF = 4;
-constexpr int LAG_MAX_CLUSTER = 8;
 constexpr int LAG_SUMS = 128;        // [8][8] G, then [8][8] C (a row per sample of the block)
-constexpr int LAG_MAX_MODEL_WARPS = 8;
+constexpr int LAG_MAX_MODEL_WARPS = 8;           // (vectors of 8 bytes: at most half as many)
+constexpr int LAG_MAX_MODEL_WARPS_REALIGNED = 4;
 constexpr int LAG_GRAM_WARPS = 4;
-// Shares of q of a sample: one per model thread (or pair of them), padded. (Realigned rows in 16-byte vectors have at most four model
-// warps, and their rings need the room.)
-__host__ __device__ constexpr int lag_q_row(int vb, bool realign) { return vb == 16 && realign ? 68 : 132; }
+// Shares of q that a model warp leaves for a sample: one per thread that owns a vector of 8 bytes, half as many for one of 16, a
+// quarter for two. (Wide slices need the room for their rings: with half as many for two as well, 413 to 420 chunks and one CTA had
+// three stages instead of four.)
+__host__ __device__ constexpr int lag_q_shares(int vb, int nc) { return vb == 8 ? 32 : (nc == 1 ? 16 : 8); }
+// Entries of a row of shares (64 or 128, absent ones zero), padded
+__host__ __device__ constexpr int lag_q_row(int vb, int nc, bool realign) { return vb == 16 && (nc == 2 || realign) ? 68 : 132; }
+static_assert(LAG_MAX_MODEL_WARPS / 2 * lag_q_shares(8, 1) <= 128 && LAG_MAX_MODEL_WARPS * lag_q_shares(16, 1) <= 128 &&
+                  LAG_MAX_MODEL_WARPS_REALIGNED * lag_q_shares(16, 1) <= 64 && LAG_MAX_MODEL_WARPS * lag_q_shares(16, 2) <= 64,
+              "a row holds the shares of all model warps");
 constexpr int LAG_REALIGN_WARPS = 4;
 constexpr int LAG_MAX_THREADS = 512;
 constexpr int LAG_GROUP = 4;         // blocks whose constants are formed together
@@ -463,7 +469,7 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
   constexpr int B = LAG_B;
   constexpr int V = 16 / (int)sizeof(XT);
   constexpr int VW = VB / (int)sizeof(XT);
-  constexpr int QROW = lag_q_row(VB, REALIGN);
+  constexpr int QROW = lag_q_row(VB, NC, REALIGN);
   extern __shared__ __align__(16) unsigned char smem[];
   const BlockParams& bp = lp.b;
   const ChainParams& p = bp.c;
@@ -549,7 +555,7 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
   const int first_part = 1 + NM;
   const int pl_copy = first_part + (MULTI ? 1 : 0), pl_const = pl_copy + lp.copy_warps, pl_feed = pl_const + 1, pl_gram = pl_feed + 1,
             pl_realign = pl_gram + NT * NW;
-  const int n16 = VB == 16 ? NM : 2 * NM;  // groups of 16 shares of q
+  const int n16 = (NM * lag_q_shares(VB, NC) + 15) / 16;  // groups of 16 shares of q
 
   if (place == 0) {
     // =========================== recurrence ==============================================================
@@ -583,7 +589,8 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
 #pragma unroll
       for (int e = 0; e < VW / 2; ++e) w[i][e] = make_float2(w1[2 * e], w1[2 * e + 1]);
     }
-    // this thread's shares of q_blk (16-byte vectors: added up with those of the lane 16 away, half of the samples each)
+    // this thread's shares of q_blk (16-byte vectors: added up with those of the lane 16 away, half of the samples each; two of
+    // them: then with those of the lane 8 away, a quarter each)
     auto put_q = [&](float (&v)[B], int blk) __attribute__((always_inline)) {
       float* qp = qpart + (blk & 1) * (B * QROW);
       if constexpr (VB == 16) {
@@ -593,9 +600,19 @@ __global__ void __launch_bounds__(LAG_MAX_THREADS, 1) chain_lag_kernel(const Lag
           const float send = hi ? v[i] : v[i + 4], keep = hi ? v[i + 4] : v[i];
           v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
         }
-        qp += (lane >> 4) * (4 * QROW) + mw * 16 + (lane & 15);
+        if constexpr (NC == 2) {
+          const bool hi8 = (lane & 8) != 0;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) qp[i * QROW] = v[i];
+          for (int i = 0; i < 2; ++i) {
+            const float send = hi8 ? v[i] : v[i + 2], keep = hi8 ? v[i + 2] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+          }
+          qp += (lane >> 3) * (2 * QROW) + mw * 8 + (lane & 7);
+        } else {
+          qp += (lane >> 4) * (4 * QROW) + mw * 16 + (lane & 15);
+        }
+#pragma unroll
+        for (int i = 0; i < (NC == 2 ? 2 : 4); ++i) qp[i * QROW] = v[i];
       } else {
         qp += mt;
 #pragma unroll

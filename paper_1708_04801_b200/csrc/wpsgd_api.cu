@@ -647,9 +647,9 @@ bool lag_kernel_fits(const wpsgd_ctx* c, bool aligned, int C, LagShape* out) {
   // A model thread owns one vector of 8 bytes in narrow slices (the rows of two blocks then stay in registers), else one or two of
   // 16: 64 fp32 chunks 1143 cycles per block with 16-byte vectors, 1236 with 8-byte ones (twice as many warps); 63 bf16 chunks
   // 1106 and 1054.
-  if (cpc > (aligned ? 512 : 256)) return false;
+  if (cpc > 2 * 32 * (aligned ? LAG_MAX_MODEL_WARPS : LAG_MAX_MODEL_WARPS_REALIGNED)) return false;
   sh.vb = cpc <= (sizeof(XT) == 4 ? 32 : 64) ? 8 : 16;
-  sh.nc = cpc <= 32 * (aligned ? (C > 1 ? 6 : 8) : 4) ? 1 : 2;
+  sh.nc = cpc <= 32 * (aligned ? (C > 1 ? 6 : LAG_MAX_MODEL_WARPS) : LAG_MAX_MODEL_WARPS_REALIGNED) ? 1 : 2;
   const int per_warp = 32 * sh.vb * sh.nc;
   sh.model_warps = (int)((cpc * 16 + per_warp - 1) / per_warp);
   // As deep a ring as there is room for. Realigning warps: a block each and both rings in multiples of four up to 64 chunks (fp32,
@@ -661,7 +661,7 @@ bool lag_kernel_fits(const wpsgd_ctx* c, bool aligned, int C, LagShape* out) {
   int others = 3 + (C > 1 ? 1 : 0) + sh.model_warps + sh.realign_warps;
   const int gram = (others + LAG_GRAM_WARPS + 1) * 32 > LAG_MAX_THREADS ? LAG_GRAM_WARPS - 1 : LAG_GRAM_WARPS;
   others += gram;
-  const int q_row = lag_q_row(sh.vb, !aligned);
+  const int q_row = lag_q_row(sh.vb, sh.nc, !aligned);
   int want = c->opt_stages > 0 ? std::max(3, c->opt_stages) : LAG_MAX_STAGES;
   for (; want >= 3; --want) {
     if (!aligned && sh.realign_rows == 1 && want % LAG_REALIGN_WARPS != 0) continue;

@@ -614,6 +614,17 @@ def test_contexts_of_two_threads_launch_one_kernel_with_different_shared_memory(
     assert not failed, (len(failed), failed[:3])
 
 
+@pytest.mark.parametrize("k,chunks,cluster", [(74, 392, 2), (4, 416, 1), (4, 372, 4)])
+def test_slices_that_fill_shared_memory_keep_a_ring_of_four_stages(P, k, chunks, cluster):
+    # with a ring of three the lagged kernel is not offered (unless its cluster size is asked for): 74 chains took a direct kernel
+    # and 1470 us instead of 213. What is asked for is what runs by itself.
+    wl = wi.config3(k=k, d=8 * chunks * cluster, m=16, n_lo=800 if k == 74 else 40, n_hi=800 if k == 74 else 40)
+    if cluster != 2:  # few chains would take more CTAs
+        assert_parity(P, wl, {"dense_variant": 10, "cluster": cluster, "stages": 4})
+        return
+    np.testing.assert_array_equal(gpu_solve(P, wl)[0], gpu_solve(P, wl, {"dense_variant": 10, "cluster": cluster})[0])
+
+
 @pytest.mark.parametrize("k,d,steps", [(4, 64, 128), (148, 128, 128), (37, 256, 256), (4, 1000, 128)])
 def test_short_runs_of_few_bf16_chains_take_the_lagged_kernel(P, k, d, steps):
     # 14 to 25 us there, 25 to 70 % more in the kernels that share the shape (and other bits: their sums are in another order)
