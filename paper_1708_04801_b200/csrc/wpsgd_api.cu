@@ -672,10 +672,17 @@ bool lag_kernel_fits(const wpsgd_ctx* c, bool aligned, int C, LagShape* out) {
   if (want < 3 || (want < 4 && C < 8 && c->opt_stages == 0 && c->opt_cluster == 0)) return false;
   // Gram teams: four of one warp, two of two or one of all, as the ring feeds them (a team holds two stages while it works). With more
   // than two teams the ring is a multiple of their number, so that a team has seen every earlier block of the stages it
-  // waits for (else a barrier's parity could stand for an older phase).
-  if (want >= 8) want -= want % 4;
-  sh.teams = want >= 8 ? 4 : (want >= 5 ? 2 : 1);
-  if (gram == 3) sh.teams = want % 3 == 0 ? 3 : 1;
+  // waits for (else a barrier's parity could stand for an older phase). Three warps, where no more fit: three teams from 6 stages
+  // on, which costs up to two of the stages; a ring of 3 does not feed them (cycles per block, squared loss, three teams and one: fp32,
+  // 2 CTAs of 449 / 512 chunks 10040 / 11230 and 7590 / 8330; 2 x 232 chunks of unaligned rows 7110 and 5840; 8 CTAs of 97
+  // chunks, one team on 8 stages and three on 6: 3000 and 2700).
+  if (gram < LAG_GRAM_WARPS) {
+    if (want >= 6) want = sh.realign_rows == 1 && !aligned ? (want >= 12 ? 12 : want) : want - want % 3;
+    sh.teams = want >= 6 && want % 3 == 0 ? 3 : 1;
+  } else {
+    if (want >= 8) want -= want % 4;
+    sh.teams = want >= 8 ? 4 : (want >= 5 ? 2 : 1);
+  }
   sh.gram_warps = gram / sh.teams;
   sh.stages = want;
   sh.smem = LagSmem(want, (size_t)cpc * 16, C, gram, sh.raw_stages, q_row).total;

@@ -509,7 +509,7 @@ def test_lagged_kernel_shapes(P, d, bf16, pad, cluster, loss, sched):
 @pytest.mark.parametrize("d,bf16,cluster", [
     (1024, False, 8), (1056, False, 8), (1284, False, 8), (1320, False, 8),  # 32 / 33 / 41 / 42 chunks of a CTA: 8- and 16-byte vectors, Gram warps on all schedulers
     (1024, True, 2), (1040, True, 2),                                        # 64 / 65 bf16 chunks
-    (1536, False, 2), (1544, False, 2), (3072, False, 2), (2000, False, 1),  # 192 / 193 / 384 chunks: one and two vectors per thread, three Gram warps
+    (1536, False, 2), (1544, False, 2), (3072, False, 2), (2000, False, 1),  # 192 / 193 / 384 chunks: one and two vectors per thread
     (1023, False, 4), (1025, False, 4), (1021, False, 2), (2049, True, 1),   # unaligned: 64 / 65 chunks (a block per warp, all warps per block), 128, 257
     (2047, False, 4), (3071, False, 4), (5999, False, 8),
 ])
@@ -527,6 +527,24 @@ def test_lagged_kernel_roles_at_their_limits(P, d, bf16, cluster, loss, sched):
             gpu_solve(P, wl, {"dense_variant": 10, "cluster": cluster})
         return
     assert_parity(P, wl, {"dense_variant": 10, "cluster": cluster})
+
+
+@pytest.mark.parametrize("d,bf16,cluster,stages", [
+    (3592, False, 2, 0), (4096, False, 2, 0), (8192, True, 2, 0),  # 449 / 512 chunks of a CTA, eight model warps: one team, a ring of 3
+    (2045, True, 2, 3), (2045, True, 2, 6), (1567, True, 2, 0),    # unaligned, 128 / 98 chunks: one team on 3 stages, three on 6 and 12
+    (1023, True, 2, 0), (799, True, 2, 0), (3711, True, 8, 0),     # a block per realigning warp, 64 / 50 / 58 chunks: rings of 12, 12 and 8
+    (4093, True, 2, 0), (2045, False, 2, 0),                       # 256 chunks, a ring of 3
+])
+@pytest.mark.parametrize("loss,sched", [(LOGISTIC, 0), (SQUARED, 1)])
+def test_lagged_kernel_teams_of_three_gram_warps(P, d, bf16, cluster, stages, loss, sched):
+    wl = wi.config2(k=3, d=d, m=48, base_steps=330)
+    wl.n_steps = np.array([330, 129, 5], dtype=np.int64)
+    wl.loss, wl.sched = loss, sched
+    if loss == SQUARED:
+        wl.y = (wl.y * 0.3).contiguous()
+    if bf16:
+        wl.X = wl.X.to(torch.bfloat16)
+    assert_parity(P, wl, {"dense_variant": 10, "cluster": cluster, "stages": stages})
 
 
 @pytest.mark.parametrize("k", [3, 240])  # tables as an argument of the stream kernel, and copied
