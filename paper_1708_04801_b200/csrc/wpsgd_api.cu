@@ -649,7 +649,10 @@ bool lag_kernel_fits(const wpsgd_ctx* c, bool aligned, int C, LagShape* out) {
   // 1106 and 1054.
   if (cpc > 2 * 32 * (aligned ? LAG_MAX_MODEL_WARPS : LAG_MAX_MODEL_WARPS_REALIGNED)) return false;
   sh.vb = cpc <= (sizeof(XT) == 4 ? 32 : 64) ? 8 : 16;
-  sh.nc = cpc <= 32 * (aligned ? (C > 1 ? 6 : LAG_MAX_MODEL_WARPS) : LAG_MAX_MODEL_WARPS_REALIGNED) ? 1 : 2;
+  // Two vectors where one would take so many warps that a Gram or copy warp had to go (fp32, unaligned rows, 8 CTAs of 65 / 97 / 128
+  // chunks: 2090, 2700, 3090 cycles per block with one, 2030, 2550, 3000 with two).
+  const int most = aligned ? (C > 1 ? 6 : LAG_MAX_MODEL_WARPS) : (sizeof(XT) == 4 && C > 1 ? 2 : LAG_MAX_MODEL_WARPS_REALIGNED);
+  sh.nc = cpc <= 32 * most ? 1 : 2;
   const int per_warp = 32 * sh.vb * sh.nc;
   sh.model_warps = (int)((cpc * 16 + per_warp - 1) / per_warp);
   // As deep a ring as there is room for. Realigning warps: a block each and both rings in multiples of four up to 64 chunks (fp32,

@@ -511,7 +511,7 @@ def test_lagged_kernel_shapes(P, d, bf16, pad, cluster, loss, sched):
     (1024, True, 2), (1040, True, 2),                                        # 64 / 65 bf16 chunks
     (1536, False, 2), (1544, False, 2), (3072, False, 2), (2000, False, 1),  # 192 / 193 / 384 chunks: one and two vectors per thread
     (1023, False, 4), (1025, False, 4), (1021, False, 2), (2049, True, 1),   # unaligned: 64 / 65 chunks (a block per warp, all warps per block), 128, 257
-    (2047, False, 4), (3071, False, 4), (5999, False, 8),
+    (2047, False, 4), (3071, False, 4), (5999, False, 8), (511, False, 2), (519, False, 2),  # 64 / 65 chunks: one and two vectors per thread
 ])
 @pytest.mark.parametrize("loss,sched", [(LOGISTIC, 0), (SQUARED, 1)])
 def test_lagged_kernel_roles_at_their_limits(P, d, bf16, cluster, loss, sched):
