@@ -722,12 +722,16 @@ wpsgd_status launch_lag(wpsgd_ctx* c, const ChainParams& p, const LagShape& sh) 
     int first[LAG_MAX_THREADS / 32], rest[LAG_MAX_THREADS / 32], nf = 0, nr = 0;
     first[nf++] = 0;
     if (sums) first[nf++] = 1 + sh.model_warps;
-    first[nf++] = constants;
-    for (int i = 0; i < sh.model_warps; ++i) rest[nr++] = 1 + i;
-    // (wide fp32 slices: the Gram warps bound the block, one goes to every scheduler; 64 chunks 1143 cycles per block, 1285 without)
-    const int g0 = sizeof(XT) == 4 && sh.cpc > 40 ? 1 : 0;
+    // Wide fp32 slices: the Gram warps bound the block, one goes to every scheduler; 64 chunks 1143 cycles per block, 1285 without.
+    // Wide aligned bf16 slices: the model warps do, and one of each goes there (the constants elsewhere); one CTA, 96 / 128 / 256 chunks
+    // 1320, 1550, 2410 without, 1240, 1330, 2210 with them; 4 CTAs of 128 / 192 chunks 1510, 1990 and 1330, 1840
+    // (up to 96 chunks clusters are 1 to 3 % slower with them).
+    const int m0 = sizeof(XT) == 2 && sh.vb == 16 && !sh.raw_stages && (sh.C == 1 || sh.cpc > 96) ? 1 : 0, g0 = m0 || (sizeof(XT) == 4 && sh.cpc > 40) ? 1 : 0;
+    first[nf++] = m0 ? sh.model_warps : constants;
     if (g0) first[nf++] = gram;
+    for (int i = 0; i < sh.model_warps - m0; ++i) rest[nr++] = 1 + i;
     for (int i = g0; i < sh.teams * sh.gram_warps; ++i) rest[nr++] = gram + i;
+    if (m0) rest[nr++] = constants;
     rest[nr++] = constants + 1;  // feeder
     for (int i = 0; i < sh.copy_warps; ++i) rest[nr++] = 1 + sh.model_warps + sums + i;
     for (int i = gram + sh.teams * sh.gram_warps; i < sh.warps; ++i) rest[nr++] = i;  // realign
