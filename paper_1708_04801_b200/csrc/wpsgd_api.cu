@@ -650,8 +650,9 @@ bool lag_kernel_fits(const wpsgd_ctx* c, bool aligned, int C, LagShape* out) {
   if (cpc > 2 * 32 * (aligned ? LAG_MAX_MODEL_WARPS : LAG_MAX_MODEL_WARPS_REALIGNED)) return false;
   sh.vb = cpc <= (sizeof(XT) == 4 ? 32 : 64) ? 8 : 16;
   // Two vectors where one would take so many warps that a Gram or copy warp had to go (fp32, unaligned rows, 8 CTAs of 65 / 97 / 128
-  // chunks: 2090, 2700, 3090 cycles per block with one, 2030, 2550, 3000 with two).
-  const int most = aligned ? (C > 1 ? 6 : LAG_MAX_MODEL_WARPS) : (sizeof(XT) == 4 && C > 1 ? 2 : LAG_MAX_MODEL_WARPS_REALIGNED);
+  // chunks: 2090, 2700, 3090 cycles per block with one, 2030, 2550, 3000 with two; aligned, 4 CTAs of 204: 3230 and 3080, bf16 2010 and
+  // 2700: those take one vector up to seven warps).
+  const int most = aligned ? (C > 1 ? (sizeof(XT) == 4 ? 6 : 7) : LAG_MAX_MODEL_WARPS) : (sizeof(XT) == 4 && C > 1 ? 2 : LAG_MAX_MODEL_WARPS_REALIGNED);
   sh.nc = cpc <= 32 * most ? 1 : 2;
   const int per_warp = 32 * sh.vb * sh.nc;
   sh.model_warps = (int)((cpc * 16 + per_warp - 1) / per_warp);

@@ -508,7 +508,7 @@ def test_lagged_kernel_shapes(P, d, bf16, pad, cluster, loss, sched):
 
 @pytest.mark.parametrize("d,bf16,cluster", [
     (1024, False, 8), (1056, False, 8), (1284, False, 8), (1320, False, 8),  # 32 / 33 / 41 / 42 chunks of a CTA: 8- and 16-byte vectors, Gram warps on all schedulers
-    (1024, True, 2), (1040, True, 2),                                        # 64 / 65 bf16 chunks
+    (1024, True, 2), (1040, True, 2), (1024, True, 1), (3584, True, 2), (3600, True, 2),  # bf16: 64 / 65 / 128 / 224 / 225 chunks
     (1536, False, 2), (1544, False, 2), (3072, False, 2), (2000, False, 1),  # 192 / 193 / 384 chunks: one and two vectors per thread
     (1023, False, 4), (1025, False, 4), (1021, False, 2), (2049, True, 1),   # unaligned: 64 / 65 chunks (a block per warp, all warps per block), 128, 257
     (2047, False, 4), (3071, False, 4), (5999, False, 8), (511, False, 2), (519, False, 2),  # 64 / 65 chunks: one and two vectors per thread
