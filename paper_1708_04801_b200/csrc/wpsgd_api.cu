@@ -580,8 +580,13 @@ wpsgd_status launch_mma(wpsgd_ctx* c, const ChainParams& p, const ClusterShape& 
   };
   if (b16) {
     const bool full = sh.cpc % 32 == 0 && (long long)sh.cpc * sh.C * 8 == c->d;
+    // Clusters of up to two CTAs have a form of their own where every warp is full (cycles per 16 samples, squared / logistic: 4096 columns
+    // 3640 / 4660 in the form for up to eight, 3530 / 4570 in it; 2560: 3370 / 4296, 3289 / 4205; with guards the other way round, 3000
+    // columns 3600 / 4500 and 3730 / 4620, 3328: 3670 / 4606 and 3780 / 4680).
     auto pick = [&](auto loss, auto is_full) -> wpsgd_status {
-      return sh.C <= 2 ? go(chain_mma16_kernel<loss.value, is_full.value, 2>) : go(chain_mma16_kernel<loss.value, is_full.value, 8>);
+      if constexpr (is_full.value)
+        if (sh.C <= 2) return go(chain_mma16_kernel<loss.value, true, 2>);
+      return go(chain_mma16_kernel<loss.value, is_full.value, 8>);
     };
     auto with_loss = [&](auto is_full) -> wpsgd_status {
       switch (c->loss) {
