@@ -910,11 +910,11 @@ double lag_estimate(const wpsgd_ctx* c, const LagShape& sh) {
   const double x = (double)sh.cpc;
   double L;
   if (F32) L = sh.C == 1 ? through(x, {{8, 725}, {16, 740}, {32, 815}, {48, 920}, {64, 1090}, {96, 1430}, {128, 1875}, {256, 3490}, {512, 6850}})
-                         : through(x, {{8, 790}, {16, 800}, {32, 840}, {48, 1000}, {64, 1130}, {96, 1500}, {128, 1940}, {256, 3640}, {384, 5560}, {512, 11200}});
-  else L = sh.C == 1 ? through(x, {{16, 785}, {32, 890}, {64, 1025}, {96, 1320}, {128, 1560}, {192, 1890}, {256, 2410}, {384, 3730}, {512, 5450}})
-                     : through(x, {{16, 885}, {48, 935}, {64, 1035}, {96, 1265}, {128, 1510}, {192, 1970}, {256, 2790}, {384, 4300}, {512, 6130}});
+                         : through(x, {{8, 790}, {16, 800}, {32, 840}, {48, 1000}, {64, 1130}, {96, 1500}, {128, 1940}, {256, 3560}, {384, 5560}, {448, 6290}, {456, 7680}, {512, 8330}});
+  else L = sh.C == 1 ? through(x, {{16, 785}, {32, 885}, {64, 1015}, {96, 1245}, {128, 1330}, {192, 1740}, {256, 2205}, {336, 3040}, {420, 3320}, {448, 4550}, {512, 5470}})
+                     : through(x, {{16, 865}, {48, 925}, {64, 1015}, {96, 1255}, {128, 1340}, {192, 1835}, {224, 2060}, {256, 2390}, {372, 3340}, {400, 4400}, {512, 4850}});
   if (sh.C == 8) L += 25.0;
-  if (sh.realign_warps) L = std::max(L, through(x, {{8, 850}, {16, 920}, {32, 1180}, {48, 1500}, {64, 1800}, {96, 2450}, {128, 3050}, {256, 9100}}));
+  if (sh.realign_warps) L = std::max(L, through(x, {{8, 800}, {16, 850}, {32, 1000}, {48, 1350}, {64, 1550}, {72, 2000}, {96, 2500}, {128, 2950}, {224, 4850}, {232, 6000}, {256, 6700}}));
   return run_estimate(c, cluster_slots(c->device, sh.C, c->steps_sorted.size()), L, 0.0, 5000.0 + 40.0 * x, 10000.0);
 }
 
