@@ -99,7 +99,8 @@ wpsgd_status wpsgd_destroy(wpsgd_ctx* ctx);
  *   "threads"         threads per node of variants 2 and 4, warps x 32 per CTA of variant 5; 0 (default): chosen from d.
  *   "prefetch"        rows in flight per chain of variants 2, 3 and of sparse variant 1; 0 (default): chosen.
  *   "stages"          blocks of rows in the shared-memory ring of the blocked kernels; 0 (default): as many as fit
- *                     (up to 4; variant 10: up to 16), else 2..8 (variant 10 takes at least 3).
+ *                     (up to 4; variant 10: up to 16), else 2..8 (variant 10 takes at least 3, and 4 or 8 in place of 5 to 7
+ *                     where rows do not start on 16 bytes and a CTA holds at most 64 chunks of one).
  *   "host_pipeline"   wpsgd_solve_host: 1 (default) copies the shards in up to four groups of nodes, longest chains
  *                     first, on a stream of the context and starts the chains of a group when its rows have arrived;
  *                     0 copies everything first.

@@ -37,9 +37,9 @@
 // the sums never turns it.
 //
 // What bounds it, and what it measured (cycles per 8 steps of the longest chain, B200 at 1965 MHz): 40 Zipf-distributed
-// nonzeros per row, d = 2^20, hinge, 64 chains: 2770 (11.55 ms for 65536 steps; 2685 before launches overlapped; one step after the other, each with a gather, a sum over 32 lanes and a
-// scatter: 3840); 5 to 10 nonzeros, d = 100000, logistic, 10 chains: 1615 (3700). With short rows the chain warp's string is
-// the longer side: margins 160, steps 500, updates 300, boundary 130 of the 1500. With long rows the chain (2400) and the
+// nonzeros per row, d = 2^20, hinge, 64 chains: 2740 (11.43 ms for 65536 steps; 2685 before launches overlapped; one step after the other, each with a gather, a sum over 32 lanes and a
+// scatter: 3840); 5 to 10 nonzeros, d = 100000, logistic, 10 chains: 1255 (3700). With short rows the chain warp's string is
+// the longer side: margins 160, steps 500, updates 300, boundary 130 of 1500 before the short form. With long rows the chain (2400) and the
 // helpers (insertion 700, products 1100, copies 400 per group) take about as long; the short form took 1615 to 1230 and, at 8
 // Zipf-distributed nonzeros, 1480 to 1270. Tried and taken back: margins from
 // the model one group back with a table per group and the model in L2 (5900 and 3300: everything that touches single

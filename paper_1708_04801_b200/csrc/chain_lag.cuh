@@ -46,15 +46,17 @@
 // peers S + 6, q sums four; the shares of q inside a CTA two (the shares of block g + 2 follow gamma_g, which took q_g).
 //
 // What bounds a block, and what it measured (B200, 1965 MHz; cycles per block of 8 samples, 4 chains that have their SMs to
-// themselves, squared and logistic loss alike): fp32, one CTA, 16 / 32 / 64 chunks of a row 740 / 815 / 1090; eight CTAs, 32 / 64 / 128
-// chunks each 845 / 1160 / 1980, 256 chunks 3720; bf16, 32 / 64 / 128 chunks 890 / 1030 / 1510; rows that do not start on 16 bytes, 32 / 64 / 128
-// chunks about 1050 / 1500 / 3000. With few chunks it is the string gamma -> update -> shares -> sum (430) -> cluster (280) -> steps
+// themselves, squared and logistic loss alike): fp32, one CTA, 16 / 32 / 64 chunks of a row 735 / 805 / 1085; eight CTAs, 32 / 64 / 128
+// chunks each 845 / 1160 / 1980, 256 chunks 3615; bf16, 32 / 64 / 128 / 256 chunks 885 / 1015 / 1330 / 2205; rows that do not start on 16 bytes,
+// 32 / 64 / 128 chunks about 1000 / 1480 / 2920. With few chunks it is the string gamma -> update -> shares -> sum (430) -> cluster (280) -> steps
 // over two blocks, and the instruction supply; from about 64 fp32 chunks per CTA on the Gram block (shared-memory reads, 8 wavefronts
 // per chunk). Before the sums of q had a warp of their own and the code was cut: 16 / 32 (eight CTAs) / 64 bf16 chunks 815 / 1235 / 1350.
 // Tried and taken back: rows by 16-byte copies of the threads instead of bulk copies (1900 against 1060 at d = 64); fp32 Gram
 // products split into three units of 32 with a lane per chunk (1164 against 908 at d = 64), or as 4 x 8 tiles with different
 // chunks in all lanes of a load (128 chunks: 2099 against 2022); partial sums to peers by plain stores that the reader polls
-// (330 cycles one way, 260 with st.async and a barrier); deeper rings than 8 stages make no difference once rows arrive in time.
+// (330 cycles one way, 260 with st.async and a barrier). Rings
+// of more than 8 stages are taken where there is room and gain at most 1 % (12 chains of 999 columns, rows from DRAM: 1083 -> 1074);
+// 5 stages cost 8 to 80 %.
 //
 // Leaving. Every wait on an mbarrier is bounded. One that runs out sets the status word and a flag in every CTA of the
 // cluster; from then on a warp skips these waits and runs to the end of its loop, so that named barriers are still met by

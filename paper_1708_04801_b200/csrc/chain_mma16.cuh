@@ -72,14 +72,6 @@ __device__ __forceinline__ void st_async_f32x4(uint32_t addr, float4 v, uint32_t
                : "memory");
 }
 
-// the same where `yes`: a predicate, not a branch
-__device__ __forceinline__ void st_async_f32x4_if(uint32_t addr, float4 v, uint32_t mbar, bool yes) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %6, 0;\n\t@p st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];\n\t}" ::"r"(addr),
-      "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(mbar), "r"((int)yes)
-      : "memory");
-}
-
 __device__ __forceinline__ void ldmatrix_x2(uint32_t (&r)[2], const void* smem_ptr) {
   const uint32_t a = (uint32_t)__cvta_generic_to_shared(smem_ptr);
   asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(a) : "memory");
